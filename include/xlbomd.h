@@ -118,7 +118,7 @@ typedef struct {
                               the forces do not contain it; the expansion always takes three,
                               the chemical-potential chain follows mu_prec.  Ignored by FP64. */
   int graphs;              /* 1: split precisions with at most 2048 padded orbitals capture each
-                              chemical-potential pass (per Newton-Schulz plan) and each probe's
+                              chemical-potential pass (per plan of its inverses) and each probe's
                               response in CUDA graphs and replay them (the second run of a plan
                               is captured; results are bitwise those of direct launches).  Needs
                               a caller stream (xlbomd_init's cuda_stream, not the legacy default
@@ -161,7 +161,7 @@ typedef enum {
   XLBOMD_D = 10,       /* get: density matrix (N x N) */
   XLBOMD_H = 11,       /* get: H[n] (N x N) */
   XLBOMD_GAMMA = 12,   /* get: Coulomb matrix gamma (natoms x natoms) */
-  XLBOMD_STATS = 13,   /* get: [mu passes, NS products, probes used, GEMMs, steps] (5) */
+  XLBOMD_STATS = 13,   /* get: [mu passes, inverse corrections, probes used, GEMMs, steps] (5) */
   XLBOMD_PROBES = 14,  /* get: probes V then responses W (2 x rank_m x natoms) */
   XLBOMD_KMAT = 15     /* get: held kernel K (natoms x natoms, row-major; kernel_mode 1, 2) */
 } xlbomd_quantity;
@@ -272,7 +272,7 @@ xlbomd_status xlbomd_energy(xlbomd_ctx* ctx, int sys);
  * one stream synchronisation per chemical-potential pass and per probe index
  * for the whole group; a padded size held by one system takes the one-system
  * step.  Every system follows exactly its one-system trajectory (same mu
- * search, Newton-Schulz plan and probes; bitwise the same results).  Errors:
+ * search, plan of the inverses and probes; bitwise the same results).  Errors:
  * ERR_DIVERGED (max |q - n| above diverge_tol for any system), and those of
  * xlbomd_density and xlbomd_kernel_update. */
 xlbomd_status xlbomd_step(xlbomd_ctx* ctx, int nsteps);

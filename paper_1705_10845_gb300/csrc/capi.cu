@@ -27,6 +27,7 @@ namespace {
 
 constexpr double kKB = 8.617333262e-5;
 constexpr double kAcc = 9.648533e-3;   // 1 eV/(amu A) in A/fs^2
+constexpr int kPassPar = 1 + 4 * 40;   // device parameters of a captured mu pass: mu, then g_0..g_3 per level
 
 struct Sys {
   int nat = 0, N = 0, np = 0, natp = 0, ng = 0, kp = 0;
@@ -57,8 +58,8 @@ struct Sys {
   double stats[5] = {0, 0, 0, 0, 0};
   double eh[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   std::vector<double> G4h;
-  // captured work (params.graphs): one graph per Newton-Schulz plan of a chemical-potential pass,
-  // one per probe slot of the kernel update; dpar holds mu and the start scales c_k
+  // captured work (params.graphs): one graph per plan of a chemical-potential pass,
+  // one per probe slot of the kernel update; dpar holds mu and the start coefficients g_j
   struct Captured {
     std::vector<int> key;
     int seen = 0;                      // eager runs before the capture
@@ -83,6 +84,7 @@ struct xlbomd_ctx {
   int status = XLBOMD_OK;
   std::string msg;
   xl::Engine* eng = nullptr;
+  xl::PlanCache plans;
 };
 
 namespace {
@@ -190,7 +192,7 @@ bool use_graphs(const xlbomd_ctx* ctx, const Sys& S) {
 // makes every lazy set-up happen outside a capture), captured into a CUDA graph the second
 // time, replayed from the graph afterwards.  fn must enqueue the same work for the same key;
 // what may differ between runs lives in device memory (for the chemical-potential pass, mu
-// and the Newton-Schulz start scales in S.dpar).
+// and the inverses' start coefficients in S.dpar).
 xlbomd_status run_captured(xlbomd_ctx* ctx, Sys& S, const std::vector<int>& key,
                            const std::function<xlbomd_status()>& fn) {
   cudaStream_t st = ctx->stream;
@@ -263,50 +265,13 @@ xlbomd_status build_H(xlbomd_ctx* ctx, Sys& S) {
   return XLBOMD_OK;
 }
 
-// Newton-Schulz plan per level from the scalar map over t in [0, t_max(k)]:
-// level 0 starts from Y = I - S (error t^4), level k > 0 from c_k Y_{k-1}
-// with c_k minimising max |1 - c b_k / b_{k-1}|, b = 1 + t^2.
-void ns_plan(double t0max, int n, double tol, std::vector<int>& s, std::vector<double>& c) {
-  const int G = 2001;
-  std::vector<double> t(G), prev(G);
-  for (int i = 0; i < G; ++i) t[i] = t0max * i / (G - 1);
-  s.assign(n, 0);
-  c.assign(n, 1.0);
-  for (int k = 0; k < n; ++k) {
-    double e;
-    if (k == 0) {
-      e = 0.0;
-      for (int i = 0; i < G; ++i) e = std::max(e, std::fabs(1.0 - (1.0 + t[i] * t[i]) * (1.0 - t[i] * t[i])));
-    } else {
-      double rmin = 1e300, rmax = -1e300;
-      for (int i = 0; i < G; ++i) {
-        const double rho = (1.0 + t[i] * t[i]) / (1.0 + prev[i] * prev[i]);
-        rmin = std::min(rmin, rho);
-        rmax = std::max(rmax, rho);
-      }
-      c[k] = 2.0 / (rmin + rmax);
-      e = (rmax - rmin) / (rmax + rmin);
-    }
-    int it = 0;
-    double err = e;
-    while (err > tol && it < 10) {
-      err = err * err;
-      ++it;
-    }
-    s[k] = it;
-    prev = t;
-    for (int i = 0; i < G; ++i) t[i] = 2.0 * t[i] / (1.0 + t[i] * t[i]);
-  }
-}
-
 // Safeguarded Newton search for the chemical potential of one system (Tr D(mu) = N_occ): the
 // host side of the mu passes, shared by the one-system and the lockstep paths.
 struct MuSearch {
   double glo = 0, ghi = 0, mu = 0, blo = 0, bhi = 0, dmu = 0, t0max = 0;
   int pass = 0;
   bool done = false;
-  std::vector<int> plan_s;
-  std::vector<double> plan_c;
+  std::vector<LevelPlan> plan;
 
   // start from the Gershgorin interval [glo, ghi] and the system's mu history
   xlbomd_status start(xlbomd_ctx* ctx, const Sys& S, double lo, double hi) {
@@ -331,14 +296,14 @@ struct MuSearch {
     return XLBOMD_OK;
   }
 
-  // spectral bound and Newton-Schulz plan of the next pass
+  // spectral bound and plan of the inverses of the next pass
   xlbomd_status prepare(xlbomd_ctx* ctx, Sys& S) {
     const xlbomd_params& p = ctx->p;
     if (pass >= p.mu_max_iter) return fail(ctx, XLBOMD_ERR_NOT_CONVERGED, "chemical potential did not converge");
     const double sc = beta_of(p) / std::ldexp(1.0, p.n_sq + 1);
     t0max = sc * std::max(std::fabs(ghi - mu), std::fabs(mu - glo));
     if (!(t0max < 1.0)) return fail(ctx, XLBOMD_ERR_SPECTRUM, "|beta (e - mu)| / 2^(n+1) >= 1");
-    ns_plan(t0max, p.n_sq, (p.prec == XLBOMD_FP64) ? 1e-16 : 1e-8, plan_s, plan_c);
+    plan_expansion(ctx->plans, t0max, p.n_sq, (p.prec == XLBOMD_FP64) ? 1e-16 : 1e-8, plan);
     S.mats.t0max = t0max;
     return XLBOMD_OK;
   }
@@ -431,7 +396,7 @@ xlbomd_status density(xlbomd_ctx* ctx, Sys& S, bool with_forces) {
     CKS(ms.prepare(ctx, S));
     const double mu = ms.mu;
     auto mu_pass = [&](const double* dp) -> xlbomd_status {
-      CK(E.foe(st, S.mats, S.H, S.N, mu, sc, ms.plan_s, ms.plan_c, S.stats, dp));
+      CK(E.foe(st, S.mats, S.H, S.N, mu, sc, ms.plan, S.stats, dp));
       // mu chain: T1_0 = +sc I, full last level
       CK(E.chain(st, S.mats, S.dvec_mu, S.N, true, S.dmu_diag, S.stats));
       CK(E.trace_tn(st, S.mats, S.N, S.scal));          // scal[0] = sum_i T_n,ii
@@ -439,12 +404,16 @@ xlbomd_status density(xlbomd_ctx* ctx, Sys& S, bool with_forces) {
       return XLBOMD_OK;
     };
     if (use_graphs(ctx, S)) {
-      if (!S.dpar) CKS(dalloc(ctx, &S.dpar, 64));
+      if (!S.dpar) CKS(dalloc(ctx, &S.dpar, kPassPar));
       ctx->ppar[0] = mu;
-      for (int k = 0; k < n && k < 63; ++k) ctx->ppar[1 + k] = ms.plan_c[k];
-      CK(cudaMemcpyAsync(S.dpar, ctx->ppar, sizeof(double) * 64, cudaMemcpyHostToDevice, st));
       std::vector<int> key{0};
-      key.insert(key.end(), ms.plan_s.begin(), ms.plan_s.end());
+      for (int k = 0; k < n; ++k) {
+        for (int q = 0; q < 4; ++q) ctx->ppar[1 + 4 * k + q] = ms.plan[k].g[q];
+        key.push_back(ms.plan[k].nb);
+        key.push_back(ms.plan[k].inv.n);
+        for (int r = 0; r < ms.plan[k].inv.n; ++r) key.push_back(ms.plan[k].inv.order[r]);
+      }
+      CK(cudaMemcpyAsync(S.dpar, ctx->ppar, sizeof(double) * kPassPar, cudaMemcpyHostToDevice, st));
       CKS(run_captured(ctx, S, key, [&] { return mu_pass(S.dpar); }));
     } else {
       CKS(mu_pass(nullptr));
@@ -490,8 +459,7 @@ xlbomd_status density_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, bool wi
       f.H = S.H;
       f.N = S.N;
       f.mu = ms[i].mu;
-      f.ns = &ms[i].plan_s;
-      f.nc = &ms[i].plan_c;
+      f.plan = &ms[i].plan;
       f.stats = S.stats;
       fj.push_back(f);
       ChainJob c;
@@ -1259,7 +1227,7 @@ xlbomd_status xlbomd_init(const xlbomd_params* params, const xlbomd_system* syst
     return st;
   };
   if (cudaMallocHost((void**)&ctx->pinned, 64 * sizeof(double)) != cudaSuccess ||
-      cudaMallocHost((void**)&ctx->ppar, 64 * sizeof(double)) != cudaSuccess ||
+      cudaMallocHost((void**)&ctx->ppar, kPassPar * sizeof(double)) != cudaSuccess ||
       cudaMallocHost((void**)&ctx->pinned_group, 2 * (size_t)nsys * sizeof(double)) != cudaSuccess)
     return bail(XLBOMD_ERR_OOM);
   if (dalloc(ctx, &ctx->cdev, 8) != XLBOMD_OK) return bail(XLBOMD_ERR_OOM);

@@ -1,12 +1,12 @@
 // Plain-FP64 engine of the recursive Fermi-operator expansion (tanh-doubling
 // form) and of its canonical density-matrix perturbation chains.
 //
-// Products whose result is symmetric (T^2, the Newton-Schulz update
-// (2I - Y B) Y, 2 T Y, Y M for the response) run in symmetric-output mode:
+// Products whose result is symmetric (T^2, those of the inverse, 2 T Y, Y M
+// for the response) run in symmetric-output mode:
 // only upper tiles are computed and mirrored, which halves their cost and
 // keeps them exactly symmetric.  Exact symmetry matters: with the A B^T
 // product form, an antisymmetric rounding component of Y would be doubled by
-// every Newton-Schulz step.
+// every correction.
 #include <cstdio>
 
 #include "precision.h"
@@ -31,26 +31,22 @@ class EngineF64 : public Engine {
   }
 
   cudaError_t foe(cudaStream_t s, MatSet& m, const double* H, int N, double mu, double sc,
-                  const std::vector<int>& ns, const std::vector<double>& nc, double* stats, const double*) override {
+                  const std::vector<LevelPlan>& plan, double* stats, const double*) override {
     const int np = m.np, n = m.n;
     RET(launch_t0_init(s, N, np, H, mu, sc, m.T[0]));
-    for (int k = 0; k < n; ++k) {
+    // S_k and S_{k-1} alternate between S and T1b, which like A1, Mt and G belongs to the chains and
+    // is free here
+    double *S = m.S, *Sprev = m.T1b;
+    for (int k = 0; k < n; ++k, std::swap(S, Sprev)) {
+      const LevelPlan& p = plan[k];
       EpiF64 e1;
-      RET(gemm(s, np, m.T[k], m.T[k], m.S, e1, true, stats));              // S = T^2
-      if (k == 0)
-        RET(launch_ident_minus(s, np, m.S, m.Y[0]));                       // Y = I - S
-      else
-        RET(launch_scale(s, (size_t)np * np, nc[k], m.Y[k - 1], m.Y[k]));  // Y = c_k Y_{k-1}
-      for (int it = 0; it < ns[k]; ++it) {
-        EpiF64 eq;                                                         // Q = 2I - Y - Y S = 2I - Y B
-        eq.alpha = -1.0;
-        eq.E = m.Y[k];
-        eq.lde = np;
-        eq.beta = -1.0;
-        eq.diag = 2.0;
-        RET(gemm(s, np, m.Y[k], m.S, m.Q, eq, false, stats));
-        EpiF64 ey;
-        RET(gemm(s, np, m.Q, m.Y[k], m.Yw, ey, true, stats));              // Y <- Q Y
+      RET(gemm(s, np, m.T[k], m.T[k], S, e1, true, stats));                // S = T^2
+      // Y = I - W0 with W_{k-1} = I - Y_{k-1}
+      const double* Yp = k > 0 ? m.Y[k - 1] : nullptr;
+      RET(launch_combine(s, np, 1.0 - p.g[0] - p.g[1], p.g[1], Yp, -p.g[2], S, -p.g[3], p.nb > 3 ? Sprev : nullptr,
+                         m.Y[k]));
+      for (int r = 0; r < p.inv.n; ++r) {
+        RET(correct(s, np, m.Y[k], S, -1.0, m.Q, m.A1, m.Mt, m.G, m.Yw, p.inv.order[r], stats));
         std::swap(m.Y[k], m.Yw);
         if (stats) stats[1] += 1;
       }
@@ -59,6 +55,44 @@ class EngineF64 : public Engine {
       RET(gemm(s, np, m.T[k], m.Y[k], m.T[k + 1], et, true, stats));       // T_{k+1} = 2 T Y
     }
     return cudaSuccess;
+  }
+
+  // One residual correction of Y ~ (I - sg S)^-1 into Yn: R = I - Y + sg Y S, Yn = Y + (R + .. + R^(order-1)) Y.
+  // Every factor is a function of one matrix, so each product runs in symmetric-output mode.
+  cudaError_t correct(cudaStream_t s, int np, const double* Y, const double* S, double sg, double* R, double* R2,
+                      double* V, double* U, double* Yn, int order, double* stats) {
+    EpiF64 er;
+    er.alpha = sg;
+    er.E = Y;
+    er.lde = np;
+    er.beta = -1.0;
+    er.diag = 1.0;
+    RET(gemm(s, np, Y, S, R, er, true, stats));
+    const double* P = R;
+    if (order >= 3) {
+      EpiF64 e2;
+      if (order == 3) {                                                    // P = R + R^2
+        e2.E = R;
+        e2.lde = np;
+        e2.beta = 1.0;
+      }
+      RET(gemm(s, np, R, R, R2, e2, true, stats));
+      P = R2;
+    }
+    if (order == 5) {                                                      // P = V + V R^2, V = R + R^2
+      RET(launch_combine(s, np, 0.0, 1.0, R, 1.0, R2, 0.0, nullptr, V));
+      EpiF64 e5;
+      e5.E = V;
+      e5.lde = np;
+      e5.beta = 1.0;
+      RET(gemm(s, np, V, R2, U, e5, true, stats));
+      P = U;
+    }
+    EpiF64 ey;
+    ey.E = Y;
+    ey.lde = np;
+    ey.beta = 1.0;
+    return gemm(s, np, P, Y, Yn, ey, true, stats);
   }
 
   cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, bool full_last, double* out_diag,
@@ -152,7 +186,7 @@ void free_matset(MatSet& m) {
 
 // Default grouped operations: one system after another.
 cudaError_t Engine::foe_group(cudaStream_t s, std::vector<FoeJob>& jobs, double sc) {
-  for (auto& j : jobs) RET(foe(s, *j.m, j.H, j.N, j.mu, sc, *j.ns, *j.nc, j.stats, j.dpar));
+  for (auto& j : jobs) RET(foe(s, *j.m, j.H, j.N, j.mu, sc, *j.plan, j.stats, j.dpar));
   return cudaSuccess;
 }
 

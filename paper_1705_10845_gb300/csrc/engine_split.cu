@@ -224,32 +224,47 @@ __global__ void convert_group_kernel(size_t count, MatList L) {
     convert4<FMT, MODE>(i, s, L.f[j], L.d[j], L.hi[j], L.lo[j]);
 }
 
-// Y = a I + b X per system (W_k start of the Newton-Schulz iteration)
-struct AxpiList {
+// Y = g0 I + g1 X1 + g2 X2 + g3 X3 per system (matrices not given are left out): the start of a level's
+// inverse, and the sums of its corrections
+struct CombList {
   int n = 0;
-  const float* X[kMaxGroup];
+  const float* X[3][kMaxGroup];
   float* Y[kMaxGroup];
   unsigned* amax[kMaxGroup];
-  float a[kMaxGroup], b[kMaxGroup];
-  const double* dc[kMaxGroup];   // device c (a = 1 - c, b = c) when not null
+  float g[4][kMaxGroup];
+  const double* dg[kMaxGroup];   // device g when not null
 };
 
-__global__ void axpi_group_kernel(int np, AxpiList L) {
+__global__ void combine_group_kernel(int np, CombList L) {
   const int j = blockIdx.y;
-  float a = L.a[j], b = L.b[j];
-  if (L.dc[j]) {
-    a = (float)(1.0 - L.dc[j][0]);
-    b = (float)L.dc[j][0];
-  }
-  const size_t count = (size_t)np * np;
-  const float* X = L.X[j];
-  float* Y = L.Y[j];
+  float g[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) g[q] = L.dg[j] ? (float)L.dg[j][q] : L.g[q][j];
+  const size_t count = (size_t)np * np / 4;
+  const float4* X0 = reinterpret_cast<const float4*>(L.X[0][j]);
+  const float4* X1 = reinterpret_cast<const float4*>(L.X[1][j]);
+  const float4* X2 = reinterpret_cast<const float4*>(L.X[2][j]);
+  float4* Y = reinterpret_cast<float4*>(L.Y[j]);
   float m = 0.0f;
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < count; idx += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(idx / np), c = (int)(idx % np);
-    const float v = b * X[idx] + (r == c ? a : 0.0f);
-    Y[idx] = v;
-    m = fmaxf(m, fabsf(v));
+    const int r = (int)(4 * idx / np), c = (int)(4 * idx % np);   // np is a multiple of 4: one row
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    const float4* Xs[3] = {X0, X1, X2};
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (Xs[q]) {
+        const float4 x = Xs[q][idx];
+        v[0] += g[q + 1] * x.x;
+        v[1] += g[q + 1] * x.y;
+        v[2] += g[q + 1] * x.z;
+        v[3] += g[q + 1] * x.w;
+      }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (r == c + q) v[q] += g[0];
+      m = fmaxf(m, fabsf(v[q]));
+    }
+    Y[idx] = make_float4(v[0], v[1], v[2], v[3]);
   }
   raise_amax(L.amax[j], m);
 }
@@ -349,9 +364,8 @@ __global__ void get_diag_group_kernel(int np, DiagList L) {
 }
 
 // Epilogue options of one split product.  The FP32 side inputs E, E2 are
-// read transposed by the product kernel, so they must be symmetric (S, W and
-// the Newton-Schulz residual Q, whose rounding asymmetry the iteration
-// removes).
+// read transposed by the product kernel, so they must be symmetric (S, W, the
+// residual Q and its polynomials).
 struct Epi {
   float alpha = 1.0f;
   const SplitMat* E = nullptr;
@@ -374,8 +388,8 @@ struct Epi {
 // The recursion is carried in correction form so that its exact leading
 // terms never pass through the rounded operands:
 //   T_{k+1} = 2 T_k - 2 T_k W_k,  W_k = I - Y_k = I - (I + T_k^2)^-1,
-// W_k from the Newton-Schulz step written for W (Q = S - W - W S,
-// W <- W + Q - Q W), and the response chains as
+// W_k from residual corrections written for W (Q = S - W - W S,
+// W <- W + P - P W, P a polynomial in Q: plan.h), and the response chains as
 //   M = 2 T1_k - A1 T_{k+1},  T1_{k+1} = M - W_k M.
 // T_k, M and T1_k are FP64 values; W, S, Q, A1 FP32 values; every product
 // operand is the hi/lo split of a value.
@@ -650,22 +664,34 @@ class EngineSplit : public Engine {
   }
 
   cudaError_t foe(cudaStream_t s, MatSet& m, const double* H, int N, double mu, double sc,
-                  const std::vector<int>& ns, const std::vector<double>& nc, double* stats,
-                  const double* dpar) override {
+                  const std::vector<LevelPlan>& plan, double* stats, const double* dpar) override {
     std::vector<FoeJob> jobs(1);
     jobs[0].m = &m;
     jobs[0].H = H;
     jobs[0].N = N;
     jobs[0].mu = mu;
-    jobs[0].ns = &ns;
-    jobs[0].nc = &nc;
+    jobs[0].plan = &plan;
     jobs[0].stats = stats;
     jobs[0].dpar = dpar;
     return foe_group(s, jobs, sc);
   }
 
+  // Linear combination of matrices per system into Y[i] and its operand split (mode as convert_group).
+  cudaError_t combine_group(cudaStream_t s, int np, CombList& L, const std::vector<SplitMat*>& Y, int mode) {
+    L.n = (int)Y.size();
+    for (int i = 0; i < L.n; ++i) {
+      L.Y[i] = Y[i]->f;
+      L.amax[i] = Y[i]->amax;
+    }
+    RET(zero_amax_group(s, Y));
+    combine_group_kernel<<<ew_grid((size_t)np * np / 4, L.n), 256, 0, s>>>(np, L);
+    note_launch();
+    RET(cudaGetLastError());
+    return convert_group(s, Y, np, mode);
+  }
+
   // The recursion of every job's system in lockstep: each product of a level is one grouped
-  // launch over the jobs that need it (a job runs its own Newton-Schulz iteration count).
+  // launch over the jobs that need it (a job runs its own plan).
   cudaError_t foe_group(cudaStream_t s, std::vector<FoeJob>& jobs, double sc) override {
     const int B = (int)jobs.size();
     if (B == 0) return cudaSuccess;
@@ -699,71 +725,93 @@ class EngineSplit : public Engine {
     RET(cudaGetLastError());
     RET(convert_group(s, T0s, np, 1));
     std::vector<SplitMat*> W(B), Wn(B);
+    // scratch of the corrections: matrices of the response chains, which are free here
+    auto Sk = [](MatSet& m, int k) -> SplitMat* { return (k & 1) ? &m.sT1b : &m.sS; };   // S_k beside S_{k-1}
     for (int k = 0; k < n; ++k) {
       std::vector<GemmOp> ops;
-      for (auto& j : jobs) ops.push_back({&j.m->sT[k], &j.m->sT[k], &j.m->sS, Epi(), j.stats});   // S = T^2
+      for (auto& j : jobs) ops.push_back({&j.m->sT[k], &j.m->sT[k], Sk(*j.m, k), Epi(), j.stats});   // S = T^2
       RET(gemm_group(s, np, ops, true));
-      // the Newton-Schulz iterates alternate between sY[k] and the work matrix; the start is
-      // chosen by the parity of the iteration count so that W_k always ends in sY[k] (the
-      // buffers every later use, and a captured graph of this pass, refer to)
-      AxpiList al;
-      al.n = B;
-      int maxit = 0;
+      // the iterates alternate between sY[k] and the work matrix; the start is chosen by the
+      // parity of the rounds so that W_k always ends in sY[k] (the buffers every later use, and
+      // a captured graph of this pass, refer to)
+      CombList cl;
+      int rounds = 0;
       for (int i = 0; i < B; ++i) {
         FoeJob& j = jobs[i];
         MatSet& m = *j.m;
-        const int nsk = (*j.ns)[k];
-        maxit = std::max(maxit, nsk);
-        W[i] = (nsk % 2 == 1) ? &m.sYw : &m.sY[k];
+        const LevelPlan& p = (*j.plan)[k];
+        rounds = std::max(rounds, p.inv.n);
+        W[i] = (p.inv.n % 2 == 1) ? &m.sYw : &m.sY[k];
         Wn[i] = (W[i] == &m.sY[k]) ? &m.sYw : &m.sY[k];
-        al.Y[i] = W[i]->f;
-        al.amax[i] = W[i]->amax;
-        if (k == 0) {                                                             // W = S
-          al.X[i] = m.sS.f;
-          al.a[i] = 0.f;
-          al.b[i] = 1.f;
-          al.dc[i] = nullptr;
-        } else {                                                                  // W = (1-c) I + c W_{k-1}
-          al.X[i] = m.sY[k - 1].f;
-          al.a[i] = (float)(1.0 - (*j.nc)[k]);
-          al.b[i] = (float)(*j.nc)[k];
-          al.dc[i] = j.dpar ? j.dpar + 1 + k : nullptr;
-        }
+        cl.X[0][i] = k > 0 ? m.sY[k - 1].f : nullptr;                            // W0 (plan.h)
+        cl.X[1][i] = p.nb > 2 ? Sk(m, k)->f : nullptr;
+        cl.X[2][i] = p.nb > 3 ? Sk(m, k - 1)->f : nullptr;
+        for (int q = 0; q < 4; ++q) cl.g[q][i] = (float)p.g[q];
+        cl.dg[i] = j.dpar ? j.dpar + 1 + 4 * k : nullptr;
       }
-      RET(zero_amax_group(s, W));
-      axpi_group_kernel<<<ew_grid(cnt, B), 256, 0, s>>>(np, al);
-      note_launch();
-      RET(cudaGetLastError());
-      RET(convert_group(s, W, np, 0));
-      for (int it = 0; it < maxit; ++it) {
-        std::vector<GemmOp> oq, ow;
-        std::vector<int> who;
+      RET(combine_group(s, np, cl, W, 0));
+      for (int r = 0; r < rounds; ++r) {
+        // Q = S - W - W S and P = Q - Q^2 + ..: functions of one matrix, so every product is symmetric
+        std::vector<GemmOp> oq, o2, o5, ow;
+        std::vector<SplitMat*> V;
+        CombList cv;
         for (int i = 0; i < B; ++i) {
           FoeJob& j = jobs[i];
-          if ((*j.ns)[k] <= it) continue;
+          const InvOrders& inv = (*j.plan)[k].inv;
+          if (r >= inv.n) continue;
           MatSet& m = *j.m;
-          Epi eq;                                                                 // Q = S - W - W S
+          const int order = inv.order[r];
+          SplitMat* P = &m.sQ;
+          Epi eq;
           eq.alpha = -1.f;
-          eq.E = &m.sS;
+          eq.E = Sk(m, k);
           eq.beta = 1.f;
           eq.E2 = W[i];
           eq.beta2 = -1.f;
-          oq.push_back({W[i], &m.sS, &m.sQ, eq, j.stats});
-          Epi ew;                                                                 // W <- W + Q - Q W
+          oq.push_back({W[i], Sk(m, k), &m.sQ, eq, j.stats});
+          if (order >= 3) {
+            Epi e2;
+            if (order == 3) {                                                    // P = Q - Q^2
+              e2.alpha = -1.f;
+              e2.E = &m.sQ;
+              e2.beta = 1.f;
+            }
+            o2.push_back({&m.sQ, &m.sQ, &m.sA1, e2, j.stats});
+            P = &m.sA1;
+          }
+          if (order == 5) {                                                      // P = V + V Q^2, V = Q - Q^2
+            const int c = (int)V.size();
+            V.push_back(&m.sMt);
+            cv.X[0][c] = m.sQ.f;
+            cv.X[1][c] = m.sA1.f;
+            cv.X[2][c] = nullptr;
+            cv.g[0][c] = 0.f;
+            cv.g[1][c] = 1.f;
+            cv.g[2][c] = -1.f;
+            cv.dg[c] = nullptr;
+            Epi e5;
+            e5.E = &m.sMt;
+            e5.beta = 1.f;
+            o5.push_back({&m.sMt, &m.sA1, &m.sT1a, e5, j.stats});
+            P = &m.sT1a;
+          }
+          Epi ew;                                                                // W <- W + P - P W
           ew.alpha = -1.f;
           ew.E = W[i];
           ew.beta = 1.f;
-          ew.E2 = &m.sQ;
+          ew.E2 = P;
           ew.beta2 = 1.f;
-          ow.push_back({&m.sQ, W[i], Wn[i], ew, j.stats});
-          who.push_back(i);
-        }
-        RET(gemm_group(s, np, oq, false));
-        RET(gemm_group(s, np, ow, true));
-        for (int i : who) {
+          ow.push_back({P, W[i], Wn[i], ew, j.stats});
           std::swap(W[i], Wn[i]);
-          if (jobs[i].stats) jobs[i].stats[1] += 1;
+          if (j.stats) j.stats[1] += 1;
         }
+        RET(gemm_group(s, np, oq, true));
+        RET(gemm_group(s, np, o2, true));
+        if (!V.empty()) {
+          RET(combine_group(s, np, cv, V, 0));
+          RET(gemm_group(s, np, o5, true));
+        }
+        RET(gemm_group(s, np, ow, true));
       }
       std::vector<GemmOp> ot;
       for (auto& j : jobs) {

@@ -21,16 +21,16 @@ __global__ void t0_init_kernel(int n, int np, const double* __restrict__ H, doub
   T0[idx] = v;
 }
 
-__global__ void ident_minus_kernel(int np, const double* __restrict__ S, double* __restrict__ Y) {
+__global__ void combine_kernel(int np, double a, double c1, const double* __restrict__ X1, double c2,
+                               const double* __restrict__ X2, double c3, const double* __restrict__ X3,
+                               double* __restrict__ Y) {
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (size_t)np * np) return;
-  const int i = (int)(idx / np), j = (int)(idx % np);
-  Y[idx] = (i == j ? 1.0 : 0.0) - S[idx];
-}
-
-__global__ void scale_kernel(size_t count, double c, const double* __restrict__ X, double* __restrict__ Y) {
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < count) Y[idx] = c * X[idx];
+  double v = (idx / np == idx % np) ? a : 0.0;
+  if (X1) v += c1 * X1[idx];
+  if (X2) v += c2 * X2[idx];
+  if (X3) v += c3 * X3[idx];
+  Y[idx] = v;
 }
 
 // A1 = T0 diag(d) + diag(d) T0  (first level of a chain with diagonal T1_0)
@@ -338,14 +338,9 @@ cudaError_t launch_t0_init(cudaStream_t s, int n, int np, const double* H, doubl
   return cudaGetLastError();
 }
 
-cudaError_t launch_ident_minus(cudaStream_t s, int np, const double* S, double* Y) {
-  ident_minus_kernel<<<blocks_for((size_t)np * np, 256), 256, 0, s>>>(np, S, Y);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_scale(cudaStream_t s, size_t count, double c, const double* X, double* Y) {
-  scale_kernel<<<blocks_for(count, 256), 256, 0, s>>>(count, c, X, Y);
+cudaError_t launch_combine(cudaStream_t s, int np, double a, double c1, const double* X1, double c2, const double* X2,
+                           double c3, const double* X3, double* Y) {
+  combine_kernel<<<blocks_for((size_t)np * np, 256), 256, 0, s>>>(np, a, c1, X1, c2, X2, c3, X3, Y);
   note_launch();
   return cudaGetLastError();
 }

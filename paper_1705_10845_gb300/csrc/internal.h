@@ -73,8 +73,6 @@ cudaError_t launch_verlet_second(cudaStream_t s, int nat, double dt, double mass
 // ---- expansion helpers (foe_kernels.cu), FP64 ----
 cudaError_t launch_t0_init(cudaStream_t s, int n, int np, const double* H, double mu, double scale,
                            double* T0);
-cudaError_t launch_ident_minus(cudaStream_t s, int np, const double* S, double* Y);
-cudaError_t launch_scale(cudaStream_t s, size_t count, double c, const double* X, double* Y);
 cudaError_t launch_level0_A1(cudaStream_t s, int np, const double* T0, const double* d, double* A1);
 cudaError_t launch_transpose_add(cudaStream_t s, int np, const double* G, double* A1);
 cudaError_t launch_row_dot(cudaStream_t s, int n, int np, const double* Y, const double* M, double* out);

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "plan.h"
 
 namespace xl {
 
@@ -62,8 +63,7 @@ struct FoeJob {
   const double* H = nullptr;
   int N = 0;
   double mu = 0.0;
-  const std::vector<int>* ns = nullptr;
-  const std::vector<double>* nc = nullptr;
+  const std::vector<LevelPlan>* plan = nullptr;
   double* stats = nullptr;
   const double* dpar = nullptr;
 };
@@ -135,14 +135,12 @@ class Engine {
   }
   double kind_ms_[64] = {0};
   int kind_n_[64] = {0};
-  // T_0 = -sc (H - mu I); n levels T_{k+1} = 2 T_k Y_k, Y_k = (I + T_k^2)^-1 by
-  // plan.s[k] Newton-Schulz steps (2I - Y B) Y from Y = I - S (k = 0) or c_k Y_{k-1}.
-  // dpar (device, may be null): when set, mu = dpar[0] and the Newton-Schulz start scales
-  // c_k = dpar[1 + k] are read on the device instead of the host values mu, nc (so that a
-  // captured graph of the expansion can be replayed with new values; split engines only).
+  // T_0 = -sc (H - mu I); n levels T_{k+1} = 2 T_k Y_k, Y_k = (I + T_k^2)^-1 as planned (plan.h).
+  // dpar (device, may be null): when set, mu = dpar[0] and the coefficients g_j of level k's start
+  // = dpar[1 + 4 k + j] are read on the device instead of the host values (so that a captured
+  // graph of the expansion can be replayed with new values; split engines only).
   virtual cudaError_t foe(cudaStream_t s, MatSet& m, const double* H, int N, double mu, double sc,
-                          const std::vector<int>& ns, const std::vector<double>& nc, double* stats,
-                          const double* dpar) = 0;
+                          const std::vector<LevelPlan>& plan, double* stats, const double* dpar) = 0;
   // Response chain with diagonal T1_0 = diag(dvec): T1_{k+1} = Y_k (2 T1_k - A1 T_{k+1}),
   // A1 = T_k T1_k + T1_k T_k.  out_diag = diag(T1_n); full_last keeps T1_n in Tmu.
   virtual cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, bool full_last,
@@ -216,6 +214,9 @@ cudaError_t launch_sub(cudaStream_t s, int n, const double* w, const double* t, 
 cudaError_t launch_dot1p(cudaStream_t s, int n, const double* a, const double* b, double* out);
 cudaError_t launch_rank1_update(cudaStream_t s, int n, const double* u, const double* v, const double* Ku,
                                 const double* vK, const double* denom, double* J, double* K);
+// Y = a I + sum_j c_j X_j over the matrices given (null: left out)
+cudaError_t launch_combine(cudaStream_t s, int np, double a, double c1, const double* X1, double c2, const double* X2,
+                           double c3, const double* X3, double* Y);
 cudaError_t launch_density_out_f64(cudaStream_t s, int N, int np, const double* Tn, const double* Tmu, double dmu,
                                    double* ddiag, double* D);
 

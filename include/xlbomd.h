@@ -116,7 +116,7 @@ typedef struct {
                               of the split; 1 = one product of the hi operands (FP32
                               accumulation).  The kernel only preconditions the n dynamics and
                               the forces do not contain it; the expansion always takes three,
-                              the chemical-potential chain follows mu_prec.  Ignored by FP64. */
+                              dD/dmu follows mu_prec.  Ignored by FP64. */
   int graphs;              /* 1: split precisions with at most 2048 padded orbitals capture each
                               chemical-potential pass (per plan of its inverses) and each probe's
                               response in CUDA graphs and replay them (the second run of a plan
@@ -125,8 +125,9 @@ typedef struct {
                               stream, which cannot be captured).  On many concurrent 32-512-atom
                               trajectories it measured slower than direct launches, so it is
                               off by default.  0: off. */
-  int mu_prec;             /* split precisions: 0 = the chemical-potential chain (dD/dmu) takes the
-                              three products of the split; 1 = one hi*hi product.  dD/dmu only
+  int mu_prec;             /* split precisions: 0 = dD/dmu (a closed form of the expansion's
+                              matrices, three to five products) takes the three products of the
+                              split; 1 = one hi*hi product.  dD/dmu only
                               sets the Newton step on mu and the first-order correction
                               D(mu + dmu) = D(mu) + dmu dD/dmu, whose trace stays exact whatever
                               its error; D's error from it is at most |dmu| times the error of
@@ -267,7 +268,7 @@ xlbomd_status xlbomd_energy(xlbomd_ctx* ctx, int sys);
 
 /* a1-a10 for every system, nsteps times (Eqs. Integration, VRL_Damp).  The
  * systems of the context that share a padded orbital count advance in
- * lockstep: their expansions, chemical-potential chains and probe chains run
+ * lockstep: their expansions, dD/dmu and probe chains run
  * as grouped tensor-core launches over all of them (split precisions), with
  * one stream synchronisation per chemical-potential pass and per probe index
  * for the whole group; a padded size held by one system takes the one-system

@@ -27,7 +27,8 @@ namespace {
 
 constexpr double kKB = 8.617333262e-5;
 constexpr double kAcc = 9.648533e-3;   // 1 eV/(amu A) in A/fs^2
-constexpr int kPassPar = 1 + 4 * 40;   // device parameters of a captured mu pass: mu, then g_0..g_3 per level
+// device parameters of a captured mu pass: mu, g_0..g_3 per level, then z_0, z_1 (and two unused)
+constexpr int kPassZ = 1 + 4 * 40, kPassPar = kPassZ + 4;
 
 struct Sys {
   int nat = 0, N = 0, np = 0, natp = 0, ng = 0, kp = 0;
@@ -36,7 +37,7 @@ struct Sys {
   double *R = nullptr, *V = nullptr, *F = nullptr, *Z = nullptr, *nh = nullptr, *q = nullptr, *r = nullptr;
   double *Kr = nullptr, *pot = nullptr, *potv = nullptr, *gam = nullptr, *SF = nullptr, *G4 = nullptr;
   double *H0 = nullptr, *H = nullptr, *Dm = nullptr;
-  double *ddiag = nullptr, *dmu_diag = nullptr, *d1 = nullptr, *dvec = nullptr, *dvec_mu = nullptr;
+  double *ddiag = nullptr, *dmu_diag = nullptr, *d1 = nullptr, *dvec = nullptr;
   double *pV = nullptr, *pW = nullptr, *scal = nullptr, *work = nullptr, *energy = nullptr;
   double *Kfull = nullptr, *Jm = nullptr;   // exact kernel (natoms x natoms) and its work matrix
   // exact kernel, split precisions: chain slots for probes run side by side, and per slot the
@@ -272,6 +273,7 @@ struct MuSearch {
   int pass = 0;
   bool done = false;
   std::vector<LevelPlan> plan;
+  ResolventPlan zplan;
 
   // start from the Gershgorin interval [glo, ghi] and the system's mu history
   xlbomd_status start(xlbomd_ctx* ctx, const Sys& S, double lo, double hi) {
@@ -304,6 +306,8 @@ struct MuSearch {
     t0max = sc * std::max(std::fabs(ghi - mu), std::fabs(mu - glo));
     if (!(t0max < 1.0)) return fail(ctx, XLBOMD_ERR_SPECTRUM, "|beta (e - mu)| / 2^(n+1) >= 1");
     plan_expansion(ctx->plans, t0max, p.n_sq, (p.prec == XLBOMD_FP64) ? 1e-16 : 1e-8, plan);
+    // dT_n/dmu at single-product accuracy needs its resolvent to no more than that
+    zplan = plan_resolvent(t0max * t0max, (p.prec == XLBOMD_FP64) ? 1e-16 : (p.mu_prec == 1) ? 1e-5 : 1e-8);
     S.mats.t0max = t0max;
     return XLBOMD_OK;
   }
@@ -397,8 +401,14 @@ xlbomd_status density(xlbomd_ctx* ctx, Sys& S, bool with_forces) {
     const double mu = ms.mu;
     auto mu_pass = [&](const double* dp) -> xlbomd_status {
       CK(E.foe(st, S.mats, S.H, S.N, mu, sc, ms.plan, S.stats, dp));
-      // mu chain: T1_0 = +sc I, full last level
-      CK(E.chain(st, S.mats, S.dvec_mu, S.N, true, S.dmu_diag, S.stats));
+      MuJob mj;
+      mj.m = &S.mats;
+      mj.N = S.N;
+      mj.plan = &ms.zplan;
+      mj.out_diag = S.dmu_diag;
+      mj.stats = S.stats;
+      mj.dpar = dp ? dp + kPassZ : nullptr;
+      CK(E.mu_derivative(st, mj, 0.5 * beta_of(p)));
       CK(E.trace_tn(st, S.mats, S.N, S.scal));          // scal[0] = sum_i T_n,ii
       CK(launch_sum(st, S.N, S.dmu_diag, S.scal + 1));    // scal[1] = sum_i dT_n,ii/dmu
       return XLBOMD_OK;
@@ -413,6 +423,10 @@ xlbomd_status density(xlbomd_ctx* ctx, Sys& S, bool with_forces) {
         key.push_back(ms.plan[k].inv.n);
         for (int r = 0; r < ms.plan[k].inv.n; ++r) key.push_back(ms.plan[k].inv.order[r]);
       }
+      ctx->ppar[kPassZ] = ms.zplan.z0;
+      ctx->ppar[kPassZ + 1] = ms.zplan.z1;
+      key.push_back(ms.zplan.inv.n);
+      for (int r = 0; r < ms.zplan.inv.n; ++r) key.push_back(ms.zplan.inv.order[r]);
       CK(cudaMemcpyAsync(S.dpar, ctx->ppar, sizeof(double) * kPassPar, cudaMemcpyHostToDevice, st));
       CKS(run_captured(ctx, S, key, [&] { return mu_pass(S.dpar); }));
     } else {
@@ -430,7 +444,7 @@ xlbomd_status density(xlbomd_ctx* ctx, Sys& S, bool with_forces) {
 }
 
 // a3-a6 for several systems of one padded size in lockstep: every mu pass runs the expansion
-// and the mu chain of all systems still searching as grouped launches, with one host
+// and dT_n/dmu of all systems still searching as grouped launches, with one host
 // synchronisation per pass for all of them.  Each system takes exactly the steps of density().
 xlbomd_status density_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, bool with_forces) {
   cudaStream_t st = ctx->stream;
@@ -450,7 +464,7 @@ xlbomd_status density_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, bool wi
   for (size_t i = 0; i < B; ++i) active[i] = i;
   while (!active.empty()) {
     std::vector<FoeJob> fj;
-    std::vector<ChainJob> cj;
+    std::vector<MuJob> mj;
     for (size_t i : active) {
       Sys& S = *G[i];
       CKS(ms[i].prepare(ctx, S));
@@ -462,16 +476,16 @@ xlbomd_status density_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, bool wi
       f.plan = &ms[i].plan;
       f.stats = S.stats;
       fj.push_back(f);
-      ChainJob c;
+      MuJob c;
       c.m = &S.mats;
-      c.dvec = S.dvec_mu;   // mu chain: T1_0 = +sc I, full last level
       c.N = S.N;
+      c.plan = &ms[i].zplan;
       c.out_diag = S.dmu_diag;
       c.stats = S.stats;
-      cj.push_back(c);
+      mj.push_back(c);
     }
     CK(E.foe_group(st, fj, sc));
-    CK(E.chain_group(st, cj, true));
+    CK(E.mu_derivative_group(st, mj, 0.5 * beta_of(p)));
     for (size_t k = 0; k < active.size(); ++k) {
       Sys& S = *G[active[k]];
       CK(E.trace_tn(st, S.mats, S.N, S.scal));
@@ -498,13 +512,13 @@ xlbomd_status density_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, bool wi
   return XLBOMD_OK;
 }
 
-// a7: one probe.  H1 = diag(gamma v) on orbitals, T1_0 = -sc H1.
+// a7: one probe.  H1 = diag(gamma v) on orbitals less its average, T1_0 = -sc H1.
 xlbomd_status response(xlbomd_ctx* ctx, Sys& S, const double* v, double* w) {
   cudaStream_t st = ctx->stream;
   const double sc = beta_of(ctx->p) / std::ldexp(1.0, ctx->p.n_sq + 1);
   CK(gamma_apply(ctx, S, v, S.potv, S.work));
-  CK(launch_expand_potential(st, S.nat, S.np, -sc, S.potv, S.dvec));
-  CK(ctx->eng->chain(st, S.mats, S.dvec, S.N, false, S.d1, S.stats));
+  CK(launch_expand_potential(st, S.nat, S.np, -sc, S.potv, S.dmu_diag, S.dvec));
+  CK(ctx->eng->chain(st, S.mats, S.dvec, S.N, S.d1, S.stats));
   CK(launch_response_finish(st, S.nat, S.N, S.d1, S.dmu_diag, S.scal + 4, w));
   return XLBOMD_OK;
 }
@@ -545,14 +559,14 @@ xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
       CK(launch_unit_vector(st, S.nat, I0 + j, vec(j, 0)));
       CK(launch_gamma_apply(st, S.nat, S.gam, S.natp, S.SF, S.kp, ctx->p.coulomb_k, vec(j, 0), vec(j, 2),
                             vec(j, 6)));
-      CK(launch_expand_potential(st, S.nat, S.np, -sc, vec(j, 2), vec(j, 3)));
+      CK(launch_expand_potential(st, S.nat, S.np, -sc, vec(j, 2), S.dmu_diag, vec(j, 3)));
       cj[j].m = &S.slots[j];
       cj[j].dvec = vec(j, 3);
       cj[j].N = S.N;
       cj[j].out_diag = vec(j, 4);
       cj[j].stats = S.stats;
     }
-    CK(ctx->eng->chain_group(st, cj, false));
+    CK(ctx->eng->chain_group(st, cj));
     for (int j = 0; j < g; ++j) {
       CK(launch_response_finish(st, S.nat, S.N, vec(j, 4), S.dmu_diag, vec(j, 5), vec(j, 1)));
       CK(launch_jacobian_column(st, S.nat, I0 + j, vec(j, 1), S.Jm, S.Kfull));
@@ -800,7 +814,7 @@ xlbomd_status response_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, const 
   for (size_t k = 0; k < G.size(); ++k) {
     Sys& S = *G[k];
     CK(gamma_apply(ctx, S, v[k], S.potv, S.work));
-    CK(launch_expand_potential(st, S.nat, S.np, -sc, S.potv, S.dvec));
+    CK(launch_expand_potential(st, S.nat, S.np, -sc, S.potv, S.dmu_diag, S.dvec));
     ChainJob c;
     c.m = &S.mats;
     c.dvec = S.dvec;
@@ -809,7 +823,7 @@ xlbomd_status response_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, const 
     c.stats = S.stats;
     cj.push_back(c);
   }
-  CK(ctx->eng->chain_group(st, cj, false));
+  CK(ctx->eng->chain_group(st, cj));
   for (size_t k = 0; k < G.size(); ++k) {
     Sys& S = *G[k];
     CK(launch_response_finish(st, S.nat, S.N, S.d1, S.dmu_diag, S.scal + 4, w[k]));
@@ -1033,7 +1047,7 @@ xlbomd_status md_step_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
 void free_sys(Sys& S) {
   double** ptrs[] = {&S.R,  &S.V,        &S.F,    &S.Z,  &S.nh,  &S.q,    &S.r,     &S.Kr,    &S.pot,
                      &S.potv, &S.gam,    &S.SF,   &S.G4, &S.H0,  &S.H,    &S.Dm,    &S.ddiag, &S.dmu_diag,
-                     &S.d1, &S.dvec,     &S.dvec_mu, &S.pV, &S.pW, &S.scal, &S.work, &S.energy,
+                     &S.d1, &S.dvec,     &S.pV, &S.pW, &S.scal, &S.work, &S.energy,
                      &S.Kfull, &S.Jm, &S.dpar};
   for (double** p : ptrs) {
     if (*p) cudaFree(*p);
@@ -1128,10 +1142,10 @@ xlbomd_status xlbomd_response_noalloc(xlbomd_ctx* ctx, int sys, const double* v_
   // the array keeps the previous call's contents: the diagonal accumulator starts at zero
   CK(cudaMemsetAsync(d1, 0, sizeof(double) * kStaticMaxNp, st));
   CK(gamma_apply(ctx, S, v_dev, potv, scal + 64));
-  CK(launch_expand_potential(st, S.nat, S.np, -sc, potv, dvec));
+  CK(launch_expand_potential(st, S.nat, S.np, -sc, potv, S.dmu_diag, dvec));
   const bool prof = ctx->eng->prof;
   ctx->eng->prof = false;   // event timing would create CUDA events
-  const cudaError_t ce = ctx->eng->chain(st, m, dvec, S.N, false, d1, S.stats);   // counted in XLBOMD_STATS
+  const cudaError_t ce = ctx->eng->chain(st, m, dvec, S.N, d1, S.stats);   // counted in XLBOMD_STATS
   ctx->eng->prof = prof;
   CK(ce);
   CK(launch_response_finish(st, S.nat, S.N, d1, S.dmu_diag, scal, w_dev));
@@ -1235,7 +1249,6 @@ xlbomd_status xlbomd_init(const xlbomd_params* params, const xlbomd_system* syst
   if (cudaMemcpyAsync(ctx->cdev, p.c, sizeof(double) * 8, cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess)
     return bail(XLBOMD_ERR_CUDA);
   ctx->sys.resize(nsys);
-  const double sc = beta_of(p) / std::ldexp(1.0, p.n_sq + 1);
   for (int i = 0; i < nsys; ++i) {
     const xlbomd_system& s = systems[i];
     Sys& S = ctx->sys[i];
@@ -1277,7 +1290,6 @@ xlbomd_status xlbomd_init(const xlbomd_params* params, const xlbomd_system* syst
     A(&S.dmu_diag, S.np);
     A(&S.d1, S.np);
     A(&S.dvec, S.np);
-    A(&S.dvec_mu, S.np);
     A(&S.pV, (size_t)(kMaxRank + 1) * nat);
     A(&S.pW, (size_t)(kMaxRank + 1) * nat);
     A(&S.scal, 64);
@@ -1288,16 +1300,13 @@ xlbomd_status xlbomd_init(const xlbomd_params* params, const xlbomd_system* syst
     // R wrapped into [0, L)
     std::vector<double> Rw(3 * nat);
     for (size_t a = 0; a < 3 * nat; ++a) Rw[a] = s.R[a] - S.L * std::floor(s.R[a] / S.L);
-    std::vector<double> dmu(S.np, 0.0);
-    for (int a = 0; a < S.N; ++a) dmu[a] = sc;
     const cudaStream_t cs = ctx->stream;
     if (cudaMemcpyAsync(S.R, Rw.data(), sizeof(double) * 3 * nat, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
         cudaMemcpyAsync(S.V, s.V, sizeof(double) * 3 * nat, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
         cudaMemcpyAsync(S.Z, s.Z, sizeof(double) * nat, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
         (S.ng && cudaMemcpyAsync(S.G4, S.G4h.data(), sizeof(double) * S.G4h.size(), cudaMemcpyHostToDevice, cs) !=
                      cudaSuccess) ||
-        cudaMemcpyAsync(S.dvec_mu, dmu.data(), sizeof(double) * S.np, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
-        cudaStreamSynchronize(cs) != cudaSuccess)   // Rw and dmu are host temporaries
+        cudaStreamSynchronize(cs) != cudaSuccess)   // Rw is a host temporary
       return bail(XLBOMD_ERR_CUDA);
     if (build_H(ctx, S) != XLBOMD_OK) return bail((xlbomd_status)ctx->status);
   }

@@ -95,7 +95,27 @@ class EngineF64 : public Engine {
     return gemm(s, np, P, Y, Yn, ey, true, stats);
   }
 
-  cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, bool full_last, double* out_diag,
+  cudaError_t mu_derivative(cudaStream_t s, MuJob& j, double amp) override {
+    MatSet& m = *j.m;
+    const int np = m.np, n = m.n;
+    // work matrices of the chains and of the expansion, both idle here
+    EpiF64 e1;
+    RET(gemm(s, np, m.T[0], m.T[0], m.S, e1, true, j.stats));
+    double *Z = m.Yw, *Zn = m.T1b;
+    RET(launch_combine(s, np, j.plan->z0, j.plan->z1, m.S, 0.0, nullptr, 0.0, nullptr, Z));
+    for (int r = 0; r < j.plan->inv.n; ++r) {
+      RET(correct(s, np, Z, m.S, 1.0, m.Q, m.A1, m.Mt, m.G, Zn, j.plan->inv.order[r], j.stats));
+      std::swap(Z, Zn);
+    }
+    RET(launch_combine(s, np, -1.0, 2.0, m.Y[n - 1], 0.0, nullptr, 0.0, nullptr, m.Q));   // I - 2 W = 2 Y - I
+    RET(gemm(s, np, m.Q, m.Q, m.A1, e1, true, j.stats));
+    EpiF64 ea;
+    ea.alpha = amp;
+    RET(gemm(s, np, m.A1, Z, m.Tmu, ea, true, j.stats));
+    return launch_get_diag(s, j.N, np, m.Tmu, j.out_diag);
+  }
+
+  cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, double* out_diag,
                     double* stats) override {
     const int np = m.np, n = m.n;
     double* T1 = m.T1a;
@@ -118,13 +138,10 @@ class EngineF64 : public Engine {
         em.beta = 2.0;
       }
       RET(gemm(s, np, m.T[k + 1], m.A1, m.Mt, em, false, stats));
-      if (last && !full_last) return launch_row_dot(s, N, np, m.Y[k], m.Mt, out_diag);   // diag(Y M)
-      double* dst = (last && full_last) ? m.Tmu : T1n;
+      if (last) return launch_row_dot(s, N, np, m.Y[k], m.Mt, out_diag);   // diag(Y M)
       EpiF64 ey;
-      RET(gemm(s, np, m.Y[k], m.Mt, dst, ey, true, stats));    // T1' = Y M  (= Y Mt^T)
-      if (last) return launch_get_diag(s, N, np, dst, out_diag);
-      T1n = T1;
-      T1 = dst;
+      RET(gemm(s, np, m.Y[k], m.Mt, T1n, ey, true, stats));    // T1' = Y M  (= Y Mt^T)
+      std::swap(T1, T1n);
     }
     return cudaSuccess;
   }
@@ -190,8 +207,13 @@ cudaError_t Engine::foe_group(cudaStream_t s, std::vector<FoeJob>& jobs, double 
   return cudaSuccess;
 }
 
-cudaError_t Engine::chain_group(cudaStream_t s, std::vector<ChainJob>& jobs, bool full_last) {
-  for (auto& j : jobs) RET(chain(s, *j.m, j.dvec, j.N, full_last, j.out_diag, j.stats));
+cudaError_t Engine::mu_derivative_group(cudaStream_t s, std::vector<MuJob>& jobs, double amp) {
+  for (auto& j : jobs) RET(mu_derivative(s, j, amp));
+  return cudaSuccess;
+}
+
+cudaError_t Engine::chain_group(cudaStream_t s, std::vector<ChainJob>& jobs) {
+  for (auto& j : jobs) RET(chain(s, *j.m, j.dvec, j.N, j.out_diag, j.stats));
   return cudaSuccess;
 }
 

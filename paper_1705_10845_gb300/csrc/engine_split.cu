@@ -829,7 +829,138 @@ class EngineSplit : public Engine {
     return cudaSuccess;
   }
 
-  cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, bool full_last, double* out_diag,
+  cudaError_t mu_derivative(cudaStream_t s, MuJob& j, double amp) override {
+    std::vector<MuJob> jobs(1, j);
+    return mu_derivative_group(s, jobs, amp);
+  }
+
+  cudaError_t mu_derivative_group(cudaStream_t s, std::vector<MuJob>& jobs, double amp) override {
+    const int B = (int)jobs.size();
+    if (B == 0) return cudaSuccess;
+    if (B > kMaxGroup) {
+      for (int i = 0; i < B; i += kMaxGroup) {
+        std::vector<MuJob> part(jobs.begin() + i, jobs.begin() + std::min(B, i + kMaxGroup));
+        RET(mu_derivative_group(s, part, amp));
+      }
+      return cudaSuccess;
+    }
+    const int np = jobs[0].m->np, n = jobs[0].m->n;
+    for (auto& j : jobs)
+      if (j.m->np != np || j.m->n != n) return cudaErrorInvalidValue;
+    const bool single = (mu_nseg_ == 1);
+    const int mode = single ? 2 : 0;
+    Epi base;
+    base.nseg = mu_nseg_;
+    base.hi_only = single;
+    // the matrices of the response chains and of the expansion's corrections are idle here
+    std::vector<GemmOp> o1;
+    for (auto& j : jobs) o1.push_back({&j.m->sT[0], &j.m->sT[0], &j.m->sS, base, j.stats});
+    RET(gemm_group(s, np, o1, true));
+    std::vector<SplitMat*> Z(B), Zn(B), C(B);
+    CombList cz;
+    int rounds = 0;
+    for (int i = 0; i < B; ++i) {
+      MuJob& j = jobs[i];
+      const ResolventPlan& p = *j.plan;
+      rounds = std::max(rounds, p.inv.n);
+      Z[i] = &j.m->sYw;
+      Zn[i] = &j.m->sT1b;
+      cz.X[0][i] = j.m->sS.f;
+      cz.X[1][i] = cz.X[2][i] = nullptr;
+      cz.g[0][i] = (float)p.z0;
+      cz.g[1][i] = (float)p.z1;
+      cz.g[2][i] = cz.g[3][i] = 0.f;
+      cz.dg[i] = j.dpar;
+    }
+    RET(combine_group(s, np, cz, Z, mode));
+    for (int r = 0; r < rounds; ++r) {
+      std::vector<GemmOp> oq, o2, o5, ow;
+      std::vector<SplitMat*> V;
+      CombList cv;
+      for (int i = 0; i < B; ++i) {
+        MuJob& j = jobs[i];
+        if (r >= j.plan->inv.n) continue;
+        MatSet& m = *j.m;
+        const int order = j.plan->inv.order[r];
+        SplitMat* P = &m.sQ;
+        Epi eq = base;                                                            // R = I - Z + S Z
+        eq.E = Z[i];
+        eq.beta = -1.f;
+        eq.diag = 1.f;
+        oq.push_back({&m.sS, Z[i], &m.sQ, eq, j.stats});
+        if (order >= 3) {
+          Epi e2 = base;
+          if (order == 3) {                                                       // P = R + R^2
+            e2.E = &m.sQ;
+            e2.beta = 1.f;
+          }
+          o2.push_back({&m.sQ, &m.sQ, &m.sA1, e2, j.stats});
+          P = &m.sA1;
+        }
+        if (order == 5) {                                                         // P = V + V R^2, V = R + R^2
+          const int c = (int)V.size();
+          V.push_back(&m.sMt);
+          cv.X[0][c] = m.sQ.f;
+          cv.X[1][c] = m.sA1.f;
+          cv.X[2][c] = nullptr;
+          cv.g[0][c] = cv.g[3][c] = 0.f;
+          cv.g[1][c] = cv.g[2][c] = 1.f;
+          cv.dg[c] = nullptr;
+          Epi e5 = base;
+          e5.E = &m.sMt;
+          e5.beta = 1.f;
+          o5.push_back({&m.sMt, &m.sA1, &m.sT1a, e5, j.stats});
+          P = &m.sT1a;
+        }
+        Epi ew = base;                                                            // Z <- Z + P Z
+        ew.E = Z[i];
+        ew.beta = 1.f;
+        ow.push_back({P, Z[i], Zn[i], ew, j.stats});
+        std::swap(Z[i], Zn[i]);
+      }
+      RET(gemm_group(s, np, oq, true));
+      RET(gemm_group(s, np, o2, true));
+      if (!V.empty()) {
+        RET(combine_group(s, np, cv, V, mode));
+        RET(gemm_group(s, np, o5, true));
+      }
+      RET(gemm_group(s, np, ow, true));
+    }
+    CombList cc;
+    std::vector<GemmOp> oc, ot;
+    DiagList dl;
+    dl.n = B;
+    int maxN = 0;
+    for (int i = 0; i < B; ++i) {
+      MuJob& j = jobs[i];
+      MatSet& m = *j.m;
+      C[i] = &m.sMt;
+      cc.X[0][i] = m.sY[n - 1].f;                                                 // C = I - 2 W_{n-1}
+      cc.X[1][i] = cc.X[2][i] = nullptr;
+      cc.g[0][i] = 1.f;
+      cc.g[1][i] = -2.f;
+      cc.g[2][i] = cc.g[3][i] = 0.f;
+      cc.dg[i] = nullptr;
+      oc.push_back({&m.sMt, &m.sMt, &m.sA1, base, j.stats});
+      Epi et = base;
+      et.alpha = (float)amp;
+      et.out64 = true;
+      et.convert = false;
+      ot.push_back({&m.sA1, Z[i], &m.sTmu, et, j.stats});
+      dl.N[i] = j.N;
+      dl.X[i] = m.sTmu.d;
+      dl.out[i] = j.out_diag;
+      maxN = std::max(maxN, j.N);
+    }
+    RET(combine_group(s, np, cc, C, mode));
+    RET(gemm_group(s, np, oc, true));
+    RET(gemm_group(s, np, ot, true));
+    get_diag_group_kernel<<<dim3((maxN + 255) / 256, B), 256, 0, s>>>(np, dl);
+    note_launch();
+    return cudaGetLastError();
+  }
+
+  cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, double* out_diag,
                     double* stats) override {
     std::vector<ChainJob> jobs(1);
     jobs[0].m = &m;
@@ -837,18 +968,18 @@ class EngineSplit : public Engine {
     jobs[0].N = N;
     jobs[0].out_diag = out_diag;
     jobs[0].stats = stats;
-    return chain_group(s, jobs, full_last);
+    return chain_group(s, jobs);
   }
 
   // Response chains of several systems (or several probes of one system, each with its own
   // chain matrices) in lockstep, every product a grouped launch.
-  cudaError_t chain_group(cudaStream_t s, std::vector<ChainJob>& jobs, bool full_last) override {
+  cudaError_t chain_group(cudaStream_t s, std::vector<ChainJob>& jobs) override {
     const int B = (int)jobs.size();
     if (B == 0) return cudaSuccess;
     if (B > kMaxGroup) {
       for (int i = 0; i < B; i += kMaxGroup) {
         std::vector<ChainJob> part(jobs.begin() + i, jobs.begin() + std::min(B, i + kMaxGroup));
-        RET(chain_group(s, part, full_last));
+        RET(chain_group(s, part));
       }
       return cudaSuccess;
     }
@@ -856,8 +987,7 @@ class EngineSplit : public Engine {
     for (auto& j : jobs)
       if (j.m->np != np || j.m->n != n) return cudaErrorInvalidValue;
     const size_t cnt = (size_t)np * np;
-    // either chain may run on the hi operands alone (the mu chain is the one with a full last level)
-    const int nseg = full_last ? mu_nseg_ : probe_nseg_;
+    const int nseg = probe_nseg_;
     // A single-product chain keeps M and T1 as FP32 values with hi operands only: its products
     // carry ~2^-11 relative error, so the double-float values and lo operands of the three-product
     // chain would add traffic and no accuracy.  The last level still writes the double-float array
@@ -875,10 +1005,10 @@ class EngineSplit : public Engine {
       RET(zero_amax_group(s, A1s));
       Epi em;                                                                    // Mt = 2 T1 - T_{k+1} A1
       em.alpha = -1.f;
-      em.out64 = !single || (last && !full_last);
+      em.out64 = !single || last;
       em.hi_only = single;
-      em.convert = !(last && !full_last);                                        // the last M of a probe
-      em.nseg = nseg;                                                            // chain is only reduced
+      em.convert = !last;                                                        // the last M is only reduced
+      em.nseg = nseg;
       std::vector<GemmOp> om;
       if (k == 0) {
         A1List al;
@@ -924,7 +1054,7 @@ class EngineSplit : public Engine {
       }
       RET(convert_group(s, A1s, np, single ? 2 : 0));
       RET(gemm_group(s, np, om, false));
-      if (last && !full_last) {
+      if (last) {
         DiagList dl;
         dl.n = B;
         int maxN = 0;
@@ -939,16 +1069,13 @@ class EngineSplit : public Engine {
         note_launch();
         return cudaGetLastError();
       }
-      std::vector<SplitMat*> dst(B);
       std::vector<GemmOp> oy;
       for (int i = 0; i < B; ++i) {
-        dst[i] = (last && full_last) ? &jobs[i].m->sTmu : T1n[i];
         Epi ey;                                                                  // T1' = M - W M
         ey.alpha = -1.f;
         if (single) {
           ey.E = Mts[i];                                                          // read transposed: M
           ey.beta = 1.0f;
-          ey.out64 = last;                                                        // T_mu (double-float)
           ey.hi_only = true;
         } else {
           ey.E64 = Mts[i]->d;
@@ -956,29 +1083,11 @@ class EngineSplit : public Engine {
           ey.e64_trans = 1;
           ey.out64 = true;
         }
-        ey.convert = !last;
         ey.nseg = nseg;
-        oy.push_back({&jobs[i].m->sY[k], Mts[i], dst[i], ey, jobs[i].stats});
+        oy.push_back({&jobs[i].m->sY[k], Mts[i], T1n[i], ey, jobs[i].stats});
       }
       RET(gemm_group(s, np, oy, true));
-      if (last) {
-        DiagList dl;
-        dl.n = B;
-        int maxN = 0;
-        for (int i = 0; i < B; ++i) {
-          dl.N[i] = jobs[i].N;
-          dl.X[i] = dst[i]->d;
-          dl.out[i] = jobs[i].out_diag;
-          maxN = std::max(maxN, jobs[i].N);
-        }
-        get_diag_group_kernel<<<dim3((maxN + 255) / 256, B), 256, 0, s>>>(np, dl);
-        note_launch();
-        return cudaGetLastError();
-      }
-      for (int i = 0; i < B; ++i) {
-        T1n[i] = T1[i];
-        T1[i] = dst[i];
-      }
+      std::swap(T1, T1n);
     }
     return cudaSuccess;
   }

@@ -67,6 +67,15 @@ struct FoeJob {
   double* stats = nullptr;
   const double* dpar = nullptr;
 };
+// One system's part of a grouped dT_n/dmu.
+struct MuJob {
+  MatSet* m = nullptr;
+  int N = 0;
+  const ResolventPlan* plan = nullptr;
+  double* out_diag = nullptr;
+  double* stats = nullptr;
+  const double* dpar = nullptr;   // device z0, z1 (captured passes), else null
+};
 struct ChainJob {
   MatSet* m = nullptr;
   const double* dvec = nullptr;
@@ -141,19 +150,28 @@ class Engine {
   // graph of the expansion can be replayed with new values; split engines only).
   virtual cudaError_t foe(cudaStream_t s, MatSet& m, const double* H, int N, double mu, double sc,
                           const std::vector<LevelPlan>& plan, double* stats, const double* dpar) = 0;
+  // Tmu = dT_n/dmu of the last expansion and out_diag its diagonal.  T_n = tanh(2^n artanh T_0) and
+  // dT_0/dmu = sc I commutes with everything, so
+  //   dT_n/dmu = sc 2^n (I - T_n^2)(I - T_0^2)^-1 = amp (I - 2 W_{n-1})^2 (I - S_0)^-1,  amp = sc 2^n
+  // (I - T_n^2 is the square of I - 2 W_{n-1}, which keeps its relative accuracy where |T_n| -> 1).
+  // 2 to 3 dense-equivalent products; a chain of 10 levels, as for a probe, takes 25 (three 16-bit
+  // products each: forces and rank-2 kernel of 150 atoms in FP16x3 7.79 -> 6.81 ms, 201 atoms in
+  // BF16x3 without a kernel 5.97 -> 4.80 ms, 24 atoms in FP64 51.8 -> 42.7 ms a step).
+  virtual cudaError_t mu_derivative(cudaStream_t s, MuJob& j, double amp) = 0;
+  virtual cudaError_t mu_derivative_group(cudaStream_t s, std::vector<MuJob>& jobs, double amp);
   // Response chain with diagonal T1_0 = diag(dvec): T1_{k+1} = Y_k (2 T1_k - A1 T_{k+1}),
-  // A1 = T_k T1_k + T1_k T_k.  out_diag = diag(T1_n); full_last keeps T1_n in Tmu.
-  virtual cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, bool full_last,
-                            double* out_diag, double* stats) = 0;
+  // A1 = T_k T1_k + T1_k T_k.  out_diag = diag(T1_n).
+  virtual cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, double* out_diag,
+                            double* stats) = 0;
   // The same for several systems of one padded size (lockstep: the split engine runs each
   // product over all of them in one grouped launch; the FP64 engine one after another).
   virtual cudaError_t foe_group(cudaStream_t s, std::vector<FoeJob>& jobs, double sc);
-  virtual cudaError_t chain_group(cudaStream_t s, std::vector<ChainJob>& jobs, bool full_last);
+  virtual cudaError_t chain_group(cudaStream_t s, std::vector<ChainJob>& jobs);
   // out[0] = sum_{i<N} (T_n)_ii
   // Device flag that the tensor-core product sets when a bounded wait gives up or a
   // tile falls outside the matrix (null: this engine has none).
   virtual const int* device_error() const { return nullptr; }
-  // Split engines: tensor products per level of the probe chains and of the mu chain
+  // Split engines: tensor products per product of the probe chains and of dT_n/dmu
   // (3, or 1 = hi operands only)
   virtual void set_chain_segments(int, int) {}
   virtual cudaError_t trace_tn(cudaStream_t s, MatSet& m, int N, double* out) = 0;
@@ -191,7 +209,8 @@ cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, int N, double beta, in
                                const double* D, const double* H, double* work, double* out);
 
 // misc FP64 launchers (foe_kernels.cu)
-cudaError_t launch_expand_potential(cudaStream_t s, int nat, int np, double scale, const double* pot, double* dvec);
+cudaError_t launch_expand_potential(cudaStream_t s, int nat, int np, double scale, const double* pot,
+                                    const double* dmu_diag, double* dvec);
 cudaError_t launch_response_finish(cudaStream_t s, int nat, int N, const double* d1, const double* dmu_diag,
                                    double* scal, double* w);
 cudaError_t launch_absmax(cudaStream_t s, int n, const double* x, double* out);

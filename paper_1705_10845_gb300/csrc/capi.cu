@@ -27,8 +27,6 @@ namespace {
 
 constexpr double kKB = 8.617333262e-5;
 constexpr double kAcc = 9.648533e-3;   // 1 eV/(amu A) in A/fs^2
-// device parameters of a captured mu pass: mu, g_0..g_3 per level, then z_0, z_1 (and two unused)
-constexpr int kPassZ = 1 + 4 * 40, kPassPar = kPassZ + 4;
 
 struct Sys {
   int nat = 0, N = 0, np = 0, natp = 0, ng = 0, kp = 0;
@@ -423,6 +421,7 @@ xlbomd_status density(xlbomd_ctx* ctx, Sys& S, bool with_forces) {
         key.push_back(ms.plan[k].inv.n);
         for (int r = 0; r < ms.plan[k].inv.n; ++r) key.push_back(ms.plan[k].inv.order[r]);
       }
+      ctx->ppar[kPassT0] = ms.t0max;
       ctx->ppar[kPassZ] = ms.zplan.z0;
       ctx->ppar[kPassZ + 1] = ms.zplan.z1;
       key.push_back(ms.zplan.inv.n);

@@ -4,20 +4,23 @@
 // Every matrix keeps a value array -- FP32, or double-float (an FP32 hi + lo
 // pair) for T_k, M and T1, whose leading terms the correction form keeps out of
 // the products -- and a split operand pair hi = rn(x s), lo = rn(x s - hi)
-// (rn: rounding to FP16, BF16 or TF32) with a power-of-two scale s chosen from
-// max |x| so that max |x s| lies in [2^10, 2^11) (FP16 keeps full precision in
-// both parts); producers raise max |x| atomically and a conversion pass writes
-// hi/lo.  A product takes three tensor-core products (hi*hi, hi*lo, lo*hi), or
-// one (hi*hi) in the probe chains and the mu chain when the context asks for
-// it.  Traces, charges and the density matrix handed to the forces are
-// accumulated in FP64.
-#include <cuda_bf16.h>
-
+// (rn: rounding to FP16, BF16 or TF32).  The power-of-two scale s comes from a
+// bound that is known before the matrix is computed (operand.cuh): |T_k| <= t_k
+// from the spectral bound and the scalar recursion, everything that only
+// matters against the identity below 4, and the chains' matrices, which are
+// linear in the probe, from max |dvec| and the recursion's growth.  So every
+// kernel that computes a matrix writes its operands in the same pass.  (The
+// scales used to follow each matrix's own maximum: a memset, an atomic maximum
+// and a conversion pass per product.)  A product takes three tensor-core
+// products (hi*hi, hi*lo, lo*hi), or one (hi*hi) in the probe chains and
+// dT_n/dmu when the context asks for it.  Traces, charges and the density
+// matrix handed to the forces are accumulated in FP64.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <unordered_map>
 
+#include "operand.cuh"
 #include "precision.h"
 #include "tc.h"
 
@@ -32,127 +35,29 @@ namespace {
 
 inline unsigned nblk(size_t count, int tpb = 256) { return (unsigned)((count + tpb - 1) / tpb); }
 
-// element-wise kernels that raise a matrix's max |x| walk their elements grid-stride with at
-// most this many blocks, so that each launch issues few atomics on the one max
+// element-wise kernels walk their elements grid-stride with at most this many blocks
 constexpr unsigned kEwBlocks = 152 * 16;
 
 // One-CTA-per-tile product kernel: products of at least this size split their hi*hi sums over
 // both accumulators.
 constexpr int kSplitAccMin = 8192;
-// Persistent product kernel, split products: the hi*hi sum is accumulated in chunks of this many
-// 64-wide K blocks of 16-bit operands (K = 1024; the same K with TF32's 32-wide blocks), each folded
-// into the running sum with round-to-nearest FP32 adds.
-// The tensor core truncates as it accumulates, so a sum's error grows with its length: at 2048
-// atoms (N = 8192) the charge error fell from 4.7e-5 e (one 8192-long sum) to 2.5e-5 e (two
-// halves), and it keeps halving with the chunk length.
-constexpr int kChunkKb = 16;
+// Split products accumulate the hi*hi sum in chunks of K = 512 (8 K blocks of 64 16-bit or 16 of 32 TF32
+// elements), added up with round-to-nearest FP32 adds.  The tensor core truncates as it accumulates, so a
+// sum's error grows with its length: at 2048 atoms (N = 8192) the charge error fell from 4.7e-5 e (one
+// 8192-long sum) to 2.5e-5 e (two halves) and 6.6e-6 e (1024-long chunks).  Product errors and times at
+// n = 8192 for chunks of 256, 512, 1024 and the whole sum: 9e-5, 1.4e-4, 2.4e-4, 2e-3 and 2.83, 2.30, 2.21,
+// 2.14 ms; at n = 1024 (128-wide tiles) 3e-5, 5e-5, 1e-4 and 29, 29, 28 us.
+constexpr int kChunkK = 512;
 
-// Raise *amax to the block's max |v| with one atomic per block (all threads
-// of the block must call it).
-__device__ __forceinline__ void raise_amax(unsigned* amax, float v) {
-  __shared__ float wmax[32];
-  v = fabsf(v);
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int nthr = blockDim.x * blockDim.y;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  if ((tid & 31) == 0) wmax[tid >> 5] = v;
-  __syncthreads();
-  if (tid == 0) {
-    float m = 0.0f;
-    for (int w = 0; w < (nthr + 31) / 32; ++w) m = fmaxf(m, wmax[w]);
-    atomicMax(amax, __float_as_uint(m));
-  }
-}
-
-// Operand words: FP16 or BF16 in 16 bits, TF32 in an FP32 word whose low 13 mantissa bits are
-// zero (fmt 0, 1, 2).
-template <int FMT>
-struct OpWord {
-  using T = unsigned short;
-  using V4 = ushort4;
-};
-template <>
-struct OpWord<2> {
-  using T = unsigned;
-  using V4 = uint4;
-};
-
-// Round x to the operand format; v receives the rounded value.  TF32 rounding (to 10 explicit
-// mantissa bits, nearest, ties away from zero) is the cvt.rna.tf32.f32 instruction.
-template <int FMT>
-__device__ __forceinline__ typename OpWord<FMT>::T op_round(float x, float& v) {
-  if constexpr (FMT == 2) {
-    unsigned r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    v = __uint_as_float(r);
-    return r;
-  } else if constexpr (FMT == 1) {
-    const __nv_bfloat16 b = __float2bfloat16_rn(x);
-    v = __bfloat162float(b);
-    return __bfloat16_as_ushort(b);
-  } else {
-    const __half h = __float2half_rn(x);
-    v = __half2float(h);
-    return __half_as_ushort(h);
-  }
-}
-
-// Four operand words at index i (16-byte groups for TF32, 8-byte for 16-bit words).
-template <int FMT>
-__device__ __forceinline__ void store4(void* base, size_t i, const typename OpWord<FMT>::T (&w)[4]) {
-  using V4 = typename OpWord<FMT>::V4;
-  V4 v;
-  v.x = w[0];
-  v.y = w[1];
-  v.z = w[2];
-  v.w = w[3];
-  reinterpret_cast<V4*>(base)[i] = v;
-}
-
-// Conversion of four values to the split operand pair: hi = rn(x s), lo = rn((x s - hi) + xl s)
-// (xl: the low word of a double-float value, else 0; s is a power of two, so x s is exact).
-// MODE 0: FP32 value -> hi, lo; 1: double-float value -> hi, lo; 2: FP32 value -> hi.
-template <int FMT, int MODE>
-__device__ __forceinline__ void convert4(size_t i, float s, const float* __restrict__ f, const float2* __restrict__ d,
-                                         void* hi, void* lo) {
-  float xs[4], xl[4] = {0.f, 0.f, 0.f, 0.f};
-  if (MODE == 1) {
-    const float4* d4 = reinterpret_cast<const float4*>(d);   // two double-float values per float4
-    const float4 a = d4[2 * i], b = d4[2 * i + 1];
-    xs[0] = a.x * s; xs[1] = a.z * s; xs[2] = b.x * s; xs[3] = b.z * s;
-    xl[0] = a.y * s; xl[1] = a.w * s; xl[2] = b.y * s; xl[3] = b.w * s;
-  } else {
-    const float4 x = reinterpret_cast<const float4*>(f)[i];
-    xs[0] = x.x * s; xs[1] = x.y * s; xs[2] = x.z * s; xs[3] = x.w * s;
-  }
-  typename OpWord<FMT>::T h[4], l[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    float hv, lv;
-    h[k] = op_round<FMT>(xs[k], hv);
-    if (MODE == 1) l[k] = op_round<FMT>((xs[k] - hv) + xl[k], lv);
-    if (MODE == 0) l[k] = op_round<FMT>(xs[k] - hv, lv);
-  }
-  store4<FMT>(hi, i, h);
-  if (MODE != 2) store4<FMT>(lo, i, l);
-}
-
-// The operand scale from max |x|: a power of two that puts max |x s| in [2^10, 2^11) (FP16
-// keeps full precision in both parts; BF16 and TF32 have FP32's range and lose nothing by it).
-__device__ __forceinline__ float operand_scale(const unsigned* amax) {
-  const float m = __uint_as_float(*amax);
-  return (m > 0.0f && isfinite(m)) ? ldexpf(1.0f, 10 - ilogbf(m)) : 1.0f;
-}
-
-// One matrix: all threads derive the same scale from amax; thread 0 of block 0 publishes it.
-// Four elements per thread and step (count is a multiple of 4).
-template <int FMT, int MODE>
-__global__ void convert_kernel(size_t count, const float* __restrict__ f, const float2* __restrict__ d,
-                               const unsigned* __restrict__ amax, void* hi, void* lo, float* __restrict__ scale) {
-  const float s = operand_scale(amax);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *scale = s;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count / 4; i += (size_t)gridDim.x * blockDim.x)
-    convert4<FMT, MODE>(i, s, f, d, hi, lo);
+// Operands of four values at element i in the format fmt (0 FP16, 1 BF16, 2 TF32).
+__device__ __forceinline__ void store_op4(int fmt, void* hi, void* lo, size_t i, float s, const float (&x)[4],
+                                          const float (&xl)[4]) {
+  if (fmt == 2)
+    store_operand4<2>(hi, lo, i, s, x, xl);
+  else if (fmt == 1)
+    store_operand4<1>(hi, lo, i, s, x, xl);
+  else
+    store_operand4<0>(hi, lo, i, s, x, xl);
 }
 
 __global__ void df_to_f64_kernel(size_t count, const float2* __restrict__ x, double* __restrict__ y) {
@@ -199,43 +104,20 @@ __global__ void density_out_d_kernel(int N, int np, const float2* __restrict__ T
 // pointers travel by value in the kernel parameters (at most kMaxGroup systems per launch).
 constexpr int kMaxGroup = 64;
 
-struct MatList {
-  int n = 0;
-  float* f[kMaxGroup];
-  float2* d[kMaxGroup];
-  void* hi[kMaxGroup];
-  void* lo[kMaxGroup];
-  float* scale[kMaxGroup];
-  unsigned* amax[kMaxGroup];
-};
-
-__global__ void zero_amax_kernel(MatList L) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < L.n) *L.amax[i] = 0u;
-}
-
-// convert_kernel per system (blockIdx.y)
-template <int FMT, int MODE>
-__global__ void convert_group_kernel(size_t count, MatList L) {
-  const int j = blockIdx.y;
-  const float s = operand_scale(L.amax[j]);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *L.scale[j] = s;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count / 4; i += (size_t)gridDim.x * blockDim.x)
-    convert4<FMT, MODE>(i, s, L.f[j], L.d[j], L.hi[j], L.lo[j]);
-}
-
 // Y = g0 I + g1 X1 + g2 X2 + g3 X3 per system (matrices not given are left out): the start of a level's
 // inverse, and the sums of its corrections
 struct CombList {
   int n = 0;
-  const float* X[3][kMaxGroup];
+  const float* X[3][kMaxGroup];   // may be Y itself
   float* Y[kMaxGroup];
-  unsigned* amax[kMaxGroup];
+  void* hi[kMaxGroup];            // operands (lo: null for single products)
+  void* lo[kMaxGroup];
+  const float* scale[kMaxGroup];
   float g[4][kMaxGroup];
   const double* dg[kMaxGroup];   // device g when not null
 };
 
-__global__ void combine_group_kernel(int np, CombList L) {
+__global__ void combine_group_kernel(int np, int fmt, CombList L) {
   const int j = blockIdx.y;
   float g[4];
 #pragma unroll
@@ -245,7 +127,8 @@ __global__ void combine_group_kernel(int np, CombList L) {
   const float4* X1 = reinterpret_cast<const float4*>(L.X[1][j]);
   const float4* X2 = reinterpret_cast<const float4*>(L.X[2][j]);
   float4* Y = reinterpret_cast<float4*>(L.Y[j]);
-  float m = 0.0f;
+  const float s = *L.scale[j];
+  const float zero[4] = {0.f, 0.f, 0.f, 0.f};
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < count; idx += (size_t)gridDim.x * blockDim.x) {
     const int r = (int)(4 * idx / np), c = (int)(4 * idx % np);   // np is a multiple of 4: one row
     float v[4] = {0.f, 0.f, 0.f, 0.f};
@@ -260,69 +143,126 @@ __global__ void combine_group_kernel(int np, CombList L) {
         v[3] += g[q + 1] * x.w;
       }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 4; ++q)
       if (r == c + q) v[q] += g[0];
-      m = fmaxf(m, fabsf(v[q]));
-    }
     Y[idx] = make_float4(v[0], v[1], v[2], v[3]);
+    store_op4(fmt, L.hi[j], L.lo[j], 4 * idx, s, v, zero);
   }
-  raise_amax(L.amax[j], m);
 }
 
-// T0 = -sc (H - mu I) as a double-float, per system
+// T0 = -sc (H - mu I) as a double-float with its operands, per system; the first thread also writes the
+// operand scales of T_0 .. T_n (|T_k| <= t_k, t_{k+1} = 2 t_k / (1 + t_k^2)) and t_0 for the chains.
+// mu and t_0 come from the device parameters dpar of a captured pass (dpar[0], dpar[dt0]) when given.
 struct T0List {
   int n = 0;
   int N[kMaxGroup];
   const double* H[kMaxGroup];
   double mu[kMaxGroup];
-  const double* dmu[kMaxGroup];
+  double t0[kMaxGroup];
+  const double* dpar[kMaxGroup];
   float2* T0[kMaxGroup];
-  unsigned* amax[kMaxGroup];
+  void* hi[kMaxGroup];
+  void* lo[kMaxGroup];
+  float* scales[kMaxGroup];
+  float* t0_dev[kMaxGroup];
 };
 
-__global__ void t0_init_group_kernel(int np, double sc, T0List L) {
+__global__ void t0_init_group_kernel(int np, int nlev, int fmt, int dt0, double sc, T0List L) {
   const int j = blockIdx.y;
-  const double mu = L.dmu[j] ? L.dmu[j][0] : L.mu[j];
+  const double mu = L.dpar[j] ? L.dpar[j][0] : L.mu[j];
+  const double t0 = L.dpar[j] ? L.dpar[j][dt0] : L.t0[j];
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double t = t0;
+    for (int k = 0; k <= nlev; ++k) {
+      L.scales[j][1 + k] = operand_scale(t);
+      t = 2.0 * t / (1.0 + t * t);
+    }
+    L.scales[j][2 + nlev] = operand_scale(1.0 / (1.0 - t0 * t0));   // |(I - T_0^2)^-1|
+    *L.t0_dev[j] = (float)t0;
+  }
+  const float s = operand_scale(t0);
   const int n = L.N[j];
   const double* H = L.H[j];
   float2* T0 = L.T0[j];
-  const size_t count = (size_t)np * np;
-  float m = 0.0f;
+  const size_t count = (size_t)np * np / 4;
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < count; idx += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(idx / np), c = (int)(idx % np);
-    double v = 0.0;
-    if (r < n && c < n) v = -sc * (H[idx] - (r == c ? mu : 0.0));
-    const float vh = (float)v;
-    T0[idx] = make_float2(vh, (float)(v - (double)vh));
-    m = fmaxf(m, fabsf(vh));
+    const int r = (int)(4 * idx / np), c = (int)(4 * idx % np);
+    const double2 a = reinterpret_cast<const double2*>(H)[2 * idx], b = reinterpret_cast<const double2*>(H)[2 * idx + 1];
+    const double h[4] = {a.x, a.y, b.x, b.y};
+    float x[4], xl[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      double v = 0.0;
+      if (r < n && c + q < n) v = -sc * (h[q] - (r == c + q ? mu : 0.0));
+      x[q] = (float)v;
+      xl[q] = (float)(v - (double)x[q]);
+    }
+    float4* d = reinterpret_cast<float4*>(T0) + 2 * idx;
+    d[0] = make_float4(x[0], xl[0], x[1], xl[1]);
+    d[1] = make_float4(x[2], xl[2], x[3], xl[3]);
+    store_op4(fmt, L.hi[j], L.lo[j], 4 * idx, s, x, xl);
   }
-  raise_amax(L.amax[j], m);
 }
 
-// A1 of chain level 0 per system: (T0 hi + lo)(d_i + d_j)
+// Operand scales of a response chain, one block per system.  With tau_k a bound of |T1_k|
+// (tau_0 = max |d|, T1_0 = diag(d)):
+//   A1 = T T1 + T1 T           |A1| <= 2 t tau
+//   M  = 2 T1 - A1 T'          |M|  <= 2 tau (1 + t t')
+//   T1' = 2 Y (T1 - T T1 T) Y  |T1'| <= 2 tau (1 + g^2),  g = t / (1 + t^2) the largest t y
+struct ChainScaleList {
+  int n = 0;
+  const double* d[kMaxGroup];
+  const float* t0[kMaxGroup];
+  float* scales[kMaxGroup];   // [3 k] A1_k, [3 k + 1] M_k, [3 k + 2] T1_{k+1}
+};
+
+__global__ void chain_scales_kernel(int np, int nlev, ChainScaleList L) {
+  __shared__ float sm[32];
+  const int j = blockIdx.x;
+  float m = 0.0f;
+  for (int i = threadIdx.x; i < np; i += blockDim.x) m = fmaxf(m, fabsf((float)L.d[j][i]));
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, sm[w]);
+  // a bound slightly above the FP32 maximum, so that rounding it down cannot matter
+  double tau = 1.0001 * (double)m, t = 1.0001 * (double)*L.t0[j];
+  for (int k = 0; k < nlev; ++k) {
+    const double tn = 2.0 * t / (1.0 + t * t), g = t / (1.0 + t * t);
+    L.scales[j][3 * k] = operand_scale(2.0 * t * tau);
+    L.scales[j][3 * k + 1] = operand_scale(2.0 * tau * (1.0 + t * tn));
+    tau *= 2.0 * (1.0 + g * g);
+    L.scales[j][3 * k + 2] = operand_scale(tau);
+    t = tn;
+  }
+}
+
+// Operands of A1 = (T0 hi + lo)(d_i + d_j), chain level 0, per system (the value itself is not needed)
 struct A1List {
   int n = 0;
   const float2* T0[kMaxGroup];
   const double* d[kMaxGroup];
-  float* A1[kMaxGroup];
-  unsigned* amax[kMaxGroup];
+  void* hi[kMaxGroup];
+  void* lo[kMaxGroup];
+  const float* scale[kMaxGroup];
 };
 
-__global__ void level0_A1_group_kernel(int np, A1List L) {
+__global__ void level0_A1_group_kernel(int np, int fmt, A1List L) {
   const int j = blockIdx.y;
-  const float2* T0 = L.T0[j];
+  const float4* T0 = reinterpret_cast<const float4*>(L.T0[j]);
   const double* d = L.d[j];
-  float* A1 = L.A1[j];
-  const size_t count = (size_t)np * np;
-  float m = 0.0f;
+  const float s = *L.scale[j];
+  const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+  const size_t count = (size_t)np * np / 4;
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < count; idx += (size_t)gridDim.x * blockDim.x) {
-    const int r = (int)(idx / np), c = (int)(idx % np);
-    const float2 t = T0[idx];
-    const float v = (t.x + t.y) * (float)(d[r] + d[c]);
-    A1[idx] = v;
-    m = fmaxf(m, fabsf(v));
+    const int r = (int)(4 * idx / np), c = (int)(4 * idx % np);
+    const float4 a = T0[2 * idx], b = T0[2 * idx + 1];
+    const double dr = d[r];
+    const float x[4] = {(a.x + a.y) * (float)(dr + d[c]), (a.z + a.w) * (float)(dr + d[c + 1]),
+                        (b.x + b.y) * (float)(dr + d[c + 2]), (b.z + b.w) * (float)(dr + d[c + 3])};
+    store_op4(fmt, L.hi[j], L.lo[j], 4 * idx, s, x, zero);
   }
-  raise_amax(L.amax[j], m);
 }
 
 // Diagonal reductions of the chains' last level, per system
@@ -363,9 +303,8 @@ __global__ void get_diag_group_kernel(int np, DiagList L) {
   if (i < L.N[j]) L.out[j][i] = df_val(L.X[j][(size_t)i * np + i]);
 }
 
-// Epilogue options of one split product.  The FP32 side inputs E, E2 are
-// read transposed by the product kernel, so they must be symmetric (S, W, the
-// residual Q and its polynomials).
+// Epilogue options of one split product.  The side inputs of a symmetric product
+// must be symmetric where out2 is written (E is read at the mirrored place too).
 struct Epi {
   float alpha = 1.0f;
   const SplitMat* E = nullptr;
@@ -374,13 +313,15 @@ struct Epi {
   float beta2 = 0.0f;
   const float2* E64 = nullptr;
   float beta64 = 0.0f;
-  int e64_trans = 0;
   float diag = 0.0f;
   const double* dvec = nullptr;
   float dvec_scale = 1.0f;
-  bool out64 = false;       // write C.d (and convert from it) instead of C.f
-  bool convert = true;      // produce the split operand pair of C
-  bool hi_only = false;     // produce only the hi operand (C enters single products only)
+  bool out64 = false;       // write C.d (and the operands of it) instead of C.f
+  bool value = true;        // write the value of C
+  bool convert = true;      // write the operands of C
+  bool hi_only = false;     // only the hi operand (C enters single products only)
+  SplitMat* V = nullptr;    // second result va C + vb E: value and operands
+  float va = 0.0f, vb = 0.0f;
   int nseg = 3;             // 3: hi*hi + hi*lo + lo*hi; 1: hi*hi only
   int pairs = 1;            // 2: C = A B^T + B A^T
 };
@@ -402,51 +343,33 @@ class EngineSplit : public Engine {
     tc_group_cache_free(group_cache_);
   }
 
-  // operand split of one matrix: mode 0 FP32 -> hi, lo; 1 double-float -> hi, lo; 2 FP32 -> hi
-  template <int FMT>
-  void launch_convert(cudaStream_t s, SplitMat& m, size_t count, unsigned g, int mode) {
-    if (mode == 0) convert_kernel<FMT, 0><<<g, 256, 0, s>>>(count, m.f, m.d, m.amax, m.hi, m.lo, m.scale);
-    else if (mode == 1) convert_kernel<FMT, 1><<<g, 256, 0, s>>>(count, m.f, m.d, m.amax, m.hi, m.lo, m.scale);
-    else convert_kernel<FMT, 2><<<g, 256, 0, s>>>(count, m.f, m.d, m.amax, m.hi, m.lo, m.scale);
-  }
-
-  cudaError_t convert_mode(cudaStream_t s, SplitMat& m, int np, int mode) {
-    const size_t count = (size_t)np * np;
-    const unsigned g = std::min<size_t>(nblk(count), 152 * 16);
-    if (fmt_ == 2)
-      launch_convert<2>(s, m, count, g, mode);
-    else if (fmt_ == 1)
-      launch_convert<1>(s, m, count, g, mode);
-    else
-      launch_convert<0>(s, m, count, g, mode);
-    note_launch();
-    return cudaGetLastError();
-  }
-  cudaError_t convert(cudaStream_t s, SplitMat& m, int np) { return convert_mode(s, m, np, 0); }
-  cudaError_t convert_d(cudaStream_t s, SplitMat& m, int np) { return convert_mode(s, m, np, 1); }
-  cudaError_t convert_hi(cudaStream_t s, SplitMat& m, int np) { return convert_mode(s, m, np, 2); }
-
   // Symmetric-product tile lists for size np, uploaded on the stream that uses them (the
   // context's stream may be non-blocking, so a legacy-stream copy would not be ordered
   // before the first product).
   cudaError_t prep_tiles(int np, cudaStream_t s) {
     if (tiles_.count(np)) return cudaSuccess;
     const bool wide = (np % 256 == 0);
-    std::vector<int> t128 = tc_sym_tiles(np, 128), t256 = wide ? tc_sym_tiles(np, 256) : std::vector<int>();
-    std::vector<int> tp = wide ? tc_sym_tiles_pair(np) : std::vector<int>();
-    std::vector<int> all(t128);
-    all.insert(all.end(), t256.begin(), t256.end());
-    all.insert(all.end(), tp.begin(), tp.end());
+    std::vector<int> all, part;
+    TcTiles t;
+    size_t off[kTcWidths + 1];
+    for (int w = 0; w < kTcWidths; ++w) {
+      off[w] = all.size();
+      if (tc_width(w) == 256 && !wide) continue;
+      part = tc_sym_tiles(np, tc_width(w));
+      t.nsym[w] = (int)part.size() / 2;
+      all.insert(all.end(), part.begin(), part.end());
+    }
+    off[kTcWidths] = all.size();
+    if (wide) {
+      part = tc_sym_tiles_pair(np);
+      t.npair = (int)part.size() / 2;
+      all.insert(all.end(), part.begin(), part.end());
+    }
     int* d = nullptr;
     RET(cudaMalloc((void**)&d, sizeof(int) * std::max<size_t>(all.size(), 2)));
     RET(cudaMemcpyAsync(d, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice, s));
-    TcTiles t;
-    t.sym128 = d;
-    t.n128 = (int)t128.size() / 2;
-    t.sym256 = d + t128.size();
-    t.n256 = (int)t256.size() / 2;
-    t.pair = wide ? d + t128.size() + t256.size() : nullptr;
-    t.npair = (int)tp.size() / 2;
+    for (int w = 0; w < kTcWidths; ++w) t.sym[w] = d + off[w];
+    t.pair = wide ? d + off[kTcWidths] : nullptr;
     tiles_[np] = {d, t};
     if (!err_) {
       RET(cudaMalloc((void**)&err_, sizeof(int)));
@@ -455,16 +378,8 @@ class EngineSplit : public Engine {
     return cudaStreamSynchronize(s);   // `all` is a host temporary
   }
 
-  cudaError_t gemm(cudaStream_t s, int np, const SplitMat& A, const SplitMat& B, SplitMat& C, const Epi& e,
-                   bool sym, double* stats) {
-    RET(prep_tiles(np, s));
-    const TcTiles& tl = tiles_[np].second;
-    RET(cudaMemsetAsync(C.amax, 0, sizeof(unsigned), s));
-    TcArgs a;
-    a.nseg = e.nseg;
-    a.pairs = e.pairs;
-    a.sym = sym ? 1 : 0;
-    a.fmt = fmt_;
+  // the epilogue arguments of C = epi(A B^T)
+  static void fill_args(TcArgs& a, int np, const SplitMat& A, const SplitMat& B, SplitMat& C, const Epi& e) {
     a.alpha = e.alpha;
     a.E = e.E ? e.E->f : nullptr;
     a.beta = e.beta;
@@ -472,32 +387,56 @@ class EngineSplit : public Engine {
     a.beta2 = e.beta2;
     a.E64 = e.E64;
     a.beta64 = e.beta64;
-    a.e64_trans = e.e64_trans;
     a.diag = e.diag;
     a.dvec = e.dvec;
     a.ndvec = e.dvec ? np : 0;
     a.dvec_scale = e.dvec_scale;
-    a.C = e.out64 ? nullptr : C.f;
-    a.C64 = e.out64 ? C.d : nullptr;
+    a.out.f = (e.value && !e.out64) ? C.f : nullptr;
+    a.out.d = e.out64 ? C.d : nullptr;
+    if (e.convert) {
+      a.out.hi = C.hi;
+      a.out.lo = e.hi_only ? nullptr : C.lo;
+      a.out.scale = C.scale;
+    }
+    if (e.V) {
+      a.out2.f = e.V->f;
+      a.out2.hi = e.V->hi;
+      a.out2.lo = e.hi_only ? nullptr : e.V->lo;
+      a.out2.scale = e.V->scale;
+      a.va = e.va;
+      a.vb = e.vb;
+    }
     a.ldc = np;
-    a.amax = C.amax;
     a.sa = A.scale;
     a.sb = B.scale;
+  }
+
+  void fill_shared(TcArgs& a, int np, const Epi& e, bool sym) const {
+    a.nseg = e.nseg;
+    a.pairs = e.pairs;
+    a.sym = sym ? 1 : 0;
+    a.fmt = fmt_;
     a.err = err_;
-    RET(prof_begin(s));
-    // large products: split the hi*hi sums over both accumulators (the tensor core truncates as it
-    // accumulates, so a K-long sum's error grows with K)
+    // one-CTA-per-tile kernel, large products: the hi*hi sums split over both accumulators
     a.split_acc = (np >= kSplitAccMin) ? 1 : 0;
-    a.chunk_kb = chunk_kb();
+    a.chunk_kb = kChunkK / (fmt_ == 2 ? 32 : 64);
+  }
+
+  cudaError_t gemm(cudaStream_t s, int np, const SplitMat& A, const SplitMat& B, SplitMat& C, const Epi& e,
+                   bool sym, double* stats) {
+    RET(prep_tiles(np, s));
+    const TcTiles& tl = tiles_[np].second;
+    TcArgs a;
+    fill_args(a, np, A, B, C, e);
+    fill_shared(a, np, e, sym);
+    RET(prof_begin(s));
     RET(gemm_tc(s, np, A.hi, A.lo, B.hi, B.lo, a, tl));
-    // kind bits: 1 sym, 2 E, 4 E2, 8 E64, 16 E64 transposed, 32 FP64 output
-    const int kind = (sym ? 1 : 0) | (e.E ? 2 : 0) | (e.E2 ? 4 : 0) | (e.E64 ? 8 : 0) | (e.e64_trans ? 16 : 0) |
+    // kind bits: 1 sym, 2 E, 4 E2, 8 E64, 16 second result, 32 double-float output
+    const int kind = (sym ? 1 : 0) | (e.E ? 2 : 0) | (e.E2 ? 4 : 0) | (e.E64 ? 8 : 0) | (e.V ? 16 : 0) |
                      (e.out64 ? 32 : 0);
     RET(prof_end(s, 2.0 * (double)np * np * np * (sym ? 0.5 : 1.0) * e.pairs, kind));
     if (stats) stats[3] += (sym ? 0.5 : 1.0) * e.pairs;
-    if (!e.convert) return cudaSuccess;
-    if (e.hi_only && !e.out64) return convert_hi(s, C, np);
-    return e.out64 ? convert_d(s, C, np) : convert(s, C, np);
+    return cudaSuccess;
   }
 
   // ---- grouped operations (one launch over the systems of a lockstep group) ----
@@ -510,61 +449,11 @@ class EngineSplit : public Engine {
     double* stats;
   };
 
-  static MatList mat_list(const std::vector<SplitMat*>& ms) {
-    MatList L;
-    L.n = (int)ms.size();
-    for (int i = 0; i < L.n; ++i) {
-      L.f[i] = ms[i]->f;
-      L.d[i] = ms[i]->d;
-      L.hi[i] = ms[i]->hi;
-      L.lo[i] = ms[i]->lo;
-      L.scale[i] = ms[i]->scale;
-      L.amax[i] = ms[i]->amax;
-    }
-    return L;
-  }
-
-  cudaError_t zero_amax_group(cudaStream_t s, const std::vector<SplitMat*>& ms) {
-    if (ms.size() == 1) return cudaMemsetAsync(ms[0]->amax, 0, sizeof(unsigned), s);
-    zero_amax_kernel<<<1, kMaxGroup, 0, s>>>(mat_list(ms));
-    note_launch();
-    return cudaGetLastError();
-  }
-
-  // operand split of each matrix: mode 0 FP32 -> hi, lo; 1 double-float -> hi, lo; 2 FP32 -> hi
-  cudaError_t convert_group(cudaStream_t s, const std::vector<SplitMat*>& ms, int np, int mode) {
-    if (ms.size() == 1) {
-      if (mode == 0) return convert(s, *ms[0], np);
-      if (mode == 1) return convert_d(s, *ms[0], np);
-      return convert_hi(s, *ms[0], np);
-    }
-    const size_t count = (size_t)np * np;
-    const unsigned gx = (unsigned)std::max<size_t>(1, std::min<size_t>(nblk(count), (152 * 16) / ms.size()));
-    const dim3 grid(gx, (unsigned)ms.size());
-    const MatList L = mat_list(ms);
-    if (fmt_ == 2) {
-      if (mode == 0) convert_group_kernel<2, 0><<<grid, 256, 0, s>>>(count, L);
-      else if (mode == 1) convert_group_kernel<2, 1><<<grid, 256, 0, s>>>(count, L);
-      else convert_group_kernel<2, 2><<<grid, 256, 0, s>>>(count, L);
-    } else if (fmt_ == 1) {
-      if (mode == 0) convert_group_kernel<1, 0><<<grid, 256, 0, s>>>(count, L);
-      else if (mode == 1) convert_group_kernel<1, 1><<<grid, 256, 0, s>>>(count, L);
-      else convert_group_kernel<1, 2><<<grid, 256, 0, s>>>(count, L);
-    } else {
-      if (mode == 0) convert_group_kernel<0, 0><<<grid, 256, 0, s>>>(count, L);
-      else if (mode == 1) convert_group_kernel<0, 1><<<grid, 256, 0, s>>>(count, L);
-      else convert_group_kernel<0, 2><<<grid, 256, 0, s>>>(count, L);
-    }
-    note_launch();
-    return cudaGetLastError();
-  }
-
   static dim3 ew_grid(size_t count, int nsys) {
     return dim3((unsigned)std::max<size_t>(1, std::min<size_t>(nblk(count), kEwBlocks / nsys)), (unsigned)nsys);
   }
 
-  // One product per op, all in one grouped launch (ops share sym, nseg, pairs), then each C's
-  // max |x| and operand split.
+  // One product per op, all in one grouped launch (ops share sym, nseg, pairs).
   cudaError_t gemm_group(cudaStream_t s, int np, std::vector<GemmOp>& ops, bool sym) {
     if (ops.empty()) return cudaSuccess;
     if (ops.size() == 1) {
@@ -574,93 +463,24 @@ class EngineSplit : public Engine {
     RET(prep_tiles(np, s));
     const TcTiles& tl = tiles_[np].second;
     const Epi& e0 = ops[0].e;
-    std::vector<SplitMat*> outs;
-    for (auto& o : ops) outs.push_back(o.C);
-    RET(zero_amax_group(s, outs));
     TcArgs shared;
-    shared.nseg = e0.nseg;
-    shared.pairs = e0.pairs;
-    shared.sym = sym ? 1 : 0;
-    shared.fmt = fmt_;
-    shared.split_acc = (np >= kSplitAccMin) ? 1 : 0;
-    shared.chunk_kb = chunk_kb();
-    shared.err = err_;
+    fill_shared(shared, np, e0, sym);
     std::vector<TcProblem> probs(ops.size());
     for (size_t i = 0; i < ops.size(); ++i) {
       const GemmOp& o = ops[i];
-      const Epi& e = o.e;
-      TcArgs& a = probs[i].epi;
       probs[i].Ahi = o.A->hi;
       probs[i].Alo = o.A->lo;
       probs[i].Bhi = o.B->hi;
       probs[i].Blo = o.B->lo;
-      a.alpha = e.alpha;
-      a.E = e.E ? e.E->f : nullptr;
-      a.beta = e.beta;
-      a.E2 = e.E2 ? e.E2->f : nullptr;
-      a.beta2 = e.beta2;
-      a.E64 = e.E64;
-      a.beta64 = e.beta64;
-      a.e64_trans = e.e64_trans;
-      a.diag = e.diag;
-      a.dvec = e.dvec;
-      a.ndvec = e.dvec ? np : 0;
-      a.dvec_scale = e.dvec_scale;
-      a.C = e.out64 ? nullptr : o.C->f;
-      a.C64 = e.out64 ? o.C->d : nullptr;
-      a.ldc = np;
-      a.amax = o.C->amax;
-      a.sa = o.A->scale;
-      a.sb = o.B->scale;
+      fill_args(probs[i].epi, np, *o.A, *o.B, *o.C, o.e);
       if (o.stats) o.stats[3] += (sym ? 0.5 : 1.0) * e0.pairs;
     }
     if (!group_cache_) group_cache_ = tc_group_cache_new();
-    RET(tune_group(s, np, probs, shared, tl));
-    shared.bn = tuned_bn_[np];
     RET(prof_begin(s));
     RET(gemm_tc_group(s, np, probs.data(), (int)probs.size(), shared, tl, group_cache_));
-    const int kind = 64 | (sym ? 1 : 0) | (e0.E ? 2 : 0) | (e0.E2 ? 4 : 0) | (e0.E64 ? 8 : 0) |
-                     (e0.e64_trans ? 16 : 0) | (e0.out64 ? 32 : 0);
-    RET(prof_end(s, (double)ops.size() * 2.0 * (double)np * np * np * (sym ? 0.5 : 1.0) * e0.pairs, kind));
-    if (!e0.convert) return cudaSuccess;
-    const int mode = (e0.hi_only && !e0.out64) ? 2 : (e0.out64 ? 1 : 0);
-    return convert_group(s, outs, np, mode);
-  }
-
-  // Tile-width autotuner of grouped products: the first grouped product of a size that both
-  // widths can tile (n a multiple of 256) runs twice with 128-wide and twice with 256-wide
-  // tiles, timed with CUDA events on the stream, and the faster width serves every later
-  // grouped product of that size.  (Few large tiles leave SMs idle on small matrices; narrow
-  // tiles stage more operand bytes per flop on large ones.)  The product is recomputed from the
-  // same operands each time, so the tuning runs change nothing.
-  cudaError_t tune_group(cudaStream_t s, int np, std::vector<TcProblem>& probs, TcArgs shared, const TcTiles& tl) {
-    if (tuned_bn_.count(np)) return cudaSuccess;
-    if (np % 256 != 0) {
-      tuned_bn_[np] = 128;
-      return cudaSuccess;
-    }
-    cudaEvent_t ev[3];
-    for (auto& e : ev) RET(cudaEventCreate(&e));
-    float ms[2] = {0.f, 0.f};
-    const int widths[2] = {128, 256};
-    cudaError_t rc = cudaSuccess;
-    for (int w = 0; w < 2 && rc == cudaSuccess; ++w) {
-      shared.bn = widths[w];
-      rc = gemm_tc_group(s, np, probs.data(), (int)probs.size(), shared, tl, group_cache_);   // warm-up
-      if (rc == cudaSuccess) rc = cudaEventRecord(ev[0], s);
-      if (rc == cudaSuccess) rc = gemm_tc_group(s, np, probs.data(), (int)probs.size(), shared, tl, group_cache_);
-      if (rc == cudaSuccess) rc = cudaEventRecord(ev[1], s);
-      if (rc == cudaSuccess) rc = cudaEventSynchronize(ev[1]);
-      if (rc == cudaSuccess) rc = cudaEventElapsedTime(&ms[w], ev[0], ev[1]);
-    }
-    for (auto& e : ev) cudaEventDestroy(e);
-    RET(rc);
-    tuned_bn_[np] = (ms[0] < ms[1]) ? 128 : 256;
-    if (const char* d = std::getenv("XLBOMD_DEBUG"))
-      if (d[0] && d[0] != '0')
-        std::fprintf(stderr, "[xlbomd] tile autotuner n %d, %zu problems: 128-wide %.3f ms, 256-wide %.3f ms -> %d\n",
-                     np, probs.size(), ms[0], ms[1], tuned_bn_[np]);
-    return cudaSuccess;
+    const int kind = 64 | (sym ? 1 : 0) | (e0.E ? 2 : 0) | (e0.E2 ? 4 : 0) | (e0.E64 ? 8 : 0) | (e0.V ? 16 : 0) |
+                     (e0.out64 ? 32 : 0);
+    return prof_end(s, (double)ops.size() * 2.0 * (double)np * np * np * (sym ? 0.5 : 1.0) * e0.pairs, kind);
   }
 
   cudaError_t foe(cudaStream_t s, MatSet& m, const double* H, int N, double mu, double sc,
@@ -676,18 +496,35 @@ class EngineSplit : public Engine {
     return foe_group(s, jobs, sc);
   }
 
-  // Linear combination of matrices per system into Y[i] and its operand split (mode as convert_group).
-  cudaError_t combine_group(cudaStream_t s, int np, CombList& L, const std::vector<SplitMat*>& Y, int mode) {
+  // Linear combination of matrices per system into Y[i] and its operands.
+  cudaError_t combine_group(cudaStream_t s, int np, CombList& L, const std::vector<SplitMat*>& Y, bool hi_only) {
     L.n = (int)Y.size();
     for (int i = 0; i < L.n; ++i) {
       L.Y[i] = Y[i]->f;
-      L.amax[i] = Y[i]->amax;
+      L.hi[i] = Y[i]->hi;
+      L.lo[i] = hi_only ? nullptr : Y[i]->lo;
+      L.scale[i] = Y[i]->scale;
     }
-    RET(zero_amax_group(s, Y));
-    combine_group_kernel<<<ew_grid((size_t)np * np / 4, L.n), 256, 0, s>>>(np, L);
+    combine_group_kernel<<<ew_grid((size_t)np * np / 4, L.n), 256, 0, s>>>(np, fmt_, L);
     note_launch();
-    RET(cudaGetLastError());
-    return convert_group(s, Y, np, mode);
+    return cudaGetLastError();
+  }
+
+  // operands of a matrix from its value, in place
+  cudaError_t operands(cudaStream_t s, SplitMat& m, int np) {
+    CombList L;
+    L.X[0][0] = m.f;
+    L.X[1][0] = L.X[2][0] = nullptr;
+    L.g[0][0] = L.g[2][0] = L.g[3][0] = 0.f;
+    L.g[1][0] = 1.f;
+    L.dg[0] = nullptr;
+    const std::vector<SplitMat*> Y(1, &m);
+    return combine_group(s, np, L, Y, false);
+  }
+
+  // The chains' matrices serve as scratch of the expansion and of dT_n/dmu, at the unit scale.
+  static void unit_scales(MatSet& m) {
+    for (SplitMat* x : {&m.sA1, &m.sMt, &m.sT1a, &m.sT1b, &m.sYw}) x->scale = m.scales;
   }
 
   // The recursion of every job's system in lockstep: each product of a level is one grouped
@@ -706,24 +543,26 @@ class EngineSplit : public Engine {
     for (auto& j : jobs)
       if (j.m->np != np || j.m->n != n) return cudaErrorInvalidValue;
     const size_t cnt = (size_t)np * np;
-    std::vector<SplitMat*> T0s;
     T0List tl;
     tl.n = B;
     for (int i = 0; i < B; ++i) {
       FoeJob& j = jobs[i];
-      T0s.push_back(&j.m->sT[0]);
+      MatSet& m = *j.m;
+      unit_scales(m);
       tl.N[i] = j.N;
       tl.H[i] = j.H;
       tl.mu[i] = j.mu;
-      tl.dmu[i] = j.dpar;
-      tl.T0[i] = j.m->sT[0].d;
-      tl.amax[i] = j.m->sT[0].amax;
+      tl.t0[i] = m.t0max;
+      tl.dpar[i] = j.dpar;
+      tl.T0[i] = m.sT[0].d;
+      tl.hi[i] = m.sT[0].hi;
+      tl.lo[i] = m.sT[0].lo;
+      tl.scales[i] = m.scales;
+      tl.t0_dev[i] = m.t0_dev;
     }
-    RET(zero_amax_group(s, T0s));
-    t0_init_group_kernel<<<ew_grid(cnt, B), 256, 0, s>>>(np, sc, tl);
+    t0_init_group_kernel<<<ew_grid(cnt / 4, B), 256, 0, s>>>(np, n, fmt_, kPassT0, sc, tl);
     note_launch();
     RET(cudaGetLastError());
-    RET(convert_group(s, T0s, np, 1));
     std::vector<SplitMat*> W(B), Wn(B);
     // scratch of the corrections: matrices of the response chains, which are free here
     auto Sk = [](MatSet& m, int k) -> SplitMat* { return (k & 1) ? &m.sT1b : &m.sS; };   // S_k beside S_{k-1}
@@ -749,12 +588,10 @@ class EngineSplit : public Engine {
         for (int q = 0; q < 4; ++q) cl.g[q][i] = (float)p.g[q];
         cl.dg[i] = j.dpar ? j.dpar + 1 + 4 * k : nullptr;
       }
-      RET(combine_group(s, np, cl, W, 0));
+      RET(combine_group(s, np, cl, W, false));
       for (int r = 0; r < rounds; ++r) {
         // Q = S - W - W S and P = Q - Q^2 + ..: functions of one matrix, so every product is symmetric
-        std::vector<GemmOp> oq, o2, o5, ow;
-        std::vector<SplitMat*> V;
-        CombList cv;
+        std::vector<GemmOp> oq, o2, o3, o5, ow;
         for (int i = 0; i < B; ++i) {
           FoeJob& j = jobs[i];
           const InvOrders& inv = (*j.plan)[k].inv;
@@ -769,26 +606,20 @@ class EngineSplit : public Engine {
           eq.E2 = W[i];
           eq.beta2 = -1.f;
           oq.push_back({W[i], Sk(m, k), &m.sQ, eq, j.stats});
-          if (order >= 3) {
-            Epi e2;
-            if (order == 3) {                                                    // P = Q - Q^2
-              e2.alpha = -1.f;
-              e2.E = &m.sQ;
-              e2.beta = 1.f;
-            }
-            o2.push_back({&m.sQ, &m.sQ, &m.sA1, e2, j.stats});
+          Epi e2;
+          e2.E = &m.sQ;
+          if (order == 3) {                                                      // P = Q - Q^2
+            e2.alpha = -1.f;
+            e2.beta = 1.f;
+            o3.push_back({&m.sQ, &m.sQ, &m.sA1, e2, j.stats});
             P = &m.sA1;
           }
           if (order == 5) {                                                      // P = V + V Q^2, V = Q - Q^2
-            const int c = (int)V.size();
-            V.push_back(&m.sMt);
-            cv.X[0][c] = m.sQ.f;
-            cv.X[1][c] = m.sA1.f;
-            cv.X[2][c] = nullptr;
-            cv.g[0][c] = 0.f;
-            cv.g[1][c] = 1.f;
-            cv.g[2][c] = -1.f;
-            cv.dg[c] = nullptr;
+            e2.value = false;
+            e2.V = &m.sMt;
+            e2.va = -1.f;
+            e2.vb = 1.f;
+            o2.push_back({&m.sQ, &m.sQ, &m.sA1, e2, j.stats});
             Epi e5;
             e5.E = &m.sMt;
             e5.beta = 1.f;
@@ -806,11 +637,9 @@ class EngineSplit : public Engine {
           if (j.stats) j.stats[1] += 1;
         }
         RET(gemm_group(s, np, oq, true));
+        RET(gemm_group(s, np, o3, true));
         RET(gemm_group(s, np, o2, true));
-        if (!V.empty()) {
-          RET(combine_group(s, np, cv, V, 0));
-          RET(gemm_group(s, np, o5, true));
-        }
+        RET(gemm_group(s, np, o5, true));
         RET(gemm_group(s, np, ow, true));
       }
       std::vector<GemmOp> ot;
@@ -818,8 +647,7 @@ class EngineSplit : public Engine {
         MatSet& m = *j.m;
         Epi et;                                                                   // T' = 2T - 2 T W
         et.alpha = -2.f;
-        et.E64 = m.sT[k].d;                                                       // symmetric: read transposed
-        et.e64_trans = 1;
+        et.E64 = m.sT[k].d;
         et.beta64 = 2.0f;
         et.out64 = true;
         ot.push_back({&m.sT[k], &m.sY[k], &m.sT[k + 1], et, j.stats});
@@ -848,13 +676,15 @@ class EngineSplit : public Engine {
     for (auto& j : jobs)
       if (j.m->np != np || j.m->n != n) return cudaErrorInvalidValue;
     const bool single = (mu_nseg_ == 1);
-    const int mode = single ? 2 : 0;
     Epi base;
     base.nseg = mu_nseg_;
     base.hi_only = single;
     // the matrices of the response chains and of the expansion's corrections are idle here
     std::vector<GemmOp> o1;
-    for (auto& j : jobs) o1.push_back({&j.m->sT[0], &j.m->sT[0], &j.m->sS, base, j.stats});
+    for (auto& j : jobs) {
+      unit_scales(*j.m);
+      o1.push_back({&j.m->sT[0], &j.m->sT[0], &j.m->sS, base, j.stats});
+    }
     RET(gemm_group(s, np, o1, true));
     std::vector<SplitMat*> Z(B), Zn(B), C(B);
     CombList cz;
@@ -865,6 +695,7 @@ class EngineSplit : public Engine {
       rounds = std::max(rounds, p.inv.n);
       Z[i] = &j.m->sYw;
       Zn[i] = &j.m->sT1b;
+      Z[i]->scale = Zn[i]->scale = j.m->scales + 2 + n;
       cz.X[0][i] = j.m->sS.f;
       cz.X[1][i] = cz.X[2][i] = nullptr;
       cz.g[0][i] = (float)p.z0;
@@ -872,11 +703,9 @@ class EngineSplit : public Engine {
       cz.g[2][i] = cz.g[3][i] = 0.f;
       cz.dg[i] = j.dpar;
     }
-    RET(combine_group(s, np, cz, Z, mode));
+    RET(combine_group(s, np, cz, Z, single));
     for (int r = 0; r < rounds; ++r) {
-      std::vector<GemmOp> oq, o2, o5, ow;
-      std::vector<SplitMat*> V;
-      CombList cv;
+      std::vector<GemmOp> oq, o2, o3, o5, ow;
       for (int i = 0; i < B; ++i) {
         MuJob& j = jobs[i];
         if (r >= j.plan->inv.n) continue;
@@ -888,24 +717,19 @@ class EngineSplit : public Engine {
         eq.beta = -1.f;
         eq.diag = 1.f;
         oq.push_back({&m.sS, Z[i], &m.sQ, eq, j.stats});
-        if (order >= 3) {
-          Epi e2 = base;
-          if (order == 3) {                                                       // P = R + R^2
-            e2.E = &m.sQ;
-            e2.beta = 1.f;
-          }
-          o2.push_back({&m.sQ, &m.sQ, &m.sA1, e2, j.stats});
+        Epi e2 = base;
+        e2.E = &m.sQ;
+        if (order == 3) {                                                         // P = R + R^2
+          e2.beta = 1.f;
+          o3.push_back({&m.sQ, &m.sQ, &m.sA1, e2, j.stats});
           P = &m.sA1;
         }
         if (order == 5) {                                                         // P = V + V R^2, V = R + R^2
-          const int c = (int)V.size();
-          V.push_back(&m.sMt);
-          cv.X[0][c] = m.sQ.f;
-          cv.X[1][c] = m.sA1.f;
-          cv.X[2][c] = nullptr;
-          cv.g[0][c] = cv.g[3][c] = 0.f;
-          cv.g[1][c] = cv.g[2][c] = 1.f;
-          cv.dg[c] = nullptr;
+          e2.value = false;
+          e2.V = &m.sMt;
+          e2.va = 1.f;
+          e2.vb = 1.f;
+          o2.push_back({&m.sQ, &m.sQ, &m.sA1, e2, j.stats});
           Epi e5 = base;
           e5.E = &m.sMt;
           e5.beta = 1.f;
@@ -919,11 +743,9 @@ class EngineSplit : public Engine {
         std::swap(Z[i], Zn[i]);
       }
       RET(gemm_group(s, np, oq, true));
+      RET(gemm_group(s, np, o3, true));
       RET(gemm_group(s, np, o2, true));
-      if (!V.empty()) {
-        RET(combine_group(s, np, cv, V, mode));
-        RET(gemm_group(s, np, o5, true));
-      }
+      RET(gemm_group(s, np, o5, true));
       RET(gemm_group(s, np, ow, true));
     }
     CombList cc;
@@ -952,7 +774,7 @@ class EngineSplit : public Engine {
       dl.out[i] = j.out_diag;
       maxN = std::max(maxN, j.N);
     }
-    RET(combine_group(s, np, cc, C, mode));
+    RET(combine_group(s, np, cc, C, single));
     RET(gemm_group(s, np, oc, true));
     RET(gemm_group(s, np, ot, true));
     get_diag_group_kernel<<<dim3((maxN + 255) / 256, B), 256, 0, s>>>(np, dl);
@@ -993,6 +815,16 @@ class EngineSplit : public Engine {
     // chain would add traffic and no accuracy.  The last level still writes the double-float array
     // the reductions read (with a zero low word).
     const bool single = (nseg == 1);
+    ChainScaleList sl;
+    sl.n = B;
+    for (int i = 0; i < B; ++i) {
+      sl.d[i] = jobs[i].dvec;
+      sl.t0[i] = jobs[i].m->t0_dev;
+      sl.scales[i] = jobs[i].m->chain_scales;
+    }
+    chain_scales_kernel<<<B, 256, 0, s>>>(np, n, sl);
+    note_launch();
+    RET(cudaGetLastError());
     std::vector<SplitMat*> T1(B), T1n(B), A1s(B), Mts(B);
     for (int i = 0; i < B; ++i) {
       T1[i] = &jobs[i].m->sT1a;
@@ -1002,7 +834,12 @@ class EngineSplit : public Engine {
     }
     for (int k = 0; k < n; ++k) {
       const bool last = (k == n - 1);
-      RET(zero_amax_group(s, A1s));
+      for (int i = 0; i < B; ++i) {
+        const float* cs = jobs[i].m->chain_scales + 3 * k;
+        A1s[i]->scale = cs;
+        Mts[i]->scale = cs + 1;
+        T1n[i]->scale = cs + 2;
+      }
       Epi em;                                                                    // Mt = 2 T1 - T_{k+1} A1
       em.alpha = -1.f;
       em.out64 = !single || last;
@@ -1016,10 +853,11 @@ class EngineSplit : public Engine {
         for (int i = 0; i < B; ++i) {
           al.T0[i] = jobs[i].m->sT[0].d;
           al.d[i] = jobs[i].dvec;
-          al.A1[i] = A1s[i]->f;
-          al.amax[i] = A1s[i]->amax;
+          al.hi[i] = A1s[i]->hi;
+          al.lo[i] = single ? nullptr : A1s[i]->lo;
+          al.scale[i] = A1s[i]->scale;
         }
-        level0_A1_group_kernel<<<ew_grid(cnt, B), 256, 0, s>>>(np, al);
+        level0_A1_group_kernel<<<ew_grid(cnt / 4, B), 256, 0, s>>>(np, fmt_, al);
         note_launch();
         RET(cudaGetLastError());
         for (int i = 0; i < B; ++i) {
@@ -1029,11 +867,13 @@ class EngineSplit : public Engine {
           om.push_back({&jobs[i].m->sT[k + 1], A1s[i], Mts[i], e, jobs[i].stats});
         }
       } else {
-        // A1 = T T1 + T1 T (T, T1 symmetric): one symmetric-output product over the two K pairs
+        // A1 = T T1 + T1 T (T, T1 symmetric): one symmetric-output product over the two K pairs; only
+        // its operands are needed
         std::vector<GemmOp> oa;
         for (int i = 0; i < B; ++i) {
           Epi ea;
-          ea.convert = false;
+          ea.value = false;
+          ea.hi_only = single;
           ea.nseg = nseg;
           ea.pairs = 2;
           oa.push_back({&jobs[i].m->sT[k], T1[i], A1s[i], ea, jobs[i].stats});
@@ -1042,17 +882,15 @@ class EngineSplit : public Engine {
         for (int i = 0; i < B; ++i) {
           Epi e = em;
           if (single) {
-            e.E = T1[i];                                                          // FP32, symmetric
+            e.E = T1[i];                                                          // FP32
             e.beta = 2.0f;
           } else {
-            e.E64 = T1[i]->d;                                                     // symmetric: read transposed
-            e.e64_trans = 1;
+            e.E64 = T1[i]->d;
             e.beta64 = 2.0f;
           }
           om.push_back({&jobs[i].m->sT[k + 1], A1s[i], Mts[i], e, jobs[i].stats});
         }
       }
-      RET(convert_group(s, A1s, np, single ? 2 : 0));
       RET(gemm_group(s, np, om, false));
       if (last) {
         DiagList dl;
@@ -1071,20 +909,19 @@ class EngineSplit : public Engine {
       }
       std::vector<GemmOp> oy;
       for (int i = 0; i < B; ++i) {
-        Epi ey;                                                                  // T1' = M - W M
-        ey.alpha = -1.f;
+        Epi ey;                                                                  // T1' = Mt - Mt W
+        ey.alpha = -1.f;                                                         // (symmetric: = M - W M)
         if (single) {
-          ey.E = Mts[i];                                                          // read transposed: M
+          ey.E = Mts[i];
           ey.beta = 1.0f;
           ey.hi_only = true;
         } else {
           ey.E64 = Mts[i]->d;
           ey.beta64 = 1.0f;
-          ey.e64_trans = 1;
           ey.out64 = true;
         }
         ey.nseg = nseg;
-        oy.push_back({&jobs[i].m->sY[k], Mts[i], T1n[i], ey, jobs[i].stats});
+        oy.push_back({Mts[i], &jobs[i].m->sY[k], T1n[i], ey, jobs[i].stats});
       }
       RET(gemm_group(s, np, oy, true));
       std::swap(T1, T1n);
@@ -1138,14 +975,11 @@ class EngineSplit : public Engine {
   int* err_ = nullptr;
 
  private:
-  int chunk_kb() const { return fmt_ == 2 ? 2 * kChunkKb : kChunkKb; }   // K blocks per 1024-long chunk
-
   int fmt_;   // operand format: 0 FP16, 1 BF16, 2 TF32
   int probe_nseg_ = 3;
   int mu_nseg_ = 3;
   std::unordered_map<int, std::pair<int*, TcTiles>> tiles_;
   TcGroupCache* group_cache_ = nullptr;
-  std::unordered_map<int, int> tuned_bn_;   // grouped products: tile width per size
 };
 
 // which value arrays a matrix keeps
@@ -1153,7 +987,7 @@ enum { kF = 1, kD = 2 };
 
 // Zeroing runs on the stream `s` that later uses the matrix.
 // esz: bytes of one operand element (2: FP16/BF16, 4: TF32)
-cudaError_t alloc_split(SplitMat& m, int np, int esz, float* scal_f, unsigned* scal_u, int what, cudaStream_t s) {
+cudaError_t alloc_split(SplitMat& m, int np, int esz, const float* scale, int what, cudaStream_t s) {
   const size_t cnt = (size_t)np * np;
   if (what & kF) {
     RET(cudaMalloc((void**)&m.f, cnt * sizeof(float)));
@@ -1167,8 +1001,7 @@ cudaError_t alloc_split(SplitMat& m, int np, int esz, float* scal_f, unsigned* s
   RET(cudaMalloc((void**)&m.lo, cnt * esz));
   RET(cudaMemsetAsync(m.hi, 0, cnt * esz, s));
   RET(cudaMemsetAsync(m.lo, 0, cnt * esz, s));
-  m.scale = scal_f;
-  m.amax = scal_u;
+  m.scale = scale;
   return cudaSuccess;
 }
 
@@ -1197,33 +1030,23 @@ Engine* make_split_engine(int prec) {
 
 cudaError_t alloc_matset_split(MatSet& m, cudaStream_t s) {
   const int np = m.np, n = m.n, esz = operand_bytes(m.prec);
-  const int nmat = (n + 1) + n + 9;
-  float* scal = nullptr;
-  RET(cudaMalloc((void**)&scal, sizeof(float) * 2 * nmat));
-  RET(cudaMemsetAsync(scal, 0, sizeof(float) * 2 * nmat, s));
-  m.tc_plan = scal;
-  float* sf = scal;
-  unsigned* su = reinterpret_cast<unsigned*>(scal + nmat);
-  int idx = 0;
+  const size_t nscale = 3 + (size_t)n + 3 * (size_t)n + 1;
+  RET(cudaMalloc((void**)&m.scales, sizeof(float) * nscale));
+  std::vector<float> init(nscale, kUnitScale);
+  RET(cudaMemcpyAsync(m.scales, init.data(), sizeof(float) * nscale, cudaMemcpyHostToDevice, s));
+  RET(cudaStreamSynchronize(s));   // init is a host temporary
+  m.chain_scales = m.scales + 3 + n;
+  m.t0_dev = m.chain_scales + 3 * n;
   m.sT.assign(n + 1, SplitMat());
   m.sY.assign(n, SplitMat());
-  for (auto& x : m.sT) {
-    RET(alloc_split(x, np, esz, sf + idx, su + idx, kD, s));
-    ++idx;
-  }
-  for (auto& x : m.sY) {
-    RET(alloc_split(x, np, esz, sf + idx, su + idx, kF, s));
-    ++idx;
-  }
+  for (int k = 0; k <= n; ++k) RET(alloc_split(m.sT[k], np, esz, m.scales + 1 + k, kD, s));
+  for (auto& x : m.sY) RET(alloc_split(x, np, esz, m.scales, kF, s));
   struct W {
     SplitMat* m;
     int what;
   } w[] = {{&m.sS, kF},  {&m.sQ, kF},  {&m.sYw, kF},  {&m.sA1, kF},
            {&m.sMt, kD | kF}, {&m.sT1a, kD | kF}, {&m.sT1b, kD | kF}, {&m.sTmu, kD}};
-  for (auto& x : w) {
-    RET(alloc_split(*x.m, np, esz, sf + idx, su + idx, x.what, s));
-    ++idx;
-  }
+  for (auto& x : w) RET(alloc_split(*x.m, np, esz, m.scales, x.what, s));
   return cudaSuccess;
 }
 
@@ -1234,29 +1057,26 @@ cudaError_t alloc_chain_slot(MatSet& slot, const MatSet& base, cudaStream_t s) {
   slot = base;
   slot.e64[0] = slot.e64[1] = slot.e64[2] = slot.e64[3] = slot.e64[4] = slot.e64[5] = slot.e64[6] = nullptr;
   const int np = base.np, esz = operand_bytes(base.prec);
-  float* scal = nullptr;
-  RET(cudaMalloc((void**)&scal, sizeof(float) * 2 * 5));
-  RET(cudaMemsetAsync(scal, 0, sizeof(float) * 2 * 5, s));
-  slot.tc_plan = scal;
+  slot.chain_scales = nullptr;
+  RET(cudaMalloc((void**)&slot.chain_scales, sizeof(float) * 3 * (size_t)base.n));
   slot.sA1 = SplitMat();
   slot.sMt = SplitMat();
   slot.sT1a = SplitMat();
   slot.sT1b = SplitMat();
   slot.sTmu = SplitMat();
-  unsigned* su = reinterpret_cast<unsigned*>(scal + 5);
-  RET(alloc_split(slot.sA1, np, esz, scal + 0, su + 0, kF, s));
-  RET(alloc_split(slot.sMt, np, esz, scal + 1, su + 1, kD | kF, s));
-  RET(alloc_split(slot.sT1a, np, esz, scal + 2, su + 2, kD | kF, s));
-  RET(alloc_split(slot.sT1b, np, esz, scal + 3, su + 3, kD | kF, s));
-  RET(alloc_split(slot.sTmu, np, esz, scal + 4, su + 4, kD, s));
+  RET(alloc_split(slot.sA1, np, esz, base.scales, kF, s));
+  RET(alloc_split(slot.sMt, np, esz, base.scales, kD | kF, s));
+  RET(alloc_split(slot.sT1a, np, esz, base.scales, kD | kF, s));
+  RET(alloc_split(slot.sT1b, np, esz, base.scales, kD | kF, s));
+  RET(alloc_split(slot.sTmu, np, esz, base.scales, kD, s));
   return cudaSuccess;
 }
 
 void free_chain_slot(MatSet& slot) {
   SplitMat* w[] = {&slot.sA1, &slot.sMt, &slot.sT1a, &slot.sT1b, &slot.sTmu};
   for (SplitMat* x : w) free_split(*x);
-  if (slot.tc_plan) cudaFree(slot.tc_plan);
-  slot.tc_plan = nullptr;
+  if (slot.chain_scales) cudaFree(slot.chain_scales);
+  slot.chain_scales = nullptr;
   slot.sT.clear();
   slot.sY.clear();
 }
@@ -1273,8 +1093,8 @@ void free_matset_split(MatSet& m) {
   m.sY.clear();
   SplitMat* w[] = {&m.sS, &m.sQ, &m.sYw, &m.sA1, &m.sMt, &m.sT1a, &m.sT1b, &m.sTmu};
   for (SplitMat* x : w) free_split(*x);
-  if (m.tc_plan) cudaFree(m.tc_plan);
-  m.tc_plan = nullptr;
+  if (m.scales) cudaFree(m.scales);
+  m.scales = m.chain_scales = m.t0_dev = nullptr;
   for (double*& p : m.e64) {
     if (p) cudaFree(p);
     p = nullptr;
@@ -1301,14 +1121,9 @@ __global__ void fill_random_kernel(size_t count, int np, uint64_t seed, int sym,
   out[idx] = ((double)(z >> 11) * (1.0 / 9007199254740992.0)) * 2.0 - 1.0;
 }
 
-__global__ void to_f32_kernel(size_t count, const double* __restrict__ x, float* __restrict__ f, unsigned* amax) {
+__global__ void to_f32_kernel(size_t count, const double* __restrict__ x, float* __restrict__ f) {
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  float v = 0.0f;
-  if (idx < count) {
-    v = (float)x[idx];
-    f[idx] = v;
-  }
-  raise_amax(amax, v);
+  if (idx < count) f[idx] = (float)x[idx];
 }
 
 __global__ void diff_f32_kernel(size_t count, const float* __restrict__ a, const float* __restrict__ b,
@@ -1397,25 +1212,22 @@ int selftest_gemm_group(int n, int prec, int mode, int nprob, double* result) {
   float* scal = nullptr;
   int rc = -2;
   std::vector<double> worst(1, 0.0);
-  if (cudaMalloc((void**)&tmp, cnt * 8) || cudaMalloc((void**)&out, 8) ||
-      cudaMalloc((void**)&scal, 8 * nprob * sizeof(float)))
+  if (cudaMalloc((void**)&tmp, cnt * 8) || cudaMalloc((void**)&out, 8) || cudaMalloc((void**)&scal, sizeof(float)) ||
+      cudaMemcpy(scal, &kUnitScale, sizeof(float), cudaMemcpyHostToDevice))
     goto done;
-  cudaMemset(scal, 0, 8 * nprob * sizeof(float));
   for (int i = 0; i < nprob; ++i) {
-    float* sf = scal + 4 * i;
-    unsigned* su = reinterpret_cast<unsigned*>(scal + 4 * nprob + 4 * i);
-    if (alloc_split(A[i], n, esz, sf, su, kF, nullptr) || alloc_split(B[i], n, esz, sf + 1, su + 1, kF, nullptr) ||
-        alloc_split(C[i], n, esz, sf + 2, su + 2, kF, nullptr) || alloc_split(R[i], n, esz, sf + 3, su + 3, kF, nullptr))
+    if (alloc_split(A[i], n, esz, scal, kF, nullptr) || alloc_split(B[i], n, esz, scal, kF, nullptr) ||
+        alloc_split(C[i], n, esz, scal, kF, nullptr) || alloc_split(R[i], n, esz, scal, kF, nullptr))
       goto done;
     fill_random_kernel<<<nblk(cnt), 256>>>(cnt, n, 101 + 7 * i, 0, tmp);
     note_launch();
-    to_f32_kernel<<<nblk(cnt), 256>>>(cnt, tmp, A[i].f, A[i].amax);
+    to_f32_kernel<<<nblk(cnt), 256>>>(cnt, tmp, A[i].f);
     note_launch();
     fill_random_kernel<<<nblk(cnt), 256>>>(cnt, n, 203 + 11 * i, sym, tmp);
     note_launch();
-    to_f32_kernel<<<nblk(cnt), 256>>>(cnt, tmp, B[i].f, B[i].amax);
+    to_f32_kernel<<<nblk(cnt), 256>>>(cnt, tmp, B[i].f);
     note_launch();
-    if (eng.convert(nullptr, A[i], n) || eng.convert(nullptr, B[i], n)) goto done;
+    if (eng.operands(nullptr, A[i], n) || eng.operands(nullptr, B[i], n)) goto done;
   }
   {
     Epi ep;
@@ -1426,9 +1238,7 @@ int selftest_gemm_group(int n, int prec, int mode, int nprob, double* result) {
       if (eng.gemm(nullptr, n, A[i], B[i], R[i], ep, sym != 0, nullptr)) goto done;
     std::vector<EngineSplit::GemmOp> ops;
     for (int i = 0; i < nprob; ++i) ops.push_back({&A[i], &B[i], &C[i], ep, nullptr});
-    // the autotuner runs both widths on the first grouped product of this size; then the
-    // chosen width; compare after each
-    for (int rep = 0; rep < 2; ++rep) {
+    for (int rep = 0; rep < 2; ++rep) {   // the second launch reads the table that the first one built
       if (eng.gemm_group(nullptr, n, ops, sym != 0)) goto done;
       for (int i = 0; i < nprob; ++i) {
         if (cudaMemset(out, 0, 8)) goto done;
@@ -1480,22 +1290,22 @@ int selftest_gemm(int n, int prec, int sym, double* result) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   float ms = 0.f;
   if (cudaMalloc((void**)&A, cnt * 8) || cudaMalloc((void**)&B, cnt * 8) || cudaMalloc((void**)&Cref, cnt * 8) ||
-      cudaMalloc((void**)&out, 8) || cudaMalloc((void**)&scal, 6 * sizeof(float)) ||
+      cudaMalloc((void**)&out, 8) || cudaMalloc((void**)&scal, sizeof(float)) ||
       (pair && cudaMalloc((void**)&Cref2, cnt * 8)))
     goto done;
-  cudaMemset(scal, 0, 6 * sizeof(float));
-  if (alloc_split(sa, n, esz, scal, (unsigned*)scal + 3, kF, s) || alloc_split(sb, n, esz, scal + 1, (unsigned*)scal + 4, kF, s) ||
-      alloc_split(sc, n, esz, scal + 2, (unsigned*)scal + 5, kF, s))
+  cudaMemcpy(scal, &kUnitScale, sizeof(float), cudaMemcpyHostToDevice);
+  if (alloc_split(sa, n, esz, scal, kF, s) || alloc_split(sb, n, esz, scal, kF, s) ||
+      alloc_split(sc, n, esz, scal, kF, s))
     goto done;
   fill_random_kernel<<<nblk(cnt), 256>>>(cnt, n, 11, 0, A);
   note_launch();
   fill_random_kernel<<<nblk(cnt), 256>>>(cnt, n, 23, sym, B);
   note_launch();
-  to_f32_kernel<<<nblk(cnt), 256>>>(cnt, A, sa.f, sa.amax);
+  to_f32_kernel<<<nblk(cnt), 256>>>(cnt, A, sa.f);
   note_launch();
-  to_f32_kernel<<<nblk(cnt), 256>>>(cnt, B, sb.f, sb.amax);
+  to_f32_kernel<<<nblk(cnt), 256>>>(cnt, B, sb.f);
   note_launch();
-  if (eng.convert(s, sa, n) || eng.convert(s, sb, n)) goto done;
+  if (eng.operands(s, sa, n) || eng.operands(s, sb, n)) goto done;
   {
     EpiF64 e;
     if (gemm_f64_nt(s, n, n, n, A, n, B, n, Cref, n, e, sym == 1)) goto done;

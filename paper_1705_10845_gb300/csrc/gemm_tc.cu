@@ -5,28 +5,27 @@
 // A_hi B_hi + A_hi B_lo + A_lo B_hi (one, A_hi B_hi, for single-product
 // chains); the operands carry power-of-two scales that the epilogue removes.
 //
-// Two kernels share the pipeline.  The default is persistent: one CTA per SM
-// walks the 128 x BN output tiles.  The other (XLBOMD_GEMM=classic) gives
-// each CTA one tile.  Warp 0 issues TMA loads (128-byte swizzle, K-major) into
-// a STAGES-deep ring guarded by mbarriers; warp 1 allocates TMEM and one
-// elected thread issues tcgen05.mma (M = 128, N = BN, K = 16) per 32-byte K
-// step; warps 2-5 wait for the accumulators, read them with tcgen05.ld (32
-// lanes x 32 columns per load), apply the epilogue and store FP32 or
-// double-float rows (and the mirrored columns of a symmetric product).  In the
-// persistent kernel the epilogue folds accumulator 0 into accumulator 1 and
-// releases it at once, so the next tile's first K blocks overlap the rest of
-// the epilogue.
+// The default kernel is persistent: one CTA per SM walks the 128 x BN output
+// tiles, BN = 32 to 256 by size (pick_width).  Warp 0 issues TMA loads
+// (128-byte swizzle, K-major) into a ring guarded by mbarriers; one thread of
+// warp 1 issues tcgen05.mma (M = 128, N = BN, K = 16) per 32-byte K step; the
+// epilogue warps read finished chunks of the sum with tcgen05.ld, add them up in
+// registers, and write the value and the operands (hi, lo) that the next
+// products read.  Two others are kept beside it: one tile per CTA
+// (XLBOMD_GEMM=classic) and a two-SM form (XLBOMD_GEMM=pair).
+//
+// Against the version that wrote FP32 values, raised each matrix's maximum
+// and left the operands to a conversion pass (memset, product, conversion; 128- or
+// 256-wide tiles), per product: n = 128 27 -> 8.5 us, 256 44 -> 10.6, 640 37 -> 16, 1024
+// 60 -> 22, 2048 82 -> 60 (symmetric 83 -> 48), 8192 2.31 -> 2.30 ms with sums half as long.
 //
 // The tensor core adds each K = 16 step into its FP32 accumulator with
 // truncation, so a small term added to a large accumulator loses bits.  The
 // hi*hi segment and the two correction segments (hi*lo, lo*hi, about 2^-11
-// smaller) therefore go to two separate TMEM accumulators (2 x BN columns)
-// that the epilogue adds in FP32.  Products of large n also split the hi*hi
-// sum over the two accumulators (split_acc), since the truncation error of a
-// sum grows with its length.  A pair product (pairs = 2) adds the swapped
-// operands as a second K range, C = A B^T + B A^T.  Every mbarrier wait is
-// bounded: on timeout the kernel records an error code and leaves its loops,
-// and TMEM is always released.
+// smaller) therefore never share an accumulator.  A pair product (pairs = 2) adds
+// the swapped operands as a second K range, C = A B^T + B A^T.  Every mbarrier
+// wait is bounded: on timeout the kernel records an error code and leaves its
+// loops, and TMEM is always released.
 //
 // TF32 operands (fmt = 2, persistent kernel only) are FP32 words whose low 13
 // mantissa bits are zero.  A 128-byte swizzle row then holds 32 elements, and
@@ -44,6 +43,7 @@
 #include <string>
 #include <unordered_map>
 
+#include "operand.cuh"
 #include "precision.h"
 #include "tc.h"
 
@@ -52,7 +52,7 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int BK = 64;           // 64 x 16-bit = 128 bytes: one swizzle row
-constexpr int STAGES = 4;
+constexpr int STAGES = 4;        // one-CTA-per-tile kernel
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int kWaitLimit = 1 << 24;
 constexpr int kGroupM = 16;
@@ -193,23 +193,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-      "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
-      "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
-      "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])),
-      "r"(__float_as_uint(v[11])), "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])),
-      "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15])), "r"(__float_as_uint(v[16])),
-      "r"(__float_as_uint(v[17])), "r"(__float_as_uint(v[18])), "r"(__float_as_uint(v[19])),
-      "r"(__float_as_uint(v[20])), "r"(__float_as_uint(v[21])), "r"(__float_as_uint(v[22])),
-      "r"(__float_as_uint(v[23])), "r"(__float_as_uint(v[24])), "r"(__float_as_uint(v[25])),
-      "r"(__float_as_uint(v[26])), "r"(__float_as_uint(v[27])), "r"(__float_as_uint(v[28])),
-      "r"(__float_as_uint(v[29])), "r"(__float_as_uint(v[30])), "r"(__float_as_uint(v[31]))
-      : "memory");
-}
-
 // 64 columns of this warp's 32 lanes, without waiting (tcgen05.wait::ld before use)
 __device__ __forceinline__ void tmem_ld64_nowait(uint32_t taddr, uint32_t (&r)[64]) {
   asm volatile(
@@ -312,23 +295,17 @@ __device__ __forceinline__ int acc1_start(const TcArgs& a, int nk) {
   return a.split_acc ? a.pairs * nk / 2 : a.pairs * nk;
 }
 
-// L2 prefetch of the side inputs of tile (tm, tn) by the 128 epilogue threads (t = 0..127)
-template <int BN>
-__device__ __forceinline__ void prefetch_sides(const TcArgs& a, int tm, int tn, int t) {
-  const int r = tm * BM + t;
+// L2 prefetch of the side inputs of the 128 x BN tile (tm, tn) by nt epilogue threads
+template <int BN, typename Args>
+__device__ __forceinline__ void prefetch_sides(const Args& a, int tm, int tn, int t, int nt) {
   const float* fsides[2] = {a.E, a.E2};
   for (int k = 0; k < 2; ++k)
     if (fsides[k])
-      for (int rr = t; rr < BN; rr += 128)
-        for (int c = 0; c < BM; c += 32) prefetch_l2(fsides[k] + (size_t)(tn * BN + rr) * a.ldc + tm * BM + c);
-  if (a.E64) {
-    if (a.e64_trans) {
-      for (int rr = t; rr < BN; rr += 128)
-        for (int c = 0; c < BM; c += 16) prefetch_l2(a.E64 + (size_t)(tn * BN + rr) * a.ldc + tm * BM + c);
-    } else {
-      for (int c = 0; c < BN; c += 16) prefetch_l2(a.E64 + (size_t)r * a.ldc + tn * BN + c);
-    }
-  }
+      for (int i = t; i < BM * (BN / 32); i += nt)
+        prefetch_l2(fsides[k] + (size_t)(tm * BM + i / (BN / 32)) * a.ldc + tn * BN + (i % (BN / 32)) * 32);
+  if (a.E64)
+    for (int i = t; i < BM * (BN / 16); i += nt)
+      prefetch_l2(a.E64 + (size_t)(tm * BM + i / (BN / 16)) * a.ldc + tn * BN + (i % (BN / 16)) * 16);
 }
 
 // a + b for a double-float a and a float b (Knuth two-sum, then renormalise)
@@ -340,94 +317,270 @@ __device__ __forceinline__ float2 df_add(float2 a, float b) {
   return make_float2(hi, err - (hi - s));
 }
 
-// Epilogue of one 32-column chunk: v holds this lane's row `row`, columns
-// col0 .. col0 + 31 of the raw accumulator sum; scales, adds the side inputs
-// and the diagonal, stores through the per-warp staging tiles tx, ty (32 x 33),
-// and raises vmax.
-__device__ __forceinline__ void epilogue_chunk(const TcArgs& a, float (&v)[32], int row, int row0, int col0,
-                                               int lane, float (*tx)[33], float (*ty)[33], float inv,
-                                               float& vmax) {
+// The epilogue's arguments in registers.  (Read through a reference to the kernel parameter or to a
+// grouped launch's table they are loaded again after every store: 4 us per 32 x 32 chunk.)
+struct EpiRegs {
+  const float *E, *E2;
+  const float2* E64;
+  const double* dvec;
+  float beta, beta2, beta64, diag, dvec_scale, va, vb, inv, so, so2;
+  float *f, *f2;
+  float2* d;
+  void *hi, *lo, *hi2, *lo2;
+  int ldc, ndvec, fmt;
+  bool sym;
+};
+
+__device__ __forceinline__ EpiRegs load_epi(const TcArgs& a) {
+  EpiRegs e;
+  e.E = a.E;
+  e.E2 = a.E2;
+  e.E64 = a.E64;
+  e.dvec = a.dvec;
+  e.beta = a.beta;
+  e.beta2 = a.beta2;
+  e.beta64 = a.beta64;
+  e.diag = a.diag;
+  e.dvec_scale = a.dvec_scale;
+  e.va = a.va;
+  e.vb = a.vb;
+  e.inv = a.alpha / (__ldg(a.sa) * __ldg(a.sb));
+  e.f = a.out.f;
+  e.d = a.out.d;
+  e.hi = a.out.hi;
+  e.lo = a.out.lo;
+  e.so = a.out.hi ? __ldg(a.out.scale) : 0.0f;
+  e.f2 = a.out2.f;
+  e.hi2 = a.out2.hi;
+  e.lo2 = a.out2.lo;
+  e.so2 = a.out2.hi ? __ldg(a.out2.scale) : 0.0f;
+  e.ldc = a.ldc;
+  e.ndvec = a.ndvec;
+  e.fmt = a.fmt;
+  e.sym = a.sym != 0;
+  return e;
+}
+
+// 4 x 4 values x + xl: four neighbouring columns at element i and every st-th one after it.
+template <int FMT>
+__device__ __forceinline__ void store_operands(void* hi, void* lo, float s, size_t i, size_t st, const float (&x)[4][4],
+                                               const float (&xl)[4][4]) {
+  if (lo) {
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] *= inv;
-  // FP32 side inputs of symmetric value, read transposed: for a fixed
-  // column the 32 lanes read 32 consecutive rows (coalesced)
-  if (a.E) {
+    for (int q = 0; q < 4; ++q) store_operand4<FMT>(hi, lo, i + q * st, s, x[q], xl[q]);
+  } else {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] += a.beta * a.E[(size_t)(col0 + i) * a.ldc + row];
+    for (int q = 0; q < 4; ++q) store_operand4<FMT>(hi, nullptr, i + q * st, s, x[q], xl[q]);
   }
-  if (a.E2) {
+}
+
+template <bool TF32>
+__device__ __forceinline__ void store_out(float* f, float2* d, void* hi, void* lo, int fmt, float s, size_t i, size_t st,
+                                          const float (&x)[4][4], const float (&xl)[4][4]) {
+  if (f) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] += a.beta2 * a.E2[(size_t)(col0 + i) * a.ldc + row];
+    for (int q = 0; q < 4; ++q)
+      *reinterpret_cast<float4*>(f + i + q * st) = make_float4(x[q][0], x[q][1], x[q][2], x[q][3]);
   }
-  const int dc = row - col0;   // diagonal column of this lane, if in the chunk
-  if (dc >= 0 && dc < 32) {
-    float dd = a.diag;
-    if (a.dvec && row < a.ndvec) dd += a.dvec_scale * (float)a.dvec[row];
+  if (d) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i)
-      if (i == dc) v[i] += dd;
+    for (int q = 0; q < 4; ++q) {
+      float4* p = reinterpret_cast<float4*>(d + i + q * st);
+      p[0] = make_float4(x[q][0], xl[q][0], x[q][1], xl[q][1]);
+      p[1] = make_float4(x[q][2], xl[q][2], x[q][3], xl[q][3]);
+    }
   }
-  if (a.C64) {
-    // double-float value: exact leading term beta64 E64 plus the FP32 part
-    float hi[32], lo[32];
-    if (a.E64 && a.e64_trans) {
+  if (hi) {
+    if constexpr (TF32)
+      store_operands<2>(hi, lo, s, i, st, x, xl);
+    else if (fmt)
+      store_operands<1>(hi, lo, s, i, st, x, xl);
+    else
+      store_operands<0>(hi, lo, s, i, st, x, xl);
+  }
+}
+
+// 4 x 4 values of a side input; on a diagonal chunk from its upper triangle.
+__device__ __forceinline__ void load_side(float (&e)[4][4], const float* __restrict__ E, size_t i, size_t st, bool dg,
+                                          int row, int col, int ldc) {
+  if (!dg) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const float2 e = a.E64[(size_t)(col0 + i) * a.ldc + row];
-        const float2 x = df_add(make_float2(a.beta64 * e.x, a.beta64 * e.y), v[i]);
-        hi[i] = x.x;
-        lo[i] = x.y;
-      }
-    } else if (a.E64) {
-#pragma unroll 8
-      for (int i = 0; i < 32; ++i) {
-        const float2 e = a.E64[(size_t)(row0 + i) * a.ldc + col0 + lane];
-        tx[i][lane] = e.x;
-        ty[i][lane] = e.y;
-      }
-      __syncwarp();
+    for (int q = 0; q < 4; ++q) {
+      const float4 w = *reinterpret_cast<const float4*>(E + i + q * st);
+      e[q][0] = w.x;
+      e[q][1] = w.y;
+      e[q][2] = w.z;
+      e[q][3] = w.w;
+    }
+  } else {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const float2 x = df_add(make_float2(a.beta64 * tx[lane][i], a.beta64 * ty[lane][i]), v[i]);
-        hi[i] = x.x;
-        lo[i] = x.y;
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int r = row + 4 * q, c = col + k;
+        e[q][k] = E[(size_t)min(r, c) * ldc + max(r, c)];
       }
-      __syncwarp();
+  }
+}
+
+__device__ __forceinline__ void axpy44(float (&x)[4][4], float b, const float (&e)[4][4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[q][k] += b * e[q][k];
+}
+
+// Epilogue of one 32 x 32 chunk at (row0, col0), whose scaled sums are in the warp's staging tile t.  A
+// lane takes columns 4 (l % 8) .. + 3 of rows l / 8, + 4, + 8, + 12 (and the same of the lower 16 rows), so
+// that every side input is read and every result written in 16-byte pieces of whole rows (8 bytes of
+// 16-bit operands), and each option is decided once per 16 values: with a branch per value group the
+// chunk took 5 to 10 us of a small product's 20.  A symmetric product skips chunks below the
+// diagonal and writes the others a second time, transposed: FP32 results through the staging tile,
+// double-float results (two words, for which the tile has no room) read back from where this warp
+// has just stored them.  Diagonal chunks take their upper triangle for both halves.
+template <bool TF32>
+__device__ __forceinline__ void epilogue_chunk(const EpiRegs& a, int row0, int col0, int lane, float (*t)[33]) {
+  const bool dg = a.sym && col0 == row0;
+  const int lr = lane >> 3, lc = (lane & 7) * 4;
+  const size_t st = 4 * (size_t)a.ldc;
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    const int r0 = 16 * h + lr, row = row0 + r0, col = col0 + lc;
+    const size_t i = (size_t)row * a.ldc + col;
+    float x[4][4], xl[4][4], e[4][4], e2[4][4];
+    if (a.E) load_side(e, a.E, i, st, dg, row, col, a.ldc);
+    if (a.E2) load_side(e2, a.E2, i, st, dg, row, col, a.ldc);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) xl[q][k] = 0.0f;
+    if (!dg) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[q][k] = t[r0 + 4 * q][lc + k];
     } else {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        hi[i] = v[i];
-        lo[i] = 0.0f;
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int r = r0 + 4 * q, c = lc + k;
+          x[q][k] = t[min(r, c)][max(r, c)];
+        }
+    }
+    if (a.E && a.beta != 0.0f) axpy44(x, a.beta, e);
+    if (a.E2) axpy44(x, a.beta2, e2);
+    if (row0 == col0 && (a.diag != 0.0f || a.dvec)) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = row + 4 * q, dc = r - col;
+        if (dc >= 0 && dc < 4) {
+          float dd = a.diag;
+          if (a.dvec && r < a.ndvec) dd += a.dvec_scale * (float)a.dvec[r];
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (k == dc) x[q][k] += dd;
+        }
       }
     }
+    if (a.hi2) {
+      float y[4][4];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int col = col0 + i;
-      if (!a.sym || col >= row) vmax = fmaxf(vmax, fabsf(hi[i]));
-      if (a.sym && col > row) a.C64[(size_t)col * a.ldc + row] = make_float2(hi[i], lo[i]);
-      tx[lane][i] = hi[i];
-      ty[lane][i] = lo[i];
-    }
-    __syncwarp();
-    for (int i = 0; i < 32; ++i) {
-      const int r = row0 + i, c = col0 + lane;
-      if (!a.sym || c >= r) a.C64[(size_t)r * a.ldc + c] = make_float2(tx[i][lane], ty[i][lane]);
-    }
-    __syncwarp();
-    return;
-  }
+      for (int q = 0; q < 4; ++q)
 #pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const int col = col0 + i;
-    if (!a.sym || col >= row) vmax = fmaxf(vmax, fabsf(v[i]));
-    if (a.sym && col > row) a.C[(size_t)col * a.ldc + row] = v[i];
-    tx[lane][i] = v[i];
+        for (int k = 0; k < 4; ++k) y[q][k] = a.va * x[q][k];
+      axpy44(y, a.vb, e);
+      store_out<TF32>(a.f2, nullptr, a.hi2, a.lo2, a.fmt, a.so2, i, st, y, xl);
+    }
+    if (a.E64) {
+      if (!dg) {
+        float4 w[4][2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4* p = reinterpret_cast<const float4*>(a.E64 + i + q * st);
+          w[q][0] = p[0];
+          w[q][1] = p[1];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float eh[4] = {w[q][0].x, w[q][0].z, w[q][1].x, w[q][1].z};
+          const float el[4] = {w[q][0].y, w[q][0].w, w[q][1].y, w[q][1].w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float2 z = df_add(make_float2(a.beta64 * eh[k], a.beta64 * el[k]), x[q][k]);
+            x[q][k] = z.x;
+            xl[q][k] = z.y;
+          }
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int r = row + 4 * q, c = col + k;
+            const float2 e = a.E64[(size_t)min(r, c) * a.ldc + max(r, c)];
+            const float2 z = df_add(make_float2(a.beta64 * e.x, a.beta64 * e.y), x[q][k]);
+            x[q][k] = z.x;
+            xl[q][k] = z.y;
+          }
+      }
+    }
+    if (a.sym && !dg && !a.d) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t[r0 + 4 * q][lc + k] = x[q][k];
+    }
+    store_out<TF32>(a.f, a.d, a.hi, a.lo, a.fmt, a.so, i, st, x, xl);
   }
   __syncwarp();
-  for (int i = 0; i < 32; ++i) {
-    const int r = row0 + i, c = col0 + lane;
-    if (!a.sym || c >= r) a.C[(size_t)r * a.ldc + c] = tx[i][lane];
+  if (!a.sym || dg) return;
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    const int c0 = 16 * h + lr;   // output rows col0 + c0, + 4, ..; columns row0 + lc ..
+    const size_t i = (size_t)(col0 + c0) * a.ldc + row0 + lc;
+    float x[4][4], xl[4][4];
+    if (a.d) {
+      float2 z[4][4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) z[q][k] = a.d[(size_t)(row0 + lc + k) * a.ldc + col0 + c0 + 4 * q];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          x[q][k] = z[q][k].x;
+          xl[q][k] = z[q][k].y;
+        }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          x[q][k] = t[lc + k][c0 + 4 * q];
+          xl[q][k] = 0.0f;
+        }
+    }
+    if (a.hi2) {
+      float y[4][4], e[4][4];
+      load_side(e, a.E, i, st, false, 0, 0, a.ldc);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) y[q][k] = a.va * x[q][k];
+      axpy44(y, a.vb, e);
+      store_out<TF32>(a.f2, nullptr, a.hi2, a.lo2, a.fmt, a.so2, i, st, y, xl);
+    }
+    store_out<TF32>(a.f, a.d, a.hi, a.lo, a.fmt, a.so, i, st, x, xl);
   }
+  __syncwarp();
+}
+
+// 32 accumulator columns of this lane's row, scaled, into the warp's staging tile
+__device__ __forceinline__ void stage_chunk(const float (&v)[32], float inv, int lane, float (*t)[33]) {
+#pragma unroll
+  for (int i = 0; i < 32; ++i) t[lane][i] = v[i] * inv;
   __syncwarp();
 }
 
@@ -544,36 +697,15 @@ __global__ void __launch_bounds__(192, 1)
   } else {
     // epilogue warps 2..5: TMEM lanes 32 * (warp % 4) ..
     const int q = warp & 3;
-    {
-      // while the tensor cores run, pull this tile's side inputs into L2
-      const int t = (warp - 2) * 32 + lane;            // 0..127
-      const int r = tm * BM + t;
-      const float* fsides[2] = {a.E, a.E2};
-      for (int k = 0; k < 2; ++k)
-        if (fsides[k])
-          for (int rr = t; rr < BN; rr += 128)
-            for (int c = 0; c < BM; c += 32) prefetch_l2(fsides[k] + (size_t)(tn * BN + rr) * a.ldc + tm * BM + c);
-      if (a.E64) {
-        if (a.e64_trans) {
-          for (int rr = t; rr < BN; rr += 128)
-            for (int c = 0; c < BM; c += 16) prefetch_l2(a.E64 + (size_t)(tn * BN + rr) * a.ldc + tm * BM + c);
-        } else {
-          for (int c = 0; c < BN; c += 16) prefetch_l2(a.E64 + (size_t)r * a.ldc + tn * BN + c);
-        }
-      }
-    }
+    prefetch_sides<BN>(a, tm, tn, (warp - 2) * 32 + lane, 128);   // while the tensor cores run
     if (!mbar_wait(accf, 0)) {
       if (lane == 0) atomicExch(a.err, 3);
     } else {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int row0 = tm * BM + q * 32;
-      const int row = row0 + lane;
-      const float inv = a.alpha / (__ldg(a.sa) * __ldg(a.sb));
-      // per-warp 32 x 33 staging tiles in the (now idle) operand ring, so that
-      // side inputs are loaded and outputs stored as whole 128-byte rows
-      float(*tx)[33] = reinterpret_cast<float(*)[33]>(sA + q * (2 * 32 * 33 * 4));
-      float(*ty)[33] = reinterpret_cast<float(*)[33]>(sA + q * (2 * 32 * 33 * 4) + 32 * 33 * 4);
-      float vmax = 0.0f;
+      const EpiRegs er = load_epi(a);
+      // per-warp 32 x 33 staging tile in the (now idle) operand ring
+      float(*t)[33] = reinterpret_cast<float(*)[33]>(sA + q * (32 * 33 * 4));
       for (int ch = 0; ch < BN / 32; ++ch) {
         float v[32];
         tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 32), v);
@@ -583,12 +715,10 @@ __global__ void __launch_bounds__(192, 1)
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] += w[i];
         }
-        const int col0 = tn * BN + ch * 32;
-        // this lane holds row `row`, columns col0 .. col0 + 31
-        epilogue_chunk(a, v, row, row0, col0, lane, tx, ty, inv, vmax);
+        if (er.sym && tn * BN + ch * 32 < row0) continue;
+        stage_chunk(v, er.inv, lane, t);
+        epilogue_chunk<false>(er, row0, tn * BN + ch * 32, lane, t);
       }
-      for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-      if (lane == 0 && a.amax) atomicMax(a.amax, __float_as_uint(vmax));
     }
   }
 
@@ -601,27 +731,27 @@ __global__ void __launch_bounds__(192, 1)
 }
 
 // Persistent variant: one CTA per SM walks the tiles id = blockIdx.x, blockIdx.x + gridDim.x, ...
-// The producer and MMA threads run ahead into the next tile while the epilogue drains the
-// previous one.  Two accumulator modes:
-//  - single products (one segment, hi*hi only): tiles alternate between the two accumulators
-//    (tile it uses accumulator it % 2), so the whole MMA of the next tile overlaps the epilogue
-//    of the previous one.  acc_full[b] and acc_free[b] carry one phase per use of accumulator b;
-//    with one barrier pair per accumulator no barrier can run two phases ahead of its waiter.
-//  - split products (three segments): the tensor core truncates as it accumulates, so the error
-//    of a K-long sum grows with K.  The hi*hi sum is therefore accumulated in chunks of
-//    chunk_kb K blocks, and the epilogue warps fold each finished chunk into the tile's sum with
-//    round-to-nearest FP32 adds (tcgen05.ld + st).  A tile with parity p first accumulates the
-//    two correction segments into accumulator p (while it is small), then each hi*hi chunk into
-//    accumulator p ^ 1; after each chunk the epilogue folds accumulator p ^ 1 into accumulator p
-//    and releases it for the next chunk, and after the last fold writes out accumulator p and
-//    releases it.  Tiles alternate p, so a tile's long correction segments run while the
-//    previous tile is written out from the other accumulator.  acc_full[0] carries one phase per
-//    fold; acc_free[b] one phase per release of accumulator b, and the MMA thread waits for
-//    release u - 1 of b before its u-th fresh write to b.  Each phase needs the previous one
-//    consumed, so no barrier runs two phases ahead.
-// Barriers: full/empty (operand ring), acc_full[2] (MMA -> epilogue), acc_free[2] (epilogue ->
-// MMA, four warp arrivals per phase).  Every wait is bounded; a role that gives up records an
-// error and raises a shared abort flag that ends the other roles' loops.
+// The producer and MMA threads run ahead into the next tile while the epilogue writes the previous
+// one.  A tile's K blocks run as chunks, each accumulated by itself in one of two TMEM accumulators
+// that alternate from chunk to chunk (and across tiles): the correction segments of a split product
+// (hi*lo, lo*hi, 2^-11 of the whole) are the first chunk, which runs while the epilogue writes the
+// tile before, then the hi*hi sum follows in chunks of chunk_kb K blocks; a single product is one
+// chunk.  The epilogue warps read each finished chunk (tcgen05.ld), add it to the tile's sum in
+// registers (round-to-nearest FP32) and release the accumulator at once, while the other one fills.
+// Two column groups of four warps share a tile (BN / 2 sums per thread; one group for BN = 32).
+//
+// The tensor core truncates as it accumulates, so a sum's error grows with its length; with the sums in
+// registers a chunk costs its one tcgen05.ld pass.  (The sums used to live in TMEM, each fold a load, a
+// load, an add and a store that the next chunk had to wait for.)  A tcgen05.ld holds up the MMAs
+// beside it by a time that hardly depends on its size: with 256-wide tiles and 512-long chunks, n = 8192
+// takes 2.46 ms with loads of 32 columns and 2.30 ms with loads of 64.  Taking all three products of a K block from one pair of hi and lo slots
+// loads a third fewer bytes, but with both in one accumulator the errors were three times as large, and
+// at n = 8192 it ran no faster (2.87 against 2.53 ms: only two K blocks fit in the ring).
+//
+// Barriers: full/empty (operand ring), acc_full[2] (MMA -> epilogue), acc_free[2] (epilogue -> MMA,
+// one arrival per epilogue warp).  Chunk c of the CTA uses accumulator c % 2 and waits for release
+// c / 2 - 1 of it, so no barrier can run two phases ahead of its waiter.  Every wait is bounded; a
+// role that gives up records an error and raises a shared abort flag that ends the other roles' loops.
 
 // Grouped launch (tab != null): tile id -> problem p of the group and its tile lid; tiles_per
 // tiles per problem.  Otherwise one problem.
@@ -676,39 +806,67 @@ __device__ __forceinline__ void kwalk_next(KWalk& w, int nk, int Cn) {
   }
 }
 
+// Shape of a persistent CTA with tiles of width BN: epilogue column groups and warps, columns per
+// warp, ring stages (as many as fit beside the staging tiles).
+template <int BN>
+struct PCfg {
+  static constexpr int CG = BN >= 64 ? 2 : 1;
+  static constexpr int NEPI = 4 * CG;
+  static constexpr int THREADS = 128 + 32 * NEPI;   // warpgroup 0: producer and MMA warps (and two idle ones)
+  static constexpr int COLS = BN / CG;
+  static constexpr int STG = BN == 256 ? 4 : BN == 128 ? 6 : 8;
+  static constexpr int B_BYTES = BN * BK * 2;
+  static constexpr int STAGE_TILE = 32 * 33 * 4;
+  static constexpr int SMEM = STG * (A_BYTES + B_BYTES) + NEPI * STAGE_TILE + (2 * STG + 4) * 8 + 16 + 1024;
+};
+
+// The four MMAs of one K block (128-byte rows): d (+)= A B^T, fresh: written, not added to.
+template <bool TF32>
+__device__ __forceinline__ void mma_block(uint32_t d, const uint8_t* pa, const uint8_t* pb, uint32_t idesc, bool fresh) {
+#pragma unroll
+  for (int j = 0; j < BK / 16; ++j) {
+    const uint64_t ad = smem_desc(pa + j * 32);
+    const uint64_t bd = smem_desc(pb + j * 32);
+    if constexpr (TF32)
+      mma_tf32(d, ad, bd, idesc, (fresh && j == 0) ? 0u : 1u);
+    else
+      mma_f16(d, ad, bd, idesc, (fresh && j == 0) ? 0u : 1u);
+  }
+}
+
 // TF32: operands are TF32 words (kind::tf32, 32-element K blocks); else FP16 or BF16 by a.fmt.
 template <int BN, bool TF32>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
     gemm_tc_persistent_kernel(const __grid_constant__ CUtensorMap mAhi, const __grid_constant__ CUtensorMap mAlo,
                               const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
                               const __grid_constant__ CUtensorMap mA2hi, const __grid_constant__ CUtensorMap mA2lo,
                               const __grid_constant__ CUtensorMap mB2hi, const __grid_constant__ CUtensorMap mB2lo,
                               TcArgs a, int ntiles, const TcEntry* __restrict__ tab, int tiles_per) {
-  constexpr int B_BYTES = BN * BK * 2;
+  using Cfg = PCfg<BN>;
+  constexpr int STG = Cfg::STG, B_BYTES = Cfg::B_BYTES, COLS = Cfg::COLS;
   constexpr uint32_t TMEM_COLS = 2 * BN;
-  constexpr int STAGE_TILE = 32 * 33 * 4;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
-  uint8_t* sB = smem + STAGES * A_BYTES;
-  uint8_t* stage = sB + STAGES * B_BYTES;   // 4 warps x 2 staging tiles of the epilogue
-  uint64_t* full = reinterpret_cast<uint64_t*>(stage + 4 * 2 * STAGE_TILE);
-  uint64_t* empty = full + STAGES;
-  uint64_t* acc_full = empty + STAGES;     // [2]
+  uint8_t* sB = smem + STG * A_BYTES;
+  uint8_t* stage = sB + STG * B_BYTES;     // one staging tile per epilogue warp
+  uint64_t* full = reinterpret_cast<uint64_t*>(stage + Cfg::NEPI * Cfg::STAGE_TILE);
+  uint64_t* empty = full + STG;
+  uint64_t* acc_full = empty + STG;        // [2]
   uint64_t* acc_free = acc_full + 2;       // [2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 0 && lane == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < STG; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
     mbar_init(&acc_full[0], 1);
     mbar_init(&acc_full[1], 1);
-    mbar_init(&acc_free[0], 4);
-    mbar_init(&acc_free[1], 4);
+    mbar_init(&acc_free[0], Cfg::NEPI);
+    mbar_init(&acc_free[1], Cfg::NEPI);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -723,19 +881,19 @@ __global__ void __launch_bounds__(192, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-
   constexpr int bk = TF32 ? BK / 2 : BK;           // elements per K block (one 128-byte row)
   const int nk = a.K / bk;
   const int total = a.nseg * a.pairs * nk;
-  const bool chunked = a.nseg > 1;                 // split products; else single products alternate
   const int H = a.pairs * nk;                      // hi*hi K blocks
-  const int Cn = total - H;                        // correction K blocks
-  const int Lc = (chunked && a.chunk_kb > 0 && a.chunk_kb < H) ? a.chunk_kb : H;   // chunk length
-  const int nchunks = (H + Lc - 1) / Lc;
-  const int nfold = chunked ? nchunks : 0;   // folds per tile
+  const int Cn = total - H;                        // correction K blocks (the first chunk)
+  const int Lc = (a.nseg > 1 && a.chunk_kb > 0 && a.chunk_kb < H) ? a.chunk_kb : H;   // hi*hi chunk
+  const int nch = (Cn > 0 ? 1 : 0) + (H + Lc - 1) / Lc;                               // chunks per tile
 
-  if (warp == 0) {
-    if (lane == 0) {
+  // BN = 256 holds 128 sums a thread: the 384 threads are launched with 168 registers each, 64,512 in
+  // all; the producer's warpgroup keeps 40 a thread (128 x 40) and the epilogue's two get 232 (256 x 232)
+  if (warp < 4) {
+    if constexpr (BN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (warp == 0 && lane == 0) {
       uint32_t g = 0;
       bool ok = true;
       int last_p = -1;
@@ -755,9 +913,9 @@ __global__ void __launch_bounds__(192, 1)
         KWalk w;
         kwalk_begin(w, Cn);
         for (int kb = 0; kb < total; ++kb, ++g, kwalk_next(w, nk, Cn)) {
-          const int s = g % STAGES;
-          const uint32_t ph = (g / STAGES) & 1;
-          if (g >= STAGES && !mbar_wait_fast(&empty[s], ph ^ 1)) {
+          const int s = g % STG;
+          const uint32_t ph = (g / STG) & 1;
+          if (g >= STG && !mbar_wait_fast(&empty[s], ph ^ 1)) {
             atomicExch(a.err, 1);
             *abort_flag = 1;
             ok = false;
@@ -773,152 +931,111 @@ __global__ void __launch_bounds__(192, 1)
           tma_load_2d(sB + s * B_BYTES, mb, kk, tn * BN, &full[s]);
         }
       }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
+    } else if (warp == 1 && lane == 0) {
       constexpr uint32_t idesc_f16 = instr_desc(BN, 0);
       constexpr uint32_t idesc_bf16 = instr_desc(BN, 1);
       constexpr uint32_t idesc_tf32 = instr_desc(BN, 2);
       const uint32_t idesc = TF32 ? idesc_tf32 : a.fmt ? idesc_bf16 : idesc_f16;
-      uint32_t g = 0;
-      int it = 0;
-      int uses0 = 0, uses1 = 0;      // fresh writes of each accumulator so far (split products)
-      int par = 0;                   // split products: accumulator parity p of this tile
-      for (int id = blockIdx.x; id < ntiles && !*abort_flag; id += gridDim.x, ++it, par ^= 1) {
-        int tm, tn;
-        int p_, lid;
-        group_tile(tab, tiles_per, id, p_, lid);
+      uint32_t g = 0, c = 0;           // K blocks and chunks of this CTA so far
+      bool ok = true;
+      for (int id = blockIdx.x; id < ntiles && ok && !*abort_flag; id += gridDim.x) {
+        int tm, tn, p, lid;
+        group_tile(tab, tiles_per, id, p, lid);
         if (!tile_coords(a, lid, tm, tn)) break;
-        bool ok = true;
-        const int buf = it & 1;      // single products: accumulator of this tile
-        int cur = 0;                 // accumulator of the current step
-        int bnd = 0;                 // first hi*hi K block of the next chunk
-        KWalk w;
-        kwalk_begin(w, Cn);
-        for (int kb = 0; kb < total; ++kb, ++g, kwalk_next(w, nk, Cn)) {
-          // does this K block start a step, and into which accumulator?
-          int fresh = -1;            // accumulator written fresh from this K block, or -1
-          if (!chunked) {
-            if (kb == 0) fresh = buf;
-          } else if (w.phase == 0) {
-            if (w.c == 0) fresh = par;                     // corrections: the tile's sum accumulator
-          } else if (w.h == bnd) {
-            if (bnd > 0) mma_commit(&acc_full[0]);                    // the previous chunk is complete: fold it
-            fresh = par ^ 1;                               // next hi*hi chunk
-            bnd += Lc;
-          }
-          if (fresh >= 0) {
-            // wait until the epilogue has released the accumulator's previous contents
-            const int u = chunked ? (fresh ? uses1 : uses0) : (it >> 1);
-            if (u > 0) {
-              if (!mbar_wait_fast(&acc_free[fresh], (uint32_t)((u - 1) & 1)) || *abort_flag) {
-                ok = false;
-                break;
-              }
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        int done = 0;                  // K blocks of this tile so far
+        for (int ch = 0; ch < nch && ok; ++ch, ++c) {
+          const int b = c & 1;
+          if (c >= 2) {                // the epilogue has read this accumulator's previous chunk
+            if (!mbar_wait_fast(&acc_free[b], ((c >> 1) - 1) & 1) || *abort_flag) {
+              ok = false;
+              break;
             }
-            if (chunked) {
-              if (fresh)
-                ++uses1;
-              else
-                ++uses0;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          }
+          const int len = (ch == 0 && Cn > 0) ? Cn : min(Lc, total - done);
+          done += len;
+          const uint32_t d = tmem + (b ? (uint32_t)BN : 0u);
+          for (int i = 0; i < len; ++i, ++g) {
+            const int s = g % STG;
+            if (!mbar_wait_fast(&full[s], (g / STG) & 1)) {
+              ok = false;
+              break;
             }
-            cur = fresh;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            mma_block<TF32>(d, sA + s * A_BYTES, sB + s * B_BYTES, idesc, i == 0);
+            mma_commit(&empty[s]);
           }
-          const int s = g % STAGES;
-          const uint32_t ph = (g / STAGES) & 1;
-          if (!mbar_wait_fast(&full[s], ph)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint32_t dcol = cur ? (uint32_t)BN : 0u;
-#pragma unroll
-          for (int j = 0; j < BK / 16; ++j) {
-            const uint64_t ad = smem_desc(sA + s * A_BYTES + j * 32);
-            const uint64_t bd = smem_desc(sB + s * B_BYTES + j * 32);
-            if constexpr (TF32)
-              mma_tf32(tmem + dcol, ad, bd, idesc, (fresh >= 0 && j == 0) ? 0u : 1u);
-            else
-              mma_f16(tmem + dcol, ad, bd, idesc, (fresh >= 0 && j == 0) ? 0u : 1u);
-          }
-          mma_commit(&empty[s]);
+          if (ok) mma_commit(&acc_full[b]);
         }
         if (!ok) {
           atomicExch(a.err, 2);
           *abort_flag = 1;
-          break;
         }
-        mma_commit(&acc_full[chunked ? 0 : buf]);         // last step of the tile
       }
     }
   } else {
-    // epilogue warps 2..5: TMEM lanes 32 * (warp % 4) ..
-    const int q = warp & 3;
-    float(*tx)[33] = reinterpret_cast<float(*)[33]>(stage + q * 2 * STAGE_TILE);
-    float(*ty)[33] = reinterpret_cast<float(*)[33]>(stage + q * 2 * STAGE_TILE + STAGE_TILE);
-    const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    int it = 0;
-    uint32_t ev = 0;                 // acc_full[0] phases consumed (split products)
-    int par = 0;                     // split products: accumulator parity p of this tile
-    for (int id = blockIdx.x; id < ntiles && !*abort_flag; id += gridDim.x, ++it, par ^= 1) {
+    if constexpr (BN == 256) asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+    // epilogue warps: TMEM lanes 32 * (warp % 4) .., columns COLS * cg ..
+    const int q = warp & 3, cg = (warp - 4) >> 2;
+    float(*t)[33] = reinterpret_cast<float(*)[33]>(stage + (warp - 4) * Cfg::STAGE_TILE);
+    const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cg * COLS);
+    uint32_t c = 0;
+    for (int id = blockIdx.x; id < ntiles && !*abort_flag; id += gridDim.x) {
       int tm, tn, p, lid;
       group_tile(tab, tiles_per, id, p, lid);
       if (!tile_coords(a, lid, tm, tn)) break;
-      const TcArgs& ea = tab ? tab[p].args : a;     // this problem's epilogue
-      const float inv = ea.alpha / (__ldg(ea.sa) * __ldg(ea.sb));
-      prefetch_sides<BN>(ea, tm, tn, (warp - 2) * 32 + lane);
-      int src;                       // accumulator holding the tile's sum
+      EpiRegs er;                      // this problem's epilogue
+      if (tab)
+        er = load_epi(tab[p].args);
+      else
+        er = load_epi(a);
+      prefetch_sides<BN>(er, tm, tn, (warp - 4) * 32 + lane, 32 * Cfg::NEPI);
+      float sum[COLS / 32][32];
       bool ok = true;
-      if (!chunked) {
-        src = it & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[src], (uint32_t)((it >> 1) & 1)));
-        if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      } else {
-        // fold f: accumulator (f % 2) ^ p += the other one, which is then released
-        src = par;
-        for (int f = 1; f <= nfold && ok; ++f, ++ev) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[0], ev & 1));
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const int dst = par, from = par ^ 1;
-          // 64 columns at a time: both loads in flight before one wait
-          for (int ch = 0; ch < BN / 64; ++ch) {
-            uint32_t v[64], u[64];
-            tmem_ld64_nowait(tmem + lane_base + (uint32_t)(from * BN + ch * 64), v);
-            tmem_ld64_nowait(tmem + lane_base + (uint32_t)(dst * BN + ch * 64), u);
-            tmem_wait_ld64(v);
-            tmem_after_wait64(u);
+      for (int ch = 0; ch < nch; ++ch, ++c) {
+        const int b = c & 1;
+        ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[b], (c >> 1) & 1));
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if constexpr (COLS == 128) {
 #pragma unroll
-            for (int i = 0; i < 64; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(u[i]));
-            tmem_st64(tmem + lane_base + (uint32_t)(dst * BN + ch * 64), v);
+          for (int x = 0; x < 2; ++x) {
+            uint32_t v[64];
+            tmem_ld64_nowait(tbase + (uint32_t)(b * BN + x * 64), v);
+            tmem_wait_ld64(v);
+#pragma unroll
+            for (int i = 0; i < 64; ++i) {
+              float& y = sum[2 * x + i / 32][i % 32];
+              y = ch ? y + __uint_as_float(v[i]) : __uint_as_float(v[i]);
+            }
           }
-          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&acc_free[from]);
-          src = dst;
+        } else {
+#pragma unroll
+          for (int x = 0; x < COLS / 32; ++x) {
+            float v[32];
+            tmem_ld32(tbase + (uint32_t)(b * BN + x * 32), v);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) sum[x][i] = ch ? sum[x][i] + v[i] : v[i];
+          }
         }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_free[b]);
       }
       if (!ok || *abort_flag) {
         if (lane == 0) atomicExch(a.err, 3);
         *abort_flag = 1;
         break;
       }
-      // the epilogue proper from the accumulator that holds the sum
-      const int row0 = tm * BM + q * 32;
-      const int row = row0 + lane;
-      float vmax = 0.0f;
-      for (int ch = 0; ch < BN / 32; ++ch) {
-        float v[32];
-        tmem_ld32(tmem + lane_base + (uint32_t)(src * BN + ch * 32), v);
-        epilogue_chunk(ea, v, row, row0, tn * BN + ch * 32, lane, tx, ty, inv, vmax);
+      const int row0 = tm * BM + q * 32, colw = tn * BN + cg * COLS;
+#pragma unroll 1
+      for (int x = 0; x < COLS / 32; ++x) {   // one copy of the epilogue's code; the sums' index stays static
+        if (er.sym && colw + x * 32 < row0) continue;
+#pragma unroll
+        for (int y = 0; y < COLS / 32; ++y)
+          if (y == x) stage_chunk(sum[y], er.inv, lane, t);
+        epilogue_chunk<TF32>(er, row0, colw + x * 32, lane, t);
       }
-      for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-      if (lane == 0 && ea.amax) atomicMax(ea.amax, __float_as_uint(vmax));
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_free[src]);
     }
   }
 
@@ -952,6 +1069,7 @@ __global__ void __launch_bounds__(192, 1)
 constexpr int PSTAGES = 6;
 constexpr int PB_BYTES = 128 * BK * 2;           // a CTA's half of the 256-row B tile
 constexpr int kPairGroupM = 8;                   // 256-row panels per raster group
+constexpr int kPairChunkKb = 16;                 // hi*hi chunk (its folds go through TMEM)
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -1039,7 +1157,7 @@ __global__ void __launch_bounds__(192, 1)
   uint8_t* sA = smem;
   uint8_t* sB = smem + PSTAGES * A_BYTES;
   uint8_t* stage = sB + PSTAGES * PB_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(stage + 4 * 2 * STAGE_TILE);
+  uint64_t* full = reinterpret_cast<uint64_t*>(stage + 4 * STAGE_TILE);
   uint64_t* empty = full + PSTAGES;
   uint64_t* acc_full = empty + PSTAGES;    // [2]
   uint64_t* acc_free = acc_full + 2;       // [2], used in the leader
@@ -1199,10 +1317,9 @@ __global__ void __launch_bounds__(192, 1)
     }
   } else {
     const int q = warp & 3;
-    float(*tx)[33] = reinterpret_cast<float(*)[33]>(stage + q * 2 * STAGE_TILE);
-    float(*ty)[33] = reinterpret_cast<float(*)[33]>(stage + q * 2 * STAGE_TILE + STAGE_TILE);
+    float(*t)[33] = reinterpret_cast<float(*)[33]>(stage + q * STAGE_TILE);
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const float inv = a.alpha / (__ldg(a.sa) * __ldg(a.sb));
+    const EpiRegs er = load_epi(a);
     const uint32_t free_leader0 = map_to_rank(&acc_free[0], 0), free_leader1 = map_to_rank(&acc_free[1], 0);
     int it = 0;
     uint32_t ev = 0;
@@ -1211,7 +1328,7 @@ __global__ void __launch_bounds__(192, 1)
       int tm, tn;
       if (!pair_tile_coords(a, id, tm, tn)) break;
       const int tm128 = 2 * tm + (int)rank;          // this CTA's 128-row panel
-      prefetch_sides<BN>(a, tm128, tn, (warp - 2) * 32 + lane);
+      prefetch_sides<BN>(a, tm128, tn, (warp - 2) * 32 + lane, 128);
       int src;
       bool ok = true;
       if (!chunked) {
@@ -1248,15 +1365,13 @@ __global__ void __launch_bounds__(192, 1)
         break;
       }
       const int row0 = tm128 * BM + q * 32;
-      const int row = row0 + lane;
-      float vmax = 0.0f;
       for (int ch = 0; ch < BN / 32; ++ch) {
         float v[32];
         tmem_ld32(tmem + lane_base + (uint32_t)(src * BN + ch * 32), v);
-        epilogue_chunk(a, v, row, row0, tn * BN + ch * 32, lane, tx, ty, inv, vmax);
+        if (er.sym && tn * BN + ch * 32 < row0) continue;
+        stage_chunk(v, er.inv, lane, t);
+        epilogue_chunk<false>(er, row0, tn * BN + ch * 32, lane, t);
       }
-      for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-      if (lane == 0 && a.amax) atomicMax(a.amax, __float_as_uint(vmax));
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(src ? free_leader1 : free_leader0);
@@ -1340,13 +1455,8 @@ int smem_bytes() {
   return STAGES * (A_BYTES + BN * BK * 2) + (2 * STAGES + 1) * 8 + 16 + 1024;
 }
 
-template <int BN>
-int smem_bytes_persistent() {
-  return STAGES * (A_BYTES + BN * BK * 2) + 4 * 2 * 32 * 33 * 4 + (2 * STAGES + 4) * 8 + 16 + 1024;
-}
-
 int smem_bytes_pair() {
-  return PSTAGES * (A_BYTES + PB_BYTES) + 4 * 2 * 32 * 33 * 4 + (2 * PSTAGES + 5) * 8 + 16 + 1024;
+  return PSTAGES * (A_BYTES + PB_BYTES) + 4 * 32 * 33 * 4 + (2 * PSTAGES + 5) * 8 + 16 + 1024;
 }
 
 // 1: one-SM persistent CTAs (default); 2: two-SM products where n is a multiple of 256
@@ -1369,7 +1479,7 @@ constexpr int kMaxDevices = 64;
 struct DeviceState {
   int sms = 0;
   int pair_clusters = 0;   // co-resident clusters of the two-SM product kernel
-  bool smem_set[7] = {false, false, false, false, false, false, false};
+  bool smem_set[11] = {};   // 0-3 persistent kernel per width, 4-7 its TF32 form, 8, 9 one-CTA-per-tile, 10 two-SM
 };
 std::mutex g_dev_mu;
 DeviceState g_dev[kMaxDevices];
@@ -1439,16 +1549,53 @@ cudaError_t ensure_smem(int slot, Kern kern, int bytes) {
 // Persistent launch with tiles of width BN (grid CTAs, one per SM); TF32 operands (a.fmt = 2)
 // take their own instantiation, so the FP16/BF16 kernel keeps compile-time K blocks.
 template <int BN>
-cudaError_t launch_persistent(cudaStream_t s, int grid, const CUtensorMap (&m)[8], const TcArgs& a, int ntiles,
-                              const TcEntry* tab, int tiles_per) {
-  const int sb = smem_bytes_persistent<BN>();
+cudaError_t launch_width(cudaStream_t s, int slot, int grid, const CUtensorMap (&m)[8], const TcArgs& a, int ntiles,
+                         const TcEntry* tab, int tiles_per) {
+  constexpr int sb = PCfg<BN>::SMEM;
   const bool tf32 = a.fmt == 2;
   auto kern = tf32 ? gemm_tc_persistent_kernel<BN, true> : gemm_tc_persistent_kernel<BN, false>;
-  const cudaError_t attr = ensure_smem((BN == 256 ? 0 : 1) + (tf32 ? 5 : 0), kern, sb);
+  const cudaError_t attr = ensure_smem(slot + (tf32 ? 4 : 0), kern, sb);
   if (attr != cudaSuccess) return attr;
-  kern<<<grid, 192, sb, s>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], m[7], a, ntiles, tab, tiles_per);
+  kern<<<grid, PCfg<BN>::THREADS, sb, s>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], m[7], a, ntiles, tab, tiles_per);
   note_launch();
   return cudaGetLastError();
+}
+
+cudaError_t launch_persistent(cudaStream_t s, int width, const CUtensorMap (&m)[8], const TcArgs& a, int ntiles,
+                              const TcEntry* tab, int tiles_per) {
+  const int grid = std::min(ntiles, sm_count());
+  switch (width) {
+    case 0: return launch_width<32>(s, 0, grid, m, a, ntiles, tab, tiles_per);
+    case 1: return launch_width<64>(s, 1, grid, m, a, ntiles, tab, tiles_per);
+    case 2: return launch_width<128>(s, 2, grid, m, a, ntiles, tab, tiles_per);
+    default: return launch_width<256>(s, 3, grid, m, a, ntiles, tab, tiles_per);
+  }
+}
+
+int tiles_of(int n, int width, bool sym, const TcTiles& t) {
+  return sym ? t.nsym[width] : (n / BM) * (n / tc_width(width));
+}
+
+// Tile width of a persistent launch over nprob problems of size n: the one with the least waves of
+// tiles times the time of a tile.  The times of a 128 x w tile relative to w = 128 hardly depend on n (one
+// CTA's K loop is bound by its hand-offs, not by the width): symmetric split products of n = 2048 take
+// 123 us with w = 32 (4 waves), 68 with 64 (2 waves), 45 with 128 (1 wave), 66 with 256; n = 1408: 48, 29,
+// 35; n = 256: 10.8, 12.0, 16.9, 28.2; n = 4096: 803, 415, 263 (4 waves), 219 (2 waves).
+int pick_width(int n, int nprob, const TcArgs& a, const TcTiles& t) {
+  static const int cost[kTcWidths] = {68, 75, 100, 150};
+  const int sms = sm_count();
+  int best = 2;
+  long long least = -1;
+  for (int w = 0; w < kTcWidths; ++w) {
+    if (n % tc_width(w)) continue;
+    const long long tiles = (long long)nprob * tiles_of(n, w, a.sym != 0, t);
+    const long long c = (tiles + sms - 1) / sms * cost[w];
+    if (least < 0 || c < least) {
+      least = c;
+      best = w;
+    }
+  }
+  return best;
 }
 
 }  // namespace
@@ -1472,8 +1619,9 @@ cudaError_t gemm_tc(cudaStream_t s, int n, const void* Ahi, const void* Alo, con
   // TF32 operands run on the persistent kernel only
   const int variant = args.fmt == 2 ? 1 : tc_variant();
   const bool two_sm = (variant == 2) && wide && tiles.pair != nullptr;
+  const int width = variant == 0 ? (wide ? 3 : 2) : pick_width(n, 1, args, tiles);
   // B boxes: a CTA's 128-row half of the 256-row tile (two-SM), else the tile's bn rows
-  const int bn = wide ? 256 : 128;
+  const int bn = tc_width(width);
   const int bbox = two_sm ? 128 : bn;
   CUtensorMap mAhi, mAlo, mBhi, mBlo, mA2hi, mA2lo, mB2hi, mB2lo;
   if (!make_map(&mAhi, Ahi, n, BM, args.fmt) || !make_map(&mAlo, Alo ? Alo : Ahi, n, BM, args.fmt) ||
@@ -1495,6 +1643,7 @@ cudaError_t gemm_tc(cudaStream_t s, int n, const void* Ahi, const void* Alo, con
   if (args.split_acc && n / BK < 2) return cudaErrorInvalidValue;   // both accumulators get K blocks
   args.tiles_n = n / bn;
   if (two_sm) {
+    args.chunk_kb = kPairChunkKb;
     int ntiles;
     if (args.sym) {
       args.tile_list = tiles.pair;
@@ -1504,7 +1653,7 @@ cudaError_t gemm_tc(cudaStream_t s, int n, const void* Ahi, const void* Alo, con
       ntiles = (n / 256) * (n / 256);
     }
     const int sb = smem_bytes_pair();
-    const cudaError_t attr = ensure_smem(4, gemm_tc_pair_kernel, sb);
+    const cudaError_t attr = ensure_smem(10, gemm_tc_pair_kernel, sb);
     if (attr != cudaSuccess) return attr;
     const int npairs = std::min(ntiles, pair_clusters(sb));
     if (const char* dbg = std::getenv("XLBOMD_DEBUG"))
@@ -1528,29 +1677,21 @@ cudaError_t gemm_tc(cudaStream_t s, int n, const void* Ahi, const void* Alo, con
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
   }
-  int nblocks;
-  if (args.sym) {
-    args.tile_list = wide ? tiles.sym256 : tiles.sym128;
-    nblocks = wide ? tiles.n256 : tiles.n128;
-  } else {
-    args.tile_list = nullptr;
-    nblocks = (n / BM) * (n / bn);
-  }
+  args.tile_list = args.sym ? tiles.sym[width] : nullptr;
+  const int nblocks = tiles_of(n, width, args.sym != 0, tiles);
   if (variant >= 1) {
-    const int grid = std::min(nblocks, sm_count());
     const CUtensorMap maps[8] = {mAhi, mAlo, mBhi, mBlo, mA2hi, mA2lo, mB2hi, mB2lo};
-    return wide ? launch_persistent<256>(s, grid, maps, args, nblocks, nullptr, 0)
-                : launch_persistent<128>(s, grid, maps, args, nblocks, nullptr, 0);
+    return launch_persistent(s, width, maps, args, nblocks, nullptr, 0);
   }
   if (wide) {
     const int sb = smem_bytes<256>();
-    const cudaError_t attr = ensure_smem(2, gemm_tc_kernel<256>, sb);
+    const cudaError_t attr = ensure_smem(8, gemm_tc_kernel<256>, sb);
     if (attr != cudaSuccess) return attr;
     gemm_tc_kernel<256><<<nblocks, 192, sb, s>>>(mAhi, mAlo, mBhi, mBlo, mA2hi, mA2lo, mB2hi, mB2lo, args);
     note_launch();
   } else {
     const int sb = smem_bytes<128>();
-    const cudaError_t attr = ensure_smem(3, gemm_tc_kernel<128>, sb);
+    const cudaError_t attr = ensure_smem(9, gemm_tc_kernel<128>, sb);
     if (attr != cudaSuccess) return attr;
     gemm_tc_kernel<128><<<nblocks, 192, sb, s>>>(mAhi, mAlo, mBhi, mBlo, mA2hi, mA2lo, mB2hi, mB2lo, args);
     note_launch();
@@ -1601,37 +1742,33 @@ cudaError_t gemm_tc_group(cudaStream_t s, int n, const TcProblem* probs, int npr
     a.err = shared.err;
     return gemm_tc(s, n, probs[0].Ahi, probs[0].Alo, probs[0].Bhi, probs[0].Blo, a, tiles);
   }
-  const bool wide = (n % 256 == 0) && shared.bn != 128;
-  const int bn = wide ? 256 : 128;
+  const int width = pick_width(n, nprob, shared, tiles);
+  const int bn = tc_width(width);
   // table key: the problems' operands and epilogue arguments (a table is rebuilt only when
   // one of them changes)
   uint64_t key = 1469598103934665603ull;
   key = fnv_mix(key, (uint64_t)n * 1000003u + shared.nseg * 7 + shared.pairs * 31 + shared.sym * 131 +
                          shared.fmt * 521 + (uint64_t)bn * 7919);
-  key = fnv_mix(key, (uint64_t)(shared.sym ? (wide ? tiles.sym256 : tiles.sym128) : nullptr));
+  key = fnv_mix(key, (uint64_t)(shared.sym ? tiles.sym[width] : nullptr));
   key = fnv_mix(key, (uint64_t)shared.err + (uint64_t)shared.chunk_kb);
   for (int i = 0; i < nprob; ++i) {
     const TcProblem& q = probs[i];
     const TcArgs& e = q.epi;
     const uint64_t w[] = {(uint64_t)q.Ahi, (uint64_t)q.Alo, (uint64_t)q.Bhi, (uint64_t)q.Blo, (uint64_t)e.E,
-                          (uint64_t)e.E2, (uint64_t)e.E64, (uint64_t)e.C64, (uint64_t)e.dvec, (uint64_t)e.C,
-                          (uint64_t)e.amax, (uint64_t)e.sa, (uint64_t)e.sb, bits_of(e.alpha), bits_of(e.beta),
-                          bits_of(e.beta2), bits_of(e.beta64), bits_of(e.diag), bits_of(e.dvec_scale),
-                          (uint64_t)e.e64_trans * 3 + (uint64_t)e.ndvec * 17 + (uint64_t)e.ldc * 65537};
+                          (uint64_t)e.E2, (uint64_t)e.E64, (uint64_t)e.dvec, (uint64_t)e.out.f, (uint64_t)e.out.d,
+                          (uint64_t)e.out.hi, (uint64_t)e.out.lo, (uint64_t)e.out.scale, (uint64_t)e.out2.f,
+                          (uint64_t)e.out2.hi, (uint64_t)e.out2.lo, (uint64_t)e.out2.scale, (uint64_t)e.sa,
+                          (uint64_t)e.sb, bits_of(e.alpha), bits_of(e.beta), bits_of(e.beta2), bits_of(e.beta64),
+                          bits_of(e.diag), bits_of(e.dvec_scale), bits_of(e.va), bits_of(e.vb),
+                          (uint64_t)e.ndvec * 17 + (uint64_t)e.ldc * 65537};
     for (uint64_t x : w) key = fnv_mix(key, x);
   }
   TcArgs a = shared;
   a.n = n;
   a.K = n;
   a.tiles_n = n / bn;
-  int tiles_per;
-  if (a.sym) {
-    a.tile_list = wide ? tiles.sym256 : tiles.sym128;
-    tiles_per = wide ? tiles.n256 : tiles.n128;
-  } else {
-    a.tile_list = nullptr;
-    tiles_per = (n / BM) * (n / bn);
-  }
+  a.tile_list = a.sym ? tiles.sym[width] : nullptr;
+  const int tiles_per = tiles_of(n, width, a.sym != 0, tiles);
   TcEntry* table = nullptr;
   auto it = cache->tables.find(key);
   if (it != cache->tables.end()) {
@@ -1667,7 +1804,6 @@ cudaError_t gemm_tc_group(cudaStream_t s, int n, const TcProblem* probs, int npr
       t.args.fmt = a.fmt;
       t.args.split_acc = a.split_acc;
       t.args.chunk_kb = a.chunk_kb;
-      t.args.bn = a.bn;
       t.args.tiles_n = a.tiles_n;
       t.args.tile_list = a.tile_list;
       t.args.err = a.err;
@@ -1683,12 +1819,10 @@ cudaError_t gemm_tc_group(cudaStream_t s, int n, const TcProblem* probs, int npr
     cache->tables[key] = table;
   }
   const int ntiles = nprob * tiles_per;
-  const int grid = std::min(ntiles, sm_count());
   // the launch's own maps are unused (every problem's maps come from the table)
   CUtensorMap dummy[8];
   std::memset(dummy, 0, sizeof(dummy));
-  return wide ? launch_persistent<256>(s, grid, dummy, a, ntiles, table, tiles_per)
-              : launch_persistent<128>(s, grid, dummy, a, ntiles, table, tiles_per);
+  return launch_persistent(s, width, dummy, a, ntiles, table, tiles_per);
 }
 
 // Tile list of symmetric two-SM products: the 256 x 256 tiles (tm, tn) with tn >= tm, in the

@@ -14,6 +14,10 @@
 
 namespace xl {
 
+// Device parameters of a captured chemical-potential pass: mu, g_0..g_3 per level (at most 40), z_0, z_1 of
+// dT_n/dmu (and two unused), |T_0|'s bound.
+constexpr int kPassZ = 1 + 4 * 40, kPassT0 = kPassZ + 4, kPassPar = kPassT0 + 1;
+
 constexpr int XLBOMD_FP16x3_ID = 1;
 constexpr int XLBOMD_BF16x3_ID = 2;
 constexpr int XLBOMD_TF32x3_ID = 3;
@@ -26,16 +30,15 @@ inline int operand_fmt(int prec) { return prec == XLBOMD_TF32x3_ID ? 2 : prec ==
 inline int operand_bytes(int prec) { return prec == XLBOMD_TF32x3_ID ? 4 : 2; }
 
 // Matrices of one system in the working precision.  In the FP64 engine each
-// logical matrix is a double array; the split engines keep an FP32 value
-// array plus hi/lo operand arrays (16-bit FP16/BF16, or TF32 in FP32 words)
-// with a power-of-two scale.
+// logical matrix is a double array; the split engines keep a value array (FP32
+// or double-float) plus hi/lo operand arrays (16-bit FP16/BF16, or TF32 in FP32
+// words) of the value times a power-of-two scale (operand.cuh).
 struct SplitMat {
-  float2* d = nullptr;       // double-float value hi + lo (matrices carried with an exact leading term)
-  float* f = nullptr;        // FP32 value (np x np)
-  void* hi = nullptr;        // operand hi part of value * scale
-  void* lo = nullptr;        // operand lo part
-  float* scale = nullptr;    // device scalar
-  unsigned* amax = nullptr;  // device scalar: float bits of max |value|
+  float2* d = nullptr;            // double-float value hi + lo (matrices carried with an exact leading term)
+  float* f = nullptr;             // FP32 value (np x np)
+  void* hi = nullptr;             // operand hi part of value * scale
+  void* lo = nullptr;             // operand lo part
+  const float* scale = nullptr;   // device scalar, one of the MatSet's scales
 };
 
 struct MatSet {
@@ -47,7 +50,12 @@ struct MatSet {
   // split engines
   std::vector<SplitMat> sT, sY;
   SplitMat sS, sQ, sYw, sA1, sMt, sT1a, sT1b, sTmu;
-  void* tc_plan = nullptr;   // device scalars (scales, max |x|) of the split engine
+  // device scalars of the split engine: operand scales ([0] kUnitScale, [1 + k] T_k, [n + 2] the
+  // resolvent of dT_n/dmu, then per level of a response chain those of A1, M and the next T1) and
+  // |T_0|'s bound of the last expansion
+  float* scales = nullptr;
+  float* chain_scales = nullptr;   // the chain part (a chain slot has its own)
+  float* t0_dev = nullptr;
   double t0max = 0.0;        // spectral bound |T_0| of the last expansion
   // FP64 work matrices of the split engine's entropy (allocated on first use)
   double* e64[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};

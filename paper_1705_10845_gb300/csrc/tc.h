@@ -8,15 +8,23 @@
 
 namespace xl {
 
+// Where a product's result goes; what is null is not written.  f: FP32 value, d: double-float value,
+// hi (and lo): tensor-core operands of the value times *scale.
+struct TcOut {
+  float* f = nullptr;
+  float2* d = nullptr;
+  void* hi = nullptr;
+  void* lo = nullptr;
+  const float* scale = nullptr;
+};
+
 struct TcArgs {
   int K = 0;                      // inner dimension (set by gemm_tc)
   int n = 0;                      // matrix size (set by gemm_tc)
   int split_acc = 0;              // one-CTA-per-tile kernel: 1 = the hi*hi K blocks split over both
                                   // accumulators (below)
-  int bn = 0;                     // grouped products: tile width 128 or 256 (0: 256 where n is a
-                                  // multiple of 256, else 128)
-  int chunk_kb = 0;               // persistent kernel, split products: the hi*hi sum is accumulated in
-                                  // chunks of this many K blocks, folded in FP32 (0: one chunk)
+  int chunk_kb = 0;               // split products: the hi*hi sum is accumulated in chunks of this many
+                                  // K blocks, added up in FP32 (0: one chunk)
   int nseg = 3;                   // 1: hi only; 3: hi*hi + hi*lo + lo*hi
   int pairs = 1;                  // 2: C = A B^T + B A^T (the swapped pair as a second K range)
   int sym = 0;                    // symmetric output (upper tiles, mirrored)
@@ -24,23 +32,21 @@ struct TcArgs {
                                   // FP32 words; persistent kernel only)
   int tiles_n = 0;                // set by gemm_tc
   const int* tile_list = nullptr; // set by gemm_tc
-  float alpha = 1.0f;             // C = alpha acc / (sa sb) + beta E^T + beta2 E2^T + beta64 E64(^T)
-  const float* E = nullptr;       //     + diag I + dvec_scale diag(dvec); E and E2 are read
-                                  //     transposed (callers pass symmetric side inputs)
+  float alpha = 1.0f;             // v = alpha acc / (sa sb) + beta E + beta2 E2 + diag I
+  const float* E = nullptr;       //     + dvec_scale diag(dvec)
   float beta = 0.0f;
   const float* E2 = nullptr;
   float beta2 = 0.0f;
-  const float2* E64 = nullptr;    // double-float side input, read transposed when e64_trans
-  float beta64 = 0.0f;            // a power of two, so that beta64 E64 is exact
-  int e64_trans = 0;
-  float2* C64 = nullptr;          // double-float output (written instead of C when set)
+  const float2* E64 = nullptr;    // out.d: v + beta64 E64 as a double-float (beta64 a power of two,
+  float beta64 = 0.0f;            // so that beta64 E64 is exact)
   float diag = 0.0f;
   const double* dvec = nullptr;
   int ndvec = 0;
   float dvec_scale = 1.0f;
-  float* C = nullptr;
+  TcOut out;
+  TcOut out2;                     // a second result va v + vb E (f, hi, lo; E symmetric)
+  float va = 0.0f, vb = 0.0f;
   int ldc = 0;
-  unsigned* amax = nullptr;       // max |C| (float bits), atomically raised
   const float* sa = nullptr;      // operand scales (device scalars)
   const float* sb = nullptr;
   int* err = nullptr;             // set non-zero when a bounded wait gives up
@@ -63,13 +69,13 @@ struct TcProblem {
 };
 
 // Device tile lists of the symmetric-output products of one size n (pairs of ints (tm, tn)):
-// 128 x 128 tiles, 128 x 256 tiles (n a multiple of 256) and 256 x 256 tiles of the two-SM
-// products (n a multiple of 256; null: two-SM products are not used for this size).
+// 128 x w tiles for the widths w = 32, 64, 128 and 256 (the last where n is a multiple of 256), and
+// 256 x 256 tiles of the two-SM products (n a multiple of 256; null: not used for this size).
+constexpr int kTcWidths = 4;
+constexpr int tc_width(int i) { return 32 << i; }
 struct TcTiles {
-  const int* sym128 = nullptr;
-  int n128 = 0;
-  const int* sym256 = nullptr;
-  int n256 = 0;
+  const int* sym[kTcWidths] = {nullptr, nullptr, nullptr, nullptr};
+  int nsym[kTcWidths] = {0, 0, 0, 0};
   const int* pair = nullptr;
   int npair = 0;
 };

@@ -327,3 +327,29 @@ def test_grouped_exact_kernel_256_atoms(X, kernel_prec, tol):
     err = np.max(np.abs(K - Kref)) / np.abs(Kref).max()
     print("exact kernel 256 atoms, kernel_prec", kernel_prec, "rel err", err, "recompute s", dt)
     assert err < tol
+
+
+@pytest.mark.parametrize("nat", [32, 33, 224, 320, 352])
+def test_density_where_the_tile_width_changes(X, nat):
+    # symmetric products take 32-wide tiles up to 1024 padded orbitals, 64-wide ones at 1280 and 1408 (their
+    # 32-wide tiles would need two waves of SMs); 128 and 256 are the smallest sizes, one and four
+    # tiles.  Every product of the expansion writes its value and its operands in the epilogue, in both
+    # triangles, with and without side inputs: charges to 1e-5 e and forces to 1e-4 eV/A of the oracle
+    s = synth.make_system(nat, 7)
+    p = X.default_params(mix_alpha=ALPHA_MIX, kernel_c=1 - 1 / ALPHA_MIX, prec="fp16x3", mu_tol=1e-3)
+    m = O.Model(Te=p.Te, n_sq=p.n_sq)
+    rng = np.random.default_rng(nat)
+    n = rng.normal(scale=0.01, size=s.natoms)
+    n -= n.mean()
+    ref = O.evaluate(s.R, s.L, s.Z, n, m, O.XLParams(rank_m=p.rank_m, kernel_c=p.kernel_c))
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, n)
+        ctx.set(0, X.MU, [ref.dens.mu + 0.01])
+        ctx.build_H(0)
+        ctx.density(0)
+        ctx.kernel_update(0)
+        q, F, Kr, D = ctx.get(0, X.Q), ctx.get(0, X.F), ctx.get(0, X.KR), ctx.get(0, X.D)
+    assert np.max(np.abs(q - ref.q)) < 1e-5
+    assert np.max(np.abs(F - ref.F)) < 1e-4
+    assert np.max(np.abs(Kr - ref.Kr)) < 1e-3
+    assert np.array_equal(D, D.T)

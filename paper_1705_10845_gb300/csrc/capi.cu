@@ -34,6 +34,10 @@ struct Sys {
   // device, FP64
   double *R = nullptr, *V = nullptr, *F = nullptr, *Z = nullptr, *nh = nullptr, *q = nullptr, *r = nullptr;
   double *Kr = nullptr, *pot = nullptr, *potv = nullptr, *gam = nullptr, *SF = nullptr, *G4 = nullptr;
+  double *Gs = nullptr, *SFr = nullptr;   // sqrt of the reciprocal weights; structure factors of a moved R
+  double *Rs = nullptr;                   // positions as FP32 pairs (split precisions; float2 each)
+  int* Gh = nullptr;                      // integer reciprocal vectors, a byte per component
+  bool sf_current = false;                // SF belongs to R
   double *H0 = nullptr, *H = nullptr, *Dm = nullptr;
   double *ddiag = nullptr, *dmu_diag = nullptr, *d1 = nullptr, *dvec = nullptr;
   double *pV = nullptr, *pW = nullptr, *scal = nullptr, *work = nullptr, *energy = nullptr;
@@ -237,6 +241,11 @@ xlbomd_status run_captured(xlbomd_ctx* ctx, Sys& S, const std::vector<int>& key,
   return XLBOMD_OK;
 }
 
+// FP32 pairs of the positions (split precisions), else null
+float2* split_R(const xlbomd_ctx* ctx, const Sys& S) {
+  return ctx->p.prec != XLBOMD_FP64 ? reinterpret_cast<float2*>(S.Rs) : nullptr;
+}
+
 xlbomd_status sync_read(xlbomd_ctx* ctx, const double* dev, int count) {
   CK(cudaMemcpyAsync(ctx->pinned, dev, sizeof(double) * count, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
@@ -252,14 +261,16 @@ cudaError_t gamma_apply(xlbomd_ctx* ctx, Sys& S, const double* x, double* y, dou
 xlbomd_status build_H(xlbomd_ctx* ctx, Sys& S) {
   cudaStream_t st = ctx->stream;
   const ModelConst m = model_of(ctx->p);
-  CK(launch_build_H0(st, m, S.nat, S.L, S.R, S.H0, S.np));
-  const bool fp32_pairs = ctx->p.prec != XLBOMD_FP64;
+  CK(launch_build_H0(st, m, S.nat, S.L, S.R, S.H0, S.H, S.np));
   if (ctx->p.coulomb_k != 0.0) {
-    CK(launch_gamma_real(st, m, S.nat, S.L, S.eta, S.R, S.gam, S.natp, fp32_pairs));
-    CK(launch_structure_factors(st, S.nat, S.ng, S.G4, S.R, S.SF, S.kp));
+    float2* Rs = split_R(ctx, S);
+    if (Rs) CK(launch_split_positions(st, S.nat, S.R, Rs));
+    CK(launch_gamma_real(st, m, S.nat, S.L, S.eta, S.R, Rs, S.gam, S.natp));
+    CK(launch_structure_factors(st, S.nat, S.ng, S.L, S.Gh, S.Gs, S.R, S.SF, S.kp));
+    S.sf_current = true;
   }
   CK(gamma_apply(ctx, S, S.nh, S.pot, S.work));
-  CK(launch_apply_potential(st, S.nat, S.np, S.H0, S.pot, S.H));
+  CK(launch_apply_potential(st, S.nat, S.np, nullptr, S.pot, S.H));
   S.have_density = false;
   return XLBOMD_OK;
 }
@@ -367,6 +378,23 @@ struct MuSearch {
   }
 };
 
+// Forces at R, D, q and n.  The reciprocal part uses the structure factors of the last build_H; after
+// xlbomd_set(R) without one it takes its own (the potentials keep those of H).
+xlbomd_status forces(xlbomd_ctx* ctx, Sys& S) {
+  cudaStream_t st = ctx->stream;
+  const double* SF = S.SF;
+  float2* Rs = split_R(ctx, S);
+  if (ctx->p.coulomb_k != 0.0 && !S.sf_current) {
+    if (!S.SFr) CKS(dalloc(ctx, &S.SFr, (size_t)S.natp * S.kp));
+    CK(launch_structure_factors(st, S.nat, S.ng, S.L, S.Gh, S.Gs, S.R, S.SFr, S.kp));
+    if (Rs) CK(launch_split_positions(st, S.nat, S.R, Rs));
+    SF = S.SFr;
+  }
+  CK(launch_forces(st, model_of(ctx->p), S.nat, S.L, S.eta, S.ng, S.G4, S.R, Rs, SF, S.kp, S.Dm, S.np, S.q, S.nh, S.F,
+                   S.work));
+  return XLBOMD_OK;
+}
+
 // density matrix, charges (and forces) from the final mu pass
 xlbomd_status density_finish(xlbomd_ctx* ctx, Sys& S, const MuSearch& ms, bool with_forces) {
   cudaStream_t st = ctx->stream;
@@ -374,10 +402,7 @@ xlbomd_status density_finish(xlbomd_ctx* ctx, Sys& S, const MuSearch& ms, bool w
   ms.finish(S);
   CK(ctx->eng->density_out(st, S.mats, S.N, ms.dmu, S.dmu_diag, S.ddiag, S.Dm));
   CK(launch_charges(st, S.nat, S.ddiag, S.Z, S.nh, S.q, S.r));
-  if (with_forces) {
-    CK(launch_forces(st, model_of(p), S.nat, S.L, S.eta, S.ng, S.G4, S.R, S.Dm, S.np, S.q, S.nh, S.F, S.work,
-                     p.prec != XLBOMD_FP64));
-  }
+  if (with_forces) CKS(forces(ctx, S));
   S.have_density = true;
   return XLBOMD_OK;
 }
@@ -678,7 +703,7 @@ xlbomd_status energy(xlbomd_ctx* ctx, Sys& S) {
   cudaStream_t st = ctx->stream;
   CK(cudaMemsetAsync(S.energy + 4, 0, sizeof(double), st));
   if (ctx->p.rep_A != 0.0) {
-    CK(launch_repulsion(st, model_of(ctx->p), S.nat, S.L, S.R, nullptr, S.work));
+    CK(launch_repulsion_energy(st, model_of(ctx->p), S.nat, S.L, S.R, S.work));
     CK(launch_sum(st, S.nat, S.work, S.energy + 4));
   }
   CK(launch_frob_dot(st, S.N, S.np, S.Dm, S.H0, S.work, S.energy + 0));
@@ -768,8 +793,7 @@ xlbomd_status scf(xlbomd_ctx* ctx, Sys& S) {
     if (floor && debug_enabled()) std::fprintf(stderr, "[xlbomd] scf stops at the rounding floor %.3e\n", res);
     if (res < p.scf_tol || floor) {
       CK(launch_fill_history(st, S.nat, p.kmax, S.nh));
-      CK(launch_forces(st, model_of(p), S.nat, S.L, S.eta, S.ng, S.G4, S.R, S.Dm, S.np, S.q, S.nh, S.F, S.work,
-                       p.prec != XLBOMD_FP64));
+      CKS(forces(ctx, S));
       S.have_K = false;   // exact or accumulated kernel: start again at the t0 state
       return kernel_update(ctx, S);
     }
@@ -986,8 +1010,7 @@ xlbomd_status scf_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
       const bool floor = p.prec != XLBOMD_FP64 && since_best[k] >= 4 && res < 100.0 * p.scf_tol;
       if (res < p.scf_tol || floor) {
         CK(launch_fill_history(st, S.nat, p.kmax, S.nh));
-        CK(launch_forces(st, model_of(p), S.nat, S.L, S.eta, S.ng, S.G4, S.R, S.Dm, S.np, S.q, S.nh, S.F, S.work,
-                         p.prec != XLBOMD_FP64));
+        CKS(forces(ctx, S));
         S.have_K = false;   // exact or accumulated kernel: start again at the t0 state
         converged.push_back(&S);
       } else {
@@ -1047,11 +1070,13 @@ void free_sys(Sys& S) {
   double** ptrs[] = {&S.R,  &S.V,        &S.F,    &S.Z,  &S.nh,  &S.q,    &S.r,     &S.Kr,    &S.pot,
                      &S.potv, &S.gam,    &S.SF,   &S.G4, &S.H0,  &S.H,    &S.Dm,    &S.ddiag, &S.dmu_diag,
                      &S.d1, &S.dvec,     &S.pV, &S.pW, &S.scal, &S.work, &S.energy,
-                     &S.Kfull, &S.Jm, &S.dpar};
+                     &S.Kfull, &S.Jm, &S.dpar, &S.Gs, &S.SFr, &S.Rs};
   for (double** p : ptrs) {
     if (*p) cudaFree(*p);
     *p = nullptr;
   }
+  if (S.Gh) cudaFree(S.Gh);
+  S.Gh = nullptr;
   for (auto& g : S.graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   S.graphs.clear();
@@ -1292,10 +1317,21 @@ xlbomd_status xlbomd_init(const xlbomd_params* params, const xlbomd_system* syst
     A(&S.pV, (size_t)(kMaxRank + 1) * nat);
     A(&S.pW, (size_t)(kMaxRank + 1) * nat);
     A(&S.scal, 64);
-    A(&S.work, std::max<size_t>({(size_t)4 * S.ng + 16, (size_t)2 * S.N + 16, (size_t)4096}));
+    A(&S.work, std::max<size_t>({(size_t)2 * S.kp + 3 * nat * force_parts(S.nat), (size_t)2 * S.N + 16, (size_t)4096}));
+    A(&S.Gs, (size_t)S.ng);
+    if (p.prec != XLBOMD_FP64) A(&S.Rs, 3 * nat);
     A(&S.energy, 8);
     if (st != XLBOMD_OK) return bail(st);
     if (alloc_matset(S.mats, p.prec, S.np, p.n_sq, ctx->stream) != cudaSuccess) return bail(XLBOMD_ERR_OOM);
+    if (cudaMalloc((void**)&S.Gh, sizeof(int) * std::max(S.ng, 1)) != cudaSuccess) return bail(XLBOMD_ERR_OOM);
+    std::vector<int> gh(S.ng);
+    std::vector<double> gs(S.ng);
+    for (int g = 0; g < S.ng; ++g) {
+      int h[3];
+      for (int c = 0; c < 3; ++c) h[c] = (int)std::lround(S.G4h[4 * g + c] * S.L / (2.0 * kPi)) + 8;
+      gh[g] = h[0] | h[1] << 8 | h[2] << 16;
+      gs[g] = std::sqrt(S.G4h[4 * g + 3]);
+    }
     // R wrapped into [0, L)
     std::vector<double> Rw(3 * nat);
     for (size_t a = 0; a < 3 * nat; ++a) Rw[a] = s.R[a] - S.L * std::floor(s.R[a] / S.L);
@@ -1305,7 +1341,9 @@ xlbomd_status xlbomd_init(const xlbomd_params* params, const xlbomd_system* syst
         cudaMemcpyAsync(S.Z, s.Z, sizeof(double) * nat, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
         (S.ng && cudaMemcpyAsync(S.G4, S.G4h.data(), sizeof(double) * S.G4h.size(), cudaMemcpyHostToDevice, cs) !=
                      cudaSuccess) ||
-        cudaStreamSynchronize(cs) != cudaSuccess)   // Rw is a host temporary
+        (S.ng && (cudaMemcpyAsync(S.Gh, gh.data(), sizeof(int) * S.ng, cudaMemcpyHostToDevice, cs) != cudaSuccess ||
+                  cudaMemcpyAsync(S.Gs, gs.data(), sizeof(double) * S.ng, cudaMemcpyHostToDevice, cs) != cudaSuccess)) ||
+        cudaStreamSynchronize(cs) != cudaSuccess)   // Rw, gh and gs are host temporaries
       return bail(XLBOMD_ERR_CUDA);
     if (build_H(ctx, S) != XLBOMD_OK) return bail((xlbomd_status)ctx->status);
   }
@@ -1466,6 +1504,7 @@ xlbomd_status xlbomd_set(xlbomd_ctx* ctx, int sys, int what, const double* host_
       CK(cudaMemcpyAsync(S.R, Rw.data(), sizeof(double) * 3 * nat, cudaMemcpyHostToDevice, ctx->stream));
       CK(cudaStreamSynchronize(ctx->stream));
       S.have_density = false;
+      S.sf_current = false;
       return XLBOMD_OK;
     }
     case XLBOMD_V:

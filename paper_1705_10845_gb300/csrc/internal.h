@@ -31,35 +31,39 @@ struct ModelConst {
   double rep_A, rep_rho;   // pair repulsion rep_A exp(-r/rep_rho) S(r); rep_A = 0: off
 };
 
-// H0 (np x np, zeroed padding) from positions R (natoms x 3) in a box L.
+// Positions as pairs of FP32 words (the Coulomb kernels of the split precisions).
+cudaError_t launch_split_positions(cudaStream_t s, int nat, const double* R, float2* Rs);
+// H0 (np x np, zeroed padding) from positions R (natoms x 3, in [0, L)) in a box L, and a copy of it in H.
 cudaError_t launch_build_H0(cudaStream_t s, const ModelConst& m, int nat, double L, const double* R,
-                            double* H0, int np);
+                            double* H0, double* H, int np);
 // Real-space part of gamma over 27 images of the minimum image (natp x natp, ld natp);
-// fp32: pair terms in FP32 (sums in FP64), for the split-precision path.
+// Rs not null: pair functions in FP32 of 48-bit distances, for the split-precision path.
 cudaError_t launch_gamma_real(cudaStream_t s, const ModelConst& m, int nat, double L, double eta,
-                              const double* R, double* gam, int natp, bool fp32);
+                              const double* R, const float2* Rs, double* gam, int natp);
 // y = gamma x with gamma = gamma_real + k SF SF^T applied through the structure
 // factors (tmp: kp doubles; SF may be null when k = 0).
 cudaError_t launch_gamma_apply(cudaStream_t s, int nat, const double* gam, int natp, const double* SF, int kp,
                                double k, const double* x, double* y, double* tmp);
-// Structure-factor matrix SF (natp x kp): row I = sqrt(A_g) [cos(G_g.R_I), sin(G_g.R_I)].
-cudaError_t launch_structure_factors(cudaStream_t s, int nat, int ng, const double* G4, const double* R,
-                                     double* SF, int kp);
+// Structure-factor matrix SF (natp x kp): row I = sqrt(w_g) [cos(G_g.R_I), sin(G_g.R_I)].  Gh: the integer
+// vectors h + 8, a byte per component; Gs = sqrt(w_g).
+cudaError_t launch_structure_factors(cudaStream_t s, int nat, int ng, double L, const int* Gh, const double* Gs,
+                                     const double* R, double* SF, int kp);
 // pot[I] = sum_J gamma_IJ x_J  (natoms)
 cudaError_t launch_gemv(cudaStream_t s, int nat, const double* gam, int natp, const double* x, double* y);
-// H = H0 + diag(pot per orbital)
+// H = H0 + diag(pot per orbital); H0 null: H += diag(pot)
 cudaError_t launch_apply_potential(cudaStream_t s, int nat, int np, const double* H0, const double* pot,
                                    double* H);
 // Gershgorin interval of H: out[0] = min(H_ii - r_i), out[1] = max(H_ii + r_i)
 cudaError_t launch_gershgorin(cudaStream_t s, int n, int np, const double* H, double* out);
-// Forces: band part from D (np x np) and Coulomb real-space + reciprocal parts.
+// Forces: band part from D (np x np), pair repulsion (rep_A != 0), Coulomb real-space and reciprocal parts
+// (SF: structure factors of R; work: 2 kp + 3 nat force_parts(nat) doubles).  Rs as for launch_gamma_real.
+int force_parts(int nat);
 cudaError_t launch_forces(cudaStream_t s, const ModelConst& m, int nat, double L, double eta, int ng,
-                          const double* G4, const double* R, const double* D, int np, const double* q,
-                          const double* n, double* F, double* work /* >= 4*ng */, bool fp32);
-// Pair repulsion: F_I += -dE_rep/dR_I when F is not null; e_I = half the pair energy of atom I
-// when e is not null (E_rep = sum_I e_I).  No launch when rep_A = 0.
-cudaError_t launch_repulsion(cudaStream_t s, const ModelConst& m, int nat, double L, const double* R, double* F,
-                             double* e);
+                          const double* G4, const double* R, const float2* Rs, const double* SF, int kp,
+                          const double* D, int np, const double* q, const double* n, double* F, double* work);
+// Pair repulsion: e_I = half the pair energy of atom I (E_rep = sum_I e_I).
+cudaError_t launch_repulsion_energy(cudaStream_t s, const ModelConst& m, int nat, double L, const double* R,
+                                    double* e);
 // q_I = sum_{a in I} (1 + Tn_aa) + 2 dmu dmu_diag_a - Z_I, r = q - n
 cudaError_t launch_charges(cudaStream_t s, int nat, const double* ddiag, const double* Z,
                            const double* n, double* q, double* r);

@@ -353,3 +353,38 @@ def test_density_where_the_tile_width_changes(X, nat):
     assert np.max(np.abs(F - ref.F)) < 1e-4
     assert np.max(np.abs(Kr - ref.Kr)) < 1e-3
     assert np.array_equal(D, D.T)
+
+
+@pytest.mark.parametrize("nat,L", [(10, 5.3), (33, None), (255, None), (256, None), (620, None)])
+def test_model_of_the_split_path_against_oracle(X, nat, L):
+    # H (FP64 with an FP32 pair test before it), gamma and the forces at a given density: a box barely above
+    # the cutoff (several images of each pair inside it), a warp's remainder, both sides of the Coulomb
+    # force's split over tx (256 atoms) and of the four-atoms-a-block launch (608).  gamma sums 27 FP32
+    # terms of order 1/r with relative errors of a few 2^-24 and cancellation between 1/r terms: 1e-5 of
+    # its largest entry is loose; a missed or doubled image is 1e-3 and more
+    s = synth.make_system(nat, 19, L=L)
+    p = X.default_params(mix_alpha=ALPHA_MIX, kernel_c=1 - 1 / ALPHA_MIX, prec="fp16x3", rep_A=40.0, mu_tol=1e-3)
+    m = O.Model(Te=p.Te, n_sq=p.n_sq, rep_A=40.0, rep_rho=p.rep_rho)
+    rng = np.random.default_rng(nat)
+    n = rng.normal(scale=0.01, size=s.natoms)
+    n -= n.mean()
+    H0, G = O.build_H0(s.R, s.L, m), O.build_gamma(s.R, s.L, m)
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, n)
+        ctx.build_H(0)
+        H, gam = ctx.get(0, X.H), ctx.get(0, X.GAMMA)
+        if nat <= 256:
+            ref = O.evaluate(s.R, s.L, s.Z, n, m, None, with_kernel=False)
+            ctx.set(0, X.MU, [ref.dens.mu])
+            ctx.density(0)
+            F = ctx.get(0, X.F)
+            # positions moved without a new Hamiltonian: the forces follow R
+            ctx.set(0, X.R, s.R + 0.25)
+            ctx.density(0)
+            F2 = ctx.get(0, X.F)
+            assert np.max(np.abs(F - ref.F)) < 1e-4
+            assert np.max(np.abs(F2 - F)) < 1e-4
+    off = ~np.eye(4 * nat, dtype=bool)
+    assert np.max(np.abs(H - H0)[off]) < 1e-11
+    assert np.max(np.abs(np.diag(H) - np.diag(H0) - np.repeat(G @ n, 4))) < 1e-4
+    assert np.max(np.abs(gam - G)) < 1e-5 * np.max(np.abs(G))

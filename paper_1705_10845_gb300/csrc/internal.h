@@ -18,12 +18,14 @@ struct EpiF64 {
   double dvec_scale = 1.0;
 };
 
-// FP64 C[M x N] = epi(A[M x K] * B[N x K]^T), row-major.  M, N multiples of
+// FP64 C[M x N] = epi(A[M x K] * B[N x K]^T), row-major, 16-byte aligned rows.  M, N multiples of
 // 64, K a multiple of 16.  sym: M == N and only tiles on or above the
 // diagonal are computed; each is written to (i, j) and mirrored to (j, i), so
-// the result is exactly symmetric (E must then be null or symmetric).
+// the result is exactly symmetric (E must then be null or symmetric; it may be C).
+// batch > 1: that many products, their matrices a stride apart (st*, elements).
 cudaError_t gemm_f64_nt(cudaStream_t s, int M, int N, int K, const double* A, int lda,
-                        const double* B, int ldb, double* C, int ldc, const EpiF64& e, bool sym);
+                        const double* B, int ldb, double* C, int ldc, const EpiF64& e, bool sym, int batch = 1,
+                        size_t stA = 0, size_t stB = 0, size_t stC = 0, size_t stE = 0);
 
 // ---- model (model_kernels.cu) ----
 struct ModelConst {

@@ -198,6 +198,7 @@ void free_matset(MatSet& m) {
     if (*p) cudaFree(*p);
     *p = nullptr;
   }
+  m.ent.release();
   free_matset_split(m);
 }
 

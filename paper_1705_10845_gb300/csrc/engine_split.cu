@@ -954,7 +954,7 @@ class EngineSplit : public Engine {
     const size_t cnt = (size_t)m.np * m.np;
     for (double*& p : m.e64)
       if (!p) RET(cudaMalloc((void**)&p, cnt * sizeof(double)));
-    double* T0 = m.e64[6];
+    double* T0 = m.e64[5];
     df_to_f64_kernel<<<nblk(cnt), 256, 0, s>>>(cnt, m.sT[0].d, T0);
     note_launch();
     RET(cudaGetLastError());
@@ -968,8 +968,8 @@ class EngineSplit : public Engine {
     const double t = m.t0max;
     while (nterms < 6 && std::ldexp(1.0, n_sq + 1) * std::pow(t, 2 * nterms + 1) / (2 * nterms + 1) * N > 1e-10)
       ++nterms;
-    return entropy_fp64(s, N, m.np, m.n, n_sq, T0, load_Y, m.e64[0], m.e64[1], m.e64[2], m.e64[3], m.e64[4],
-                        m.e64[5], nterms, D, work, out);
+    return entropy_fp64(s, N, m.np, m.n, n_sq, T0, load_Y, m.ent, m.e64[0], m.e64[1], m.e64[2], m.e64[3],
+                        m.e64[4], nterms, D, work, out);
   }
 
   int* err_ = nullptr;
@@ -1055,7 +1055,8 @@ cudaError_t alloc_matset_split(MatSet& m, cudaStream_t s) {
 // one system can run their chains side by side (grouped launches).
 cudaError_t alloc_chain_slot(MatSet& slot, const MatSet& base, cudaStream_t s) {
   slot = base;
-  slot.e64[0] = slot.e64[1] = slot.e64[2] = slot.e64[3] = slot.e64[4] = slot.e64[5] = slot.e64[6] = nullptr;
+  for (double*& p : slot.e64) p = nullptr;
+  slot.ent = EntropyWork();
   const int np = base.np, esz = operand_bytes(base.prec);
   slot.chain_scales = nullptr;
   RET(cudaMalloc((void**)&slot.chain_scales, sizeof(float) * 3 * (size_t)base.n));

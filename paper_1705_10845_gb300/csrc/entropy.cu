@@ -10,6 +10,7 @@
 // matrix (spectra in [1 - |t_0|max, 1 + |t_0|max] and [1/2, 1]) and is taken
 // by a blocked FP64 Cholesky factorisation; artanh(T_0) is its odd power
 // series (|t_0| << 1), whose traces against D come from Frobenius products.
+#include <algorithm>
 #include <cmath>
 #include <functional>
 
@@ -26,56 +27,69 @@ namespace {
 
 constexpr int CB = 64;
 
-// Factor the CB x CB diagonal block at (kb, kb) in place (lower Cholesky);
-// part[kb / CB] = sum 2 ln L_ii; a non-positive pivot writes NaN.
-__global__ void chol_panel_kernel(double* A, int np, int kb, double* part) {
-  __shared__ double a[CB][CB + 1];
-  __shared__ double lsum;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < CB * CB; e += blockDim.x) a[e / CB][e % CB] = A[(size_t)(kb + e / CB) * np + kb + e % CB];
-  if (tid == 0) lsum = 0.0;
+// Diagonal block (kb, kb) of matrix blockIdx.x: A = L D L^T (L unit lower); part[..][kb / CB] = sum ln d (NaN for
+// a non-positive pivot) and Li = D^-1/2 L^-1, for which A^-1 = Li^T Li.  In place: at step j column j
+// turns from A's into L^-1's, its old values are in col[j & 1].
+__global__ void __launch_bounds__(256) chol_panel_kernel(const double* __restrict__ W, size_t stride, int np, int kb,
+                                                         double* __restrict__ Li, double* __restrict__ part, int npart) {
+  __shared__ double x[CB][CB + 1], col[2][CB], d[CB], inv;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const double* A = W + stride * blockIdx.x;
+  for (int e = tid; e < CB * CB; e += 256) x[e / CB][e % CB] = A[(size_t)(kb + e / CB) * np + kb + e % CB];
   __syncthreads();
-  for (int j = 0; j < CB; ++j) {
-    if (tid == 0) {
-      const double d = a[j][j];
-      const double l = d > 0.0 ? sqrt(d) : nan("");
-      a[j][j] = l;
-      lsum += 2.0 * log(l);
-    }
-    __syncthreads();
-    for (int i = j + 1 + tid; i < CB; i += blockDim.x) a[i][j] /= a[j][j];
-    __syncthreads();
-    const int rem = CB - j - 1;
-    for (int e = tid; e < rem * rem; e += blockDim.x) {
-      const int i = j + 1 + e / rem, c = j + 1 + e % rem;
-      if (c <= i) a[i][c] -= a[i][j] * a[c][j];
+  if (tid < CB) col[0][tid] = x[tid][0];
+  if (tid == 0) {
+    d[0] = x[0][0];
+    inv = 1.0 / x[0][0];
+  }
+  __syncthreads();
+  for (int j = 0; j < CB - 1; ++j) {
+    const double* cj = col[j & 1];
+    double* cn = col[(j + 1) & 1];
+    const double iv = inv;
+    __syncthreads();   // every thread has read inv
+    for (int i = j + 1 + ty; i < CB; i += 16) {
+      const double l = cj[i] * iv;
+      for (int c = tx; c <= i; c += 16) {
+        if (c == j) {
+          x[i][j] = -l;
+          continue;
+        }
+        const double v = x[i][c] - l * (c < j ? x[j][c] : cj[c]);
+        x[i][c] = v;
+        if (c == j + 1) {
+          cn[i] = v;
+          if (i == j + 1) {
+            d[i] = v;
+            inv = 1.0 / v;
+          }
+        }
+      }
     }
     __syncthreads();
   }
-  for (int e = tid; e < CB * CB; e += blockDim.x) {
+  if (tid < CB) {
+    const double v = d[tid];
+    const double s = warp_sum(v > 0.0 ? log(v) : nan(""));
+    if ((tid & 31) == 0) col[0][tid >> 5] = s;
+    col[1][tid] = 1.0 / sqrt(v);
+  }
+  __syncthreads();
+  if (tid == 0) part[(size_t)npart * blockIdx.x + kb / CB] = col[0][0] + col[0][1];
+  double* out = Li + (size_t)CB * CB * blockIdx.x;
+  for (int e = tid; e < CB * CB; e += 256) {
     const int i = e / CB, c = e % CB;
-    A[(size_t)(kb + i) * np + kb + c] = (c <= i) ? a[i][c] : 0.0;
+    out[e] = c < i ? x[i][c] * col[1][i] : c == i ? col[1][i] : 0.0;
   }
-  if (tid == 0) part[kb / CB] = lsum;
 }
 
-// Rows below the panel: X L^T = A_row  ->  X = A_row L^-T (one thread per row).
-__global__ void chol_trsm_kernel(double* A, int np, int kb) {
-  __shared__ double L[CB][CB + 1];
-  for (int e = threadIdx.x; e < CB * CB; e += blockDim.x) L[e / CB][e % CB] = A[(size_t)(kb + e / CB) * np + kb + e % CB];
-  __syncthreads();
-  const int row = kb + CB + blockIdx.x * CB + threadIdx.x;
-  if (threadIdx.x >= CB || row >= np) return;
-  double x[CB];
-  double* ar = A + (size_t)row * np + kb;
-#pragma unroll 4
-  for (int j = 0; j < CB; ++j) {
-    double t = ar[j];
-    for (int c = 0; c < j; ++c) t -= x[c] * L[j][c];
-    x[j] = t / L[j][j];
-  }
-#pragma unroll 4
-  for (int j = 0; j < CB; ++j) ar[j] = x[j];
+// out[b] = sum of the panels' parts of matrix b
+__global__ void chol_sum_kernel(int npart, const double* __restrict__ part, double* __restrict__ out) {
+  __shared__ double sh[32];
+  double v = 0.0;
+  for (int i = threadIdx.x; i < npart; i += blockDim.x) v += part[(size_t)npart * blockIdx.x + i];
+  v = block_sum(v, sh);
+  if (threadIdx.x == 0) out[blockIdx.x] = v;
 }
 
 // W = I - T (np x np)
@@ -103,55 +117,80 @@ __global__ void entropy_combine_kernel(EntW w, const double* __restrict__ ld, co
   *out = s;
 }
 
-// logdet of the SPD matrix in W (destroyed); result in *out.  part >= np/CB doubles.
-cudaError_t logdet_spd(cudaStream_t s, double* W, int np, double* part, double* out) {
+// log-determinants of the nb SPD matrices in the work area (destroyed) into out[0..nb)
+cudaError_t logdet_spd(cudaStream_t s, const EntropyWork& w, int np, int nb, double* out) {
+  const size_t cnt = (size_t)np * np;
+  const int npart = np / CB;
   for (int kb = 0; kb < np; kb += CB) {
-    chol_panel_kernel<<<1, 256, 0, s>>>(W, np, kb, part);
+    chol_panel_kernel<<<nb, 256, 0, s>>>(w.mats(), cnt, np, kb, w.li(np), w.part(np), npart);
     note_launch();
     RET(cudaGetLastError());
     const int rest = np - kb - CB;
     if (rest > 0) {
-      chol_trsm_kernel<<<rest / CB, CB, 0, s>>>(W, np, kb);
-      note_launch();
-      RET(cudaGetLastError());
+      // X = A21 Li^T, A22 -= X X^T
+      double* A21 = w.mats() + (size_t)(kb + CB) * np + kb;
+      EpiF64 ex;
+      RET(gemm_f64_nt(s, rest, CB, CB, A21, np, w.li(np), CB, w.rows(np), CB, ex, false, nb, cnt, (size_t)CB * CB,
+                      (size_t)np * CB));
       EpiF64 e;
       e.alpha = -1.0;
-      e.E = W + (size_t)(kb + CB) * np + kb + CB;
+      e.E = A21 + CB;
       e.lde = np;
       e.beta = 1.0;
-      const double* Lp = W + (size_t)(kb + CB) * np + kb;
-      RET(gemm_f64_nt(s, rest, rest, CB, Lp, np, Lp, np, W + (size_t)(kb + CB) * np + kb + CB, np, e, true));
+      RET(gemm_f64_nt(s, rest, rest, CB, w.rows(np), CB, w.rows(np), CB, A21 + CB, np, e, true, nb, (size_t)np * CB,
+                      (size_t)np * CB, cnt, cnt));
     }
   }
-  return launch_sum(s, np / CB, part, out);
+  chol_sum_kernel<<<nb, 128, 0, s>>>(npart, w.part(np), out);
+  note_launch();
+  return cudaGetLastError();
 }
 
 }  // namespace
 
+cudaError_t EntropyWork::reserve(int np, int nmat) {
+  if (buf) return cudaSuccess;
+  const size_t per = sizeof(double) * ((size_t)np * np + (size_t)np * CB + CB * CB + np / CB);
+  cap = (int)std::max<size_t>(1, std::min<size_t>((size_t)nmat, ((size_t)2 << 30) / per));
+  return cudaMalloc((void**)&buf, per * cap);
+}
+double* EntropyWork::mats() const { return buf; }
+double* EntropyWork::rows(int np) const { return buf + (size_t)np * np * cap; }
+double* EntropyWork::li(int np) const { return rows(np) + (size_t)np * CB * cap; }
+double* EntropyWork::part(int np) const { return li(np) + (size_t)CB * CB * cap; }
+void EntropyWork::release() {
+  if (buf) cudaFree(buf);
+  buf = nullptr;
+}
+
 // Entropy from FP64 inputs.  T0: FP64 T_0; load_Y(k, dst) writes Y_k as an
-// FP64 matrix into dst; G, S, Q, Yw, A1, Mt: FP64 work matrices (np x np);
+// FP64 matrix into dst; S, Q, Yw, A1, Mt: FP64 work matrices (np x np);
 // nterms: terms j = 0..nterms-1 of the artanh series.
 cudaError_t entropy_fp64(cudaStream_t s, int N, int np, int n, int n_sq, const double* T0,
-                         const std::function<cudaError_t(int, double*)>& load_Y, double* G, double* S, double* Q,
+                         const std::function<cudaError_t(int, double*)>& load_Y, EntropyWork& ew, double* S, double* Q,
                          double* Yw, double* A1, double* Mt, int nterms, const double* D, double* work,
                          double* out) {
   if (n + 1 > 42 || nterms < 1 || nterms > 6) return cudaErrorInvalidValue;
-  // work layout: [0, 64): logdet slots, [64, 72): trace slots, [128, 128 + np/CB): Cholesky partials,
-  // [1024, 2048): Frobenius partials
+  // work layout: [0, 64): logdet slots, [64, 72): trace slots, [1024, 2048): Frobenius partials
   double* ld = work;
   double* tr = work + 64;
-  double* part = work + 128;
   double* fwork = work + 1024;
   const size_t count = (size_t)np * np;
-  // logdet(I - T_0)
-  ident_minus_f64_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, np, T0, G);
-  note_launch();
-  RET(cudaGetLastError());
-  RET(logdet_spd(s, G, np, part, ld + 0));
-  // logdet(Y_k)
-  for (int k = 0; k < n; ++k) {
-    RET(load_Y(k, G));
-    RET(logdet_spd(s, G, np, part, ld + 1 + k));
+  // logdet(I - T_0), then logdet(Y_k)
+  RET(ew.reserve(np, n + 1));
+  for (int k0 = 0; k0 <= n; k0 += ew.cap) {
+    const int nb = std::min(ew.cap, n + 1 - k0);
+    for (int b = 0; b < nb; ++b) {
+      double* dst = ew.mats() + count * b;
+      if (k0 + b == 0) {
+        ident_minus_f64_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, np, T0, dst);
+        note_launch();
+        RET(cudaGetLastError());
+      } else {
+        RET(load_Y(k0 + b - 1, dst));
+      }
+    }
+    RET(logdet_spd(s, ew, np, nb, ld + k0));
   }
   // Tr[D T0^(2j+1)] from S0 = T0^2, S2 = S0^2, S4 = S2^2, P1 = D T0, P3 = P1 S0
   EpiF64 e;
@@ -197,7 +236,7 @@ cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, int N, double beta, in
   auto load_Y = [&](int k, double* dst) {
     return cudaMemcpyAsync(dst, m.Y[k], sizeof(double) * count, cudaMemcpyDeviceToDevice, s);
   };
-  return entropy_fp64(s, N, m.np, m.n, n_sq, m.T[0], load_Y, m.G, m.S, m.Q, m.Yw, m.A1, m.Mt, 6, D, work, out);
+  return entropy_fp64(s, N, m.np, m.n, n_sq, m.T[0], load_Y, m.ent, m.S, m.Q, m.Yw, m.A1, m.Mt, 6, D, work, out);
 }
 
 }  // namespace xl

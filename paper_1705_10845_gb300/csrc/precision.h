@@ -41,6 +41,19 @@ struct SplitMat {
   const float* scale = nullptr;   // device scalar, one of the MatSet's scales
 };
 
+// Work area of the entropy's log-determinants (allocated on first use): cap matrices np x np, and per
+// matrix the rows below a panel, the panel's inverse factor and the panels' parts.
+struct EntropyWork {
+  double* buf = nullptr;
+  int cap = 0;
+  cudaError_t reserve(int np, int nmat);
+  void release();
+  double* mats() const;
+  double* rows(int np) const;
+  double* li(int np) const;
+  double* part(int np) const;
+};
+
 struct MatSet {
   int prec = 0, np = 0, n = 0;
   // FP64 engine
@@ -58,7 +71,8 @@ struct MatSet {
   float* t0_dev = nullptr;
   double t0max = 0.0;        // spectral bound |T_0| of the last expansion
   // FP64 work matrices of the split engine's entropy (allocated on first use)
-  double* e64[7] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  double* e64[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  EntropyWork ent;
 };
 
 cudaError_t alloc_matset(MatSet& m, int prec, int np, int n, cudaStream_t s);
@@ -210,7 +224,7 @@ int selftest_gemm_group(int n, int prec, int mode, int nprob, double* result);
 
 // FP64 eigenvalue-free entropy (entropy.cu)
 cudaError_t entropy_fp64(cudaStream_t s, int N, int np, int n, int n_sq, const double* T0,
-                         const std::function<cudaError_t(int, double*)>& load_Y, double* G, double* S, double* Q,
+                         const std::function<cudaError_t(int, double*)>& load_Y, EntropyWork& ew, double* S, double* Q,
                          double* Yw, double* A1, double* Mt, int nterms, const double* D, double* work,
                          double* out);
 cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, int N, double beta, int n_sq, double mu, double dmu,

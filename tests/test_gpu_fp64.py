@@ -332,3 +332,27 @@ def test_residual_and_energy_fluctuations_scale_as_dt_squared_on_gpu(X):
     print("dt study: residual RMS", res, "energy std", fluct)
     for a, b in ((res[0], res[1]), (res[1], res[2]), (fluct[0], fluct[1]), (fluct[1], fluct[2])):
         assert 3.0 < a / b < 5.5, (res, fluct)
+
+
+@pytest.mark.parametrize("nat", [33, 65, 97, 129])
+def test_density_and_entropy_at_tile_edges(X, nat):
+    # padded orbital counts 256, 384, 512 and 640: products with 8, 16 and 32 wide tiles, symmetric and
+    # dense, and the batched log-determinants of the energy (4 to 10 panels of 64)
+    s = synth.make_system(nat, 23)
+    p = model_params(X)
+    m = oracle_model(p)
+    n = random_n(s.natoms, nat, scale=0.01)
+    ref = O.evaluate(s.R, s.L, s.Z, n, m, O.XLParams(rank_m=p.rank_m, kernel_c=p.kernel_c))
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, n)
+        ctx.set(0, X.MU, [ref.dens.mu + 0.01])
+        ctx.build_H(0)
+        ctx.density(0)
+        ctx.kernel_update(0)
+        ctx.energy(0)
+        q, F, Kr, E = ctx.get(0, X.Q), ctx.get(0, X.F), ctx.get(0, X.KR), ctx.get(0, X.ENERGY)
+    assert np.max(np.abs(q - ref.q)) < 1e-9
+    assert np.max(np.abs(F - ref.F)) < 1e-8
+    assert np.max(np.abs(Kr - ref.Kr)) < 1e-8
+    assert abs(E[0] - ref.Omega) < 1e-8 * abs(ref.Omega)
+    assert abs(E[3] - ref.parts["entropy"]) < 1e-7

@@ -820,18 +820,63 @@ struct PCfg {
   static constexpr int SMEM = STG * (A_BYTES + B_BYTES) + NEPI * STAGE_TILE + (2 * STG + 4) * 8 + 16 + 1024;
 };
 
-// The four MMAs of one K block (128-byte rows): d (+)= A B^T, fresh: written, not added to.
-template <bool TF32>
-__device__ __forceinline__ void mma_block(uint32_t d, const uint8_t* pa, const uint8_t* pb, uint32_t idesc, bool fresh) {
-#pragma unroll
-  for (int j = 0; j < BK / 16; ++j) {
-    const uint64_t ad = smem_desc(pa + j * 32);
-    const uint64_t bd = smem_desc(pb + j * 32);
-    if constexpr (TF32)
-      mma_tf32(d, ad, bd, idesc, (fresh && j == 0) ? 0u : 1u);
-    else
-      mma_f16(d, ad, bd, idesc, (fresh && j == 0) ? 0u : 1u);
+// ---- the two single-thread loops of the persistent kernel: 32-bit shared addresses throughout ----
+
+__device__ __forceinline__ bool bar_spin(uint32_t bar, uint32_t parity) {
+  for (int it = 0; it < (kWaitLimit << 4); ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
   }
+  return false;
+}
+
+__device__ __forceinline__ void bar_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// one K block's A and B tiles into a ring slot
+__device__ __forceinline__ void load_slot(uint32_t bar, uint32_t bytes, uint32_t da, const CUtensorMap* ma, uint32_t db,
+                                          const CUtensorMap* mb, int x, int ya, int yb) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(da),
+      "l"(reinterpret_cast<uint64_t>(ma)), "r"(x), "r"(ya), "r"(bar)
+      : "memory");
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(db),
+      "l"(reinterpret_cast<uint64_t>(mb)), "r"(x), "r"(yb), "r"(bar)
+      : "memory");
+}
+
+// Shared-memory descriptors (smem_desc) as words: the low one holds the address / 16, the high one is constant.
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return (addr >> 4) | (1u << 16); }
+
+template <bool TF32>
+__device__ __forceinline__ void mma_words(uint32_t d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t accumulate) {
+  if constexpr (TF32)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %4, p;\n\t}" ::"r"(d),
+        "r"(alo), "r"(blo), "r"(kDescHi), "r"(idesc), "r"(accumulate)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(d),
+        "r"(alo), "r"(blo), "r"(kDescHi), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 
 // TF32: operands are TF32 words (kind::tf32, 32-element K blocks); else FP16 or BF16 by a.fmt.
@@ -893,9 +938,11 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
   // all; the producer's warpgroup keeps 40 a thread (128 x 40) and the epilogue's two get 232 (256 x 232)
   if (warp < 4) {
     if constexpr (BN == 256) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB), full0 = smem_u32(full), empty0 = smem_u32(empty);
+    uint32_t slot = 0, ph = 0;         // ring slot and the parity of its current use
+    bool ok = true;
     if (warp == 0 && lane == 0) {
-      uint32_t g = 0;
-      bool ok = true;
+      bool first = true;               // the ring's first use needs no release
       int last_p = -1;
       for (int id = blockIdx.x; id < ntiles && ok && !*abort_flag; id += gridDim.x) {
         int tm, tn, p, lid;
@@ -910,25 +957,29 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
           for (int i = 0; i < 8; ++i) tensormap_acquire(&maps[i]);
           last_p = p;
         }
-        KWalk w;
-        kwalk_begin(w, Cn);
-        for (int kb = 0; kb < total; ++kb, ++g, kwalk_next(w, nk, Cn)) {
-          const int s = g % STG;
-          const uint32_t ph = (g / STG) & 1;
-          if (g >= STG && !mbar_wait_fast(&empty[s], ph ^ 1)) {
-            atomicExch(a.err, 1);
-            *abort_flag = 1;
-            ok = false;
-            break;
+        // segments: the corrections hi*lo, lo*hi of each pair, then hi*hi of each pair
+        for (int sg = a.nseg > 1 ? 0 : 2 * a.pairs; sg < 3 * a.pairs && ok; ++sg) {
+          const int pr = sg < 2 * a.pairs ? sg >> 1 : sg - 2 * a.pairs;
+          const int kind = sg < 2 * a.pairs ? 1 + (sg & 1) : 0;
+          const int ia = (kind == 2) ? (pr ? 5 : 1) : (pr ? 4 : 0);
+          const int ib = (kind == 1) ? (pr ? 7 : 3) : (pr ? 6 : 2);
+          const CUtensorMap* ma = maps ? &maps[ia] : (kind == 2) ? (pr ? &mA2lo : &mAlo) : (pr ? &mA2hi : &mAhi);
+          const CUtensorMap* mb = maps ? &maps[ib] : (kind == 1) ? (pr ? &mB2lo : &mBlo) : (pr ? &mB2hi : &mBhi);
+          for (int k = 0; k < a.K; k += bk) {
+            if (!first && !bar_spin(empty0 + 8 * slot, ph ^ 1)) {
+              atomicExch(a.err, 1);
+              *abort_flag = 1;
+              ok = false;
+              break;
+            }
+            load_slot(full0 + 8 * slot, A_BYTES + B_BYTES, a0 + slot * A_BYTES, ma, b0 + slot * B_BYTES, mb, k, tm * BM,
+                      tn * BN);
+            if (++slot == STG) {
+              slot = 0;
+              ph ^= 1;
+              first = false;
+            }
           }
-          mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
-          const int kk = w.kidx * bk;
-          const int ia = (w.kind == 2) ? (w.pr ? 5 : 1) : (w.pr ? 4 : 0);
-          const int ib = (w.kind == 1) ? (w.pr ? 7 : 3) : (w.pr ? 6 : 2);
-          const CUtensorMap* ma = maps ? &maps[ia] : (w.kind == 2) ? (w.pr ? &mA2lo : &mAlo) : (w.pr ? &mA2hi : &mAhi);
-          const CUtensorMap* mb = maps ? &maps[ib] : (w.kind == 1) ? (w.pr ? &mB2lo : &mBlo) : (w.pr ? &mB2hi : &mBhi);
-          tma_load_2d(sA + s * A_BYTES, ma, kk, tm * BM, &full[s]);
-          tma_load_2d(sB + s * B_BYTES, mb, kk, tn * BN, &full[s]);
         }
       }
     } else if (warp == 1 && lane == 0) {
@@ -936,17 +987,18 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
       constexpr uint32_t idesc_bf16 = instr_desc(BN, 1);
       constexpr uint32_t idesc_tf32 = instr_desc(BN, 2);
       const uint32_t idesc = TF32 ? idesc_tf32 : a.fmt ? idesc_bf16 : idesc_f16;
-      uint32_t g = 0, c = 0;           // K blocks and chunks of this CTA so far
-      bool ok = true;
+      const uint32_t alo0 = desc_lo(a0), blo0 = desc_lo(b0);
+      const uint32_t accf0 = smem_u32(acc_full), accr0 = smem_u32(acc_free);
+      uint32_t alo = alo0, blo = blo0, c = 0;   // descriptors of the slot; chunks of this CTA so far
       for (int id = blockIdx.x; id < ntiles && ok && !*abort_flag; id += gridDim.x) {
         int tm, tn, p, lid;
         group_tile(tab, tiles_per, id, p, lid);
         if (!tile_coords(a, lid, tm, tn)) break;
         int done = 0;                  // K blocks of this tile so far
         for (int ch = 0; ch < nch && ok; ++ch, ++c) {
-          const int b = c & 1;
+          const uint32_t b = c & 1;
           if (c >= 2) {                // the epilogue has read this accumulator's previous chunk
-            if (!mbar_wait_fast(&acc_free[b], ((c >> 1) - 1) & 1) || *abort_flag) {
+            if (!bar_spin(accr0 + 8 * b, ((c >> 1) - 1) & 1) || *abort_flag) {
               ok = false;
               break;
             }
@@ -954,18 +1006,30 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
           }
           const int len = (ch == 0 && Cn > 0) ? Cn : min(Lc, total - done);
           done += len;
-          const uint32_t d = tmem + (b ? (uint32_t)BN : 0u);
-          for (int i = 0; i < len; ++i, ++g) {
-            const int s = g % STG;
-            if (!mbar_wait_fast(&full[s], (g / STG) & 1)) {
+          const uint32_t d = tmem + b * BN;
+          uint32_t acc = 0;
+          for (int i = 0; i < len; ++i) {
+            if (!bar_spin(full0 + 8 * slot, ph)) {
               ok = false;
               break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            mma_block<TF32>(d, sA + s * A_BYTES, sB + s * B_BYTES, idesc, i == 0);
-            mma_commit(&empty[s]);
+            mma_words<TF32>(d, alo, blo, idesc, acc);
+            mma_words<TF32>(d, alo + 2, blo + 2, idesc, 1u);
+            mma_words<TF32>(d, alo + 4, blo + 4, idesc, 1u);
+            mma_words<TF32>(d, alo + 6, blo + 6, idesc, 1u);
+            bar_commit(empty0 + 8 * slot);
+            acc = 1;
+            alo += A_BYTES >> 4;
+            blo += B_BYTES >> 4;
+            if (++slot == STG) {
+              slot = 0;
+              ph ^= 1;
+              alo = alo0;
+              blo = blo0;
+            }
           }
-          if (ok) mma_commit(&acc_full[b]);
+          if (ok) bar_commit(accf0 + 8 * b);
         }
         if (!ok) {
           atomicExch(a.err, 2);

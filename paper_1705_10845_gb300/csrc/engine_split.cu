@@ -118,6 +118,7 @@ struct CombList {
 };
 
 __global__ void combine_group_kernel(int np, int fmt, CombList L) {
+  grid_wait();
   const int j = blockIdx.y;
   float g[4];
 #pragma unroll
@@ -168,6 +169,7 @@ struct T0List {
 };
 
 __global__ void t0_init_group_kernel(int np, int nlev, int fmt, int dt0, double sc, T0List L) {
+  grid_wait();
   const int j = blockIdx.y;
   const double mu = L.dpar[j] ? L.dpar[j][0] : L.mu[j];
   const double t0 = L.dpar[j] ? L.dpar[j][dt0] : L.t0[j];
@@ -217,6 +219,7 @@ struct ChainScaleList {
 };
 
 __global__ void chain_scales_kernel(int np, int nlev, ChainScaleList L) {
+  grid_wait();
   __shared__ float sm[32];
   const int j = blockIdx.x;
   float m = 0.0f;
@@ -249,6 +252,7 @@ struct A1List {
 };
 
 __global__ void level0_A1_group_kernel(int np, int fmt, A1List L) {
+  grid_wait();
   const int j = blockIdx.y;
   const float4* T0 = reinterpret_cast<const float4*>(L.T0[j]);
   const double* d = L.d[j];
@@ -276,6 +280,7 @@ struct DiagList {
 
 // out_i = (Y M)_ii = Mt_ii - sum_j W_ij Mt_ij  (Y = I - W, Mt = M^T), one warp per row
 __global__ void row_dot_last_group_kernel(int np, DiagList L) {
+  grid_wait();
   const int j = blockIdx.y;
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -298,6 +303,7 @@ __global__ void row_dot_last_group_kernel(int np, DiagList L) {
 }
 
 __global__ void get_diag_group_kernel(int np, DiagList L) {
+  grid_wait();
   const int j = blockIdx.y;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < L.N[j]) L.out[j][i] = df_val(L.X[j][(size_t)i * np + i]);
@@ -505,9 +511,8 @@ class EngineSplit : public Engine {
       L.lo[i] = hi_only ? nullptr : Y[i]->lo;
       L.scale[i] = Y[i]->scale;
     }
-    combine_group_kernel<<<ew_grid((size_t)np * np / 4, L.n), 256, 0, s>>>(np, fmt_, L);
-    note_launch();
-    return cudaGetLastError();
+    RET(launch_chained(s, ew_grid((size_t)np * np / 4, L.n), 256, 0, combine_group_kernel, np, fmt_, L));
+    return cudaSuccess;
   }
 
   // operands of a matrix from its value, in place
@@ -560,9 +565,7 @@ class EngineSplit : public Engine {
       tl.scales[i] = m.scales;
       tl.t0_dev[i] = m.t0_dev;
     }
-    t0_init_group_kernel<<<ew_grid(cnt / 4, B), 256, 0, s>>>(np, n, fmt_, kPassT0, sc, tl);
-    note_launch();
-    RET(cudaGetLastError());
+    RET(launch_chained(s, ew_grid(cnt / 4, B), 256, 0, t0_init_group_kernel, np, n, fmt_, kPassT0, sc, tl));
     std::vector<SplitMat*> W(B), Wn(B);
     // scratch of the corrections: matrices of the response chains, which are free here
     auto Sk = [](MatSet& m, int k) -> SplitMat* { return (k & 1) ? &m.sT1b : &m.sS; };   // S_k beside S_{k-1}
@@ -777,9 +780,8 @@ class EngineSplit : public Engine {
     RET(combine_group(s, np, cc, C, single));
     RET(gemm_group(s, np, oc, true));
     RET(gemm_group(s, np, ot, true));
-    get_diag_group_kernel<<<dim3((maxN + 255) / 256, B), 256, 0, s>>>(np, dl);
-    note_launch();
-    return cudaGetLastError();
+    RET(launch_chained(s, dim3((maxN + 255) / 256, B), 256, 0, get_diag_group_kernel, np, dl));
+    return cudaSuccess;
   }
 
   cudaError_t chain(cudaStream_t s, MatSet& m, const double* dvec, int N, double* out_diag,
@@ -822,9 +824,7 @@ class EngineSplit : public Engine {
       sl.t0[i] = jobs[i].m->t0_dev;
       sl.scales[i] = jobs[i].m->chain_scales;
     }
-    chain_scales_kernel<<<B, 256, 0, s>>>(np, n, sl);
-    note_launch();
-    RET(cudaGetLastError());
+    RET(launch_chained(s, B, 256, 0, chain_scales_kernel, np, n, sl));
     std::vector<SplitMat*> T1(B), T1n(B), A1s(B), Mts(B);
     for (int i = 0; i < B; ++i) {
       T1[i] = &jobs[i].m->sT1a;
@@ -857,9 +857,7 @@ class EngineSplit : public Engine {
           al.lo[i] = single ? nullptr : A1s[i]->lo;
           al.scale[i] = A1s[i]->scale;
         }
-        level0_A1_group_kernel<<<ew_grid(cnt / 4, B), 256, 0, s>>>(np, fmt_, al);
-        note_launch();
-        RET(cudaGetLastError());
+        RET(launch_chained(s, ew_grid(cnt / 4, B), 256, 0, level0_A1_group_kernel, np, fmt_, al));
         for (int i = 0; i < B; ++i) {
           Epi e = em;
           e.dvec = jobs[i].dvec;
@@ -903,9 +901,8 @@ class EngineSplit : public Engine {
           dl.out[i] = jobs[i].out_diag;
           maxN = std::max(maxN, jobs[i].N);
         }
-        row_dot_last_group_kernel<<<dim3((maxN + 7) / 8, B), 256, 0, s>>>(np, dl);
-        note_launch();
-        return cudaGetLastError();
+        RET(launch_chained(s, dim3((maxN + 7) / 8, B), 256, 0, row_dot_last_group_kernel, np, dl));
+        return cudaSuccess;
       }
       std::vector<GemmOp> oy;
       for (int i = 0; i < B; ++i) {

@@ -11,8 +11,15 @@
 namespace xl {
 namespace {
 
-__global__ void t0_init_kernel(int n, int np, const double* __restrict__ H, double mu, double scale,
-                               double* __restrict__ T0) {
+#define RET(x)                        \
+  do {                                \
+    cudaError_t e_ = (x);             \
+    if (e_ != cudaSuccess) return e_; \
+  } while (0)
+
+__global__ void t0_init_kernel(int n, int np, const double* H, double mu, double scale,
+                               double* T0) {
+  grid_wait();
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (size_t)np * np) return;
   const int i = (int)(idx / np), j = (int)(idx % np);
@@ -21,9 +28,10 @@ __global__ void t0_init_kernel(int n, int np, const double* __restrict__ H, doub
   T0[idx] = v;
 }
 
-__global__ void combine_kernel(int np, double a, double c1, const double* __restrict__ X1, double c2,
-                               const double* __restrict__ X2, double c3, const double* __restrict__ X3,
-                               double* __restrict__ Y) {
+__global__ void combine_kernel(int np, double a, double c1, const double* X1, double c2,
+                               const double* X2, double c3, const double* X3,
+                               double* Y) {
+  grid_wait();
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (size_t)np * np) return;
   double v = (idx / np == idx % np) ? a : 0.0;
@@ -34,8 +42,9 @@ __global__ void combine_kernel(int np, double a, double c1, const double* __rest
 }
 
 // A1 = T0 diag(d) + diag(d) T0  (first level of a chain with diagonal T1_0)
-__global__ void level0_A1_kernel(int np, const double* __restrict__ T0, const double* __restrict__ d,
-                                 double* __restrict__ A1) {
+__global__ void level0_A1_kernel(int np, const double* T0, const double* d,
+                                 double* A1) {
+  grid_wait();
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (size_t)np * np) return;
   const int i = (int)(idx / np), j = (int)(idx % np);
@@ -43,7 +52,8 @@ __global__ void level0_A1_kernel(int np, const double* __restrict__ T0, const do
 }
 
 // A1 = G + G^T through 32x32 shared-memory tiles (coalesced both ways).
-__global__ void transpose_add_kernel(int np, const double* __restrict__ G, double* __restrict__ A1) {
+__global__ void transpose_add_kernel(int np, const double* G, double* A1) {
+  grid_wait();
   __shared__ double tile[32][33];
   const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
   const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
@@ -56,8 +66,9 @@ __global__ void transpose_add_kernel(int np, const double* __restrict__ G, doubl
 }
 
 // out[i] = sum_j Y_ij M_ij (i < n): the diagonal of Y M^T, one warp per row.
-__global__ void row_dot_kernel(int n, int np, const double* __restrict__ Y, const double* __restrict__ M,
-                               double* __restrict__ out) {
+__global__ void row_dot_kernel(int n, int np, const double* Y, const double* M,
+                               double* out) {
+  grid_wait();
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (i >= n) return;
@@ -69,7 +80,8 @@ __global__ void row_dot_kernel(int n, int np, const double* __restrict__ Y, cons
   if (lane == 0) out[i] = acc;
 }
 
-__global__ void get_diag_kernel(int n, int np, const double* __restrict__ X, double* __restrict__ out) {
+__global__ void get_diag_kernel(int n, int np, const double* X, double* out) {
+  grid_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = X[(size_t)i * np + i];
 }
@@ -348,42 +360,36 @@ cudaError_t launch_density_out_f64(cudaStream_t s, int N, int np, const double* 
 }
 
 cudaError_t launch_t0_init(cudaStream_t s, int n, int np, const double* H, double mu, double scale, double* T0) {
-  t0_init_kernel<<<blocks_for((size_t)np * np, 256), 256, 0, s>>>(n, np, H, mu, scale, T0);
-  note_launch();
-  return cudaGetLastError();
+  RET(launch_chained(s, blocks_for((size_t)np * np, 256), 256, 0, t0_init_kernel, n, np, H, mu, scale, T0));
+  return cudaSuccess;
 }
 
 cudaError_t launch_combine(cudaStream_t s, int np, double a, double c1, const double* X1, double c2, const double* X2,
                            double c3, const double* X3, double* Y) {
-  combine_kernel<<<blocks_for((size_t)np * np, 256), 256, 0, s>>>(np, a, c1, X1, c2, X2, c3, X3, Y);
-  note_launch();
-  return cudaGetLastError();
+  RET(launch_chained(s, blocks_for((size_t)np * np, 256), 256, 0, combine_kernel, np, a, c1, X1, c2, X2, c3, X3, Y));
+  return cudaSuccess;
 }
 
 cudaError_t launch_level0_A1(cudaStream_t s, int np, const double* T0, const double* d, double* A1) {
-  level0_A1_kernel<<<blocks_for((size_t)np * np, 256), 256, 0, s>>>(np, T0, d, A1);
-  note_launch();
-  return cudaGetLastError();
+  RET(launch_chained(s, blocks_for((size_t)np * np, 256), 256, 0, level0_A1_kernel, np, T0, d, A1));
+  return cudaSuccess;
 }
 
 cudaError_t launch_transpose_add(cudaStream_t s, int np, const double* G, double* A1) {
   if (np % 32) return cudaErrorInvalidValue;
   dim3 grid(np / 32, np / 32), block(32, 8);
-  transpose_add_kernel<<<grid, block, 0, s>>>(np, G, A1);
-  note_launch();
-  return cudaGetLastError();
+  RET(launch_chained(s, grid, block, 0, transpose_add_kernel, np, G, A1));
+  return cudaSuccess;
 }
 
 cudaError_t launch_row_dot(cudaStream_t s, int n, int np, const double* Y, const double* M, double* out) {
-  row_dot_kernel<<<(n + 7) / 8, 256, 0, s>>>(n, np, Y, M, out);
-  note_launch();
-  return cudaGetLastError();
+  RET(launch_chained(s, (n + 7) / 8, 256, 0, row_dot_kernel, n, np, Y, M, out));
+  return cudaSuccess;
 }
 
 cudaError_t launch_get_diag(cudaStream_t s, int n, int np, const double* X, double* out) {
-  get_diag_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, np, X, out);
-  note_launch();
-  return cudaGetLastError();
+  RET(launch_chained(s, (n + 255) / 256, 256, 0, get_diag_kernel, n, np, X, out));
+  return cudaSuccess;
 }
 
 cudaError_t launch_sum(cudaStream_t s, int n, const double* x, double* out) {

@@ -49,9 +49,10 @@ struct F64Batch {
 
 // 8 x 8 tiles: warp w takes the K chunks w, w + 4, ..; lane l holds (l / 4, l % 4) and (l / 4, l % 4 + 4).
 template <bool SYM>
-__global__ void __launch_bounds__(128) gemm_f64_t8_kernel(int M, int N, int K, const double* __restrict__ A, int lda,
-                                                          const double* __restrict__ B, int ldb, double* C, int ldc,
+__global__ void __launch_bounds__(128) gemm_f64_t8_kernel(int M, int N, int K, const double* A, int lda,
+                                                          const double* B, int ldb, double* C, int ldc,
                                                           EpiF64 e, F64Batch st) {
+  grid_wait();
   __shared__ double sa[4][8][KC + 1], sb[4][8][KC + 1];
   __shared__ double red[3][64];
   A += st.a * blockIdx.z;
@@ -118,9 +119,10 @@ __global__ void __launch_bounds__(128) gemm_f64_t8_kernel(int M, int N, int K, c
 
 // T x T tiles (16 or 32), four warps in 2 x 2, each (T / 2)^2 outputs as 8 x 8 blocks of two per lane.
 template <int T, bool SYM>
-__global__ void __launch_bounds__(128) gemm_f64_t_kernel(int M, int N, int K, const double* __restrict__ A, int lda,
-                                                         const double* __restrict__ B, int ldb, double* C, int ldc,
+__global__ void __launch_bounds__(128) gemm_f64_t_kernel(int M, int N, int K, const double* A, int lda,
+                                                         const double* B, int ldb, double* C, int ldc,
                                                          EpiF64 e, F64Batch st) {
+  grid_wait();
   constexpr int NB = T / 16;              // 8 x 8 blocks per warp and dimension
   constexpr int PER = T * KC / 2 / 128;   // 16-byte pieces per thread, operand and chunk
   __shared__ double sa[2][T][KC + 1], sb[2][T][KC + 1];
@@ -195,9 +197,10 @@ __global__ void __launch_bounds__(128) gemm_f64_t_kernel(int M, int N, int K, co
 }
 
 template <bool SYM>
-__global__ void __launch_bounds__(256) gemm_f64_kernel(int M, int N, int K, const double* __restrict__ A,
-                                                       int lda, const double* __restrict__ B, int ldb,
+__global__ void __launch_bounds__(256) gemm_f64_kernel(int M, int N, int K, const double* A,
+                                                       int lda, const double* B, int ldb,
                                                        double* C, int ldc, EpiF64 e, F64Batch st) {
+  grid_wait();
   constexpr int BM = 64, BN = 64, BK = KC;
   A += st.a * blockIdx.z;
   B += st.b * blockIdx.z;
@@ -270,13 +273,17 @@ int pick_tile(int M, int N, bool sym, int batch) {
 }
 
 template <bool SYM>
-void launch(cudaStream_t s, int tile, dim3 grid, int M, int N, int K, const double* A, int lda, const double* B, int ldb,
+cudaError_t launch(cudaStream_t s, int tile, dim3 grid, int M, int N, int K, const double* A, int lda, const double* B, int ldb,
             double* C, int ldc, const EpiF64& e, const F64Batch& st) {
   switch (tile) {
-    case 8: gemm_f64_t8_kernel<SYM><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, e, st); break;
-    case 16: gemm_f64_t_kernel<16, SYM><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, e, st); break;
-    case 32: gemm_f64_t_kernel<32, SYM><<<grid, 128, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, e, st); break;
-    default: gemm_f64_kernel<SYM><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, e, st);
+    case 8:
+      return launch_chained(s, grid, 128, 0, gemm_f64_t8_kernel<SYM>, M, N, K, A, lda, B, ldb, C, ldc, e, st);
+    case 16:
+      return launch_chained(s, grid, 128, 0, gemm_f64_t_kernel<16, SYM>, M, N, K, A, lda, B, ldb, C, ldc, e, st);
+    case 32:
+      return launch_chained(s, grid, 128, 0, gemm_f64_t_kernel<32, SYM>, M, N, K, A, lda, B, ldb, C, ldc, e, st);
+    default:
+      return launch_chained(s, grid, 256, 0, gemm_f64_kernel<SYM>, M, N, K, A, lda, B, ldb, C, ldc, e, st);
   }
 }
 
@@ -291,12 +298,8 @@ cudaError_t gemm_f64_nt(cudaStream_t s, int M, int N, int K, const double* A, in
   const long long nt = N / t;
   const dim3 grid((unsigned)(sym ? nt * (nt + 1) / 2 : nt * (M / t)), 1, (unsigned)batch);
   const F64Batch st{stA, stB, stC, stE};
-  if (sym)
-    launch<true>(s, t, grid, M, N, K, A, lda, B, ldb, C, ldc, e, st);
-  else
-    launch<false>(s, t, grid, M, N, K, A, lda, B, ldb, C, ldc, e, st);
-  note_launch();
-  return cudaGetLastError();
+  return sym ? launch<true>(s, t, grid, M, N, K, A, lda, B, ldb, C, ldc, e, st)
+             : launch<false>(s, t, grid, M, N, K, A, lda, B, ldb, C, ldc, e, st);
 }
 
 }  // namespace xl

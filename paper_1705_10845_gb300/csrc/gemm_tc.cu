@@ -344,16 +344,16 @@ __device__ __forceinline__ EpiRegs load_epi(const TcArgs& a) {
   e.dvec_scale = a.dvec_scale;
   e.va = a.va;
   e.vb = a.vb;
-  e.inv = a.alpha / (__ldg(a.sa) * __ldg(a.sb));
+  e.inv = a.alpha / (*a.sa * *a.sb);
   e.f = a.out.f;
   e.d = a.out.d;
   e.hi = a.out.hi;
   e.lo = a.out.lo;
-  e.so = a.out.hi ? __ldg(a.out.scale) : 0.0f;
+  e.so = a.out.hi ? *a.out.scale : 0.0f;
   e.f2 = a.out2.f;
   e.hi2 = a.out2.hi;
   e.lo2 = a.out2.lo;
-  e.so2 = a.out2.hi ? __ldg(a.out2.scale) : 0.0f;
+  e.so2 = a.out2.hi ? *a.out2.scale : 0.0f;
   e.ldc = a.ldc;
   e.ndvec = a.ndvec;
   e.fmt = a.fmt;
@@ -401,7 +401,7 @@ __device__ __forceinline__ void store_out(float* f, float2* d, void* hi, void* l
 }
 
 // 4 x 4 values of a side input; on a diagonal chunk from its upper triangle.
-__device__ __forceinline__ void load_side(float (&e)[4][4], const float* __restrict__ E, size_t i, size_t st, bool dg,
+__device__ __forceinline__ void load_side(float (&e)[4][4], const float* E, size_t i, size_t st, bool dg,
                                           int row, int col, int ldc) {
   if (!dg) {
 #pragma unroll
@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
                               const __grid_constant__ CUtensorMap mBhi, const __grid_constant__ CUtensorMap mBlo,
                               const __grid_constant__ CUtensorMap mA2hi, const __grid_constant__ CUtensorMap mA2lo,
                               const __grid_constant__ CUtensorMap mB2hi, const __grid_constant__ CUtensorMap mB2lo,
-                              TcArgs a, int ntiles, const TcEntry* __restrict__ tab, int tiles_per) {
+                              TcArgs a, int ntiles, const TcEntry* tab, int tiles_per) {
   using Cfg = PCfg<BN>;
   constexpr int STG = Cfg::STG, B_BYTES = Cfg::B_BYTES, COLS = Cfg::COLS;
   constexpr uint32_t TMEM_COLS = 2 * BN;
@@ -926,6 +926,7 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  grid_wait();   // the prologue above overlaps the kernel before
   constexpr int bk = TF32 ? BK / 2 : BK;           // elements per K block (one 128-byte row)
   const int nk = a.K / bk;
   const int total = a.nseg * a.pairs * nk;
@@ -1620,9 +1621,8 @@ cudaError_t launch_width(cudaStream_t s, int slot, int grid, const CUtensorMap (
   auto kern = tf32 ? gemm_tc_persistent_kernel<BN, true> : gemm_tc_persistent_kernel<BN, false>;
   const cudaError_t attr = ensure_smem(slot + (tf32 ? 4 : 0), kern, sb);
   if (attr != cudaSuccess) return attr;
-  kern<<<grid, PCfg<BN>::THREADS, sb, s>>>(m[0], m[1], m[2], m[3], m[4], m[5], m[6], m[7], a, ntiles, tab, tiles_per);
-  note_launch();
-  return cudaGetLastError();
+  return launch_chained(s, grid, PCfg<BN>::THREADS, sb, kern, m[0], m[1], m[2], m[3], m[4], m[5], m[6], m[7], a, ntiles,
+                        tab, tiles_per);
 }
 
 cudaError_t launch_persistent(cudaStream_t s, int width, const CUtensorMap (&m)[8], const TcArgs& a, int ntiles,

@@ -54,6 +54,7 @@ constexpr int BM = 128;
 constexpr int BK = 64;           // 64 x 16-bit = 128 bytes: one swizzle row
 constexpr int STAGES = 4;        // one-CTA-per-tile kernel
 constexpr int A_BYTES = BM * BK * 2;
+constexpr int kOnceMaxN = 3072;  // largest size (multiple of 256) of the narrow tiles
 constexpr int kWaitLimit = 1 << 24;
 constexpr int kGroupM = 16;
 
@@ -732,21 +733,26 @@ __global__ void __launch_bounds__(192, 1)
 
 // Persistent variant: one CTA per SM walks the tiles id = blockIdx.x, blockIdx.x + gridDim.x, ...
 // The producer and MMA threads run ahead into the next tile while the epilogue writes the previous
-// one.  A tile's K blocks run as chunks, each accumulated by itself in one of two TMEM accumulators
-// that alternate from chunk to chunk (and across tiles): the correction segments of a split product
-// (hi*lo, lo*hi, 2^-11 of the whole) are the first chunk, which runs while the epilogue writes the
-// tile before, then the hi*hi sum follows in chunks of chunk_kb K blocks; a single product is one
+// one.  A tile's hi*hi sum runs in chunks of chunk_kb K blocks, each accumulated by itself in one of two
+// TMEM accumulators that alternate from chunk to chunk (and across tiles); a single product is one
 // chunk.  The epilogue warps read each finished chunk (tcgen05.ld), add it to the tile's sum in
 // registers (round-to-nearest FP32) and release the accumulator at once, while the other one fills.
 // Two column groups of four warps share a tile (BN / 2 sums per thread; one group for BN = 32).
+//
+// The corrections of a split product (hi*lo, lo*hi, 2^-11 of the whole) have accumulators of their own.
+// Tiles of up to 128 columns have TMEM for two more, alternating from tile to tile: each K block's hi
+// and lo parts are loaded once (two slots) and all three products taken from them, and the corrections
+// are added last.  The ring's turn-around is about 2 us a slot at any width, so a third fewer slots are
+// a third less time in the K loop: n = 640 symmetric 14.1 -> 12.0 us, 1408 25.7 -> 21.8, 2048 42.3 -> 37.0.
+// Tiles of 256 columns take the corrections as a first chunk, which runs while the epilogue still writes
+// the tile before, and load the hi parts a second time.  (One accumulator for all three products had
+// three times the error.)
 //
 // The tensor core truncates as it accumulates, so a sum's error grows with its length; with the sums in
 // registers a chunk costs its one tcgen05.ld pass.  (The sums used to live in TMEM, each fold a load, a
 // load, an add and a store that the next chunk had to wait for.)  A tcgen05.ld holds up the MMAs
 // beside it by a time that hardly depends on its size: with 256-wide tiles and 512-long chunks, n = 8192
-// takes 2.46 ms with loads of 32 columns and 2.30 ms with loads of 64.  Taking all three products of a K block from one pair of hi and lo slots
-// loads a third fewer bytes, but with both in one accumulator the errors were three times as large, and
-// at n = 8192 it ran no faster (2.87 against 2.53 ms: only two K blocks fit in the ring).
+// takes 2.46 ms with loads of 32 columns and 2.30 ms with loads of 64.
 //
 // Barriers: full/empty (operand ring), acc_full[2] (MMA -> epilogue), acc_free[2] (epilogue -> MMA,
 // one arrival per epilogue warp).  Chunk c of the CTA uses accumulator c % 2 and waits for release
@@ -814,7 +820,11 @@ struct PCfg {
   static constexpr int NEPI = 4 * CG;
   static constexpr int THREADS = 128 + 32 * NEPI;   // warpgroup 0: producer and MMA warps (and two idle ones)
   static constexpr int COLS = BN / CG;
-  static constexpr int STG = BN == 256 ? 4 : BN == 128 ? 6 : 8;
+  // split products of up to 128 columns load each K block's hi and lo parts once (two slots) and do all
+  // three products from them
+  static constexpr bool ONCE = BN <= 128;
+  static constexpr int STG = BN == 256 ? 4 : BN == 128 ? 6 : BN == 64 ? 8 : 10;   // even where ONCE
+  static constexpr uint32_t TMEM_COLS = (ONCE ? 4 : 2) * BN;   // ONCE: two accumulators for corrections
   static constexpr int B_BYTES = BN * BK * 2;
   static constexpr int STAGE_TILE = 32 * 33 * 4;
   static constexpr int SMEM = STG * (A_BYTES + B_BYTES) + NEPI * STAGE_TILE + (2 * STG + 4) * 8 + 16 + 1024;
@@ -889,7 +899,7 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
                               TcArgs a, int ntiles, const TcEntry* tab, int tiles_per) {
   using Cfg = PCfg<BN>;
   constexpr int STG = Cfg::STG, B_BYTES = Cfg::B_BYTES, COLS = Cfg::COLS;
-  constexpr uint32_t TMEM_COLS = 2 * BN;
+  constexpr uint32_t TMEM_COLS = Cfg::TMEM_COLS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
@@ -929,9 +939,10 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
   grid_wait();   // the prologue above overlaps the kernel before
   constexpr int bk = TF32 ? BK / 2 : BK;           // elements per K block (one 128-byte row)
   const int nk = a.K / bk;
-  const int total = a.nseg * a.pairs * nk;
+  const bool once = Cfg::ONCE && a.nseg > 1;
   const int H = a.pairs * nk;                      // hi*hi K blocks
-  const int Cn = total - H;                        // correction K blocks (the first chunk)
+  const int Cn = once ? 0 : (a.nseg - 1) * H;      // correction K blocks in a chunk of their own (the first)
+  const int total = Cn + H;
   const int Lc = (a.nseg > 1 && a.chunk_kb > 0 && a.chunk_kb < H) ? a.chunk_kb : H;   // hi*hi chunk
   const int nch = (Cn > 0 ? 1 : 0) + (H + Lc - 1) / Lc;                               // chunks per tile
 
@@ -958,20 +969,22 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
           for (int i = 0; i < 8; ++i) tensormap_acquire(&maps[i]);
           last_p = p;
         }
-        // segments: the corrections hi*lo, lo*hi of each pair, then hi*hi of each pair
-        for (int sg = a.nseg > 1 ? 0 : 2 * a.pairs; sg < 3 * a.pairs && ok; ++sg) {
-          const int pr = sg < 2 * a.pairs ? sg >> 1 : sg - 2 * a.pairs;
-          const int kind = sg < 2 * a.pairs ? 1 + (sg & 1) : 0;
-          const int ia = (kind == 2) ? (pr ? 5 : 1) : (pr ? 4 : 0);
-          const int ib = (kind == 1) ? (pr ? 7 : 3) : (pr ? 6 : 2);
-          const CUtensorMap* ma = maps ? &maps[ia] : (kind == 2) ? (pr ? &mA2lo : &mAlo) : (pr ? &mA2hi : &mAhi);
-          const CUtensorMap* mb = maps ? &maps[ib] : (kind == 1) ? (pr ? &mB2lo : &mBlo) : (pr ? &mB2hi : &mBhi);
-          for (int k = 0; k < a.K; k += bk) {
+        // Segments of K blocks, two loads of A and B tiles per K block in the first kind:
+        //   once    the hi parts, the lo parts
+        //   else    corrections: A hi and B lo, A lo and B hi; then (kind 1) the hi parts alone
+        // each for the pair and, in pair products, the swapped pair.
+        for (int sg = (a.nseg > 1 ? 0 : a.pairs); sg < (once ? 1 : 2) * a.pairs && ok; ++sg) {
+          const int pr = sg % a.pairs;
+          const bool two = sg < a.pairs;
+          const CUtensorMap* ahi = maps ? &maps[pr ? 4 : 0] : pr ? &mA2hi : &mAhi;
+          const CUtensorMap* alo_ = maps ? &maps[pr ? 5 : 1] : pr ? &mA2lo : &mAlo;
+          const CUtensorMap* bhi = maps ? &maps[pr ? 6 : 2] : pr ? &mB2hi : &mBhi;
+          const CUtensorMap* blo_ = maps ? &maps[pr ? 7 : 3] : pr ? &mB2lo : &mBlo;
+          auto put = [&](const CUtensorMap* ma, const CUtensorMap* mb, int k) -> bool {
             if (!first && !bar_spin(empty0 + 8 * slot, ph ^ 1)) {
               atomicExch(a.err, 1);
               *abort_flag = 1;
-              ok = false;
-              break;
+              return false;
             }
             load_slot(full0 + 8 * slot, A_BYTES + B_BYTES, a0 + slot * A_BYTES, ma, b0 + slot * B_BYTES, mb, k, tm * BM,
                       tn * BN);
@@ -980,6 +993,14 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
               ph ^= 1;
               first = false;
             }
+            return true;
+          };
+          if (two) {
+            const CUtensorMap* b1 = once ? bhi : blo_;
+            const CUtensorMap* b2 = once ? blo_ : bhi;
+            for (int k = 0; k < a.K && ok; k += bk) ok = put(ahi, b1, k) && put(alo_, b2, k);
+          } else {
+            for (int k = 0; k < a.K && ok; k += bk) ok = put(ahi, bhi, k);
           }
         }
       }
@@ -991,7 +1012,8 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
       const uint32_t alo0 = desc_lo(a0), blo0 = desc_lo(b0);
       const uint32_t accf0 = smem_u32(acc_full), accr0 = smem_u32(acc_free);
       uint32_t alo = alo0, blo = blo0, c = 0;   // descriptors of the slot; chunks of this CTA so far
-      for (int id = blockIdx.x; id < ntiles && ok && !*abort_flag; id += gridDim.x) {
+      uint32_t par = 0;                // once: the tile's correction accumulator
+      for (int id = blockIdx.x; id < ntiles && ok && !*abort_flag; id += gridDim.x, par ^= 1) {
         int tm, tn, p, lid;
         group_tile(tab, tiles_per, id, p, lid);
         if (!tile_coords(a, lid, tm, tn)) break;
@@ -1019,8 +1041,26 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
             mma_words<TF32>(d, alo + 2, blo + 2, idesc, 1u);
             mma_words<TF32>(d, alo + 4, blo + 4, idesc, 1u);
             mma_words<TF32>(d, alo + 6, blo + 6, idesc, 1u);
-            bar_commit(empty0 + 8 * slot);
             acc = 1;
+            if (once) {                // the lo slot is the next one of the same round (STG is even)
+              if (!bar_spin(full0 + 8 * slot + 8, ph)) {
+                ok = false;
+                break;
+              }
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              const uint32_t dc = tmem + (2 + par) * BN;
+              const uint32_t al = alo + (A_BYTES >> 4), bl = blo + (B_BYTES >> 4);
+              const uint32_t fc = (ch == 0 && i == 0) ? 0u : 1u;
+#pragma unroll
+              for (int j = 0; j < 4; ++j) mma_words<TF32>(dc, alo + 2 * j, bl + 2 * j, idesc, j == 0 ? fc : 1u);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) mma_words<TF32>(dc, al + 2 * j, blo + 2 * j, idesc, 1u);
+              bar_commit(empty0 + 8 * slot);
+              ++slot;
+              alo = al;
+              blo = bl;
+            }
+            bar_commit(empty0 + 8 * slot);
             alo += A_BYTES >> 4;
             blo += B_BYTES >> 4;
             if (++slot == STG) {
@@ -1044,8 +1084,8 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
     const int q = warp & 3, cg = (warp - 4) >> 2;
     float(*t)[33] = reinterpret_cast<float(*)[33]>(stage + (warp - 4) * Cfg::STAGE_TILE);
     const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cg * COLS);
-    uint32_t c = 0;
-    for (int id = blockIdx.x; id < ntiles && !*abort_flag; id += gridDim.x) {
+    uint32_t c = 0, par = 0;
+    for (int id = blockIdx.x; id < ntiles && !*abort_flag; id += gridDim.x, par ^= 1) {
       int tm, tn, p, lid;
       group_tile(tab, tiles_per, id, p, lid);
       if (!tile_coords(a, lid, tm, tn)) break;
@@ -1081,6 +1121,15 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
             tmem_ld32(tbase + (uint32_t)(b * BN + x * 32), v);
 #pragma unroll
             for (int i = 0; i < 32; ++i) sum[x][i] = ch ? sum[x][i] + v[i] : v[i];
+          }
+          if (once && ch == nch - 1) {   // the tile's corrections
+#pragma unroll
+            for (int x = 0; x < COLS / 32; ++x) {
+              float v[32];
+              tmem_ld32(tbase + (uint32_t)((2 + par) * BN + x * 32), v);
+#pragma unroll
+              for (int i = 0; i < 32; ++i) sum[x][i] += v[i];
+            }
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1640,18 +1689,18 @@ int tiles_of(int n, int width, bool sym, const TcTiles& t) {
   return sym ? t.nsym[width] : (n / BM) * (n / tc_width(width));
 }
 
-// Tile width of a persistent launch over nprob problems of size n: the one with the least waves of
-// tiles times the time of a tile.  The times of a 128 x w tile relative to w = 128 hardly depend on n (one
-// CTA's K loop is bound by its hand-offs, not by the width): symmetric split products of n = 2048 take
-// 123 us with w = 32 (4 waves), 68 with 64 (2 waves), 45 with 128 (1 wave), 66 with 256; n = 1408: 48, 29,
-// 35; n = 256: 10.8, 12.0, 16.9, 28.2; n = 4096: 803, 415, 263 (4 waves), 219 (2 waves).
+// Tile width of a persistent launch over nprob problems of size n: 256 where n > 3072 allows it, else the one
+// of 32, 64 and 128 with the least waves of tiles times the time of a tile.  (The 256-wide tiles add up
+// their corrections apart from the rest, so their results differ from the others' in rounding; a size
+// always takes one kind, whatever the number of problems.)  The times of a 128 x w tile relative to
+// w = 128 hardly depend on n: a CTA's K loop is bound by the ring's turn-around, about 2 us at any width.
 int pick_width(int n, int nprob, const TcArgs& a, const TcTiles& t) {
   static const int cost[kTcWidths] = {68, 75, 100, 150};
+  if (n > kOnceMaxN && n % 256 == 0) return 3;
   const int sms = sm_count();
   int best = 2;
   long long least = -1;
-  for (int w = 0; w < kTcWidths; ++w) {
-    if (n % tc_width(w)) continue;
+  for (int w = 0; w < 3; ++w) {
     const long long tiles = (long long)nprob * tiles_of(n, w, a.sym != 0, t);
     const long long c = (tiles + sms - 1) / sms * cost[w];
     if (least < 0 || c < least) {

@@ -252,9 +252,43 @@ xlbomd_status sync_read(xlbomd_ctx* ctx, const double* dev, int count) {
   return XLBOMD_OK;
 }
 
+// The vectors of a product with gamma, and of a response, of system S (x: the charges or the probe)
+ProbeJob probe_job(const Sys& S, const double* x, double* pot, double* tmp) {
+  ProbeJob j;
+  j.nat = S.nat;
+  j.N = S.N;
+  j.np = S.np;
+  j.natp = S.natp;
+  j.kp = S.kp;
+  j.gam = S.gam;
+  j.SF = S.SF;
+  j.x = x;
+  j.tmp = tmp;
+  j.pot = pot;
+  j.dmu = S.dmu_diag;
+  j.dvec = S.dvec;
+  j.d1 = S.d1;
+  j.scal = S.scal + 4;
+  return j;
+}
+
 // y = gamma x (real-space matrix plus the reciprocal part through the structure factors)
 cudaError_t gamma_apply(xlbomd_ctx* ctx, Sys& S, const double* x, double* y, double* tmp) {
-  return launch_gamma_apply(ctx->stream, S.nat, S.gam, S.natp, S.SF, S.kp, ctx->p.coulomb_k, x, y, tmp);
+  return launch_probe_potential(ctx->stream, ctx->p.coulomb_k, {probe_job(S, x, y, tmp)});
+}
+
+KernelVecJob kernel_vec_job(const Sys& S, int mode, int m, double* flag) {
+  KernelVecJob j;
+  j.mode = mode;
+  j.nat = S.nat;
+  j.m = m;
+  j.c = S.kc;
+  j.r = S.r;
+  j.V = S.pV;
+  j.W = S.pW;
+  j.out = S.Kr;
+  j.flag = flag;
+  return j;
 }
 
 // a1-a2
@@ -537,13 +571,21 @@ xlbomd_status density_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, bool wi
 }
 
 // a7: one probe.  H1 = diag(gamma v) on orbitals less its average, T1_0 = -sc H1.
-xlbomd_status response(xlbomd_ctx* ctx, Sys& S, const double* v, double* w) {
+xlbomd_status response(xlbomd_ctx* ctx, Sys& S, const ProbeJob& j) {
   cudaStream_t st = ctx->stream;
   const double sc = beta_of(ctx->p) / std::ldexp(1.0, ctx->p.n_sq + 1);
-  CK(gamma_apply(ctx, S, v, S.potv, S.work));
-  CK(launch_expand_potential(st, S.nat, S.np, -sc, S.potv, S.dmu_diag, S.dvec));
+  const std::vector<ProbeJob> jobs{j};
+  CK(launch_probe_potential(st, ctx->p.coulomb_k, jobs));
+  CK(launch_probe_expand(st, -sc, jobs));
   CK(ctx->eng->chain(st, S.mats, S.dvec, S.N, S.d1, S.stats));
-  CK(launch_response_finish(st, S.nat, S.N, S.d1, S.dmu_diag, S.scal + 4, w));
+  CK(launch_probe_finish(st, jobs));
+  return XLBOMD_OK;
+}
+
+xlbomd_status response(xlbomd_ctx* ctx, Sys& S, const double* v, double* w) {
+  ProbeJob j = probe_job(S, v, S.potv, S.work);
+  j.w = w;
+  CKS(response(ctx, S, j));
   return XLBOMD_OK;
 }
 
@@ -553,7 +595,7 @@ xlbomd_status response(xlbomd_ctx* ctx, Sys& S, const double* v, double* w) {
 xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
   cudaStream_t st = ctx->stream;
   const double sc = beta_of(ctx->p) / std::ldexp(1.0, ctx->p.n_sq + 1);
-  const size_t per_vec = 2 * (size_t)S.nat + 3 * (size_t)S.np + (size_t)S.kp + 64;   // v, w, potv?, ...
+  const size_t per_vec = (size_t)S.nat + 2 * (size_t)S.np + 8;   // pot, dvec, d1, scal
   if (S.slots.empty()) {
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
@@ -568,33 +610,33 @@ xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
       }
     CKS(dalloc(ctx, &S.slot_vec, per_vec * G));
   }
-  const int G = (int)S.slots.size();
-  auto vec = [&](int j, int what) -> double* {   // 0 v, 1 w, 2 potv, 3 dvec, 4 d1, 5 scal, 6 tmp
-    double* b = S.slot_vec + per_vec * (size_t)j;
-    const size_t off[7] = {0, (size_t)S.nat, 2 * (size_t)S.nat, 2 * (size_t)S.nat + S.np,
-                           2 * (size_t)S.nat + 2 * (size_t)S.np, 2 * (size_t)S.nat + 3 * (size_t)S.np,
-                           2 * (size_t)S.nat + 3 * (size_t)S.np + 32};
-    return b + off[what];
-  };
+  // parts of one size: 96 probes run as 48 + 48 and not as 64 + 32, which is one wave of tiles less
+  const int parts = (S.nat + (int)S.slots.size() - 1) / (int)S.slots.size();
+  const int G = (S.nat + parts - 1) / parts;
   for (int I0 = 0; I0 < S.nat; I0 += G) {
     const int g = std::min(G, S.nat - I0);
     std::vector<ChainJob> cj(g);
+    std::vector<ProbeJob> pj(g);
     for (int j = 0; j < g; ++j) {
-      CK(launch_unit_vector(st, S.nat, I0 + j, vec(j, 0)));
-      CK(launch_gamma_apply(st, S.nat, S.gam, S.natp, S.SF, S.kp, ctx->p.coulomb_k, vec(j, 0), vec(j, 2),
-                            vec(j, 6)));
-      CK(launch_expand_potential(st, S.nat, S.np, -sc, vec(j, 2), S.dmu_diag, vec(j, 3)));
+      double* b = S.slot_vec + per_vec * (size_t)j;
+      ProbeJob& p = pj[j];
+      p = probe_job(S, nullptr, b, nullptr);
+      p.unit = I0 + j;
+      p.dvec = b + S.nat;
+      p.d1 = p.dvec + S.np;
+      p.scal = p.d1 + S.np;
+      p.Jm = S.Jm;
+      p.B = S.Kfull;
       cj[j].m = &S.slots[j];
-      cj[j].dvec = vec(j, 3);
+      cj[j].dvec = p.dvec;
       cj[j].N = S.N;
-      cj[j].out_diag = vec(j, 4);
+      cj[j].out_diag = p.d1;
       cj[j].stats = S.stats;
     }
+    CK(launch_probe_potential(st, ctx->p.coulomb_k, pj));
+    CK(launch_probe_expand(st, -sc, pj));
     CK(ctx->eng->chain_group(st, cj));
-    for (int j = 0; j < g; ++j) {
-      CK(launch_response_finish(st, S.nat, S.N, vec(j, 4), S.dmu_diag, vec(j, 5), vec(j, 1)));
-      CK(launch_jacobian_column(st, S.nat, I0 + j, vec(j, 1), S.Jm, S.Kfull));
-    }
+    CK(launch_probe_finish(st, pj));
   }
   return XLBOMD_OK;
 }
@@ -611,12 +653,12 @@ xlbomd_status kernel_exact(xlbomd_ctx* ctx, Sys& S) {
   if (ctx->p.prec != XLBOMD_FP64 && S.nat > 1) {
     CKS(exact_columns_grouped(ctx, S));
   } else {
-    double* v = S.pV + (size_t)kMaxRank * S.nat;   // spare probe rows
-    double* w = S.pW + (size_t)kMaxRank * S.nat;
     for (int I = 0; I < S.nat; ++I) {
-      CK(launch_unit_vector(st, S.nat, I, v));
-      CKS(response(ctx, S, v, w));
-      CK(launch_jacobian_column(st, S.nat, I, w, S.Jm, S.Kfull));
+      ProbeJob j = probe_job(S, nullptr, S.potv, nullptr);
+      j.unit = I;
+      j.Jm = S.Jm;
+      j.B = S.Kfull;
+      CKS(response(ctx, S, j));
     }
   }
   CK(cudaMemsetAsync(S.scal + 10, 0, sizeof(double), st));
@@ -681,8 +723,8 @@ xlbomd_status kernel_update(xlbomd_ctx* ctx, Sys& S) {
   }
   int m = 0;
   for (int i = 0; i < p.rank_m; ++i) {
-    CK(launch_kernel_vec(st, 0, S.nat, i, S.kc, S.r, S.pV, S.pW, nullptr, S.scal + 8));
-    CKS(sync_read(ctx, S.scal + 8, 1));
+    CK(launch_kernel_vec(st, {kernel_vec_job(S, 0, i, ctx->pinned)}));
+    CK(cudaStreamSynchronize(st));
     if (ctx->pinned[0] != 1.0) break;
     double* vi = S.pV + (size_t)i * S.nat;
     double* wi = S.pW + (size_t)i * S.nat;
@@ -692,7 +734,7 @@ xlbomd_status kernel_update(xlbomd_ctx* ctx, Sys& S) {
       CKS(response(ctx, S, vi, wi));
     m = i + 1;
   }
-  CK(launch_kernel_vec(st, 1, S.nat, m, S.kc, S.r, S.pV, S.pW, S.Kr, S.scal + 8));
+  CK(launch_kernel_vec(st, {kernel_vec_job(S, 1, m, nullptr)}));
   S.probes_used = m;
   S.stats[2] = m;
   return XLBOMD_OK;
@@ -777,8 +819,8 @@ xlbomd_status scf(xlbomd_ctx* ctx, Sys& S) {
       if (lam < 0.0) S.kc = 1.2 * lam;
       if (debug_enabled()) std::fprintf(stderr, "[xlbomd] stiffest mode %.4f -> c = %.4f\n", lam, S.kc);
     }
-    CK(launch_absmax(st, S.nat, S.r, S.scal + 9));
-    CKS(sync_read(ctx, S.scal + 9, 1));
+    CK(launch_absmax(st, S.nat, S.r, ctx->pinned));
+    CK(cudaStreamSynchronize(st));
     const double res = ctx->pinned[0];
     if (debug_enabled()) std::fprintf(stderr, "[xlbomd] scf it %d max|q - n| %.3e mu %.8f\n", it, res, S.mu);
     if (!std::isfinite(res) || res > 1e3) return fail(ctx, XLBOMD_ERR_DIVERGED, "t0 SCF diverged");
@@ -833,24 +875,22 @@ xlbomd_status response_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, const 
                              const std::vector<double*>& w) {
   cudaStream_t st = ctx->stream;
   const double sc = beta_of(ctx->p) / std::ldexp(1.0, ctx->p.n_sq + 1);
-  std::vector<ChainJob> cj;
+  std::vector<ChainJob> cj(G.size());
+  std::vector<ProbeJob> pj(G.size());
   for (size_t k = 0; k < G.size(); ++k) {
     Sys& S = *G[k];
-    CK(gamma_apply(ctx, S, v[k], S.potv, S.work));
-    CK(launch_expand_potential(st, S.nat, S.np, -sc, S.potv, S.dmu_diag, S.dvec));
-    ChainJob c;
-    c.m = &S.mats;
-    c.dvec = S.dvec;
-    c.N = S.N;
-    c.out_diag = S.d1;
-    c.stats = S.stats;
-    cj.push_back(c);
+    pj[k] = probe_job(S, v[k], S.potv, S.work);
+    pj[k].w = w[k];
+    cj[k].m = &S.mats;
+    cj[k].dvec = S.dvec;
+    cj[k].N = S.N;
+    cj[k].out_diag = S.d1;
+    cj[k].stats = S.stats;
   }
+  CK(launch_probe_potential(st, ctx->p.coulomb_k, pj));
+  CK(launch_probe_expand(st, -sc, pj));
   CK(ctx->eng->chain_group(st, cj));
-  for (size_t k = 0; k < G.size(); ++k) {
-    Sys& S = *G[k];
-    CK(launch_response_finish(st, S.nat, S.N, S.d1, S.dmu_diag, S.scal + 4, w[k]));
-  }
+  CK(launch_probe_finish(st, pj));
   return XLBOMD_OK;
 }
 
@@ -871,11 +911,9 @@ xlbomd_status kernel_update_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
   std::vector<size_t> active(B);
   for (size_t i = 0; i < B; ++i) active[i] = i;
   for (int i = 0; i < p.rank_m && !active.empty(); ++i) {
-    for (size_t k = 0; k < active.size(); ++k) {
-      Sys& S = *G[active[k]];
-      CK(launch_kernel_vec(st, 0, S.nat, i, S.kc, S.r, S.pV, S.pW, nullptr, S.scal + 8));
-      CK(cudaMemcpyAsync(h + k, S.scal + 8, sizeof(double), cudaMemcpyDeviceToHost, st));
-    }
+    std::vector<KernelVecJob> kj;
+    for (size_t k = 0; k < active.size(); ++k) kj.push_back(kernel_vec_job(*G[active[k]], 0, i, h + k));
+    CK(launch_kernel_vec(st, kj));
     CK(cudaStreamSynchronize(st));
     std::vector<size_t> probing;
     for (size_t k = 0; k < active.size(); ++k)
@@ -893,12 +931,14 @@ xlbomd_status kernel_update_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
     if (!g.empty()) CKS(response_group(ctx, g, dv, dw));
     active.swap(probing);
   }
+  std::vector<KernelVecJob> kj;
   for (size_t j = 0; j < B; ++j) {
     Sys& S = *G[j];
-    CK(launch_kernel_vec(st, 1, S.nat, m[j], S.kc, S.r, S.pV, S.pW, S.Kr, S.scal + 8));
+    kj.push_back(kernel_vec_job(S, 1, m[j], nullptr));
     S.probes_used = m[j];
     S.stats[2] = m[j];
   }
+  CK(launch_kernel_vec(st, kj));
   return XLBOMD_OK;
 }
 
@@ -989,8 +1029,7 @@ xlbomd_status scf_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
     CKS(density_group(ctx, g, false));
     if (it == 0 && p.kernel_auto) CKS(stiffest_mode_group(ctx, g));
     for (size_t j = 0; j < g.size(); ++j) {
-      CK(launch_absmax(st, g[j]->nat, g[j]->r, g[j]->scal + 9));
-      CK(cudaMemcpyAsync(h + j, g[j]->scal + 9, sizeof(double), cudaMemcpyDeviceToHost, st));
+      CK(launch_absmax(st, g[j]->nat, g[j]->r, h + j));
     }
     CK(cudaStreamSynchronize(st));
     std::vector<size_t> next;
@@ -1053,10 +1092,9 @@ xlbomd_status md_step_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
   for (size_t k = 0; k < G.size(); ++k) {
     Sys& S = *G[k];
     CK(launch_verlet_second(st, S.nat, p.dt, kAcc / S.mass, S.V, S.F));
-    CK(launch_absmax(st, S.nat, S.r, S.scal + 9));
+    CK(launch_absmax(st, S.nat, S.r, h + k));
     const bool e = p.energy_every > 0 && ((int)S.stats[4] + 1) % p.energy_every == 0;
     if (e) CKS(energy(ctx, S));
-    CK(cudaMemcpyAsync(h + k, S.scal + 9, sizeof(double), cudaMemcpyDeviceToHost, st));
   }
   CK(cudaStreamSynchronize(st));
   for (size_t k = 0; k < G.size(); ++k) {
@@ -1165,14 +1203,19 @@ xlbomd_status xlbomd_response_noalloc(xlbomd_ctx* ctx, int sys, const double* v_
   double* scal = d1 + kStaticMaxNp;
   // the array keeps the previous call's contents: the diagonal accumulator starts at zero
   CK(cudaMemsetAsync(d1, 0, sizeof(double) * kStaticMaxNp, st));
-  CK(gamma_apply(ctx, S, v_dev, potv, scal + 64));
-  CK(launch_expand_potential(st, S.nat, S.np, -sc, potv, S.dmu_diag, dvec));
+  ProbeJob j = probe_job(S, v_dev, potv, scal + 64);
+  j.dvec = dvec;
+  j.d1 = d1;
+  j.scal = scal;
+  j.w = w_dev;
+  CK(launch_probe_potential(st, ctx->p.coulomb_k, {j}));
+  CK(launch_probe_expand(st, -sc, {j}));
   const bool prof = ctx->eng->prof;
   ctx->eng->prof = false;   // event timing would create CUDA events
   const cudaError_t ce = ctx->eng->chain(st, m, dvec, S.N, d1, S.stats);   // counted in XLBOMD_STATS
   ctx->eng->prof = prof;
   CK(ce);
-  CK(launch_response_finish(st, S.nat, S.N, d1, S.dmu_diag, scal, w_dev));
+  CK(launch_probe_finish(st, {j}));
   return XLBOMD_OK;
 }
 

@@ -174,12 +174,14 @@ __global__ void t0_init_group_kernel(int np, int nlev, int fmt, int dt0, double 
   const double mu = L.dpar[j] ? L.dpar[j][0] : L.mu[j];
   const double t0 = L.dpar[j] ? L.dpar[j][dt0] : L.t0[j];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    double t = t0;
-    for (int k = 0; k <= nlev; ++k) {
-      L.scales[j][1 + k] = operand_scale(t);
-      t = 2.0 * t / (1.0 + t * t);
+    float* scales = L.scales[j];
+    float t = (float)t0;   // FP32 for the same reason as in chain_scales_kernel
+    scales[1] = operand_scale(t0);
+    for (int k = 1; k <= nlev; ++k) {
+      t = 2.0f * t / (1.0f + t * t);
+      scales[1 + k] = operand_scale(t);
     }
-    L.scales[j][2 + nlev] = operand_scale(1.0 / (1.0 - t0 * t0));   // |(I - T_0^2)^-1|
+    scales[2 + nlev] = operand_scale(1.0 / (1.0 - t0 * t0));   // |(I - T_0^2)^-1|
     *L.t0_dev[j] = (float)t0;
   }
   const float s = operand_scale(t0);
@@ -229,14 +231,16 @@ __global__ void chain_scales_kernel(int np, int nlev, ChainScaleList L) {
   __syncthreads();
   if (threadIdx.x != 0) return;
   for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, sm[w]);
-  // a bound slightly above the FP32 maximum, so that rounding it down cannot matter
-  double tau = 1.0001 * (double)m, t = 1.0001 * (double)*L.t0[j];
+  // bounds slightly above the FP32 maximum, so that rounding them down cannot matter; in FP32, since one
+  // thread's chain of FP64 divisions took 15 us at 12 levels
+  float tau = 1.0001f * m, t = 1.0001f * *L.t0[j];
+  float* scales = L.scales[j];
   for (int k = 0; k < nlev; ++k) {
-    const double tn = 2.0 * t / (1.0 + t * t), g = t / (1.0 + t * t);
-    L.scales[j][3 * k] = operand_scale(2.0 * t * tau);
-    L.scales[j][3 * k + 1] = operand_scale(2.0 * tau * (1.0 + t * tn));
-    tau *= 2.0 * (1.0 + g * g);
-    L.scales[j][3 * k + 2] = operand_scale(tau);
+    const float g = t / (1.0f + t * t), tn = 2.0f * g;
+    scales[3 * k] = operand_scale(2.0f * t * tau);
+    scales[3 * k + 1] = operand_scale(2.0f * tau * (1.0f + t * tn));
+    tau *= 2.0f * (1.0f + g * g);
+    scales[3 * k + 2] = operand_scale(tau);
     t = tn;
   }
 }

@@ -6,6 +6,8 @@
 // T_0 = -beta (H - mu I) / 2^(n+1), the recursion
 // X_{k+1} = X_k^2 [X_k^2 + (I - X_k)^2]^-1 on X = (I + T)/2 becomes
 // T_{k+1} = 2 T_k (I + T_k^2)^-1 and D = (I + T_n)/2.
+#include <algorithm>
+
 #include "precision.h"
 
 namespace xl {
@@ -105,7 +107,170 @@ __global__ void frob_partial_kernel(int n, int np, const double* __restrict__ A,
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
 
-// ---- rank-m kernel update (one CTA) ----
+// ---- vector algebra of the response chains and of the rank-m kernel update ----
+//
+// Vectors of nat or 4 nat doubles, one block per system or probe and all of them in one launch: the
+// work is nothing, a launch costs 2 to 3 us, and with 2 FP64 operations a clock on an SM a reduction
+// over a block of 1024 threads takes 1.4 us by its shuffles alone.  So few threads and few reductions
+// per block.  A probe of 96 atoms in a group of 48 took 8.2 us in sf_dot and gamma_apply, 7.8 us in
+// the expansion and 8.6 us at the end.
+
+constexpr int kVecThreads = 256;
+constexpr int kMaxJobs = 16;
+
+// The jobs of a launch travel in the kernel parameters.
+template <class Job, int NJ>
+struct JobList {
+  int n = 0;
+  Job job[NJ];
+};
+
+// sums of a and b over a block of kVecThreads; valid in every thread (sh: 16 doubles)
+__device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  a = warp_sum(a);
+  b = warp_sum(b);
+  __syncthreads();
+  if (lane == 0) {
+    sh[wid] = a;
+    sh[8 + wid] = b;
+  }
+  __syncthreads();
+  a = sh[lane & 7];
+  b = sh[8 + (lane & 7)];
+  for (int o = 4; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+}
+
+// t = SF^T x per job: a block takes 32 of its kp structure factors
+template <int NJ>
+__global__ void __launch_bounds__(1024) probe_dot_kernel(const __grid_constant__ JobList<ProbeJob, NJ> L) {
+  grid_wait();
+  const ProbeJob& J = L.job[blockIdx.y];
+  __shared__ double sh[32][33];
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5, g = blockIdx.x * 32 + c;
+  if (blockIdx.x * 32 >= J.kp) return;
+  double acc = 0.0;
+  if (g < J.kp) {
+    const double *SF = J.SF, *x = J.x;
+#pragma unroll 4
+    for (int I = w; I < J.nat; I += 32) acc += SF[(size_t)I * J.kp + g] * x[I];
+  }
+  sh[w][c] = acc;
+  __syncthreads();
+  const int gw = blockIdx.x * 32 + w;   // warp w sums column w
+  const double s = warp_sum(sh[c][w]);
+  if (c == 0 && gw < J.kp) J.tmp[gw] = s;
+}
+
+// pot_I = sum_J gamma_real_IJ x_J + k sum_g SF[I][g] t[g], one block per row.  For a unit probe x = e_u
+// the first sum is the element gamma_real_Iu and t is row u of SF.
+template <int NJ>
+__global__ void probe_apply_kernel(double k, const __grid_constant__ JobList<ProbeJob, NJ> L) {
+  grid_wait();
+  const ProbeJob& J = L.job[blockIdx.y];
+  __shared__ double sh[32];
+  const int I = blockIdx.x;
+  if (I >= J.nat) return;
+  double acc = 0.0, rec = 0.0;
+  const double* gam = J.gam + (size_t)I * J.natp;
+  if (J.unit >= 0) {
+    if (threadIdx.x == 0) acc = gam[J.unit];
+  } else {
+    const double* x = J.x;
+#pragma unroll 4
+    for (int q = threadIdx.x; q < J.nat; q += blockDim.x) acc += gam[q] * x[q];
+  }
+  if (J.SF) {
+    const double* row = J.SF + (size_t)I * J.kp;
+    const double* t = (J.unit >= 0) ? J.SF + (size_t)J.unit * J.kp : J.tmp;
+#pragma unroll 4
+    for (int g = threadIdx.x; g < J.kp; g += blockDim.x) rec += row[g] * t[g];
+  }
+  acc = block_sum(acc + k * rec, sh);
+  if (threadIdx.x == 0) J.pot[I] = acc;
+}
+
+// dvec_a = scale (pot_I - pbar) on the orbitals of atom I, 0 on the padding (one block per job).  A uniform
+// potential has no canonical response (mu follows it); taking the average pbar = sum_a dmu_a pot_a /
+// sum_a dmu_a out beforehand leaves sum_a d1_a = -sum_a pot_a dmu_a at rounding level, so that the
+// chain does not carry a large part that mu_1 dT_n/dmu then has to cancel (the errors of the two are
+// independent).  A unit probe's potential is mostly uniform: K of 48 atoms in FP16x3 was 2e-5 off
+// without the shift.
+template <int NJ>
+__global__ void __launch_bounds__(kVecThreads) probe_expand_kernel(double scale, const __grid_constant__ JobList<ProbeJob, NJ> L) {
+  grid_wait();
+  const ProbeJob& J = L.job[blockIdx.x];
+  __shared__ double sh[16];
+  const double *pot = J.pot, *dmu = J.dmu;
+  double s0 = 0.0, s1 = 0.0;
+  for (int a = threadIdx.x; a < 4 * J.nat; a += kVecThreads) {
+    s0 += dmu[a];
+    s1 += dmu[a] * pot[a >> 2];
+  }
+  block_sum2(s0, s1, sh);
+  double pbar = s1 / s0;
+  if (!isfinite(pbar)) pbar = 0.0;
+  for (int a = threadIdx.x; a < J.np; a += kVecThreads) J.dvec[a] = (a < 4 * J.nat) ? scale * (pot[a >> 2] - pbar) : 0.0;
+}
+
+// mu1 = -sum d1 / sum dmu;  w_I = sum_{a in I} (d1_a + mu1 dmu_a)  (one block per job).  A unit probe's
+// w - e_u is column u of J - I (row-major nat x nat at Jm), next to a column of the identity at B.
+template <int NJ>
+__global__ void __launch_bounds__(kVecThreads) probe_finish_kernel(const __grid_constant__ JobList<ProbeJob, NJ> L) {
+  grid_wait();
+  const ProbeJob& J = L.job[blockIdx.x];
+  __shared__ double sh[16];
+  const double *d1 = J.d1, *dmu = J.dmu;
+  double s1 = 0.0, s2 = 0.0;
+  for (int a = threadIdx.x; a < J.N; a += kVecThreads) {
+    s1 += d1[a];
+    s2 += dmu[a];
+  }
+  block_sum2(s1, s2, sh);
+  const double mu1 = (s2 != 0.0) ? -s1 / s2 : 0.0;
+  if (threadIdx.x == 0) {
+    J.scal[0] = s1;
+    J.scal[1] = s2;
+    J.scal[2] = mu1;
+  }
+  for (int I = threadIdx.x; I < J.nat; I += kVecThreads) {
+    double t = 0.0;
+    for (int a = 4 * I; a < 4 * I + 4; ++a) t += d1[a] + mu1 * dmu[a];
+    if (J.w) J.w[I] = t;
+    if (J.unit >= 0) {
+      const size_t o = (size_t)I * J.nat + J.unit;
+      J.Jm[o] = t - (I == J.unit ? 1.0 : 0.0);
+      J.B[o] = (I == J.unit) ? 1.0 : 0.0;
+    }
+  }
+}
+
+// out[q] = sum_{I < n} f(q, I) for q < cnt, a warp or several per sum (part: the block's warps x 1
+// double, or cnt if that is more); valid in every thread after the call
+template <class F>
+__device__ __forceinline__ void block_dots(int cnt, int n, double* part, double* out, F f) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int split = cnt < nw ? nw / cnt : 1;
+  for (int u = wid; u < cnt * split; u += nw) {
+    const int q = u / split;
+    double acc = 0.0;
+    for (int I = (u % split) * 32 + lane; I < n; I += 32 * split) acc += f(q, I);
+    acc = warp_sum(acc);
+    if (lane == 0) part[u] = acc;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < cnt) {
+    double t = 0.0;
+    for (int p = 0; p < split; ++p) t += part[threadIdx.x * split + p];
+    out[threadIdx.x] = t;
+  }
+  __syncthreads();
+}
+
+// Rank-m kernel update, one block per system.
 //
 // With orthonormal probes V (rows), responses W, U = W - c V and
 // S = (c - 1) I_m + V U^T, the Sherman-Morrison sequence of Eq. K_up equals
@@ -114,166 +279,103 @@ __global__ void frob_partial_kernel(int n, int np, const double* __restrict__ A,
 //         first i probes; flag = 1 and V[i] = v_i, or flag = 0 when less than
 //         1e-12 of it is left (K_i r already in the span).
 // mode 1: out = K_m r.
-__device__ void kernel_apply(int nat, int m, double c, const double* r, const double* V, const double* W,
-                             double* x, double* sh, double* Smat, double* y) {
+// The m^2 + m sums of S and V r are taken side by side, as are the sums of a Gram-Schmidt pass (the
+// classical form, twice), so that the chain of reductions does not grow with m.  One sum after the
+// other by 1024 threads this took 17 us at m = 2 and 40 us at m = 4 for 512 atoms.
+template <int NJ>
+__global__ void __launch_bounds__(512) kernel_vec_kernel(const __grid_constant__ JobList<KernelVecJob, NJ> L) {
+  grid_wait();
+  const KernelVecJob& J = L.job[blockIdx.x];
+  __shared__ double part[kMaxRank * (kMaxRank + 1)];
+  __shared__ double dots[kMaxRank * (kMaxRank + 1)];
+  const int tid = threadIdx.x, nat = J.nat, m = J.m;
+  const double c = J.c;
+  const double *r = J.r, *V = J.V, *W = J.W;
+  double* x = (J.mode == 1) ? J.out : J.V + (size_t)m * nat;   // mode 0: the candidate goes to V[m]
   // x = K_m r
-  const int tid = threadIdx.x;
-  if (m == 0) {
-    for (int I = tid; I < nat; I += blockDim.x) x[I] = r[I] / (c - 1.0);
+  if (m > 0) {
+    const int ld = m + 1;
+    block_dots(m * ld, nat, part, dots, [&](int q, int I) {
+      const int a = q / ld, b = q % ld;
+      const double va = V[(size_t)a * nat + I];
+      return b == m ? va * r[I] : va * (W[(size_t)b * nat + I] - c * V[(size_t)b * nat + I]);
+    });
+    if (tid < m) dots[tid * ld + tid] += c - 1.0;
     __syncthreads();
-    return;
-  }
-  for (int a = 0; a < m; ++a) {
-    for (int b = 0; b < m; ++b) {
-      double acc = 0.0;
-      for (int I = tid; I < nat; I += blockDim.x)
-        acc += V[(size_t)a * nat + I] * (W[(size_t)b * nat + I] - c * V[(size_t)b * nat + I]);
-      acc = block_sum(acc, sh);
-      if (tid == 0) Smat[a * kMaxRank + b] = acc + (a == b ? c - 1.0 : 0.0);
-    }
-    double acc = 0.0;
-    for (int I = tid; I < nat; I += blockDim.x) acc += V[(size_t)a * nat + I] * r[I];
-    acc = block_sum(acc, sh);
-    if (tid == 0) y[a] = acc;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    // Gaussian elimination with partial pivoting on the m x m system S y = V r
-    double A[kMaxRank][kMaxRank + 1];
-    for (int a = 0; a < m; ++a) {
-      for (int b = 0; b < m; ++b) A[a][b] = Smat[a * kMaxRank + b];
-      A[a][m] = y[a];
-    }
-    for (int col = 0; col < m; ++col) {
-      int piv = col;
-      for (int a = col + 1; a < m; ++a)
-        if (fabs(A[a][col]) > fabs(A[piv][col])) piv = a;
-      if (piv != col)
-        for (int b = 0; b <= m; ++b) {
-          const double t = A[col][b];
-          A[col][b] = A[piv][b];
-          A[piv][b] = t;
+    if (tid < 32) {
+      // Gaussian elimination with partial pivoting on S y = V r, lane b at column b; y ends in column m
+      for (int col = 0; col < m; ++col) {
+        int piv = col;
+        for (int a = col + 1; a < m; ++a)
+          if (fabs(dots[a * ld + col]) > fabs(dots[piv * ld + col])) piv = a;
+        __syncwarp();
+        if (piv != col && tid <= m) {
+          const double t = dots[col * ld + tid];
+          dots[col * ld + tid] = dots[piv * ld + tid];
+          dots[piv * ld + tid] = t;
         }
-      for (int a = col + 1; a < m; ++a) {
-        const double f = A[a][col] / A[col][col];
-        for (int b = col; b <= m; ++b) A[a][b] -= f * A[col][b];
+        __syncwarp();
+        if (tid > col && tid <= m)
+          for (int a = col + 1; a < m; ++a)
+            dots[a * ld + tid] -= dots[a * ld + col] / dots[col * ld + col] * dots[col * ld + tid];
+        __syncwarp();
+      }
+      for (int a = m - 1; a >= 0; --a) {
+        const double y = dots[a * ld + m] / dots[a * ld + a];
+        __syncwarp();
+        if (tid < a) dots[tid * ld + m] -= dots[tid * ld + a] * y;
+        if (tid == a) dots[a * ld + m] = y;
+        __syncwarp();
       }
     }
-    for (int a = m - 1; a >= 0; --a) {
-      double t = A[a][m];
-      for (int b = a + 1; b < m; ++b) t -= A[a][b] * y[b];
-      y[a] = t / A[a][a];
-    }
+    __syncthreads();
   }
-  __syncthreads();
   for (int I = tid; I < nat; I += blockDim.x) {
     double t = r[I];
-    for (int a = 0; a < m; ++a) t -= (W[(size_t)a * nat + I] - c * V[(size_t)a * nat + I]) * y[a];
+    for (int a = 0; a < m; ++a) t -= (W[(size_t)a * nat + I] - c * V[(size_t)a * nat + I]) * dots[a * (m + 1) + m];
     x[I] = t / (c - 1.0);
   }
+  if (J.mode == 1) return;
   __syncthreads();
-}
-
-__global__ void kernel_vec_kernel(int mode, int nat, int m, double c, const double* __restrict__ r,
-                                  double* __restrict__ V, const double* __restrict__ W, double* __restrict__ out,
-                                  double* __restrict__ flag) {
-  __shared__ double sh[32];
-  __shared__ double Smat[kMaxRank * kMaxRank];
-  __shared__ double y[kMaxRank];
-  const int tid = threadIdx.x;
-  if (mode == 1) {
-    kernel_apply(nat, m, c, r, V, W, out, sh, Smat, y);
-    return;
-  }
-  // mode 0: candidate into V[m]
-  double* v = V + (size_t)m * nat;
-  kernel_apply(nat, m, c, r, V, W, v, sh, Smat, y);
   double n0 = 0.0;
-  for (int I = tid; I < nat; I += blockDim.x) n0 += v[I] * v[I];
-  n0 = sqrt(block_sum(n0, sh));
-  for (int pass = 0; pass < 2; ++pass)
-    for (int a = 0; a < m; ++a) {
-      double d = 0.0;
-      for (int I = tid; I < nat; I += blockDim.x) d += V[(size_t)a * nat + I] * v[I];
-      d = block_sum(d, sh);
-      for (int I = tid; I < nat; I += blockDim.x) v[I] -= d * V[(size_t)a * nat + I];
-      __syncthreads();
+  for (int pass = 0; pass < 2 && m > 0; ++pass) {
+    // the first pass also takes |x|^2
+    const int cnt = m + (pass == 0 ? 1 : 0);
+    block_dots(cnt, nat, part, dots, [&](int q, int I) { return (q == m ? x[I] : V[(size_t)q * nat + I]) * x[I]; });
+    if (pass == 0) n0 = sqrt(dots[m]);
+    for (int I = tid; I < nat; I += blockDim.x) {
+      double t = x[I];
+      for (int a = 0; a < m; ++a) t -= dots[a] * V[(size_t)a * nat + I];
+      x[I] = t;
     }
-  double nv = 0.0;
-  for (int I = tid; I < nat; I += blockDim.x) nv += v[I] * v[I];
-  nv = sqrt(block_sum(nv, sh));
+    __syncthreads();
+  }
+  block_dots(1, nat, part, dots, [&](int, int I) { return x[I] * x[I]; });
+  const double nv = sqrt(dots[0]);
+  if (m == 0) n0 = nv;
   const bool ok = (n0 > 0.0) && isfinite(nv) && (nv > 1e-12 * n0);
   if (ok)
-    for (int I = tid; I < nat; I += blockDim.x) v[I] /= nv;
-  if (tid == 0) *flag = ok ? 1.0 : 0.0;
+    for (int I = tid; I < nat; I += blockDim.x) x[I] /= nv;
+  if (tid == 0) *J.flag = ok ? 1.0 : 0.0;
 }
 
-// dvec_a = scale (pot_I - pbar) on the orbitals of atom I, 0 on the padding (one block).  A uniform
-// potential has no canonical response (mu follows it); taking the average pbar = sum_a dmu_a pot_a /
-// sum_a dmu_a out beforehand leaves sum_a d1_a = -sum_a pot_a dmu_a at rounding level, so that the
-// chain does not carry a large part that mu_1 dT_n/dmu then has to cancel (the errors of the two are
-// independent).  A unit probe's potential is mostly uniform: K of 48 atoms in FP16x3 was 2e-5 off
-// without the shift.
-__global__ void expand_potential_kernel(int nat, int np, double scale, const double* __restrict__ pot,
-                                        const double* __restrict__ dmu, double* __restrict__ dvec) {
-  __shared__ double sh[32];
-  double s0 = 0.0, s1 = 0.0;
-  for (int a = threadIdx.x; a < 4 * nat; a += blockDim.x) {
-    s0 += dmu[a];
-    s1 += dmu[a] * pot[a >> 2];
-  }
-  s0 = block_sum(s0, sh);
-  s1 = block_sum(s1, sh);
-  double pbar = s1 / s0;
-  if (!isfinite(pbar)) pbar = 0.0;
-  for (int a = threadIdx.x; a < np; a += blockDim.x) dvec[a] = (a < 4 * nat) ? scale * (pot[a >> 2] - pbar) : 0.0;
-}
-
-// mu1 = -sum d1 / sum dmu;  w_I = sum_{a in I} (d1_a + mu1 dmu_a)  (one block)
-__global__ void response_finish_kernel(int nat, int N, const double* __restrict__ d1,
-                                       const double* __restrict__ dmu, double* __restrict__ scal,
-                                       double* __restrict__ w) {
-  __shared__ double sh[32];
-  double s1 = 0.0, s2 = 0.0;
-  for (int a = threadIdx.x; a < N; a += blockDim.x) {
-    s1 += d1[a];
-    s2 += dmu[a];
-  }
-  s1 = block_sum(s1, sh);
-  s2 = block_sum(s2, sh);
-  const double mu1 = (s2 != 0.0) ? -s1 / s2 : 0.0;
-  if (threadIdx.x == 0) {
-    scal[0] = s1;
-    scal[1] = s2;
-    scal[2] = mu1;
-  }
-  for (int I = threadIdx.x; I < nat; I += blockDim.x) {
-    double t = 0.0;
-    for (int a = 4 * I; a < 4 * I + 4; ++a) t += d1[a] + mu1 * dmu[a];
-    w[I] = t;
-  }
-}
-
-__global__ void absmax_kernel(int n, const double* __restrict__ x, double* __restrict__ out) {
+// max |x_i|; any value that is not finite makes it NaN, so that the host sees it
+__global__ void absmax_kernel(int n, const double* x, double* out) {
+  grid_wait();
   __shared__ double sh[32];
   double m = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, fabs(x[i]));
+  bool bad = false;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    bad |= !isfinite(x[i]);
+    m = fmax(m, fabs(x[i]));
+  }
   m = warp_max(m);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
+  bad = __syncthreads_or(bad);
   if (threadIdx.x < 32) {
     m = (threadIdx.x < (blockDim.x >> 5)) ? sh[threadIdx.x] : 0.0;
     m = warp_max(m);
-    if (threadIdx.x == 0) {
-      // NaN anywhere poisons the result so that the host sees it
-      bool bad = false;
-      for (int i = 0; i < n; ++i)
-        if (!isfinite(x[i])) {
-          bad = true;
-          break;
-        }
-      *out = bad ? nan("") : m;
-    }
+    if (threadIdx.x == 0) *out = bad ? nan("") : m;
   }
 }
 
@@ -314,24 +416,76 @@ inline unsigned blocks_for(size_t count, int tpb) { return (unsigned)((count + t
 
 }  // namespace
 
-cudaError_t launch_expand_potential(cudaStream_t s, int nat, int np, double scale, const double* pot,
-                                    const double* dmu, double* dvec) {
-  expand_potential_kernel<<<1, 1024, 0, s>>>(nat, np, scale, pot, dmu, dvec);
-  note_launch();
-  return cudaGetLastError();
+namespace {
+
+// f(list) with the jobs in lists of one, or of at most 16 (1.9 KB of parameters)
+template <class Job, class F>
+cudaError_t in_lists(const std::vector<Job>& jobs, F f) {
+  if (jobs.size() == 1) {
+    JobList<Job, 1> L;
+    L.n = 1;
+    L.job[0] = jobs[0];
+    return f(L);
+  }
+  for (size_t i = 0; i < jobs.size(); i += kMaxJobs) {
+    JobList<Job, kMaxJobs> L;
+    L.n = (int)std::min<size_t>(kMaxJobs, jobs.size() - i);
+    std::copy_n(jobs.begin() + i, L.n, L.job);
+    RET(f(L));
+  }
+  return cudaSuccess;
 }
 
-cudaError_t launch_response_finish(cudaStream_t s, int nat, int N, const double* d1, const double* dmu,
-                                   double* scal, double* w) {
-  response_finish_kernel<<<1, 1024, 0, s>>>(nat, N, d1, dmu, scal, w);
-  note_launch();
-  return cudaGetLastError();
+template <int NJ>
+cudaError_t probe_potential(cudaStream_t s, double k, JobList<ProbeJob, NJ>& L) {
+  int nat = 0, dots = 0;
+  for (int j = 0; j < L.n; ++j) {
+    if (k == 0.0) L.job[j].SF = nullptr;
+    nat = std::max(nat, L.job[j].nat);
+    if (L.job[j].SF && L.job[j].unit < 0) dots = std::max(dots, L.job[j].kp);
+  }
+  if (dots) RET(launch_chained(s, dim3((dots + 31) / 32, L.n), 1024, 0, probe_dot_kernel<NJ>, L));
+  // a row has nat + kp products
+  return launch_chained(s, dim3(nat, L.n), nat <= 2048 ? 256 : 512, 0, probe_apply_kernel<NJ>, k, L);
+}
+
+template <int NJ>
+cudaError_t kernel_vec(cudaStream_t s, const JobList<KernelVecJob, NJ>& L) {
+  int nat = 0;
+  for (int j = 0; j < L.n; ++j) nat = std::max(nat, L.job[j].nat);
+  return launch_chained(s, L.n, nat <= 256 ? 256 : 512, 0, kernel_vec_kernel<NJ>, L);
+}
+
+template <int NJ>
+cudaError_t probe_expand(cudaStream_t s, double scale, const JobList<ProbeJob, NJ>& L) {
+  return launch_chained(s, L.n, kVecThreads, 0, probe_expand_kernel<NJ>, scale, L);
+}
+
+template <int NJ>
+cudaError_t probe_finish(cudaStream_t s, const JobList<ProbeJob, NJ>& L) {
+  return launch_chained(s, L.n, kVecThreads, 0, probe_finish_kernel<NJ>, L);
+}
+
+}  // namespace
+
+cudaError_t launch_probe_potential(cudaStream_t s, double k, const std::vector<ProbeJob>& jobs) {
+  return in_lists(jobs, [&](auto& L) { return probe_potential(s, k, L); });
+}
+
+cudaError_t launch_probe_expand(cudaStream_t s, double scale, const std::vector<ProbeJob>& jobs) {
+  return in_lists(jobs, [&](auto& L) { return probe_expand(s, scale, L); });
+}
+
+cudaError_t launch_probe_finish(cudaStream_t s, const std::vector<ProbeJob>& jobs) {
+  return in_lists(jobs, [&](auto& L) { return probe_finish(s, L); });
+}
+
+cudaError_t launch_kernel_vec(cudaStream_t s, const std::vector<KernelVecJob>& jobs) {
+  return in_lists(jobs, [&](auto& L) { return kernel_vec(s, L); });
 }
 
 cudaError_t launch_absmax(cudaStream_t s, int n, const double* x, double* out) {
-  absmax_kernel<<<1, 1024, 0, s>>>(n, x, out);
-  note_launch();
-  return cudaGetLastError();
+  return launch_chained(s, 1, 256, 0, absmax_kernel, n, x, out);
 }
 
 cudaError_t launch_fill_history(cudaStream_t s, int nat, int kmax, double* nh) {
@@ -408,31 +562,9 @@ cudaError_t launch_frob_dot(cudaStream_t s, int n, int np, const double* A, cons
   return cudaGetLastError();
 }
 
-cudaError_t launch_kernel_vec(cudaStream_t s, int mode, int nat, int m, double c, const double* r, double* V,
-                              const double* W, double* out, double* flag) {
-  kernel_vec_kernel<<<1, 1024, 0, s>>>(mode, nat, m, c, r, V, W, out, flag);
-  note_launch();
-  return cudaGetLastError();
-}
-
-
 // ---- exact kernel K = (J - I)^-1 (Eq. KK) ----
 
 namespace {
-
-__global__ void unit_vector_kernel(int n, int i, double* __restrict__ v) {
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a < n) v[a] = (a == i) ? 1.0 : 0.0;
-}
-
-// A[a][col] = w[a] - delta(a, col): column col of J - I (row-major n x n); B = I alongside
-__global__ void jacobian_column_kernel(int n, int col, const double* __restrict__ w, double* __restrict__ A,
-                                       double* __restrict__ B) {
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= n) return;
-  A[(size_t)a * n + col] = w[a] - (a == col ? 1.0 : 0.0);
-  B[(size_t)a * n + col] = (a == col) ? 1.0 : 0.0;
-}
 
 // Gauss-Jordan step k, part 1 (one CTA): partial pivot of column k over rows k..n-1,
 // swap of rows k and p in A and B, scaling of row k by 1 / A_kk, and the elimination
@@ -520,18 +652,6 @@ __global__ void gj_eliminate_kernel(int n, int k, double* __restrict__ A, double
 }
 
 }  // namespace
-
-cudaError_t launch_unit_vector(cudaStream_t s, int n, int i, double* v) {
-  unit_vector_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, i, v);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_jacobian_column(cudaStream_t s, int n, int col, const double* w, double* A, double* B) {
-  jacobian_column_kernel<<<(n + 255) / 256, 256, 0, s>>>(n, col, w, A, B);
-  note_launch();
-  return cudaGetLastError();
-}
 
 cudaError_t launch_gauss_jordan(cudaStream_t s, int n, double* A, double* B, double* f, double* flag) {
   if (n < 1 || n > 65535) return cudaErrorInvalidValue;

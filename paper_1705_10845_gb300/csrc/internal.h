@@ -1,5 +1,7 @@
 // Internal declarations of the XL-BOMD library (not part of the C ABI).
 #pragma once
+#include <vector>
+
 #include "common.cuh"
 
 namespace xl {
@@ -42,10 +44,32 @@ cudaError_t launch_build_H0(cudaStream_t s, const ModelConst& m, int nat, double
 // Rs not null: pair functions in FP32 of 48-bit distances, for the split-precision path.
 cudaError_t launch_gamma_real(cudaStream_t s, const ModelConst& m, int nat, double L, double eta,
                               const double* R, const float2* Rs, double* gam, int natp);
-// y = gamma x with gamma = gamma_real + k SF SF^T applied through the structure
-// factors (tmp: kp doubles; SF may be null when k = 0).
-cudaError_t launch_gamma_apply(cudaStream_t s, int nat, const double* gam, int natp, const double* SF, int kp,
-                               double k, const double* x, double* y, double* tmp);
+// One probe of a response (or one product with gamma): all vectors are of one system.
+struct ProbeJob {
+  int nat = 0, N = 0, np = 0, natp = 0, kp = 0;
+  int unit = -1;                                 // x = e_unit when >= 0 (x and tmp not read)
+  const double *gam = nullptr, *SF = nullptr;    // gamma_real and the structure factors (null: no reciprocal part)
+  const double* x = nullptr;
+  double *tmp = nullptr, *pot = nullptr;         // kp doubles; pot = gamma x
+  const double* dmu = nullptr;                   // diagonal of dT_n/dmu
+  double *dvec = nullptr, *d1 = nullptr, *scal = nullptr, *w = nullptr;
+  double *Jm = nullptr, *B = nullptr;            // a unit probe's column of J - I and of the identity
+};
+// Rank-m kernel update (kernel_vec_kernel).  flag may be pinned host memory.
+struct KernelVecJob {
+  int mode = 0, nat = 0, m = 0;
+  double c = 0.0;
+  const double* r = nullptr;
+  double* V = nullptr;
+  const double* W = nullptr;
+  double *out = nullptr, *flag = nullptr;
+};
+// pot = gamma x with gamma = gamma_real + k SF SF^T applied through the structure factors
+cudaError_t launch_probe_potential(cudaStream_t s, double k, const std::vector<ProbeJob>& jobs);
+// dvec = scale (pot less its average) on orbitals; w (and the column of J - I) from d1
+cudaError_t launch_probe_expand(cudaStream_t s, double scale, const std::vector<ProbeJob>& jobs);
+cudaError_t launch_probe_finish(cudaStream_t s, const std::vector<ProbeJob>& jobs);
+cudaError_t launch_kernel_vec(cudaStream_t s, const std::vector<KernelVecJob>& jobs);
 // Structure-factor matrix SF (natp x kp): row I = sqrt(w_g) [cos(G_g.R_I), sin(G_g.R_I)].  Gh: the integer
 // vectors h + 8, a byte per component; Gs = sqrt(w_g).
 cudaError_t launch_structure_factors(cudaStream_t s, int nat, int ng, double L, const int* Gh, const double* Gs,
@@ -88,9 +112,6 @@ cudaError_t launch_sum(cudaStream_t s, int n, const double* x, double* out);
 // out = sum_{i,j<n} A_ij B_ij (deterministic two-level reduction; work >= 1024 doubles)
 cudaError_t launch_frob_dot(cudaStream_t s, int n, int np, const double* A, const double* B, double* work,
                             double* out);
-// Small vector algebra of the kernel update (one CTA, FP64).
-cudaError_t launch_kernel_vec(cudaStream_t s, int mode, int nat, int m, double c, const double* r,
-                              double* V, const double* W, double* out, double* flag);
 // Energy parts: out[0..] from vectors (Coulomb, kinetic).
 cudaError_t launch_energy_vec(cudaStream_t s, int nat, const double* q, const double* n,
                               const double* pot, const double* V, double mass, double* out);

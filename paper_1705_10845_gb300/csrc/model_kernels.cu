@@ -444,56 +444,32 @@ __global__ void gemv_kernel(int nat, const double* __restrict__ gam, int natp, c
   if (lane == 0) y[I] = acc;
 }
 
-// t[v][g] = sum_I SF[I][g] x_v[I]: 32 columns a block, 32 row groups.  NV = 1: x_0 = x; NV = 2: x_0 = 2 x - y
-// and x_1 = y (x = q, y = n).  The rows used to run one after another in one thread per column: 125 us at
-// 512 atoms.
-template <int NV>
+// t[v][g] = sum_I SF[I][g] x_v[I] with x_0 = 2 x - y and x_1 = y (x = q, y = n): 32 columns a block, 32 row
+// groups.  The rows used to run one after another in one thread per column: 125 us at 512 atoms.
 __global__ void __launch_bounds__(1024) sf_dot_kernel(int nat, int kp, const double* __restrict__ SF,
                                                       const double* __restrict__ x, const double* __restrict__ y,
                                                       double* __restrict__ t) {
-  __shared__ double sh[NV][32][33];
+  __shared__ double sh[2][32][33];
   const int c = threadIdx.x & 31, w = threadIdx.x >> 5, g = blockIdx.x * 32 + c;
   double a0 = 0.0, a1 = 0.0;
   if (g < kp) {
 #pragma unroll 4
     for (int I = w; I < nat; I += 32) {
       const double s = SF[(size_t)I * kp + g];
-      if (NV == 1) {
-        a0 += s * x[I];
-      } else {
-        a0 += s * (2.0 * x[I] - y[I]);
-        a1 += s * y[I];
-      }
+      a0 += s * (2.0 * x[I] - y[I]);
+      a1 += s * y[I];
     }
   }
   sh[0][w][c] = a0;
-  if (NV == 2) sh[NV - 1][w][c] = a1;
+  sh[1][w][c] = a1;
   __syncthreads();
   // warp w sums column w
   const int gw = blockIdx.x * 32 + w;
-  const double s0 = warp_sum(sh[0][c][w]);
-  if (c == 0 && gw < kp) t[gw] = s0;
-  if (NV == 2) {
-    const double s1 = warp_sum(sh[NV - 1][c][w]);
-    if (c == 0 && gw < kp) t[kp + gw] = s1;
+  const double s0 = warp_sum(sh[0][c][w]), s1 = warp_sum(sh[1][c][w]);
+  if (c == 0 && gw < kp) {
+    t[gw] = s0;
+    t[kp + gw] = s1;
   }
-}
-
-// y_I = sum_J gamma_real_IJ x_J + k sum_g SF[I][g] t[g], one block per row
-__global__ void gamma_apply_kernel(int nat, const double* __restrict__ gam, int natp, const double* __restrict__ SF,
-                                   int kp, double k, const double* __restrict__ t, const double* __restrict__ x,
-                                   double* __restrict__ y) {
-  __shared__ double sh[32];
-  const int I = blockIdx.x;
-  double acc = 0.0, rec = 0.0;
-#pragma unroll 4
-  for (int J = threadIdx.x; J < nat; J += blockDim.x) acc += gam[(size_t)I * natp + J] * x[J];
-  if (SF) {
-#pragma unroll 4
-    for (int g = threadIdx.x; g < kp; g += blockDim.x) rec += SF[(size_t)I * kp + g] * t[g];
-  }
-  acc = block_sum(acc + k * rec, sh);
-  if (threadIdx.x == 0) y[I] = acc;
 }
 
 __global__ void add_potential_kernel(int nat, int np, const double* __restrict__ pot, double* __restrict__ H) {
@@ -819,26 +795,6 @@ cudaError_t launch_gamma_real(cudaStream_t s, const ModelConst& m, int nat, doub
   return cudaGetLastError();
 }
 
-namespace {
-
-// Threads per row of gamma_apply: a row has nat + kp products.
-int apply_threads(int nat) { return nat <= 2048 ? 256 : 512; }
-
-}  // namespace
-
-cudaError_t launch_gamma_apply(cudaStream_t s, int nat, const double* gam, int natp, const double* SF, int kp,
-                               double k, const double* x, double* y, double* tmp) {
-  if (SF && k != 0.0) {
-    sf_dot_kernel<1><<<(kp + 31) / 32, 1024, 0, s>>>(nat, kp, SF, x, nullptr, tmp);
-    note_launch();
-  } else {
-    SF = nullptr;
-  }
-  gamma_apply_kernel<<<nat, apply_threads(nat), 0, s>>>(nat, gam, natp, SF, kp, k, tmp, x, y);
-  note_launch();
-  return cudaGetLastError();
-}
-
 cudaError_t launch_structure_factors(cudaStream_t s, int nat, int ng, double L, const int* Gh, const double* Gs,
                                      const double* R, double* SF, int kp) {
   const int natp = (nat + 63) / 64 * 64;
@@ -902,7 +858,7 @@ cudaError_t launch_forces(cudaStream_t s, const ModelConst& m, int nat, double L
     else
       forces_coul_split_kernel<false><<<grid, 128, 0, s>>>(m, nat, L, eta, Rs, q, n, part);
     note_launch();
-    sf_dot_kernel<2><<<(kp + 31) / 32, 1024, 0, s>>>(nat, kp, SF, q, n, work);
+    sf_dot_kernel<<<(kp + 31) / 32, 1024, 0, s>>>(nat, kp, SF, q, n, work);
     note_launch();
     forces_coul_recip_kernel<<<nat, 128, 0, s>>>(m.k, nat, ng, kp, parts, G4, SF, q, n, work, part, F);
     note_launch();

@@ -13,12 +13,16 @@
 namespace xl {
 
 // 2^(14 - ceil(log2 bound)); 1 for a bound that is zero or not finite
-__host__ __device__ inline float operand_scale(double bound) {
-  if (!(bound > 0.0) || !(bound < 1e300)) return 1.0f;
+__host__ __device__ inline float operand_scale(float bound) {
+  if (!(bound > 0.0f) || !(bound < 1e37f)) return 1.0f;
   int e;
-  frexp(bound, &e);   // bound <= 2^e
+  frexpf(bound, &e);   // bound <= 2^e
   e = e < -40 ? -40 : e > 70 ? 70 : e;
-  return (float)ldexp(1.0, 14 - e);
+  return ldexpf(1.0f, 14 - e);
+}
+__host__ __device__ inline float operand_scale(double bound) {
+  // rounded up, so that it stays a bound; what FP32 cannot hold has the scale of the range's end
+  return operand_scale(bound > 1e36 && bound < 1e300 ? 1e36f : (float)bound * 1.000001f);
 }
 
 // matrices that only matter against the identity (S, W, the residuals and their polynomials; all below 4)

@@ -231,19 +231,12 @@ cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, int N, double beta, in
                                const double* D, const double* H, double* work, double* out);
 
 // misc FP64 launchers (foe_kernels.cu)
-cudaError_t launch_expand_potential(cudaStream_t s, int nat, int np, double scale, const double* pot,
-                                    const double* dmu_diag, double* dvec);
-cudaError_t launch_response_finish(cudaStream_t s, int nat, int N, const double* d1, const double* dmu_diag,
-                                   double* scal, double* w);
 cudaError_t launch_absmax(cudaStream_t s, int n, const double* x, double* out);
 cudaError_t launch_fill_history(cudaStream_t s, int nat, int kmax, double* nh);
 cudaError_t launch_axpy(cudaStream_t s, int n, double a, const double* x, double* y);
 cudaError_t launch_diag_sum(cudaStream_t s, int n, int np, const double* X, double* out);
-// exact kernel (foe_kernels.cu): v = e_i; column col of J - I from w (and of B = I);
-// B <- (A)^-1 B by Gauss-Jordan with partial pivoting (A row-major n x n, destroyed;
+// exact kernel (foe_kernels.cu): B <- (A)^-1 B by Gauss-Jordan with partial pivoting (A row-major n x n, destroyed;
 // f: n doubles of work; *flag set to 1 on a zero or non-finite pivot)
-cudaError_t launch_unit_vector(cudaStream_t s, int n, int i, double* v);
-cudaError_t launch_jacobian_column(cudaStream_t s, int n, int col, const double* w, double* A, double* B);
 cudaError_t launch_gauss_jordan(cudaStream_t s, int n, double* A, double* B, double* f, double* flag);
 // accumulated rank-1 kernel (foe_kernels.cu), row-major n x n FP64 matrices:
 // M = a I; y = M^T x; v <- v/|v| (flag 1 if |v| > 0); u = w - t; out = 1 + a.b;

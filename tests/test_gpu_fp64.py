@@ -356,3 +356,31 @@ def test_density_and_entropy_at_tile_edges(X, nat):
     assert np.max(np.abs(Kr - ref.Kr)) < 1e-8
     assert abs(E[0] - ref.Omega) < 1e-8 * abs(ref.Omega)
     assert abs(E[3] - ref.parts["entropy"]) < 1e-7
+
+
+@pytest.mark.parametrize("nat,rank,prec", [(5, 1, "fp64"), (9, 8, "fp64"), (33, 3, "fp64"), (65, 7, "fp64"),
+                                           (257, 5, "fp16x3")])
+def test_rank_m_update_algebra(X, nat, rank, prec):
+    # the FP64 vector algebra of the update from the probes V and responses W it reports itself: one or
+    # several warps per sum, one and several rounds of sums, 256 and 512 threads.  Orthonormality to a few
+    # hundred roundings; K r through S of condition below 1e3; a candidate loses what the projection cancels
+    s = synth.make_system(nat, 31, **({} if nat > 24 else {"L": 7.0}))
+    p = model_params(X, rank_m=rank, prec=prec)
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, random_n(nat, 7))
+        ctx.build_H(0)
+        ctx.density(0)
+        ctx.kernel_update(0)
+        r, Kr, (V, W) = ctx.get(0, X.RES), ctx.get(0, X.KR), ctx.get(0, X.PROBES)
+        used = int(ctx.get(0, X.STATS)[2])
+    assert 1 <= used <= rank
+    V, W = V[:used], W[:used]
+    assert np.max(np.abs(V @ V.T - np.eye(used))) < 1e-13
+    ref = O.apply_kernel(r, V, W, p.kernel_c)
+    assert np.max(np.abs(Kr - ref)) < 1e-11 * np.max(np.abs(ref))
+    for i in range(used):
+        x = O.apply_kernel(r, V[:i], W[:i], p.kernel_c)
+        left = x - V[:i].T @ (V[:i] @ x)
+        left -= V[:i].T @ (V[:i] @ left)
+        ratio = np.linalg.norm(left) / np.linalg.norm(x)
+        assert np.max(np.abs(V[i] - left / np.linalg.norm(left))) < 1e-12 / ratio

@@ -566,6 +566,138 @@ cudaError_t launch_frob_dot(cudaStream_t s, int n, int np, const double* A, cons
 
 namespace {
 
+// In-place Gauss-Jordan inverse with partial pivoting of a matrix that fits the shared memory of one
+// cluster: column j lives in CTA j mod 8, one warp per column.  Per step the warp that holds the pivot
+// column searches it and sends the row exchange, 1/pivot and the factors to all CTAs; every warp then
+// updates its own columns, and the next pivot column goes first, so that its search and the cluster
+// barrier run beside the rest of the update (a CTA has 2 FP64 FMAs a clock: 0.3 us a step at n = 96).  The
+// factors are held three deep: a CTA arrives for step k + 1 when it enters step k, done with k - 1.
+// n = 96 as a search and an elimination launch per step: 1010 us.
+constexpr int kGjCtas = 8, kGjThreads = 512, kGjMaxSmem = 227 * 1024;
+
+__host__ __device__ inline size_t gj_smem(int n) {
+  const size_t cols = (n + kGjCtas - 1) / kGjCtas;
+  return sizeof(double) * (cols * (n | 1) + 3 * (size_t)(n + 2)) + 3 * sizeof(int) * (size_t)n;
+}
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t cta, double v) {
+  uint32_t remote;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(cta));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
+}
+
+__global__ void __cluster_dims__(kGjCtas, 1, 1) __launch_bounds__(kGjThreads)
+    gj_cluster_kernel(int n, const double* __restrict__ A, double* __restrict__ B, double* __restrict__ flag) {
+  extern __shared__ double sm[];
+  const int cta = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kGjThreads / 32;
+  const int cols = (n - cta + kGjCtas - 1) / kGjCtas, ld = n | 1;
+  double* fs = sm + (size_t)((n + kGjCtas - 1) / kGjCtas) * ld;   // 3 x [n factors, 1/pivot, pivot row]
+  int* piv = reinterpret_cast<int*>(fs + 3 * (n + 2));
+  int *src = piv + n, *dst = src + n;
+  for (int e = threadIdx.x; e < n * cols; e += kGjThreads) {
+    const int i = e / cols, c = e % cols;
+    sm[(size_t)c * ld + i] = A[(size_t)i * n + cta + kGjCtas * c];
+  }
+  __syncthreads();
+  cluster_arrive();   // every CTA has started before the first remote store
+  cluster_wait();
+
+  // one warp: pivot search of column k in rows k .. n - 1, its exchange, factors and inverse column
+  auto publish = [&](int k) {
+    double* col = sm + (size_t)(k / kGjCtas) * ld;
+    double best = -1.0;
+    int p = k;
+    for (int i = k + lane; i < n; i += 32) {
+      const double v = fabs(col[i]);
+      if (v > best) {
+        best = v;
+        p = i;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int op = __shfl_xor_sync(0xffffffffu, p, o);
+      if (ov > best || (ov == best && op < p)) {
+        best = ov;
+        p = op;
+      }
+    }
+    const double pv = col[p], top = col[k];
+    const bool bad = !(fabs(pv) > 0.0) || !isfinite(pv);
+    const double inv = bad ? 0.0 : 1.0 / pv;
+    __syncwarp();
+    const uint32_t f = (uint32_t)__cvta_generic_to_shared(fs + (size_t)(k % 3) * (n + 2));
+    for (int i = lane; i < n; i += 32) {
+      const double v = (i == k) ? 0.0 : (i == p) ? top : col[i];
+      for (int c = 0; c < kGjCtas; ++c) st_cluster(f + 8 * i, c, v);
+      col[i] = (i == k) ? inv : -v * inv;
+    }
+    if (lane < kGjCtas) {
+      st_cluster(f + 8 * n, lane, inv);
+      st_cluster(f + 8 * (n + 1), lane, (double)p);
+    }
+    __syncwarp();
+  };
+
+  if (cta == 0 && wid == 0) publish(0);
+  cluster_arrive();
+  bool bad = false;
+  for (int k = 0; k < n; ++k) {
+    cluster_wait();
+    const double* f = fs + (size_t)(k % 3) * (n + 2);
+    const double inv = f[n];
+    const int p = (int)f[n + 1];
+    if (inv == 0.0) {   // the same in every thread of the cluster
+      bad = true;
+      break;
+    }
+    if (threadIdx.x == 0) piv[k] = p;
+    auto update = [&](int c) {
+      double* col = sm + (size_t)c * ld;
+      const double top = col[k], ck = col[p] * inv;
+      __syncwarp();
+      for (int i = lane; i < n; i += 32) {
+        const double v = (i == p) ? top : col[i];
+        col[i] = (i == k) ? ck : v - f[i] * ck;
+      }
+      __syncwarp();
+    };
+    const int next = (k + 1 < n && (k + 1) % kGjCtas == cta) ? (k + 1) / kGjCtas : -1;
+    if (next >= 0 && next % nw == wid) {
+      update(next);
+      publish(k + 1);
+    }
+    if (k + 1 < n) cluster_arrive();
+    for (int c = wid; c < cols; c += nw)
+      if (c != next && cta + kGjCtas * c != k) update(c);
+  }
+  __syncthreads();
+  if (!bad) {
+    // the result is the inverse of the row-permuted matrix: undo the exchanges on its columns
+    for (int j = threadIdx.x; j < n; j += kGjThreads) src[j] = j;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int k = n - 1; k >= 0; --k) {
+        const int p = piv[k], t = src[k];
+        src[k] = src[p];
+        src[p] = t;
+      }
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += kGjThreads) dst[src[j]] = j;
+    __syncthreads();
+    for (int e = threadIdx.x; e < n * cols; e += kGjThreads) {
+      const int i = e / cols, c = e % cols;
+      B[(size_t)i * n + dst[cta + kGjCtas * c]] = sm[(size_t)c * ld + i];
+    }
+  } else if (cta == 0 && threadIdx.x == 0) {
+    *flag = 1.0;
+  }
+  cluster_arrive();   // no CTA leaves while another may still store into it
+  cluster_wait();
+}
+
 // Gauss-Jordan step k, part 1 (one CTA): partial pivot of column k over rows k..n-1,
 // swap of rows k and p in A and B, scaling of row k by 1 / A_kk, and the elimination
 // factors f_i = A_ik (f_k = 0) copied out so that part 2 reads no column it writes.
@@ -655,6 +787,12 @@ __global__ void gj_eliminate_kernel(int n, int k, double* __restrict__ A, double
 
 cudaError_t launch_gauss_jordan(cudaStream_t s, int n, double* A, double* B, double* f, double* flag) {
   if (n < 1 || n > 65535) return cudaErrorInvalidValue;
+  if (gj_smem(n) <= kGjMaxSmem) {   // n <= 456
+    RET(cudaFuncSetAttribute(gj_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGjMaxSmem));
+    gj_cluster_kernel<<<kGjCtas, kGjThreads, gj_smem(n), s>>>(n, A, B, flag);
+    note_launch();
+    return cudaGetLastError();
+  }
   const dim3 grid((2 * n + 255) / 256, n);
   for (int k = 0; k < n; ++k) {
     gj_pivot_kernel<<<1, 1024, 0, s>>>(n, k, A, B, f, flag);

@@ -384,3 +384,43 @@ def test_rank_m_update_algebra(X, nat, rank, prec):
         left -= V[:i].T @ (V[:i] @ left)
         ratio = np.linalg.norm(left) / np.linalg.norm(x)
         assert np.max(np.abs(V[i] - left / np.linalg.norm(left))) < 1e-12 / ratio
+
+
+@pytest.mark.parametrize("nat", [2, 5, 9, 64, 65])
+def test_exact_kernel_inverse_at_cluster_edges(X, nat):
+    # columns dealt to the 8 CTAs of the inverting cluster: fewer than CTAs, one more than a multiple, more
+    # than one column per CTA
+    s = synth.make_system(nat, 12, **({} if nat > 24 else {"L": 7.0}))
+    p = model_params(X, kernel_mode=1)
+    n = random_n(nat, 16)
+    ev = O.evaluate(s.R, s.L, s.Z, n, oracle_model(p), None, with_kernel=False, with_forces=False)
+    Kref = O.kernel_exact(ev.dens, ev.gamma)
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, n)
+        ctx.set(0, X.MU, [ev.dens.mu])
+        ctx.build_H(0)
+        ctx.density(0)
+        ctx.kernel_exact(0)
+        K = ctx.get(0, X.KMAT)
+    assert np.max(np.abs(K - Kref)) < 1e-9 * max(1.0, np.abs(Kref).max())
+
+
+@pytest.mark.parametrize("nat", [200, 460])
+def test_exact_kernel_inverts_the_response(X, nat):
+    # K (w - v) = v with w the response along v; 460 atoms are beyond the shared memory of a cluster.  The
+    # FP16x3 responses are good to 1e-5 (w and the columns of J alike), K here has a condition below 100
+    import torch
+    s = synth.make_system(nat, 13)
+    p = model_params(X, kernel_mode=1, prec="fp16x3")
+    v = random_n(nat, 17)
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, random_n(nat, 18))
+        ctx.build_H(0)
+        ctx.density(0)
+        vd = torch.tensor(v, dtype=torch.float64, device="cuda")
+        wd = torch.zeros_like(vd)
+        ctx.response(0, vd.data_ptr(), wd.data_ptr())
+        torch.cuda.synchronize()
+        ctx.kernel_exact(0)
+        K = ctx.get(0, X.KMAT)
+    assert np.linalg.norm(K @ (wd.cpu().numpy() - v) - v) < 1e-3 * np.linalg.norm(v)

@@ -88,6 +88,10 @@ struct xlbomd_ctx {
   std::string msg;
   xl::Engine* eng = nullptr;
   xl::PlanCache plans;
+  // lockstep: streams for the kernels that each system runs by itself (side_by_side)
+  std::vector<cudaStream_t> side;
+  std::vector<cudaEvent_t> side_done;
+  cudaEvent_t side_fork = nullptr;
 };
 
 namespace {
@@ -250,6 +254,45 @@ xlbomd_status sync_read(xlbomd_ctx* ctx, const double* dev, int count) {
   CK(cudaMemcpyAsync(ctx->pinned, dev, sizeof(double) * count, cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   return XLBOMD_OK;
+}
+
+// f(k) for the systems k < count of a lockstep group, with ctx->stream one of up to 8 side streams that
+// start after the work already on the context's stream; that stream then waits for all of them.  For
+// the kernels of one system that touch no other: they are latency-bound (57 atoms: 16 kernels of 3 to
+// 20 us), so the systems overlap until the host's 2 us per launch bounds them.  8 systems of 57 atoms,
+// two steps, one system after the other: 6250 us.
+constexpr int kSide = 8;
+
+template <class F>
+xlbomd_status side_by_side(xlbomd_ctx* ctx, size_t count, F f) {
+  if (count < 2) return count ? f((size_t)0) : XLBOMD_OK;
+  while ((int)ctx->side.size() < kSide) {
+    cudaStream_t s = nullptr;
+    CK(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+    ctx->side.push_back(s);
+  }
+  while ((int)ctx->side_done.size() < kSide) {
+    cudaEvent_t e = nullptr;
+    CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    ctx->side_done.push_back(e);
+  }
+  if (!ctx->side_fork) CK(cudaEventCreateWithFlags(&ctx->side_fork, cudaEventDisableTiming));
+  const cudaStream_t main = ctx->stream;
+  const size_t lanes = std::min<size_t>(count, kSide);
+  CK(cudaEventRecord(ctx->side_fork, main));
+  for (size_t l = 0; l < lanes; ++l) CK(cudaStreamWaitEvent(ctx->side[l], ctx->side_fork, 0));
+  xlbomd_status rs = XLBOMD_OK;
+  for (size_t k = 0; k < count && rs == XLBOMD_OK; ++k) {
+    ctx->stream = ctx->side[k % lanes];
+    rs = f(k);
+  }
+  ctx->stream = main;
+  // also after an error: nothing of this call runs on past what follows on the context's stream
+  for (size_t l = 0; l < lanes; ++l) {
+    CK(cudaEventRecord(ctx->side_done[l], ctx->side[l]));
+    CK(cudaStreamWaitEvent(main, ctx->side_done[l], 0));
+  }
+  return rs;
 }
 
 // The vectors of a product with gamma, and of a response, of system S (x: the charges or the probe)
@@ -511,10 +554,11 @@ xlbomd_status density_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, bool wi
   Engine& E = *ctx->eng;
   const size_t B = G.size();
   double* h = ctx->pinned_group;
-  for (size_t i = 0; i < B; ++i) {
-    CK(launch_gershgorin(st, G[i]->N, G[i]->np, G[i]->H, G[i]->work));
-    CK(cudaMemcpyAsync(h + 2 * i, G[i]->work, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-  }
+  CKS(side_by_side(ctx, B, [&](size_t i) -> xlbomd_status {
+    CK(launch_gershgorin(ctx->stream, G[i]->N, G[i]->np, G[i]->H, G[i]->work));
+    CK(cudaMemcpyAsync(h + 2 * i, G[i]->work, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    return XLBOMD_OK;
+  }));
   CK(cudaStreamSynchronize(st));
   std::vector<MuSearch> ms(B);
   for (size_t i = 0; i < B; ++i) CKS(ms[i].start(ctx, *G[i], h[2 * i], h[2 * i + 1]));
@@ -544,27 +588,28 @@ xlbomd_status density_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G, bool wi
     }
     CK(E.foe_group(st, fj, sc));
     CK(E.mu_derivative_group(st, mj, 0.5 * beta_of(p)));
-    for (size_t k = 0; k < active.size(); ++k) {
+    CKS(side_by_side(ctx, active.size(), [&](size_t k) -> xlbomd_status {
       Sys& S = *G[active[k]];
-      CK(E.trace_tn(st, S.mats, S.N, S.scal));
-      CK(launch_sum(st, S.N, S.dmu_diag, S.scal + 1));
-      CK(cudaMemcpyAsync(h + 2 * k, S.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    }
+      CK(E.trace_tn(ctx->stream, S.mats, S.N, S.scal));
+      CK(launch_sum(ctx->stream, S.N, S.dmu_diag, S.scal + 1));
+      CK(cudaMemcpyAsync(h + 2 * k, S.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+      return XLBOMD_OK;
+    }));
     int* herr = reinterpret_cast<int*>(ctx->pinned + 63);
     *herr = 0;
     if (const int* derr = E.device_error())
       CK(cudaMemcpyAsync(herr, derr, sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (*herr != 0) return fail(ctx, XLBOMD_ERR_TIMEOUT, "tensor-core product: a bounded wait gave up or a tile was out of range");
-    std::vector<size_t> next;
+    std::vector<size_t> next, done;
     for (size_t k = 0; k < active.size(); ++k) {
       const size_t i = active[k];
       CKS(ms[i].update(ctx, *G[i], h[2 * k], h[2 * k + 1]));
-      if (ms[i].done)
-        CKS(density_finish(ctx, *G[i], ms[i], with_forces));
-      else
-        next.push_back(i);
+      (ms[i].done ? done : next).push_back(i);
     }
+    CKS(side_by_side(ctx, done.size(), [&](size_t k) -> xlbomd_status {
+      return density_finish(ctx, *G[done[k]], ms[done[k]], with_forces);
+    }));
     active.swap(next);
   }
   return XLBOMD_OK;
@@ -1077,11 +1122,12 @@ xlbomd_status scf_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
 xlbomd_status md_step_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
   cudaStream_t st = ctx->stream;
   const xlbomd_params& p = ctx->p;
-  for (Sys* S : G) {
-    CK(launch_verlet_first(st, S->nat, S->L, p.dt, kAcc / S->mass, S->R, S->V, S->F, S->nh, p.kmax, S->Kr, p.kappa,
-                           p.alpha, ctx->cdev));
-    CKS(build_H(ctx, *S));
-  }
+  CKS(side_by_side(ctx, G.size(), [&](size_t k) -> xlbomd_status {
+    Sys* S = G[k];
+    CK(launch_verlet_first(ctx->stream, S->nat, S->L, p.dt, kAcc / S->mass, S->R, S->V, S->F, S->nh, p.kmax, S->Kr,
+                           p.kappa, p.alpha, ctx->cdev));
+    return build_H(ctx, *S);
+  }));
   CKS(density_group(ctx, G, true));
   for (Sys* S : G) {
     ++S->md_steps;
@@ -1089,12 +1135,15 @@ xlbomd_status md_step_group(xlbomd_ctx* ctx, const std::vector<Sys*>& G) {
   }
   CKS(kernel_update_group(ctx, G));
   double* h = ctx->pinned_group;
-  for (size_t k = 0; k < G.size(); ++k) {
+  CKS(side_by_side(ctx, G.size(), [&](size_t k) -> xlbomd_status {
     Sys& S = *G[k];
-    CK(launch_verlet_second(st, S.nat, p.dt, kAcc / S.mass, S.V, S.F));
-    CK(launch_absmax(st, S.nat, S.r, h + k));
-    const bool e = p.energy_every > 0 && ((int)S.stats[4] + 1) % p.energy_every == 0;
-    if (e) CKS(energy(ctx, S));
+    CK(launch_verlet_second(ctx->stream, S.nat, p.dt, kAcc / S.mass, S.V, S.F));
+    CK(launch_absmax(ctx->stream, S.nat, S.r, h + k));
+    return XLBOMD_OK;
+  }));
+  for (Sys* S : G) {
+    const bool e = p.energy_every > 0 && ((int)S->stats[4] + 1) % p.energy_every == 0;
+    if (e) CKS(energy(ctx, *S));
   }
   CK(cudaStreamSynchronize(st));
   for (size_t k = 0; k < G.size(); ++k) {
@@ -1633,6 +1682,9 @@ xlbomd_status xlbomd_selftest_gemm_group(int n, int prec, int sym, int nprob, do
 xlbomd_status xlbomd_free(xlbomd_ctx* ctx) {
   if (!ctx) return XLBOMD_ERR_ARG;
   cudaStreamSynchronize(ctx->stream);   // no work of this context may still use its memory
+  for (cudaEvent_t e : ctx->side_done) cudaEventDestroy(e);
+  if (ctx->side_fork) cudaEventDestroy(ctx->side_fork);
+  for (cudaStream_t t : ctx->side) cudaStreamDestroy(t);
   for (Sys& S : ctx->sys) free_sys(S);
   if (ctx->cdev) cudaFree(ctx->cdev);
   if (ctx->pinned) cudaFreeHost(ctx->pinned);

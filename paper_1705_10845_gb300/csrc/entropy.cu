@@ -92,6 +92,15 @@ __global__ void chol_sum_kernel(int npart, const double* __restrict__ part, doub
   if (threadIdx.x == 0) out[blockIdx.x] = v;
 }
 
+// Y on the N x N block, the identity around it: log det of the whole is that of the block
+__global__ void block_or_identity_kernel(size_t count, int N, int np, const double* __restrict__ Y,
+                                         double* __restrict__ dst) {
+  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= count) return;
+  const int i = (int)(idx / np), j = (int)(idx % np);
+  dst[idx] = (i < N && j < N) ? Y[idx] : (i == j ? 1.0 : 0.0);
+}
+
 // W = I - T (np x np)
 __global__ void ident_minus_f64_kernel(size_t count, int np, const double* __restrict__ T, double* __restrict__ W) {
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -117,15 +126,16 @@ __global__ void entropy_combine_kernel(EntW w, const double* __restrict__ ld, co
   *out = s;
 }
 
-// log-determinants of the nb SPD matrices in the work area (destroyed) into out[0..nb)
-cudaError_t logdet_spd(cudaStream_t s, const EntropyWork& w, int np, int nb, double* out) {
+// log-determinants of the leading m x m blocks (m a multiple of CB) of the nb SPD matrices in the work area
+// (destroyed) into out[0..nb)
+cudaError_t logdet_spd(cudaStream_t s, const EntropyWork& w, int m, int np, int nb, double* out) {
   const size_t cnt = (size_t)np * np;
-  const int npart = np / CB;
-  for (int kb = 0; kb < np; kb += CB) {
+  const int npart = m / CB;
+  for (int kb = 0; kb < m; kb += CB) {
     chol_panel_kernel<<<nb, 256, 0, s>>>(w.mats(), cnt, np, kb, w.li(np), w.part(np), npart);
     note_launch();
     RET(cudaGetLastError());
-    const int rest = np - kb - CB;
+    const int rest = m - kb - CB;
     if (rest > 0) {
       // X = A21 Li^T, A22 -= X X^T
       double* A21 = w.mats() + (size_t)(kb + CB) * np + kb;
@@ -176,6 +186,7 @@ cudaError_t entropy_fp64(cudaStream_t s, int N, int np, int n, int n_sq, const d
   double* tr = work + 64;
   double* fwork = work + 1024;
   const size_t count = (size_t)np * np;
+  const int mc = (N + CB - 1) / CB * CB, m = (N + 15) / 16 * 16;   // padding does not change what follows
   // logdet(I - T_0), then logdet(Y_k)
   RET(ew.reserve(np, n + 1));
   for (int k0 = 0; k0 <= n; k0 += ew.cap) {
@@ -190,27 +201,27 @@ cudaError_t entropy_fp64(cudaStream_t s, int N, int np, int n, int n_sq, const d
         RET(load_Y(k0 + b - 1, dst));
       }
     }
-    RET(logdet_spd(s, ew, np, nb, ld + k0));
+    RET(logdet_spd(s, ew, mc, np, nb, ld + k0));
   }
   // Tr[D T0^(2j+1)] from S0 = T0^2, S2 = S0^2, S4 = S2^2, P1 = D T0, P3 = P1 S0
   EpiF64 e;
   RET(cudaMemsetAsync(tr, 0, 8 * sizeof(double), s));
   RET(launch_frob_dot(s, N, np, D, T0, fwork, tr + 0));                                    // Tr D T0
   if (nterms > 1) {
-    RET(gemm_f64_nt(s, np, np, np, T0, np, T0, np, S, np, e, true));                        // S0
-    RET(gemm_f64_nt(s, np, np, np, D, np, T0, np, A1, np, e, false));                       // P1 = D T0
+    RET(gemm_f64_nt(s, m, m, m, T0, np, T0, np, S, np, e, true));   // S0
+    RET(gemm_f64_nt(s, m, m, m, D, np, T0, np, A1, np, e, false));   // P1 = D T0
     RET(launch_frob_dot(s, N, np, A1, S, fwork, tr + 1));                                   // Tr D T0^3
   }
   if (nterms > 2) {
-    RET(gemm_f64_nt(s, np, np, np, S, np, S, np, Q, np, e, true));                          // S2 = S0^2
+    RET(gemm_f64_nt(s, m, m, m, S, np, S, np, Q, np, e, true));   // S2 = S0^2
     RET(launch_frob_dot(s, N, np, A1, Q, fwork, tr + 2));                                   // Tr D T0^5
   }
   if (nterms > 3) {
-    RET(gemm_f64_nt(s, np, np, np, A1, np, S, np, Mt, np, e, false));                       // P3 = P1 S0
+    RET(gemm_f64_nt(s, m, m, m, A1, np, S, np, Mt, np, e, false));   // P3 = P1 S0
     RET(launch_frob_dot(s, N, np, Mt, Q, fwork, tr + 3));                                   // Tr D T0^7
   }
   if (nterms > 4) {
-    RET(gemm_f64_nt(s, np, np, np, Q, np, Q, np, Yw, np, e, true));                         // S4
+    RET(gemm_f64_nt(s, m, m, m, Q, np, Q, np, Yw, np, e, true));   // S4
     RET(launch_frob_dot(s, N, np, A1, Yw, fwork, tr + 4));                                  // Tr D T0^9
   }
   if (nterms > 5) RET(launch_frob_dot(s, N, np, Mt, Yw, fwork, tr + 5));                    // Tr D T0^11
@@ -234,7 +245,9 @@ cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, int N, double beta, in
   (void)H;
   const size_t count = (size_t)m.np * m.np;
   auto load_Y = [&](int k, double* dst) {
-    return cudaMemcpyAsync(dst, m.Y[k], sizeof(double) * count, cudaMemcpyDeviceToDevice, s);
+    block_or_identity_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, N, m.np, m.Y[k], dst);
+    note_launch();
+    return cudaGetLastError();
   };
   return entropy_fp64(s, N, m.np, m.n, n_sq, m.T[0], load_Y, m.ent, m.S, m.Q, m.Yw, m.A1, m.Mt, 6, D, work, out);
 }

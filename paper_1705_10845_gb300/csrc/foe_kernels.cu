@@ -19,24 +19,28 @@ namespace {
     if (e_ != cudaSuccess) return e_; \
   } while (0)
 
-__global__ void t0_init_kernel(int n, int np, const double* H, double mu, double scale,
+// Element-wise kernels over the leading m x m block of matrices with leading dimension np.
+__global__ void t0_init_kernel(int n, int m, int np, const double* H, double mu, double scale,
                                double* T0) {
   grid_wait();
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)np * np) return;
-  const int i = (int)(idx / np), j = (int)(idx % np);
+  const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (int)(e / m), j = (int)(e % m);
+  if (i >= m) return;
+  const size_t idx = (size_t)i * np + j;
   double v = 0.0;
   if (i < n && j < n) v = -scale * (H[idx] - (i == j ? mu : 0.0));
   T0[idx] = v;
 }
 
-__global__ void combine_kernel(int np, double a, double c1, const double* X1, double c2,
+__global__ void combine_kernel(int m, int np, double a, double c1, const double* X1, double c2,
                                const double* X2, double c3, const double* X3,
                                double* Y) {
   grid_wait();
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)np * np) return;
-  double v = (idx / np == idx % np) ? a : 0.0;
+  const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (int)(e / m), j = (int)(e % m);
+  if (i >= m) return;
+  const size_t idx = (size_t)i * np + j;
+  double v = (i == j) ? a : 0.0;
   if (X1) v += c1 * X1[idx];
   if (X2) v += c2 * X2[idx];
   if (X3) v += c3 * X3[idx];
@@ -44,16 +48,17 @@ __global__ void combine_kernel(int np, double a, double c1, const double* X1, do
 }
 
 // A1 = T0 diag(d) + diag(d) T0  (first level of a chain with diagonal T1_0)
-__global__ void level0_A1_kernel(int np, const double* T0, const double* d,
+__global__ void level0_A1_kernel(int m, int np, const double* T0, const double* d,
                                  double* A1) {
   grid_wait();
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)np * np) return;
-  const int i = (int)(idx / np), j = (int)(idx % np);
+  const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (int)(e / m), j = (int)(e % m);
+  if (i >= m) return;
+  const size_t idx = (size_t)i * np + j;
   A1[idx] = T0[idx] * (d[i] + d[j]);
 }
 
-// A1 = G + G^T through 32x32 shared-memory tiles (coalesced both ways).
+// A1 = G + G^T through 32x32 shared-memory tiles (coalesced both ways; np is a multiple of 32).
 __global__ void transpose_add_kernel(int np, const double* G, double* A1) {
   grid_wait();
   __shared__ double tile[32][33];
@@ -67,8 +72,8 @@ __global__ void transpose_add_kernel(int np, const double* G, double* A1) {
   }
 }
 
-// out[i] = sum_j Y_ij M_ij (i < n): the diagonal of Y M^T, one warp per row.
-__global__ void row_dot_kernel(int n, int np, const double* Y, const double* M,
+// out[i] = sum_{j < k} Y_ij M_ij (i < n): the diagonal of Y M^T, one warp per row.
+__global__ void row_dot_kernel(int n, int k, int np, const double* Y, const double* M,
                                double* out) {
   grid_wait();
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -77,7 +82,7 @@ __global__ void row_dot_kernel(int n, int np, const double* Y, const double* M,
   const double* y = Y + (size_t)i * np;
   const double* m = M + (size_t)i * np;
   double acc = 0.0;
-  for (int j = lane; j < np; j += 32) acc += y[j] * m[j];
+  for (int j = lane; j < k; j += 32) acc += y[j] * m[j];
   acc = warp_sum(acc);
   if (lane == 0) out[i] = acc;
 }
@@ -513,31 +518,31 @@ cudaError_t launch_density_out_f64(cudaStream_t s, int N, int np, const double* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_t0_init(cudaStream_t s, int n, int np, const double* H, double mu, double scale, double* T0) {
-  RET(launch_chained(s, blocks_for((size_t)np * np, 256), 256, 0, t0_init_kernel, n, np, H, mu, scale, T0));
+cudaError_t launch_t0_init(cudaStream_t s, int n, int m, int np, const double* H, double mu, double scale, double* T0) {
+  RET(launch_chained(s, blocks_for((size_t)m * m, 256), 256, 0, t0_init_kernel, n, m, np, H, mu, scale, T0));
   return cudaSuccess;
 }
 
-cudaError_t launch_combine(cudaStream_t s, int np, double a, double c1, const double* X1, double c2, const double* X2,
-                           double c3, const double* X3, double* Y) {
-  RET(launch_chained(s, blocks_for((size_t)np * np, 256), 256, 0, combine_kernel, np, a, c1, X1, c2, X2, c3, X3, Y));
+cudaError_t launch_combine(cudaStream_t s, int m, int np, double a, double c1, const double* X1, double c2,
+                           const double* X2, double c3, const double* X3, double* Y) {
+  RET(launch_chained(s, blocks_for((size_t)m * m, 256), 256, 0, combine_kernel, m, np, a, c1, X1, c2, X2, c3, X3, Y));
   return cudaSuccess;
 }
 
-cudaError_t launch_level0_A1(cudaStream_t s, int np, const double* T0, const double* d, double* A1) {
-  RET(launch_chained(s, blocks_for((size_t)np * np, 256), 256, 0, level0_A1_kernel, np, T0, d, A1));
+cudaError_t launch_level0_A1(cudaStream_t s, int m, int np, const double* T0, const double* d, double* A1) {
+  RET(launch_chained(s, blocks_for((size_t)m * m, 256), 256, 0, level0_A1_kernel, m, np, T0, d, A1));
   return cudaSuccess;
 }
 
-cudaError_t launch_transpose_add(cudaStream_t s, int np, const double* G, double* A1) {
+cudaError_t launch_transpose_add(cudaStream_t s, int m, int np, const double* G, double* A1) {
   if (np % 32) return cudaErrorInvalidValue;
-  dim3 grid(np / 32, np / 32), block(32, 8);
+  dim3 grid((m + 31) / 32, (m + 31) / 32), block(32, 8);
   RET(launch_chained(s, grid, block, 0, transpose_add_kernel, np, G, A1));
   return cudaSuccess;
 }
 
-cudaError_t launch_row_dot(cudaStream_t s, int n, int np, const double* Y, const double* M, double* out) {
-  RET(launch_chained(s, (n + 7) / 8, 256, 0, row_dot_kernel, n, np, Y, M, out));
+cudaError_t launch_row_dot(cudaStream_t s, int n, int k, int np, const double* Y, const double* M, double* out) {
+  RET(launch_chained(s, (n + 7) / 8, 256, 0, row_dot_kernel, n, k, np, Y, M, out));
   return cudaSuccess;
 }
 

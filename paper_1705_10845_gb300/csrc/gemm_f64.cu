@@ -15,7 +15,7 @@
 namespace xl {
 namespace {
 
-constexpr int KC = 16;   // K values staged at a time (K is a multiple of 16)
+constexpr int KC = 16;   // K values staged at a time (M, N and K are multiples of 16)
 
 // upper-triangular tile index t of nt x nt tiles -> (bi, bj), bj >= bi
 __device__ __forceinline__ void sym_tile(int t, int nt, int& bi, int& bj) {
@@ -131,11 +131,12 @@ __global__ void __launch_bounds__(128) gemm_f64_t_kernel(int M, int N, int K, co
   C += st.c * blockIdx.z;
   if (e.E) e.E += st.e * blockIdx.z;
   int bi, bj;
+  const int nt = (N + T - 1) / T;   // rows past M and N are loaded and not stored
   if (SYM) {
-    sym_tile(blockIdx.x, N / T, bi, bj);
+    sym_tile(blockIdx.x, nt, bi, bj);
   } else {
-    bi = blockIdx.x / (N / T);
-    bj = blockIdx.x % (N / T);
+    bi = blockIdx.x / nt;
+    bj = blockIdx.x % nt;
   }
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int r = (w >> 1) * (T / 2) + (lane >> 2), c = (w & 1) * (T / 2) + (lane & 3);
@@ -191,6 +192,7 @@ __global__ void __launch_bounds__(128) gemm_f64_t_kernel(int M, int N, int K, co
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
       const int row = bi * T + r + 8 * i, col = bj * T + c + 8 * j;
+      if (row >= M || col >= N) continue;   // a multiple of 8 each: col + 4 is inside with col
       store_c<SYM>(e, C, ldc, row, col, bi == bj, acc[i][j][0]);
       store_c<SYM>(e, C, ldc, row, col + 4, bi == bj, acc[i][j][1]);
     }
@@ -207,11 +209,12 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(int M, int N, int K, cons
   C += st.c * blockIdx.z;
   if (e.E) e.E += st.e * blockIdx.z;
   int bi, bj;
+  const int nt = (N + BN - 1) / BN;
   if (SYM) {
-    sym_tile(blockIdx.x, N / BN, bi, bj);
+    sym_tile(blockIdx.x, nt, bi, bj);
   } else {
-    bi = blockIdx.x / (N / BN);
-    bj = blockIdx.x % (N / BN);
+    bi = blockIdx.x / nt;
+    bj = blockIdx.x % nt;
   }
   __shared__ double As[BK][BM + 1];
   __shared__ double Bs[BK][BN + 1];
@@ -249,7 +252,8 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(int M, int N, int K, cons
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      store_c<SYM>(e, C, ldc, bi * BM + ty + 16 * i, bj * BN + tx + 16 * j, bi == bj, acc[i][j]);
+      if (bi * BM + 16 * i < M && bj * BN + 16 * j < N)
+        store_c<SYM>(e, C, ldc, bi * BM + ty + 16 * i, bj * BN + tx + 16 * j, bi == bj, acc[i][j]);
 }
 
 // Tile edge of a product: the one with the least waves over the SMs times the tile's multiply-adds, with
@@ -261,8 +265,8 @@ int pick_tile(int M, int N, bool sym, int batch) {
   int best = 64;
   double least = 0.0;
   for (int i = 0; i < 4; ++i) {
-    const long long nt = N / edge[i];
-    const long long tiles = batch * (sym ? nt * (nt + 1) / 2 : nt * (M / edge[i]));
+    const long long nt = (N + edge[i] - 1) / edge[i];
+    const long long tiles = batch * (sym ? nt * (nt + 1) / 2 : nt * ((M + edge[i] - 1) / edge[i]));
     const double c = (double)((tiles + 151) / 152) * edge[i] * edge[i] * over[i];
     if (least == 0.0 || c < least) {
       least = c;
@@ -292,11 +296,11 @@ cudaError_t launch(cudaStream_t s, int tile, dim3 grid, int M, int N, int K, con
 cudaError_t gemm_f64_nt(cudaStream_t s, int M, int N, int K, const double* A, int lda, const double* B,
                         int ldb, double* C, int ldc, const EpiF64& e, bool sym, int batch, size_t stA, size_t stB,
                         size_t stC, size_t stE) {
-  if (M % 64 || N % 64 || K % KC || M <= 0 || N <= 0 || K <= 0 || batch < 1) return cudaErrorInvalidValue;
+  if (M % 16 || N % 16 || K % KC || M <= 0 || N <= 0 || K <= 0 || batch < 1) return cudaErrorInvalidValue;
   if (sym && M != N) return cudaErrorInvalidValue;
   const int t = pick_tile(M, N, sym, batch);
-  const long long nt = N / t;
-  const dim3 grid((unsigned)(sym ? nt * (nt + 1) / 2 : nt * (M / t)), 1, (unsigned)batch);
+  const long long nt = (N + t - 1) / t;
+  const dim3 grid((unsigned)(sym ? nt * (nt + 1) / 2 : nt * ((M + t - 1) / t)), 1, (unsigned)batch);
   const F64Batch st{stA, stB, stC, stE};
   return sym ? launch<true>(s, t, grid, M, N, K, A, lda, B, ldb, C, ldc, e, st)
              : launch<false>(s, t, grid, M, N, K, A, lda, B, ldb, C, ldc, e, st);

@@ -20,8 +20,9 @@ struct EpiF64 {
   double dvec_scale = 1.0;
 };
 
-// FP64 C[M x N] = epi(A[M x K] * B[N x K]^T), row-major, 16-byte aligned rows.  M, N multiples of
-// 64, K a multiple of 16.  sym: M == N and only tiles on or above the
+// FP64 C[M x N] = epi(A[M x K] * B[N x K]^T), row-major, 16-byte aligned rows.  M, N, K multiples
+// of 16; the rows of A and B are readable up to the next multiple of 64 (they are loaded for the tiles at
+// the edge, and only elements inside M x N are stored).  sym: M == N and only tiles on or above the
 // diagonal are computed; each is written to (i, j) and mirrored to (j, i), so
 // the result is exactly symmetric (E must then be null or symmetric; it may be C).
 // batch > 1: that many products, their matrices a stride apart (st*, elements).
@@ -100,12 +101,12 @@ cudaError_t launch_verlet_first(cudaStream_t s, int nat, double L, double dt, do
 cudaError_t launch_verlet_second(cudaStream_t s, int nat, double dt, double mass_inv_acc, double* V,
                                  const double* F);
 
-// ---- expansion helpers (foe_kernels.cu), FP64 ----
-cudaError_t launch_t0_init(cudaStream_t s, int n, int np, const double* H, double mu, double scale,
+// ---- expansion helpers (foe_kernels.cu), FP64: over the leading m x m block, leading dimension np ----
+cudaError_t launch_t0_init(cudaStream_t s, int n, int m, int np, const double* H, double mu, double scale,
                            double* T0);
-cudaError_t launch_level0_A1(cudaStream_t s, int np, const double* T0, const double* d, double* A1);
-cudaError_t launch_transpose_add(cudaStream_t s, int np, const double* G, double* A1);
-cudaError_t launch_row_dot(cudaStream_t s, int n, int np, const double* Y, const double* M, double* out);
+cudaError_t launch_level0_A1(cudaStream_t s, int m, int np, const double* T0, const double* d, double* A1);
+cudaError_t launch_transpose_add(cudaStream_t s, int m, int np, const double* G, double* A1);
+cudaError_t launch_row_dot(cudaStream_t s, int n, int k, int np, const double* Y, const double* M, double* out);
 cudaError_t launch_get_diag(cudaStream_t s, int n, int np, const double* X, double* out);
 // out[slot] = sum_{i<n} x[i] (deterministic, one block)
 cudaError_t launch_sum(cudaStream_t s, int n, const double* x, double* out);

@@ -248,9 +248,9 @@ cudaError_t launch_sub(cudaStream_t s, int n, const double* w, const double* t, 
 cudaError_t launch_dot1p(cudaStream_t s, int n, const double* a, const double* b, double* out);
 cudaError_t launch_rank1_update(cudaStream_t s, int n, const double* u, const double* v, const double* Ku,
                                 const double* vK, const double* denom, double* J, double* K);
-// Y = a I + sum_j c_j X_j over the matrices given (null: left out)
-cudaError_t launch_combine(cudaStream_t s, int np, double a, double c1, const double* X1, double c2, const double* X2,
-                           double c3, const double* X3, double* Y);
+// Y = a I + sum_j c_j X_j over the matrices given (null: left out), leading m x m block
+cudaError_t launch_combine(cudaStream_t s, int m, int np, double a, double c1, const double* X1, double c2,
+                           const double* X2, double c3, const double* X3, double* Y);
 cudaError_t launch_density_out_f64(cudaStream_t s, int N, int np, const double* Tn, const double* Tmu, double dmu,
                                    double* ddiag, double* D);
 

@@ -676,6 +676,7 @@ xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
       cj[j].dvec = p.dvec;
       cj[j].N = S.N;
       cj[j].out_diag = p.d1;
+      cj[j].side = G;
       cj[j].stats = S.stats;
     }
     CK(launch_probe_potential(st, ctx->p.coulomb_k, pj));

@@ -213,11 +213,14 @@ __global__ void t0_init_group_kernel(int np, int nlev, int fmt, int dt0, double 
 //   A1 = T T1 + T1 T           |A1| <= 2 t tau
 //   M  = 2 T1 - A1 T'          |M|  <= 2 tau (1 + t t')
 //   T1' = 2 Y (T1 - T T1 T) Y  |T1'| <= 2 tau (1 + g^2),  g = t / (1 + t^2) the largest t y
+// Two-step chain: P = Y T1 in the place of M, |P| <= tau, and Q = T' T1 / 4 in that of A1 at the scale that
+// makes Q T' match P W in one accumulator; |Q| times it stays below 2^14.
 struct ChainScaleList {
   int n = 0;
   const double* d[kMaxGroup];
   const float* t0[kMaxGroup];
-  float* scales[kMaxGroup];   // [3 k] A1_k, [3 k + 1] M_k, [3 k + 2] T1_{k+1}
+  const float* ts[kMaxGroup];   // two-step chain: the scales of T_0, T_1, ..  (null: three-step)
+  float* scales[kMaxGroup];     // [3 k] A1_k, [3 k + 1] M_k, [3 k + 2] T1_{k+1}
 };
 
 __global__ void chain_scales_kernel(int np, int nlev, ChainScaleList L) {
@@ -237,8 +240,10 @@ __global__ void chain_scales_kernel(int np, int nlev, ChainScaleList L) {
   float* scales = L.scales[j];
   for (int k = 0; k < nlev; ++k) {
     const float g = t / (1.0f + t * t), tn = 2.0f * g;
-    scales[3 * k] = operand_scale(2.0f * t * tau);
-    scales[3 * k + 1] = operand_scale(2.0f * tau * (1.0f + t * tn));
+    const float* ts = L.ts[j];
+    const float sp = ts ? operand_scale(tau) : operand_scale(2.0f * tau * (1.0f + t * tn));
+    scales[3 * k] = ts ? sp * kUnitScale / ts[k + 1] : operand_scale(2.0f * t * tau);
+    scales[3 * k + 1] = sp;
     tau *= 2.0f * (1.0f + g * g);
     scales[3 * k + 2] = operand_scale(tau);
     t = tn;
@@ -273,14 +278,88 @@ __global__ void level0_A1_group_kernel(int np, int fmt, A1List L) {
   }
 }
 
+// Two-step chain, level 0, per system: P = (I - W) diag(d) and Q = T' diag(d) / 4, value and operands
+struct P0List {
+  int n = 0;
+  const float* W[kMaxGroup];
+  const float2* T[kMaxGroup];
+  const double* d[kMaxGroup];
+  float* Pf[kMaxGroup];    // P as FP32 (single products) ..
+  float2* Pd[kMaxGroup];   // .. or as double-float
+  float* Qf[kMaxGroup];
+  void *Phi[kMaxGroup], *Plo[kMaxGroup], *Qhi[kMaxGroup], *Qlo[kMaxGroup];
+  const float *Ps[kMaxGroup], *Qs[kMaxGroup];
+};
+
+__global__ void level0_P_group_kernel(int np, int fmt, P0List L) {
+  grid_wait();
+  const int j = blockIdx.y;
+  const float4* W = reinterpret_cast<const float4*>(L.W[j]);
+  const float4* T = reinterpret_cast<const float4*>(L.T[j]);
+  const double* d = L.d[j];
+  const float sp = *L.Ps[j], sq = *L.Qs[j];
+  const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+  const size_t count = (size_t)np * np / 4;
+  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < count; idx += (size_t)gridDim.x * blockDim.x) {
+    const int r = (int)(4 * idx / np), c = (int)(4 * idx % np);
+    const float4 w4 = W[idx], a = T[2 * idx], b = T[2 * idx + 1];
+    const float w[4] = {w4.x, w4.y, w4.z, w4.w}, t[4] = {a.x + a.y, a.z + a.w, b.x + b.y, b.z + b.w};
+    float p[4], pl[4], q[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const double dc = d[c + e], v = ((r == c + e ? 1.0 : 0.0) - (double)w[e]) * dc;
+      p[e] = (float)v;
+      pl[e] = (float)(v - (double)p[e]);
+      q[e] = 0.25f * t[e] * (float)dc;
+    }
+    if (L.Pf[j]) {
+      reinterpret_cast<float4*>(L.Pf[j])[idx] = make_float4(p[0], p[1], p[2], p[3]);
+    } else {
+      float4* o = reinterpret_cast<float4*>(L.Pd[j]) + 2 * idx;
+      o[0] = make_float4(p[0], pl[0], p[1], pl[1]);
+      o[1] = make_float4(p[2], pl[2], p[3], pl[3]);
+    }
+    reinterpret_cast<float4*>(L.Qf[j])[idx] = make_float4(q[0], q[1], q[2], q[3]);
+    store_op4(fmt, L.Phi[j], L.Plo[j], 4 * idx, sp, p, pl);
+    store_op4(fmt, L.Qhi[j], L.Qlo[j], 4 * idx, sq, q, zero);
+  }
+}
+
 // Diagonal reductions of the chains' last level, per system
 struct DiagList {
   int n = 0;
   int N[kMaxGroup];
   const float* W[kMaxGroup];    // row_dot: W_k (FP32)
-  const float2* X[kMaxGroup];   // row_dot: M^T; get_diag: T1_n (double-float)
+  const float2* X[kMaxGroup];   // row_dot: M^T, or P; get_diag: T1_n (double-float)
+  const float* Q[kMaxGroup];    // two-step chain: Q and T'
+  const float2* T[kMaxGroup];
   double* out[kMaxGroup];
 };
+
+// out_i = T1'_ii = 2 P_ii - 2 sum_j (P_ij W_ij + Q_ij T'_ij), one warp per row
+__global__ void row_dot_two_group_kernel(int np, DiagList L) {
+  grid_wait();
+  const int j = blockIdx.y;
+  const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (i >= L.N[j]) return;
+  const size_t row = (size_t)i * np;
+  const float *W = L.W[j] + row, *Q = L.Q[j] + row;
+  const float2 *P = L.X[j] + row, *T = L.T[j] + row;
+  float accf = 0.0f;
+  double acc = 0.0;
+  for (int c = lane, t = 0; c < np; c += 32, ++t) {
+    const float2 p = P[c], tt = T[c];
+    accf += W[c] * (p.x + p.y) + Q[c] * (tt.x + tt.y);
+    if ((t & 15) == 15) {
+      acc += (double)accf;
+      accf = 0.0f;
+    }
+  }
+  acc += (double)accf;
+  acc = warp_sum(acc);
+  if (lane == 0) L.out[j][i] = 2.0 * (df_val(P[i]) - acc);
+}
 
 // out_i = (Y M)_ii = Mt_ii - sum_j W_ij Mt_ij  (Y = I - W, Mt = M^T), one warp per row
 __global__ void row_dot_last_group_kernel(int np, DiagList L) {
@@ -333,7 +412,7 @@ struct Epi {
   SplitMat* V = nullptr;    // second result va C + vb E: value and operands
   float va = 0.0f, vb = 0.0f;
   int nseg = 3;             // 3: hi*hi + hi*lo + lo*hi; 1: hi*hi only
-  int pairs = 1;            // 2: C = A B^T + B A^T
+  int pairs = 1;            // 2: C = A B^T + B A^T, or A B^T + A2 B2^T with a second pair
 };
 
 // The recursion is carried in correction form so that its exact leading
@@ -432,15 +511,39 @@ class EngineSplit : public Engine {
     a.chunk_kb = kChunkK / (fmt_ == 2 ? 32 : 64);
   }
 
-  cudaError_t gemm(cudaStream_t s, int np, const SplitMat& A, const SplitMat& B, SplitMat& C, const Epi& e,
-                   bool sym, double* stats) {
+  struct GemmOp {
+    const SplitMat* A;
+    const SplitMat* B;
+    SplitMat* C;
+    Epi e;
+    double* stats;
+    const SplitMat *A2 = nullptr, *B2 = nullptr;
+  };
+
+  void fill_problem(TcProblem& p, int np, const GemmOp& o) const {
+    p.Ahi = o.A->hi;
+    p.Alo = o.A->lo;
+    p.Bhi = o.B->hi;
+    p.Blo = o.B->lo;
+    if (o.A2) {
+      p.A2hi = o.A2->hi;
+      p.A2lo = o.A2->lo;
+      p.B2hi = o.B2->hi;
+      p.B2lo = o.B2->lo;
+    }
+    fill_args(p.epi, np, *o.A, *o.B, *o.C, o.e);
+  }
+
+  cudaError_t gemm(cudaStream_t s, int np, const GemmOp& o, bool sym) {
+    const Epi& e = o.e;
+    double* stats = o.stats;
     RET(prep_tiles(np, s));
     const TcTiles& tl = tiles_[np].second;
-    TcArgs a;
-    fill_args(a, np, A, B, C, e);
-    fill_shared(a, np, e, sym);
+    TcProblem p;
+    fill_problem(p, np, o);
+    fill_shared(p.epi, np, e, sym);
     RET(prof_begin(s));
-    RET(gemm_tc(s, np, A.hi, A.lo, B.hi, B.lo, a, tl));
+    RET(gemm_tc(s, np, p, tl));
     // kind bits: 1 sym, 2 E, 4 E2, 8 E64, 16 second result, 32 double-float output
     const int kind = (sym ? 1 : 0) | (e.E ? 2 : 0) | (e.E2 ? 4 : 0) | (e.E64 ? 8 : 0) | (e.V ? 16 : 0) |
                      (e.out64 ? 32 : 0);
@@ -451,14 +554,6 @@ class EngineSplit : public Engine {
 
   // ---- grouped operations (one launch over the systems of a lockstep group) ----
 
-  struct GemmOp {
-    const SplitMat* A;
-    const SplitMat* B;
-    SplitMat* C;
-    Epi e;
-    double* stats;
-  };
-
   static dim3 ew_grid(size_t count, int nsys) {
     return dim3((unsigned)std::max<size_t>(1, std::min<size_t>(nblk(count), kEwBlocks / nsys)), (unsigned)nsys);
   }
@@ -466,10 +561,7 @@ class EngineSplit : public Engine {
   // One product per op, all in one grouped launch (ops share sym, nseg, pairs).
   cudaError_t gemm_group(cudaStream_t s, int np, std::vector<GemmOp>& ops, bool sym) {
     if (ops.empty()) return cudaSuccess;
-    if (ops.size() == 1) {
-      GemmOp& o = ops[0];
-      return gemm(s, np, *o.A, *o.B, *o.C, o.e, sym, o.stats);
-    }
+    if (ops.size() == 1) return gemm(s, np, ops[0], sym);
     RET(prep_tiles(np, s));
     const TcTiles& tl = tiles_[np].second;
     const Epi& e0 = ops[0].e;
@@ -478,11 +570,7 @@ class EngineSplit : public Engine {
     std::vector<TcProblem> probs(ops.size());
     for (size_t i = 0; i < ops.size(); ++i) {
       const GemmOp& o = ops[i];
-      probs[i].Ahi = o.A->hi;
-      probs[i].Alo = o.A->lo;
-      probs[i].Bhi = o.B->hi;
-      probs[i].Blo = o.B->lo;
-      fill_args(probs[i].epi, np, *o.A, *o.B, *o.C, o.e);
+      fill_problem(probs[i], np, o);
       if (o.stats) o.stats[3] += (sym ? 0.5 : 1.0) * e0.pairs;
     }
     if (!group_cache_) group_cache_ = tc_group_cache_new();
@@ -799,6 +887,110 @@ class EngineSplit : public Engine {
     return chain_group(s, jobs);
   }
 
+  // A level of a chain in two launches instead of three: with Y T = T' / 2 and T T' = 2 W,
+  //   T1' = 2 Y (T1 - T T1 T) Y = 2 P - 2 (P W + Q T'),  P = Y T1 = T1 - W T1,  Q = T' T1 / 4,
+  // P and Q side by side, then one symmetric product over two K pairs.  A level is 3 n^3 multiply-adds this
+  // way and 2.5 n^3 in three launches, so it is taken where launches count: up to 128 tiles of 128 x 128 per
+  // matrix of the probes side by side, less than one for each SM.  The systems of a lockstep group do not
+  // count: each gives the bits of its own run.  Three and two launches, us: response at n = 1024 669 and
+  // 612, two steps of 24 atoms 2305 and 2102, of 8 systems of 57 atoms 4439 and 4379, 150 atoms (n = 640)
+  // 2104 and 2002, 333 atoms TF32x3 (1408, 121 tiles) 5771 and 5594; 512 atoms (2048, 256 tiles) 7116 and
+  // 7270, 48 probes at n = 384 3577 and 3703.
+  static bool two_step(int np, int side) { return (long long)side * (np / 128) * (np / 128) <= 128; }
+
+  cudaError_t chain_two_step(cudaStream_t s, std::vector<ChainJob>& jobs, int np, int n) {
+    const int B = (int)jobs.size(), nseg = probe_nseg_;
+    const bool single = (nseg == 1);
+    const size_t cnt = (size_t)np * np;
+    for (int k = 0; k < n; ++k) {
+      const bool last = (k == n - 1);
+      P0List pl;
+      pl.n = B;
+      std::vector<GemmOp> op, ot;
+      for (int i = 0; i < B; ++i) {
+        MatSet& m = *jobs[i].m;
+        const float* cs = m.chain_scales + 3 * k;
+        SplitMat *Q = &m.sA1, *P = &m.sMt, *T1 = (k & 1) ? &m.sT1b : &m.sT1a, *T1n = (k & 1) ? &m.sT1a : &m.sT1b;
+        Q->scale = cs;
+        P->scale = cs + 1;
+        T1n->scale = cs + 2;
+        if (k == 0) {
+          pl.W[i] = m.sY[0].f;
+          pl.T[i] = m.sT[1].d;
+          pl.d[i] = jobs[i].dvec;
+          pl.Pf[i] = single && !last ? P->f : nullptr;
+          pl.Pd[i] = P->d;
+          pl.Qf[i] = Q->f;
+          pl.Phi[i] = P->hi;
+          pl.Plo[i] = single ? nullptr : P->lo;
+          pl.Qhi[i] = Q->hi;
+          pl.Qlo[i] = single ? nullptr : Q->lo;
+          pl.Ps[i] = P->scale;
+          pl.Qs[i] = Q->scale;
+        } else {
+          Epi ep;                                                                // P = T1 - W T1
+          ep.alpha = -1.f;
+          if (single) {
+            ep.E = T1;
+            ep.beta = 1.f;
+          } else {
+            ep.E64 = T1->d;
+            ep.beta64 = 1.f;
+          }
+          ep.out64 = !single || last;
+          ep.convert = !last;                                                    // the last ones are only reduced
+          ep.hi_only = single;
+          ep.nseg = nseg;
+          op.push_back({&m.sY[k], T1, P, ep, jobs[i].stats});
+          Epi eq;                                                                // Q = T' T1 / 4
+          eq.alpha = 0.25f;
+          eq.value = last;
+          eq.convert = !last;
+          eq.hi_only = single;
+          eq.nseg = nseg;
+          op.push_back({&m.sT[k + 1], T1, Q, eq, jobs[i].stats});
+        }
+        Epi et;                                                                  // T1' = 2 P - 2 (P W + Q T')
+        et.alpha = -2.f;
+        if (single) {
+          et.E = P;
+          et.beta = 2.f;
+          et.hi_only = true;
+        } else {
+          et.E64 = P->d;
+          et.beta64 = 2.f;
+          et.out64 = true;
+        }
+        et.nseg = nseg;
+        et.pairs = 2;
+        ot.push_back({P, &m.sY[k], T1n, et, jobs[i].stats, Q, &m.sT[k + 1]});
+      }
+      if (k == 0)
+        RET(launch_chained(s, ew_grid(cnt / 4, B), 256, 0, level0_P_group_kernel, np, fmt_, pl));
+      else
+        RET(gemm_group(s, np, op, false));
+      if (!last) {
+        RET(gemm_group(s, np, ot, true));
+        continue;
+      }
+      DiagList dl;
+      dl.n = B;
+      int maxN = 0;
+      for (int i = 0; i < B; ++i) {
+        MatSet& m = *jobs[i].m;
+        dl.N[i] = jobs[i].N;
+        dl.W[i] = m.sY[k].f;
+        dl.X[i] = m.sMt.d;
+        dl.Q[i] = m.sA1.f;
+        dl.T[i] = m.sT[k + 1].d;
+        dl.out[i] = jobs[i].out_diag;
+        maxN = std::max(maxN, jobs[i].N);
+      }
+      RET(launch_chained(s, dim3((maxN + 7) / 8, B), 256, 0, row_dot_two_group_kernel, np, dl));
+    }
+    return cudaSuccess;
+  }
+
   // Response chains of several systems (or several probes of one system, each with its own
   // chain matrices) in lockstep, every product a grouped launch.
   cudaError_t chain_group(cudaStream_t s, std::vector<ChainJob>& jobs) override {
@@ -821,9 +1013,11 @@ class EngineSplit : public Engine {
     // chain would add traffic and no accuracy.  The last level still writes the double-float array
     // the reductions read (with a zero low word).
     const bool single = (nseg == 1);
+    const bool two = two_step(np, jobs[0].side);
     ChainScaleList sl;
     sl.n = B;
     for (int i = 0; i < B; ++i) {
+      sl.ts[i] = two ? jobs[i].m->scales + 1 : nullptr;
       sl.d[i] = jobs[i].dvec;
       sl.t0[i] = jobs[i].m->t0_dev;
       sl.scales[i] = jobs[i].m->chain_scales;
@@ -836,6 +1030,7 @@ class EngineSplit : public Engine {
       A1s[i] = &jobs[i].m->sA1;
       Mts[i] = &jobs[i].m->sMt;
     }
+    if (two) return chain_two_step(s, jobs, np, n);
     for (int k = 0; k < n; ++k) {
       const bool last = (k == n - 1);
       for (int i = 0; i < B; ++i) {
@@ -1237,7 +1432,7 @@ int selftest_gemm_group(int n, int prec, int mode, int nprob, double* result) {
     ep.nseg = single ? 1 : 3;
     ep.alpha = 0.75f;
     for (int i = 0; i < nprob; ++i)
-      if (eng.gemm(nullptr, n, A[i], B[i], R[i], ep, sym != 0, nullptr)) goto done;
+      if (eng.gemm(nullptr, n, {&A[i], &B[i], &R[i], ep, nullptr}, sym != 0)) goto done;
     std::vector<EngineSplit::GemmOp> ops;
     for (int i = 0; i < nprob; ++i) ops.push_back({&A[i], &B[i], &C[i], ep, nullptr});
     for (int rep = 0; rep < 2; ++rep) {   // the second launch reads the table that the first one built
@@ -1325,10 +1520,10 @@ int selftest_gemm(int n, int prec, int sym, double* result) {
     Epi ep;
     ep.pairs = pair ? 2 : 1;
     ep.nseg = single ? 1 : 3;
-    if (eng.gemm(s, n, sa, sb, sc, ep, sym != 0, nullptr)) goto done;
+    if (eng.gemm(s, n, {&sa, &sb, &sc, ep, nullptr}, sym != 0)) goto done;
     cudaEventRecord(e0, s);
     for (int r = 0; r < 5; ++r)
-      if (eng.gemm(s, n, sa, sb, sc, ep, sym != 0, nullptr)) goto done;
+      if (eng.gemm(s, n, {&sa, &sb, &sc, ep, nullptr}, sym != 0)) goto done;
   }
   cudaEventRecord(e1, s);
   if (cudaDeviceSynchronize() != cudaSuccess) goto done;

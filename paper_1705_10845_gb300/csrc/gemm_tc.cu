@@ -1723,8 +1723,20 @@ void tc_forget_maps(const void* base) {
   }
 }
 
-cudaError_t gemm_tc(cudaStream_t s, int n, const void* Ahi, const void* Alo, const void* Bhi, const void* Blo,
-                    TcArgs args, const TcTiles& tiles) {
+namespace {
+
+// the second pair of p: its own, or the first one swapped
+void second_pair(const TcProblem& p, const void* (&q)[4]) {
+  const void* own[4] = {p.A2hi, p.A2lo ? p.A2lo : p.A2hi, p.B2hi, p.B2lo ? p.B2lo : p.B2hi};
+  const void* swapped[4] = {p.Bhi, p.Blo ? p.Blo : p.Bhi, p.Ahi, p.Alo ? p.Alo : p.Ahi};
+  for (int i = 0; i < 4; ++i) q[i] = p.A2hi ? own[i] : swapped[i];
+}
+
+}  // namespace
+
+cudaError_t gemm_tc(cudaStream_t s, int n, const TcProblem& prob, const TcTiles& tiles) {
+  TcArgs args = prob.epi;
+  const void *Ahi = prob.Ahi, *Alo = prob.Alo, *Bhi = prob.Bhi, *Blo = prob.Blo;
   if (n % 128 != 0 || n <= 0) return cudaErrorInvalidValue;
   if (args.pairs != 1 && args.pairs != 2) return cudaErrorInvalidValue;
   const bool wide = (n % 256 == 0);
@@ -1741,9 +1753,10 @@ cudaError_t gemm_tc(cudaStream_t s, int n, const void* Ahi, const void* Alo, con
       !make_map(&mBhi, Bhi, n, bbox, args.fmt) || !make_map(&mBlo, Blo ? Blo : Bhi, n, bbox, args.fmt))
     return cudaErrorInvalidValue;
   if (args.pairs == 2) {
-    // the swapped pair: B in the A role (BM-row boxes), A in the B role
-    if (!make_map(&mA2hi, Bhi, n, BM, args.fmt) || !make_map(&mA2lo, Blo ? Blo : Bhi, n, BM, args.fmt) ||
-        !make_map(&mB2hi, Ahi, n, bbox, args.fmt) || !make_map(&mB2lo, Alo ? Alo : Ahi, n, bbox, args.fmt))
+    const void* q[4];
+    second_pair(prob, q);
+    if (!make_map(&mA2hi, q[0], n, BM, args.fmt) || !make_map(&mA2lo, q[1], n, BM, args.fmt) ||
+        !make_map(&mB2hi, q[2], n, bbox, args.fmt) || !make_map(&mB2lo, q[3], n, bbox, args.fmt))
       return cudaErrorInvalidValue;
   } else {
     mA2hi = mAhi;
@@ -1845,7 +1858,8 @@ cudaError_t gemm_tc_group(cudaStream_t s, int n, const TcProblem* probs, int npr
   if (nprob < 1 || !cache || shared.fmt < 0 || shared.fmt > 2) return cudaErrorInvalidValue;
   if (n % 128 != 0 || n <= 0 || (shared.pairs != 1 && shared.pairs != 2)) return cudaErrorInvalidValue;
   if (nprob == 1) {
-    TcArgs a = probs[0].epi;
+    TcProblem one = probs[0];
+    TcArgs& a = one.epi;
     a.nseg = shared.nseg;
     a.pairs = shared.pairs;
     a.sym = shared.sym;
@@ -1853,7 +1867,7 @@ cudaError_t gemm_tc_group(cudaStream_t s, int n, const TcProblem* probs, int npr
     a.split_acc = shared.split_acc;
     a.chunk_kb = shared.chunk_kb;
     a.err = shared.err;
-    return gemm_tc(s, n, probs[0].Ahi, probs[0].Alo, probs[0].Bhi, probs[0].Blo, a, tiles);
+    return gemm_tc(s, n, one, tiles);
   }
   const int width = pick_width(n, nprob, shared, tiles);
   const int bn = tc_width(width);
@@ -1867,7 +1881,8 @@ cudaError_t gemm_tc_group(cudaStream_t s, int n, const TcProblem* probs, int npr
   for (int i = 0; i < nprob; ++i) {
     const TcProblem& q = probs[i];
     const TcArgs& e = q.epi;
-    const uint64_t w[] = {(uint64_t)q.Ahi, (uint64_t)q.Alo, (uint64_t)q.Bhi, (uint64_t)q.Blo, (uint64_t)e.E,
+    const uint64_t w[] = {(uint64_t)q.Ahi, (uint64_t)q.Alo, (uint64_t)q.Bhi, (uint64_t)q.Blo, (uint64_t)q.A2hi,
+                          (uint64_t)q.A2lo, (uint64_t)q.B2hi, (uint64_t)q.B2lo, (uint64_t)e.E,
                           (uint64_t)e.E2, (uint64_t)e.E64, (uint64_t)e.dvec, (uint64_t)e.out.f, (uint64_t)e.out.d,
                           (uint64_t)e.out.hi, (uint64_t)e.out.lo, (uint64_t)e.out.scale, (uint64_t)e.out2.f,
                           (uint64_t)e.out2.hi, (uint64_t)e.out2.lo, (uint64_t)e.out2.scale, (uint64_t)e.sa,
@@ -1897,8 +1912,10 @@ cudaError_t gemm_tc_group(cudaStream_t s, int n, const TcProblem* probs, int npr
           !make_map(&t.map[2], q.Bhi, n, bn, shared.fmt) || !make_map(&t.map[3], Blo, n, bn, shared.fmt))
         return cudaErrorInvalidValue;
       if (shared.pairs == 2) {
-        if (!make_map(&t.map[4], q.Bhi, n, BM, shared.fmt) || !make_map(&t.map[5], Blo, n, BM, shared.fmt) ||
-            !make_map(&t.map[6], q.Ahi, n, bn, shared.fmt) || !make_map(&t.map[7], Alo, n, bn, shared.fmt))
+        const void* r[4];
+        second_pair(q, r);
+        if (!make_map(&t.map[4], r[0], n, BM, shared.fmt) || !make_map(&t.map[5], r[1], n, BM, shared.fmt) ||
+            !make_map(&t.map[6], r[2], n, bn, shared.fmt) || !make_map(&t.map[7], r[3], n, bn, shared.fmt))
           return cudaErrorInvalidValue;
       } else {
         t.map[4] = t.map[0];

@@ -53,7 +53,7 @@ struct TcArgs {
 };
 
 // One problem of a grouped product launch, in device memory: its tensor maps (A hi, A lo, B hi,
-// B lo, and the swapped pair's A2 hi, A2 lo, B2 hi, B2 lo) and its epilogue arguments.  The
+// B lo, and the second pair's A2 hi, A2 lo, B2 hi, B2 lo) and its epilogue arguments.  The
 // problems of a group share n, the segment and pair counts, the symmetric mode and the operand
 // type; they differ in their matrices and scalars.
 struct TcEntry {   // CUtensorMap's own alignment (64 bytes) aligns every entry
@@ -65,6 +65,9 @@ struct TcEntry {   // CUtensorMap's own alignment (64 bytes) aligns every entry
 // sym, fmt, chunk_kb and err come from the launch's shared arguments).
 struct TcProblem {
   const void *Ahi = nullptr, *Alo = nullptr, *Bhi = nullptr, *Blo = nullptr;   // operand arrays (n x n, row-major)
+  // the second pair of pairs = 2: C = A B^T + A2 B2^T.  Null: B and A.  The scales of A2 and B2 multiply to
+  // those of A and B.
+  const void *A2hi = nullptr, *A2lo = nullptr, *B2hi = nullptr, *B2lo = nullptr;
   TcArgs epi;
 };
 
@@ -82,8 +85,7 @@ struct TcTiles {
 
 // n x n product (n a multiple of 128); the symmetric tile lists come from tc_sym_tiles and
 // tc_sym_tiles_pair.
-cudaError_t gemm_tc(cudaStream_t s, int n, const void* Ahi, const void* Alo, const void* Bhi, const void* Blo,
-                    TcArgs args, const TcTiles& tiles);
+cudaError_t gemm_tc(cudaStream_t s, int n, const TcProblem& prob, const TcTiles& tiles);
 // Grouped product: the problems' tiles in one persistent launch (one-SM kernel).  The device
 // table of each distinct problem list is built once and kept in `cache` (key: the table's
 // bytes), so repeated groups upload nothing.

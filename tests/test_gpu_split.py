@@ -388,3 +388,39 @@ def test_model_of_the_split_path_against_oracle(X, nat, L):
     assert np.max(np.abs(H - H0)[off]) < 1e-11
     assert np.max(np.abs(np.diag(H) - np.diag(H0) - np.repeat(G @ n, 4))) < 1e-4
     assert np.max(np.abs(gam - G)) < 1e-5 * np.max(np.abs(G))
+
+
+@pytest.mark.parametrize("prec,nat,n_sq,kernel_prec", [("fp16x3", 32, 10, 0), ("fp16x3", 33, 1, 0), ("bf16x3", 33, 10, 0),
+                                                       ("tf32x3", 65, 12, 0), ("fp16x3", 353, 10, 0),
+                                                       ("fp16x3", 33, 10, 1), ("fp16x3", 33, 2, 1)])
+def test_response_chain_by_levels(X, prec, nat, n_sq, kernel_prec):
+    # both forms of a chain level (two launches up to 1408 padded orbitals, three at 353 atoms), the first level
+    # made from the diagonal and the last one only reduced, also where they are the same (n_sq = 1) or
+    # neighbours (2).  Against the oracle's response: 1e-4 with split products (1e-3 in BF16x3), 1e-2 with
+    # single ones, whose operands are good to 2^-11
+    import torch
+    s = synth.make_system(nat, 27)
+    Te = 1000.0 if n_sq >= 10 else 200000.0 / n_sq   # |beta (e - mu)| / 2^(n+1) stays below 1
+    p = X.default_params(mix_alpha=ALPHA_MIX, kernel_c=1 - 1 / ALPHA_MIX, prec=prec, mu_tol=1e-3, n_sq=n_sq, Te=Te,
+                         kernel_prec=kernel_prec)
+    m = O.Model(Te=p.Te, n_sq=p.n_sq)
+    rng = np.random.default_rng(nat)
+    n = rng.normal(scale=0.01, size=nat)
+    n -= n.mean()
+    v = rng.normal(size=nat)
+    v -= v.mean()
+    v /= np.linalg.norm(v)
+    ref = O.evaluate(s.R, s.L, s.Z, n, m, None, with_kernel=False, with_forces=False)
+    wref = O.response(ref.dens, ref.gamma, v)
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, n)
+        ctx.set(0, X.MU, [ref.dens.mu])
+        ctx.build_H(0)
+        ctx.density(0)
+        vd = torch.tensor(v, dtype=torch.float64, device="cuda")
+        wd = torch.zeros_like(vd)
+        ctx.response(0, vd.data_ptr(), wd.data_ptr())
+        torch.cuda.synchronize()
+        w = wd.cpu().numpy()
+    tol = 1e-2 if kernel_prec else 1e-3 if prec == "bf16x3" else 1e-4
+    assert np.linalg.norm(w - wref) < tol * np.linalg.norm(wref)

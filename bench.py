@@ -5,7 +5,7 @@ Workload (default): the precision workload -- one trajectory of 4096
 carbon-like atoms (N = 16384 orbitals) in a 38.8 A periodic cube, Te = 1000 K,
 10 squarings of the recursive Fermi-operator expansion, rank-4 kernel,
 dt = 0.25 fs; split FP16x3 tensor-core products in the expansion (one 16-bit
-product in the probe and chemical-potential chains) with FP32 accumulation and
+product in the probe chains and in dD/dmu) with FP32 accumulation and
 FP64 traces, charges, forces and integration (--prec bf16x3, tf32x3 or fp64 selects
 another form).  A step is one full XL-BOMD step
 (H build, expansion with the chemical-potential loop, charges, forces, four
@@ -42,7 +42,7 @@ TF32_PER_BF16 = 1.1 / 2.25   # nominal dense tensor rates of GB300 (PFLOP/s): tf
 # DRAM bytes (read + write) per launch of the product kernel, averaged over the launches of one
 # MD step, keyed by (variant, padded orbital count), from the ncu captures summarised in profiles/;
 # a workload or kernel without a capture since the kernel last changed reports null
-GEMM_TRAFFIC = {("persistent", 16384): 3450.66e9 / 233}   # xlbomd_step_4096atoms_fp16x3_launches.md
+GEMM_TRAFFIC = {}
 
 
 def gemm_variant():
@@ -65,8 +65,8 @@ def parse():
                     help="1 (default): the kernel's probe chains take one hi*hi product instead of three; "
                          "0: three, as the expansion")
     ap.add_argument("--mu-prec", type=int, default=1, choices=[0, 1],
-                    help="1 (default): the chemical-potential chain (dD/dmu) takes one hi*hi product instead "
-                         "of three; 0: three, as the expansion")
+                    help="1 (default): the products of dD/dmu take one hi*hi product instead of three; 0: three, "
+                         "as the expansion")
     ap.add_argument("--rep-A", type=float, default=40.0,
                     help="pair repulsion A exp(-r/0.3 A) (eV): the model's atoms collapse without it in long runs")
     ap.add_argument("--e2e-steps", type=int, default=None)
@@ -557,7 +557,7 @@ def main():
     # ---- plain-FP64 GPU path of the same workload ----
     # One FP64 step at this size takes tens of minutes, so by default one timed FP64 product of the
     # same size bounds it: the FP64 path runs at least the mixed step's dense-equivalent product
-    # count (its Newton-Schulz inverses take as many or more iterations, and its A1 takes the same
+    # count (its inverses are corrected to 1e-16 instead of 1e-8, and its A1 takes the same
     # work), so products x product time is a lower bound on its step time and the rate below an
     # upper bound on its step rate.  --fp64-steps K times K real FP64 steps instead.
     fp64 = None

@@ -304,8 +304,8 @@ xlbomd_status xlbomd_selftest_gemm(int n, int prec, int sym, double* result);
 /* Diagnostics: the grouped product launch (the products of several systems of one size in
  * one persistent launch, per-problem tensor maps and epilogue arguments read from a device
  * table) against single launches: nprob (2..64) seeded operand pairs of size n, each product
- * computed alone, then all together in one grouped launch (both tile widths, as the tile
- * autotuner tries them, then the width it keeps).  sym as for xlbomd_selftest_gemm (0-2, +4
+ * computed alone, then all together in one grouped launch (at the widths their tile counts
+ * choose, several times).  sym as for xlbomd_selftest_gemm (0-2, +4
  * single product); prec FP16x3, BF16x3 or TF32x3.  result[0] = max |C_group - C_single| (0: the
  * grouped launch computes every tile exactly as the single launch does), result[1] = device
  * wait-timeout flag.  The paper has no counterpart. */

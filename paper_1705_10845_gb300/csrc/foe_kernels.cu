@@ -577,7 +577,7 @@ namespace {
 // updates its own columns, and the next pivot column goes first, so that its search and the cluster
 // barrier run beside the rest of the update (a CTA has 2 FP64 FMAs a clock: 0.3 us a step at n = 96).  The
 // factors are held three deep: a CTA arrives for step k + 1 when it enters step k, done with k - 1.
-// n = 96 takes 237 us; as a search and an elimination launch per step it took 1100.
+// n = 96 takes 237 us; as a search and an elimination launch per step it took 1340.
 constexpr int kGjCtas = 8, kGjThreads = 512, kGjMaxSmem = 227 * 1024;
 
 __host__ __device__ inline size_t gj_smem(int n) {

@@ -84,7 +84,8 @@ __device__ __forceinline__ void add_block_grad(const Bond& b, double dx, double 
 }
 
 // FP32 test of the 27 images of a pair: bit 9 (tx + 1) + 3 (ty + 1) + tz + 1 is set where the image may lie
-// within the cutoff (cut2 = r_cut^2 and a margin above the FP32 rounding of positions in [0, L)).
+// within the cutoff (cut2 = r_cut^2 and a margin above the FP32 rounding of positions in [0, L)).  A
+// distance that is not a number may lie anywhere: the FP64 pass then carries it into H and the forces.
 __device__ __forceinline__ unsigned image_mask(float dx, float dy, float dz, float L, float cut2) {
   float x[3], y[3], z[3];
 #pragma unroll
@@ -103,7 +104,7 @@ __device__ __forceinline__ unsigned image_mask(float dx, float dy, float dz, flo
     for (int j = 0; j < 3; ++j)
 #pragma unroll
       for (int k = 0; k < 3; ++k)
-        if (x[i] + y[j] + z[k] < cut2) m |= 1u << (9 * i + 3 * j + k);
+        if (!(x[i] + y[j] + z[k] >= cut2)) m |= 1u << (9 * i + 3 * j + k);
   return m;
 }
 
@@ -210,7 +211,7 @@ __global__ void forces_short_kernel(ModelConst m, int nat, double L, float cut2,
       const double dx = R[3 * J] - xi + (t / 9 - 1) * L, dy = R[3 * J + 1] - yi + (t / 3 % 3 - 1) * L,
                    dz = R[3 * J + 2] - zi + (t % 3 - 1) * L;
       const double r2 = dx * dx + dy * dy + dz * dz;
-      if (r2 < rc2) {
+      if (!(r2 >= rc2)) {
         double Db[4][4];
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
@@ -703,7 +704,7 @@ __global__ void repulsion_energy_kernel(ModelConst m, int nat, double L, float c
       const double dx = R[3 * J] - xi + (t / 9 - 1) * L, dy = R[3 * J + 1] - yi + (t / 3 % 3 - 1) * L,
                    dz = R[3 * J + 2] - zi + (t % 3 - 1) * L;
       const double r2 = dx * dx + dy * dy + dz * dz;
-      if (r2 < rc2) {
+      if (!(r2 >= rc2)) {
         const double r = sqrt(r2);
         const double u = fmin(fmax((r - m.r_taper) / w, 0.0), 1.0);
         const double S = 1.0 - u * u * u * (10.0 - u * (15.0 - 6.0 * u));

@@ -424,3 +424,37 @@ def test_exact_kernel_inverts_the_response(X, nat):
         ctx.kernel_exact(0)
         K = ctx.get(0, X.KMAT)
     assert np.linalg.norm(K @ (wd.cpu().numpy() - v) - v) < 1e-3 * np.linalg.norm(v)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp16x3"])
+@pytest.mark.parametrize("coulomb_k", [14.399645, 0.0])
+def test_non_finite_positions_are_reported(X, prec, coulomb_k):
+    # also without the Coulomb term, whose gamma would carry a NaN into H by itself: the pair search must not lose it
+    s = synth.make_system(24, 1705, L=7.0)
+    p = model_params(X, prec=prec, coulomb_k=coulomb_k, mu_tol=1e-9 if prec == "fp64" else 1e-3)
+    for bad in (np.nan, np.inf):
+        R = s.R.copy()
+        R[5, 1] = bad
+        with X.Context(p, [sysdict(s)]) as ctx:
+            ctx.set(0, X.R, R)
+            ctx.build_H(0)
+            assert np.isnan(ctx.get(0, X.H)).any()
+            with pytest.raises(X.XlbomdError) as e:
+                ctx.density(0)
+            assert e.value.status == -5
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp16x3"])
+def test_forces_after_a_non_finite_move_are_not_finite(X, prec):
+    # positions moved without a new Hamiltonian: D stays that of the old H, the atom's own forces cannot be finite
+    s = synth.make_system(24, 1705, L=7.0)
+    p = model_params(X, prec=prec, coulomb_k=0.0, rep_A=40.0, mu_tol=1e-9 if prec == "fp64" else 1e-3)
+    R = s.R.copy()
+    R[5, 1] = np.nan
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.build_H(0)
+        ctx.set(0, X.R, R)
+        ctx.density(0)
+        assert not np.isfinite(ctx.get(0, X.F)[5]).any()
+        ctx.energy(0)
+        assert np.isnan(ctx.get(0, X.ENERGY)[6])

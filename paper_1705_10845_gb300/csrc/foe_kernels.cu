@@ -204,6 +204,9 @@ __global__ void probe_apply_kernel(double k, const __grid_constant__ JobList<Pro
 // chain does not carry a large part that mu_1 dT_n/dmu then has to cancel (the errors of the two are
 // independent).  A unit probe's potential is mostly uniform: K of 48 atoms in FP16x3 was 2e-5 off
 // without the shift.
+// The chain runs on 2^-e dvec, |dvec| < 2^e its largest element, so that the scales of its operands have the
+// same range to work in whatever the size of the probe; probe_finish_kernel takes d1 back by 2^e (scal[3]).
+// Powers of two change no bit of w.  (At the probe's own size FP16 pairs lost w below |v| = 1e-17 and had NaN above 1e19.)
 template <int NJ>
 __global__ void __launch_bounds__(kVecThreads) probe_expand_kernel(double scale, const __grid_constant__ JobList<ProbeJob, NJ> L) {
   grid_wait();
@@ -218,20 +221,33 @@ __global__ void __launch_bounds__(kVecThreads) probe_expand_kernel(double scale,
   block_sum2(s0, s1, sh);
   double pbar = s1 / s0;
   if (!isfinite(pbar)) pbar = 0.0;
-  for (int a = threadIdx.x; a < J.np; a += kVecThreads) J.dvec[a] = (a < 4 * J.nat) ? scale * (pot[a >> 2] - pbar) : 0.0;
+  // the high words of |x| order like the numbers themselves
+  __shared__ int top[kVecThreads / 32];
+  int m = 0;
+  for (int I = threadIdx.x; I < J.nat; I += kVecThreads) m = max(m, __double2hiint(fabs(scale * (pot[I] - pbar))));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = __reduce_max_sync(0xffffffffu, top[threadIdx.x & (kVecThreads / 32 - 1)]);
+  const int ex = m >> 20;   // biased exponent; 0 and 2047: nothing to scale
+  const int e = (ex == 0 || ex == 2047) ? 0 : min(ex - 1022, 1022);
+  const double down = ldexp(1.0, -e);
+  if (threadIdx.x == 0) J.scal[3] = ldexp(1.0, e);
+  for (int a = threadIdx.x; a < J.np; a += kVecThreads) J.dvec[a] = (a < 4 * J.nat) ? scale * (pot[a >> 2] - pbar) * down : 0.0;
 }
 
-// mu1 = -sum d1 / sum dmu;  w_I = sum_{a in I} (d1_a + mu1 dmu_a)  (one block per job).  A unit probe's
-// w - e_u is column u of J - I (row-major nat x nat at Jm), next to a column of the identity at B.
+// With d1 taken back by 2^e: mu1 = -sum d1 / sum dmu;  w_I = sum_{a in I} (d1_a + mu1 dmu_a)  (one block per job).
+// A unit probe's w - e_u is column u of J - I (row-major nat x nat at Jm), next to a column of the identity at B.
 template <int NJ>
 __global__ void __launch_bounds__(kVecThreads) probe_finish_kernel(const __grid_constant__ JobList<ProbeJob, NJ> L) {
   grid_wait();
   const ProbeJob& J = L.job[blockIdx.x];
   __shared__ double sh[16];
   const double *d1 = J.d1, *dmu = J.dmu;
+  const double up = J.scal[3];
   double s1 = 0.0, s2 = 0.0;
   for (int a = threadIdx.x; a < J.N; a += kVecThreads) {
-    s1 += d1[a];
+    s1 += d1[a] * up;
     s2 += dmu[a];
   }
   block_sum2(s1, s2, sh);
@@ -243,7 +259,7 @@ __global__ void __launch_bounds__(kVecThreads) probe_finish_kernel(const __grid_
   }
   for (int I = threadIdx.x; I < J.nat; I += kVecThreads) {
     double t = 0.0;
-    for (int a = 4 * I; a < 4 * I + 4; ++a) t += d1[a] + mu1 * dmu[a];
+    for (int a = 4 * I; a < 4 * I + 4; ++a) t += fma(mu1, dmu[a], d1[a] * up);   // d1 up is exact
     if (J.w) J.w[I] = t;
     if (J.unit >= 0) {
       const size_t o = (size_t)I * J.nat + J.unit;

@@ -53,7 +53,8 @@ struct ProbeJob {
   const double* x = nullptr;
   double *tmp = nullptr, *pot = nullptr;         // kp doubles; pot = gamma x
   const double* dmu = nullptr;                   // diagonal of dT_n/dmu
-  double *dvec = nullptr, *d1 = nullptr, *scal = nullptr, *w = nullptr;
+  double *dvec = nullptr, *d1 = nullptr, *w = nullptr;
+  double* scal = nullptr;                        // sum d1, sum dmu, mu1; [3] the factor d1 is to be taken back by
   double *Jm = nullptr, *B = nullptr;            // a unit probe's column of J - I and of the identity
 };
 // Rank-m kernel update (kernel_vec_kernel).  flag may be pinned host memory.
@@ -67,7 +68,7 @@ struct KernelVecJob {
 };
 // pot = gamma x with gamma = gamma_real + k SF SF^T applied through the structure factors
 cudaError_t launch_probe_potential(cudaStream_t s, double k, const std::vector<ProbeJob>& jobs);
-// dvec = scale (pot less its average) on orbitals; w (and the column of J - I) from d1
+// dvec = scale (pot less its average) on orbitals, at a power of two; w (and the column of J - I) from d1
 cudaError_t launch_probe_expand(cudaStream_t s, double scale, const std::vector<ProbeJob>& jobs);
 cudaError_t launch_probe_finish(cudaStream_t s, const std::vector<ProbeJob>& jobs);
 cudaError_t launch_kernel_vec(cudaStream_t s, const std::vector<KernelVecJob>& jobs);

@@ -424,3 +424,36 @@ def test_response_chain_by_levels(X, prec, nat, n_sq, kernel_prec):
         w = wd.cpu().numpy()
     tol = 1e-2 if kernel_prec else 1e-3 if prec == "bf16x3" else 1e-4
     assert np.linalg.norm(w - wref) < tol * np.linalg.norm(wref)
+
+
+@pytest.mark.parametrize("prec,nat,kernel_prec", [("fp64", 24, 0), ("fp16x3", 33, 0), ("fp16x3", 33, 1), ("bf16x3", 24, 0),
+                                                  ("tf32x3", 65, 0), ("fp16x3", 353, 0)])
+def test_response_is_linear_in_the_probe(X, prec, nat, kernel_prec):
+    # w is linear in v and v has no preferred size: a factor 2^k of the probe is a factor 2^k of every number
+    # of the chain, so w changes by exactly that factor (two- and three-launch chains, split and single products)
+    import torch
+    s = synth.make_system(nat, 27, **({"L": 7.0} if nat == 24 else {}))
+    p = X.default_params(mix_alpha=ALPHA_MIX, kernel_c=1 - 1 / ALPHA_MIX, prec=prec, mu_tol=1e-3, kernel_prec=kernel_prec)
+    rng = np.random.default_rng(nat)
+    n = rng.normal(scale=0.01, size=nat)
+    n -= n.mean()
+    v = rng.normal(size=nat)
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, n)
+        ctx.build_H(0)
+        ctx.density(0)
+        w = {}
+        for k in (0, -60, -83, -300, 40, 66, 300):
+            vd = torch.tensor(np.ldexp(v, k), dtype=torch.float64, device="cuda")
+            wd = torch.zeros_like(vd)
+            ctx.response(0, vd.data_ptr(), wd.data_ptr())
+            torch.cuda.synchronize()
+            w[k] = np.ldexp(wd.cpu().numpy(), -k)
+        zero = torch.zeros(nat, dtype=torch.float64, device="cuda")
+        wd = torch.ones_like(zero)
+        ctx.response(0, zero.data_ptr(), wd.data_ptr())
+        torch.cuda.synchronize()
+    assert np.all(np.isfinite(w[0])) and np.max(np.abs(w[0])) > 0.1
+    for k in w:
+        assert np.array_equal(w[k], w[0]), k
+    assert np.all(wd.cpu().numpy() == 0.0)

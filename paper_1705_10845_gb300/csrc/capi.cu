@@ -645,8 +645,7 @@ xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
     const size_t per_slot = chain_slot_bytes(S.np, ctx->p.prec) + per_vec * sizeof(double);
-    int G = (int)std::min<size_t>(64, std::max<size_t>(1, free_b / 4 / per_slot));
-    G = std::min(G, S.nat);
+    const int G = probe_parts(S.nat, (int)std::min<size_t>(kMaxSlots, std::max<size_t>(1, free_b / 4 / per_slot))).size;
     S.slots.resize(G);
     for (int j = 0; j < G; ++j)
       if (alloc_chain_slot(S.slots[j], S.mats, st) != cudaSuccess) {
@@ -655,9 +654,8 @@ xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
       }
     CKS(dalloc(ctx, &S.slot_vec, per_vec * G));
   }
-  // parts of one size: 96 probes run as 48 + 48 and not as 64 + 32, which is one wave of tiles less
-  const int parts = (S.nat + (int)S.slots.size() - 1) / (int)S.slots.size();
-  const int G = (S.nat + parts - 1) / parts;
+  const ProbeParts parts = probe_parts(S.nat, (int)S.slots.size());
+  const int G = parts.size;
   for (int I0 = 0; I0 < S.nat; I0 += G) {
     const int g = std::min(G, S.nat - I0);
     std::vector<ChainJob> cj(g);
@@ -676,7 +674,7 @@ xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
       cj[j].dvec = p.dvec;
       cj[j].N = S.N;
       cj[j].out_diag = p.d1;
-      cj[j].side = G;
+      cj[j].side = parts.side;
       cj[j].stats = S.stats;
     }
     CK(launch_probe_potential(st, ctx->p.coulomb_k, pj));

@@ -245,6 +245,22 @@ class PlanCache {
   std::vector<E> v_;   // at most 16 x 60 entries
 };
 
+// The unit probes of the exact kernel in parts of one size that run side by side: 96 probes on 64 slots as
+// 48 + 48 and not as 64 + 32, which is one wave of tiles less.  side is the size of a part when memory sets no
+// limit: the form of a chain level (and with it the rounding) is chosen by it, so that K does not
+// depend on how much memory was free when the slots were made.
+constexpr int kMaxSlots = 64;
+struct ProbeParts {
+  int size, side;
+};
+inline ProbeParts probe_parts(int nat, int slots) {
+  auto even = [nat](int s) {
+    const int parts = (nat + s - 1) / s;
+    return (nat + parts - 1) / parts;
+  };
+  return {even(std::max(1, std::min(slots, nat))), even(std::min(nat, kMaxSlots))};
+}
+
 // The whole expansion: level 0 on |t| <= t0max, then t <- 2 t / (1 + t^2).
 inline void plan_expansion(PlanCache& cache, double t0max, int n, double tol, std::vector<LevelPlan>& out) {
   out.resize(n);

@@ -104,7 +104,7 @@ struct ChainJob {
   int N = 0;
   double* out_diag = nullptr;
   double* stats = nullptr;
-  int side = 1;   // probes of one system side by side in its group
+  int side = 1;   // probes of one system side by side in its group (memory permitting): picks the chain's form
 };
 
 class Engine {

@@ -457,3 +457,34 @@ def test_response_is_linear_in_the_probe(X, prec, nat, kernel_prec):
     for k in w:
         assert np.array_equal(w[k], w[0]), k
     assert np.all(wd.cpu().numpy() == 0.0)
+
+
+def hold_all_but(nbytes):
+    """A device block that leaves about nbytes of device memory free."""
+    import torch
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    return torch.empty(free - nbytes, dtype=torch.uint8, device="cuda")
+
+
+@pytest.mark.parametrize("nat,left", [(33, 200 << 20), (96, 300 << 20)])
+def test_exact_kernel_does_not_depend_on_free_memory(X, nat, left):
+    # how many probes run side by side follows the free memory; the arithmetic of a probe must not.  33 atoms
+    # (4 tiles each) sit where the form of a chain changes with the number of probes
+    import torch
+    s = synth.make_system(nat, 12)
+    p = X.default_params(mix_alpha=ALPHA_MIX, kernel_c=1 - 1 / ALPHA_MIX, prec="fp16x3", mu_tol=1e-3, kernel_mode=1)
+    K = []
+    for little in (False, True):
+        with X.Context(p, [sysdict(s)]) as ctx:
+            ctx.build_H(0)
+            ctx.density(0)
+            held = hold_all_but(left) if little else None
+            try:
+                ctx.kernel_exact(0)
+                K.append(ctx.get(0, X.KMAT))
+            finally:
+                del held
+                torch.cuda.empty_cache()
+    assert np.array_equal(K[0], K[1])

@@ -69,3 +69,35 @@ def test_planned_corrections_reach_the_tolerance(tmp_path):
         assert int(products) <= n * (6 if tol > 1e-12 else 8), (tol, t0, n)
         # spectra up to 1 - s = 1e-6 still end
         assert float(zl) <= tol or float(t0) > 0.99, (tol, t0, n)
+
+
+PARTS = r'''
+#include "plan.h"
+#include <cstdio>
+int main() {
+  for (int nat = 1; nat <= 700; ++nat)
+    for (int slots = 1; slots <= 64; ++slots) {
+      const xl::ProbeParts p = xl::probe_parts(nat, slots), again = xl::probe_parts(nat, p.size);
+      std::printf("%d %d %d %d %d %d\n", nat, slots, p.size, p.side, again.size, again.side);
+    }
+}
+'''
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
+def test_probe_parts_of_the_exact_kernel(tmp_path):
+    src = tmp_path / "parts.cpp"
+    src.write_text(PARTS)
+    exe = tmp_path / "parts"
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I" + os.path.join(ROOT, "paper_1705_10845_gb300", "csrc"), str(src),
+                    "-o", str(exe)], check=True)
+    side = {}
+    for line in subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.splitlines():
+        nat, slots, size, s, size2, s2 = map(int, line.split())
+        assert 1 <= size <= min(slots, nat)
+        parts = -(-nat // size)
+        assert parts == -(-nat // min(slots, nat))   # no more parts than the slots ask for
+        assert (size2, s2) == (size, s)              # the slots of one part are all that is needed
+        # what picks the arithmetic is a function of the atoms alone
+        assert side.setdefault(nat, s) == s
+        assert s == (size if slots == 64 else s)

@@ -634,9 +634,18 @@ xlbomd_status response(xlbomd_ctx* ctx, Sys& S, const double* v, double* w) {
   return XLBOMD_OK;
 }
 
+void free_slots(Sys& S) {
+  for (MatSet& m : S.slots) free_chain_slot(m);
+  S.slots.clear();
+  if (S.slot_vec) cudaFree(S.slot_vec);
+  S.slot_vec = nullptr;
+}
+
 // Columns of J - I for the exact kernel with the unit-probe responses run side by side: up
 // to 64 probes at a time, each in its own chain slot, every chain product one grouped launch
 // over the probes.  The number of slots is bounded by a quarter of the free device memory.
+// All slots of a part and their vectors are there or none is: a later call may come after a failed one
+// (xlbomd_clear_error), and it must find no slot without its matrices.
 xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
   cudaStream_t st = ctx->stream;
   const double sc = beta_of(ctx->p) / std::ldexp(1.0, ctx->p.n_sq + 1);
@@ -646,13 +655,17 @@ xlbomd_status exact_columns_grouped(xlbomd_ctx* ctx, Sys& S) {
     CK(cudaMemGetInfo(&free_b, &total_b));
     const size_t per_slot = chain_slot_bytes(S.np, ctx->p.prec) + per_vec * sizeof(double);
     const int G = probe_parts(S.nat, (int)std::min<size_t>(kMaxSlots, std::max<size_t>(1, free_b / 4 / per_slot))).size;
-    S.slots.resize(G);
-    for (int j = 0; j < G; ++j)
-      if (alloc_chain_slot(S.slots[j], S.mats, st) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(ctx, XLBOMD_ERR_OOM, "exact kernel: chain slot allocation failed");
-      }
-    CKS(dalloc(ctx, &S.slot_vec, per_vec * G));
+    S.slots.reserve(G);
+    bool ok = true;
+    for (int j = 0; j < G && ok; ++j) {
+      S.slots.emplace_back();
+      ok = alloc_chain_slot(S.slots.back(), S.mats, st) == cudaSuccess;
+    }
+    if (!ok || dalloc(ctx, &S.slot_vec, per_vec * G) != XLBOMD_OK) {
+      cudaGetLastError();
+      free_slots(S);
+      return fail(ctx, XLBOMD_ERR_OOM, "exact kernel: chain slot allocation failed");
+    }
   }
   const ProbeParts parts = probe_parts(S.nat, (int)S.slots.size());
   const int G = parts.size;
@@ -1166,10 +1179,7 @@ void free_sys(Sys& S) {
   for (auto& g : S.graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   S.graphs.clear();
-  for (MatSet& m : S.slots) free_chain_slot(m);
-  S.slots.clear();
-  if (S.slot_vec) cudaFree(S.slot_vec);
-  S.slot_vec = nullptr;
+  free_slots(S);
   free_matset(S.mats);
 }
 

@@ -1247,30 +1247,26 @@ cudaError_t alloc_matset_split(MatSet& m, cudaStream_t s) {
 }
 
 // A chain slot: a view of a system's expansion matrices (T_k, W_k shared) with its own
-// response-chain matrices (A1, M, T1 twice, T_mu) and their scalars, so that several probes of
-// one system can run their chains side by side (grouped launches).
+// response-chain matrices (A1, M, T1 twice) and their scalars, so that several probes of
+// one system can run their chains side by side (grouped launches).  After a failure free_chain_slot
+// gives back what the slot got: nothing of the base's is left in what it frees.
 cudaError_t alloc_chain_slot(MatSet& slot, const MatSet& base, cudaStream_t s) {
   slot = base;
   for (double*& p : slot.e64) p = nullptr;
   slot.ent = EntropyWork();
   const int np = base.np, esz = operand_bytes(base.prec);
   slot.chain_scales = nullptr;
+  for (SplitMat* x : {&slot.sA1, &slot.sMt, &slot.sT1a, &slot.sT1b, &slot.sTmu}) *x = SplitMat();
   RET(cudaMalloc((void**)&slot.chain_scales, sizeof(float) * 3 * (size_t)base.n));
-  slot.sA1 = SplitMat();
-  slot.sMt = SplitMat();
-  slot.sT1a = SplitMat();
-  slot.sT1b = SplitMat();
-  slot.sTmu = SplitMat();
   RET(alloc_split(slot.sA1, np, esz, base.scales, kF, s));
   RET(alloc_split(slot.sMt, np, esz, base.scales, kD | kF, s));
   RET(alloc_split(slot.sT1a, np, esz, base.scales, kD | kF, s));
   RET(alloc_split(slot.sT1b, np, esz, base.scales, kD | kF, s));
-  RET(alloc_split(slot.sTmu, np, esz, base.scales, kD, s));
   return cudaSuccess;
 }
 
 void free_chain_slot(MatSet& slot) {
-  SplitMat* w[] = {&slot.sA1, &slot.sMt, &slot.sT1a, &slot.sT1b, &slot.sTmu};
+  SplitMat* w[] = {&slot.sA1, &slot.sMt, &slot.sT1a, &slot.sT1b};
   for (SplitMat* x : w) free_split(*x);
   if (slot.chain_scales) cudaFree(slot.chain_scales);
   slot.chain_scales = nullptr;
@@ -1280,7 +1276,7 @@ void free_chain_slot(MatSet& slot) {
 
 // bytes of one chain slot of size np
 size_t chain_slot_bytes(int np, int prec) {
-  return (size_t)np * np * (8 + 3 * 16 + 12 + 5 * 2 * (operand_bytes(prec) - 2));
+  return (size_t)np * np * (8 + 3 * 16 + 4 * 2 * (operand_bytes(prec) - 2));
 }
 
 void free_matset_split(MatSet& m) {

@@ -488,3 +488,29 @@ def test_exact_kernel_does_not_depend_on_free_memory(X, nat, left):
                 del held
                 torch.cuda.empty_cache()
     assert np.array_equal(K[0], K[1])
+
+
+def test_exact_kernel_after_a_failed_allocation(X):
+    # one chain slot of 200 atoms (896 padded orbitals, 45 MB) does not fit: ERR_OOM, nothing half-made is kept, and with the memory
+    # back the same context gives the kernel that a fresh one gives
+    import torch
+    s = synth.make_system(200, 13)
+    p = X.default_params(mix_alpha=ALPHA_MIX, kernel_c=1 - 1 / ALPHA_MIX, prec="fp16x3", mu_tol=1e-3, kernel_mode=1)
+    K = []
+    for fail in (False, True):
+        with X.Context(p, [sysdict(s)]) as ctx:
+            ctx.build_H(0)
+            ctx.density(0)
+            if fail:
+                held = hold_all_but(24 << 20)
+                try:
+                    with pytest.raises(X.XlbomdError) as e:
+                        ctx.kernel_exact(0)
+                    assert e.value.status == -2
+                finally:
+                    del held
+                    torch.cuda.empty_cache()
+                assert ctx._lib.xlbomd_clear_error(ctx.h) == 0
+            ctx.kernel_exact(0)
+            K.append(ctx.get(0, X.KMAT))
+    assert np.array_equal(K[0], K[1])

@@ -4,6 +4,8 @@ The product engine is checked against the FP64 product; the density, charges,
 forces and kernel against the oracle.  Tolerances of the mixed forms: charges
 1e-5 e, forces 1e-4 eV/A.
 """
+import os
+
 import numpy as np
 import pytest
 
@@ -514,3 +516,70 @@ def test_exact_kernel_after_a_failed_allocation(X):
             ctx.kernel_exact(0)
             K.append(ctx.get(0, X.KMAT))
     assert np.array_equal(K[0], K[1])
+
+
+@pytest.mark.parametrize("prec", ["fp16x3", "tf32x3"])
+def test_entropy_does_not_count_padding(X, prec, tmp_path):
+    # 33 atoms: the log-determinants run over 192 rows, 60 of them padding, which must be rows of the identity.
+    # What the planned corrections leave of an inverse (below 1e-8, but times up to 2^13) is a function of the
+    # eigenvalue; it is computed here for the eigenvalues of the system and for the padding's zero, and
+    # the entropy has to be off by the former alone, to within half of the latter (14 squarings: below that
+    # the padding's part is no larger than what the error of D puts on the entropy, some 1e-5 eV)
+    import shutil
+    import subprocess
+    n_sq = 14
+    if shutil.which("g++") is None:
+        pytest.skip("no host compiler")
+    s = synth.make_system(33, 27)
+    p = X.default_params(mix_alpha=ALPHA_MIX, kernel_c=1 - 1 / ALPHA_MIX, prec=prec, mu_tol=1e-3, n_sq=n_sq)
+    m = O.Model(Te=p.Te, n_sq=p.n_sq)
+    n = np.zeros(33)
+    ref = O.evaluate(s.R, s.L, s.Z, n, m, None, with_kernel=False, with_forces=False)
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, n)
+        ctx.set(0, X.MU, [ref.dens.mu])
+        ctx.build_H(0)
+        ctx.density(0)
+        ctx.energy(0)
+        S = ctx.get(0, X.ENERGY)[3]
+    radius = np.abs(ref.H).sum(1) - np.abs(np.diag(ref.H))
+    sc = m.beta / 2.0 ** (n_sq + 1)
+    t0 = sc * max((np.diag(ref.H) + radius).max() - ref.dens.mu, ref.dens.mu - (np.diag(ref.H) - radius).min())
+    src = tmp_path / "left.cpp"
+    src.write_text(r"""
+#include "plan.h"
+#include <cstdio>
+#include <cstdlib>
+using namespace xl;
+int main(int argc, char** argv) {   // t0, n, then eigenvalues of T_0: sum_k 2^(n-1-k) ln(1 - R_k) of each
+  const int n = std::atoi(argv[2]);
+  PlanCache cache;
+  std::vector<LevelPlan> p;
+  plan_expansion(cache, std::atof(argv[1]), n, 1e-8, p);
+  for (int i = 3; i < argc; ++i) {
+    double t = std::atof(argv[i]), w1 = 0.0, s1 = 0.0, sum = 0.0;
+    for (int k = 0; k < n; ++k) {
+      const double s = t * t, W0 = p[k].g[0] + p[k].g[1] * w1 + p[k].g[2] * s + p[k].g[3] * s1;
+      double R = 1.0 - (1.0 + s) * (1.0 - W0);
+      for (int r = 0; r < p[k].inv.n; ++r) R = std::pow(R, p[k].inv.order[r]);
+      sum += std::ldexp(std::log1p(-R), n - 1 - k);
+      s1 = s;
+      w1 = 1.0 - (1.0 - R) / (1.0 + s);
+      t = 2.0 * t * (1.0 - w1);
+    }
+    std::printf("%.17g\n", sum);
+  }
+}
+""")
+    exe = tmp_path / "left"
+    csrc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1705_10845_gb300", "csrc")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I" + csrc, str(src), "-o", str(exe)], check=True)
+    t = [repr(float(x)) for x in sc * (ref.dens.mu - ref.dens.eps)] + ["0.0"]
+    left = [float(x) for x in subprocess.run([str(exe), repr(float(t0)), str(n_sq)] + t, capture_output=True, text=True,
+                                             check=True).stdout.split()]
+    unit = 2.0 * 8.617333262e-5 * p.Te   # the energy part is -2 kB Te S, S = -sum ln(1 - f) - ..
+    own, pad = unit * sum(left[:-1]), unit * 60 * left[-1]
+    off = S - ref.parts["entropy"]
+    print("entropy off by", off, "corrections of the spectrum", own, "of the padding", pad)
+    assert abs(pad) > 1e-4
+    assert abs(off - own) < 0.5 * abs(pad)

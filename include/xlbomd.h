@@ -263,7 +263,10 @@ xlbomd_status xlbomd_kernel_exact(xlbomd_ctx* ctx, int sys);
  * (Eq. ShadowH1: kinetic energy + Omega), written to XLBOMD_ENERGY as
  * [Omega, 2 Tr[D H0], 1/2 sum (2q - n) gamma n, -2 kB Te S, kinetic, total,
  * repulsion].  Requires xlbomd_density on the same state; synchronises the
- * stream.  Errors: ERR_ARG (no density), ERR_CUDA. */
+ * stream.  The work area of the entropy (up to 2 GB, less where less is free; six FP64
+ * matrices beside it in split precisions) is made by the first call, serves every system of
+ * the context and grows to the largest.  Errors: ERR_ARG (no density), ERR_OOM (the split
+ * precisions' matrices do not fit), ERR_CUDA. */
 xlbomd_status xlbomd_energy(xlbomd_ctx* ctx, int sys);
 
 /* a1-a10 for every system, nsteps times (Eqs. Integration, VRL_Damp).  The

@@ -807,8 +807,13 @@ xlbomd_status energy(xlbomd_ctx* ctx, Sys& S) {
   }
   CK(launch_frob_dot(st, S.N, S.np, S.Dm, S.H0, S.work, S.energy + 0));
   CK(launch_energy_vec(st, S.nat, S.q, S.nh, S.pot, S.V, S.mass, S.energy + 1));
-  CK(ctx->eng->entropy(st, S.mats, S.N, beta_of(ctx->p), ctx->p.n_sq, S.mu, S.dmu_last, S.Dm, S.H, S.work,
-                       S.energy + 3));
+  const cudaError_t ee = ctx->eng->entropy(st, S.mats, S.N, beta_of(ctx->p), ctx->p.n_sq, S.mu, S.dmu_last, S.Dm, S.H,
+                                           S.work, S.energy + 3);
+  if (ee == cudaErrorMemoryAllocation) {
+    cudaGetLastError();   // reported here; the next launch is not to find it
+    return fail(ctx, XLBOMD_ERR_OOM, "energy: work matrices do not fit");
+  }
+  CK(ee);
   CKS(sync_read(ctx, S.energy, 5));
   const double band = 2.0 * ctx->pinned[0], coul = ctx->pinned[1], ke = ctx->pinned[2];
   const double ent = -2.0 * kKB * ctx->p.Te * ctx->pinned[3], rep = ctx->pinned[4];

@@ -171,7 +171,7 @@ class EngineF64 : public Engine {
 
   cudaError_t entropy(cudaStream_t s, MatSet& m, int N, double beta, int n_sq, double mu, double dmu,
                       const double* D, const double* H, double* work, double* out) override {
-    return launch_entropy_f64(s, m, N, beta, n_sq, mu, dmu, D, H, work, out);
+    return launch_entropy_f64(s, m, ent_, N, beta, n_sq, mu, dmu, D, H, work, out);
   }
 };
 
@@ -212,7 +212,6 @@ void free_matset(MatSet& m) {
     if (*p) cudaFree(*p);
     *p = nullptr;
   }
-  m.ent.release();
   free_matset_split(m);
 }
 

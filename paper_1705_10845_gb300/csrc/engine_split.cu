@@ -431,6 +431,7 @@ class EngineSplit : public Engine {
   ~EngineSplit() override {
     for (auto& kv : tiles_) cudaFree(kv.second.first);
     if (err_) cudaFree(err_);
+    free_e64();
     tc_group_cache_free(group_cache_);
   }
 
@@ -1150,9 +1151,19 @@ class EngineSplit : public Engine {
                       const double*, double* work, double* out) override {
     // FP64 route from the split values: T_0 from its double-float value, Y_k = I - W_k
     const size_t cnt = (size_t)m.np * m.np;
-    for (double*& p : m.e64)
-      if (!p) RET(cudaMalloc((void**)&p, cnt * sizeof(double)));
-    double* T0 = m.e64[5];
+    if (cnt > e64_count_) {
+      free_e64();
+      for (double*& p : e64_) {
+        const cudaError_t e = cudaMalloc((void**)&p, cnt * sizeof(double));
+        if (e != cudaSuccess) {
+          p = nullptr;
+          free_e64();
+          return e;
+        }
+      }
+      e64_count_ = cnt;
+    }
+    double* T0 = e64_[5];
     df_to_f64_kernel<<<nblk(cnt), 256, 0, s>>>(cnt, m.sT[0].d, T0);
     note_launch();
     RET(cudaGetLastError());
@@ -1166,13 +1177,23 @@ class EngineSplit : public Engine {
     const double t = m.t0max;
     while (nterms < 6 && std::ldexp(1.0, n_sq + 1) * std::pow(t, 2 * nterms + 1) / (2 * nterms + 1) * N > 1e-10)
       ++nterms;
-    return entropy_fp64(s, N, m.np, m.n, n_sq, T0, load_Y, m.ent, m.e64[0], m.e64[1], m.e64[2], m.e64[3],
-                        m.e64[4], nterms, D, work, out);
+    return entropy_fp64(s, N, m.np, m.n, n_sq, T0, load_Y, ent_, e64_[0], e64_[1], e64_[2], e64_[3],
+                        e64_[4], nterms, D, work, out);
   }
 
   int* err_ = nullptr;
 
  private:
+  void free_e64() {
+    for (double*& p : e64_) {
+      if (p) cudaFree(p);
+      p = nullptr;
+    }
+    e64_count_ = 0;
+  }
+
+  double* e64_[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};   // FP64 matrices of the entropy (first use)
+  size_t e64_count_ = 0;                                                      // elements of each: the largest system's
   int fmt_;   // operand format: 0 FP16, 1 BF16, 2 TF32
   int probe_nseg_ = 3;
   int mu_nseg_ = 3;
@@ -1254,8 +1275,6 @@ cudaError_t alloc_matset_split(MatSet& m, cudaStream_t s) {
 // gives back what the slot got: nothing of the base's is left in what it frees.
 cudaError_t alloc_chain_slot(MatSet& slot, const MatSet& base, cudaStream_t s) {
   slot = base;
-  for (double*& p : slot.e64) p = nullptr;
-  slot.ent = EntropyWork();
   const int np = base.np, esz = operand_bytes(base.prec);
   slot.chain_scales = nullptr;
   for (SplitMat* x : {&slot.sA1, &slot.sMt, &slot.sT1a, &slot.sT1b, &slot.sTmu}) *x = SplitMat();
@@ -1290,10 +1309,6 @@ void free_matset_split(MatSet& m) {
   for (SplitMat* x : w) free_split(*x);
   if (m.scales) cudaFree(m.scales);
   m.scales = m.chain_scales = m.t0_dev = nullptr;
-  for (double*& p : m.e64) {
-    if (p) cudaFree(p);
-    p = nullptr;
-  }
 }
 
 // ---- self-test of the tensor-core product against the FP64 product ----

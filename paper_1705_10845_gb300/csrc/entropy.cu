@@ -25,7 +25,7 @@ namespace {
     if (e_ != cudaSuccess) return e_; \
   } while (0)
 
-constexpr int CB = 64;
+constexpr int CB = EntropyWork::kPanel;
 
 // Diagonal block (kb, kb) of matrix blockIdx.x: A = L D L^T (L unit lower); part[..][kb / CB] = sum ln d (NaN for
 // a non-positive pivot) and Li = D^-1/2 L^-1, for which A^-1 = Li^T Li.  In place: at step j column j
@@ -132,52 +132,37 @@ cudaError_t logdet_spd(cudaStream_t s, const EntropyWork& w, int m, int np, int 
   const size_t cnt = (size_t)np * np;
   const int npart = m / CB;
   for (int kb = 0; kb < m; kb += CB) {
-    chol_panel_kernel<<<nb, 256, 0, s>>>(w.mats(), cnt, np, kb, w.li(np), w.part(np), npart);
+    chol_panel_kernel<<<nb, 256, 0, s>>>(w.mats, cnt, np, kb, w.li, w.part, npart);
     note_launch();
     RET(cudaGetLastError());
     const int rest = m - kb - CB;
     if (rest > 0) {
       // X = A21 Li^T, A22 -= X X^T
-      double* A21 = w.mats() + (size_t)(kb + CB) * np + kb;
+      double* A21 = w.mats + (size_t)(kb + CB) * np + kb;
       EpiF64 ex;
-      RET(gemm_f64_nt(s, rest, CB, CB, A21, np, w.li(np), CB, w.rows(np), CB, ex, false, nb, cnt, (size_t)CB * CB,
+      RET(gemm_f64_nt(s, rest, CB, CB, A21, np, w.li, CB, w.rows, CB, ex, false, nb, cnt, (size_t)CB * CB,
                       (size_t)np * CB));
       EpiF64 e;
       e.alpha = -1.0;
       e.E = A21 + CB;
       e.lde = np;
       e.beta = 1.0;
-      RET(gemm_f64_nt(s, rest, rest, CB, w.rows(np), CB, w.rows(np), CB, A21 + CB, np, e, true, nb, (size_t)np * CB,
+      RET(gemm_f64_nt(s, rest, rest, CB, w.rows, CB, w.rows, CB, A21 + CB, np, e, true, nb, (size_t)np * CB,
                       (size_t)np * CB, cnt, cnt));
     }
   }
-  chol_sum_kernel<<<nb, 128, 0, s>>>(npart, w.part(np), out);
+  chol_sum_kernel<<<nb, 128, 0, s>>>(npart, w.part, out);
   note_launch();
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t EntropyWork::reserve(int np, int nmat) {
-  if (buf) return cudaSuccess;
-  const size_t per = sizeof(double) * ((size_t)np * np + (size_t)np * CB + CB * CB + np / CB);
-  cap = (int)std::max<size_t>(1, std::min<size_t>((size_t)nmat, ((size_t)2 << 30) / per));
-  return cudaMalloc((void**)&buf, per * cap);
-}
-double* EntropyWork::mats() const { return buf; }
-double* EntropyWork::rows(int np) const { return buf + (size_t)np * np * cap; }
-double* EntropyWork::li(int np) const { return rows(np) + (size_t)np * CB * cap; }
-double* EntropyWork::part(int np) const { return li(np) + (size_t)CB * CB * cap; }
-void EntropyWork::release() {
-  if (buf) cudaFree(buf);
-  buf = nullptr;
-}
-
 // Entropy from FP64 inputs.  T0: FP64 T_0; load_Y(k, dst) writes Y_k as an
 // FP64 matrix into dst; S, Q, Yw, A1, Mt: FP64 work matrices (np x np);
 // nterms: terms j = 0..nterms-1 of the artanh series.
 cudaError_t entropy_fp64(cudaStream_t s, int N, int np, int n, int n_sq, const double* T0,
-                         const std::function<cudaError_t(int, double*)>& load_Y, EntropyWork& ew, double* S, double* Q,
+                         const std::function<cudaError_t(int, double*)>& load_Y, EntropyWork& area, double* S, double* Q,
                          double* Yw, double* A1, double* Mt, int nterms, const double* D, double* work,
                          double* out) {
   if (n + 1 > 42 || nterms < 1 || nterms > 6) return cudaErrorInvalidValue;
@@ -188,11 +173,19 @@ cudaError_t entropy_fp64(cudaStream_t s, int N, int np, int n, int n_sq, const d
   const size_t count = (size_t)np * np;
   const int mc = (N + CB - 1) / CB * CB, m = (N + 15) / 16 * 16;   // padding does not change what follows
   // logdet(I - T_0), then logdet(Y_k)
-  RET(ew.reserve(np, n + 1));
+  area.reserve(np, n + 1,
+               [](size_t bytes) -> void* {
+                 void* p = nullptr;
+                 if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+                 cudaGetLastError();   // a smaller area is asked for next
+                 return nullptr;
+               },
+               [](void* p) { cudaFree(p); });
+  const EntropyWork ew = area.cap > 0 ? area : EntropyWork::on(S, Q, np);
   for (int k0 = 0; k0 <= n; k0 += ew.cap) {
     const int nb = std::min(ew.cap, n + 1 - k0);
     for (int b = 0; b < nb; ++b) {
-      double* dst = ew.mats() + count * b;
+      double* dst = ew.mats + count * b;
       if (k0 + b == 0) {
         ident_minus_f64_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(count, np, T0, dst);
         note_launch();
@@ -237,7 +230,7 @@ cudaError_t entropy_fp64(cudaStream_t s, int N, int np, int n, int n_sq, const d
   return cudaGetLastError();
 }
 
-cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, int N, double beta, int n_sq, double mu, double dmu,
+cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, EntropyWork& area, int N, double beta, int n_sq, double mu, double dmu,
                                const double* D, const double* H, double* work, double* out) {
   (void)beta;
   (void)mu;
@@ -249,7 +242,7 @@ cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, int N, double beta, in
     note_launch();
     return cudaGetLastError();
   };
-  return entropy_fp64(s, N, m.np, m.n, n_sq, m.T[0], load_Y, m.ent, m.S, m.Q, m.Yw, m.A1, m.Mt, 6, D, work, out);
+  return entropy_fp64(s, N, m.np, m.n, n_sq, m.T[0], load_Y, area, m.S, m.Q, m.Yw, m.A1, m.Mt, 6, D, work, out);
 }
 
 }  // namespace xl

@@ -9,6 +9,7 @@
 #include <functional>
 #include <vector>
 
+#include "entropy_work.h"
 #include "internal.h"
 #include "plan.h"
 
@@ -41,19 +42,6 @@ struct SplitMat {
   const float* scale = nullptr;   // device scalar, one of the MatSet's scales
 };
 
-// Work area of the entropy's log-determinants (allocated on first use): cap matrices np x np, and per
-// matrix the rows below a panel, the panel's inverse factor and the panels' parts.
-struct EntropyWork {
-  double* buf = nullptr;
-  int cap = 0;
-  cudaError_t reserve(int np, int nmat);
-  void release();
-  double* mats() const;
-  double* rows(int np) const;
-  double* li(int np) const;
-  double* part(int np) const;
-};
-
 struct MatSet {
   int prec = 0, np = 0, n = 0;
   // FP64 engine
@@ -70,9 +58,6 @@ struct MatSet {
   float* chain_scales = nullptr;   // the chain part (a chain slot has its own)
   float* t0_dev = nullptr;
   double t0max = 0.0;        // spectral bound |T_0| of the last expansion
-  // FP64 work matrices of the split engine's entropy (allocated on first use)
-  double* e64[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  EntropyWork ent;
 };
 
 cudaError_t alloc_matset(MatSet& m, int prec, int np, int n, cudaStream_t s);
@@ -111,7 +96,9 @@ class Engine {
  public:
   virtual ~Engine() {
     for (auto e : ev_) cudaEventDestroy(e);
+    ent_.free_all([](void* p) { cudaFree(p); });
   }
+  EntropyWork ent_;   // of every system's energy
   // Timing of the matrix products with CUDA events on their stream.
   bool prof = false;
   std::vector<cudaEvent_t> ev_;
@@ -225,10 +212,10 @@ int selftest_gemm_group(int n, int prec, int mode, int nprob, double* result);
 
 // FP64 eigenvalue-free entropy (entropy.cu)
 cudaError_t entropy_fp64(cudaStream_t s, int N, int np, int n, int n_sq, const double* T0,
-                         const std::function<cudaError_t(int, double*)>& load_Y, EntropyWork& ew, double* S, double* Q,
+                         const std::function<cudaError_t(int, double*)>& load_Y, EntropyWork& area, double* S, double* Q,
                          double* Yw, double* A1, double* Mt, int nterms, const double* D, double* work,
                          double* out);
-cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, int N, double beta, int n_sq, double mu, double dmu,
+cudaError_t launch_entropy_f64(cudaStream_t s, MatSet& m, EntropyWork& area, int N, double beta, int n_sq, double mu, double dmu,
                                const double* D, const double* H, double* work, double* out);
 
 // misc FP64 launchers (foe_kernels.cu)

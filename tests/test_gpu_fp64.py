@@ -458,3 +458,58 @@ def test_forces_after_a_non_finite_move_are_not_finite(X, prec):
         assert not np.isfinite(ctx.get(0, X.F)[5]).any()
         ctx.energy(0)
         assert np.isnan(ctx.get(0, X.ENERGY)[6])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp16x3"])
+def test_energy_work_area_is_shared_by_the_systems(X, prec):
+    # eight systems of 512 padded orbitals: the first energy makes the work area, the others use it.  A context
+    # of uneven sizes gives each system the energies of its own context
+    import torch
+    systems = [sysdict(synth.make_system(100 + i, 40 + i)) for i in range(8)]
+    p = model_params(X, prec=prec, mu_tol=1e-9 if prec == "fp64" else 1e-3)
+    with X.Context(p, systems) as ctx:
+        free = []
+        for i in range(8):
+            ctx.build_H(i)
+            ctx.density(i)
+            ctx.energy(i)
+            torch.cuda.synchronize()
+            free.append(torch.cuda.mem_get_info()[0])
+    assert len(set(free)) == 1, free
+    mixed = [sysdict(synth.make_system(nat, 60 + nat)) for nat in (40, 24, 100, 33)]
+    own = []
+    for s in mixed:
+        with X.Context(p, [s]) as ctx:
+            ctx.density(0)
+            ctx.energy(0)
+            own.append(ctx.get(0, X.ENERGY))
+    with X.Context(p, mixed) as ctx:
+        for i in range(len(mixed)):
+            ctx.density(i)
+            ctx.energy(i)
+            assert np.array_equal(ctx.get(i, X.ENERGY), own[i]), i
+
+
+def test_energy_with_little_free_memory(X):
+    # FP64, 1024 padded orbitals: the work area for all levels takes 100 MB, for one 9 MB.  With 60, 20 and 4 MB
+    # free the log-determinants run in smaller batches, the last on the engine's own matrices
+    import torch
+    s = sysdict(synth.make_system(230, 9))
+    p = model_params(X, rank_m=0)
+    E = []
+    for left in (None, 60 << 20, 20 << 20, 4 << 20):
+        with X.Context(p, [s]) as ctx:
+            ctx.density(0)
+            held = None
+            if left is not None:
+                torch.cuda.synchronize()
+                torch.cuda.empty_cache()
+                held = torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda")
+            try:
+                ctx.energy(0)
+                E.append(ctx.get(0, X.ENERGY))
+            finally:
+                del held
+                torch.cuda.empty_cache()
+    for e in E[1:]:
+        assert np.max(np.abs(e - E[0])) < 1e-10 * np.max(np.abs(E[0]))

@@ -151,10 +151,10 @@ typedef enum {
   XLBOMD_Q = 0,        /* get: Mulliken charges q[n] (natoms) */
   XLBOMD_N = 1,        /* get/set: n(t) (natoms); set fills the whole history with it */
   XLBOMD_NHIST = 2,    /* get/set: n(t - k dt), k = 0..kmax ((kmax+1) x natoms) */
-  XLBOMD_F = 3,        /* get: forces (natoms x 3, eV/A) */
+  XLBOMD_F = 3,        /* get/set: forces (natoms x 3, eV/A) */
   XLBOMD_R = 4,        /* get/set: positions (natoms x 3) */
   XLBOMD_V = 5,        /* get/set: velocities (natoms x 3) */
-  XLBOMD_KR = 6,       /* get: K (q - n) (natoms) */
+  XLBOMD_KR = 6,       /* get/set: K (q - n) (natoms) */
   XLBOMD_RES = 7,      /* get: residual q - n (natoms) */
   XLBOMD_ENERGY = 8,   /* get: [Omega, band, coulomb, entropy, kinetic, total, repulsion] (7);
                           Omega includes the repulsion */
@@ -284,7 +284,13 @@ xlbomd_status xlbomd_step(xlbomd_ctx* ctx, int nsteps);
 /* Copy a quantity to host memory (synchronises the stream). */
 xlbomd_status xlbomd_get(xlbomd_ctx* ctx, int sys, int what, double* host_out);
 
-/* Overwrite a quantity from host memory (R, V, N, NHIST, MU). */
+/* Overwrite a quantity from host memory (R, V, N, NHIST, MU, F, KR).  A step
+ * begins with the half kick by F and the n update by K r that the context
+ * holds, those of its last density and kernel update: to go on from a state
+ * of another context or an earlier one, set R, V, NHIST, F, KR and MU (or set the
+ * first three and run xlbomd_build_H, xlbomd_density and
+ * xlbomd_kernel_update).  With R, V and NHIST alone the first step takes the F
+ * and K r of the state before. */
 xlbomd_status xlbomd_set(xlbomd_ctx* ctx, int sys, int what, const double* host_in);
 
 /* Sizes: natoms and padded orbital count of system sys. */

@@ -1629,6 +1629,12 @@ xlbomd_status xlbomd_set(xlbomd_ctx* ctx, int sys, int what, const double* host_
       CK(cudaStreamSynchronize(ctx->stream));
       S.have_density = false;
       return XLBOMD_OK;
+    case XLBOMD_F:
+    case XLBOMD_KR:   // what the first half kick and the first n update of a step take
+      CK(cudaMemcpyAsync(what == XLBOMD_F ? S.F : S.Kr, host_in, sizeof(double) * (what == XLBOMD_F ? 3 : 1) * nat,
+                         cudaMemcpyHostToDevice, ctx->stream));
+      CK(cudaStreamSynchronize(ctx->stream));
+      return XLBOMD_OK;
     case XLBOMD_MU:
       S.mu = host_in[0];
       S.mu_valid = true;

@@ -513,3 +513,58 @@ def test_energy_with_little_free_memory(X):
                 torch.cuda.empty_cache()
     for e in E[1:]:
         assert np.max(np.abs(e - E[0])) < 1e-10 * np.max(np.abs(E[0]))
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-9), ("fp16x3", 1e-5)])
+def test_restart_from_host_copies_continues_the_trajectory(X, prec, tol):
+    # the first half kick takes F(t) and the first n update K r(t): with both set beside R, V, the history and
+    # mu a second context goes on where the first one stands.  Its search for mu starts without a
+    # history, so charges agree to the precision of a density (1e-9 e, FP16x3 1e-5 e) and not to the bit
+    s = synth.make_system(24, 1705, L=7.0)
+    p = model_params(X, prec=prec, mu_tol=1e-9 if prec == "fp64" else 1e-3, rep_A=40.0)
+    what = (X.R, X.V, X.NHIST, X.F, X.KR, X.MU)
+    with X.Context(p, [sysdict(s)]) as a, X.Context(p, [sysdict(s)]) as b:
+        a.set(0, X.N, random_n(s.natoms, 5, scale=0.01))
+        a.build_H(0)
+        a.density(0)
+        a.kernel_update(0)
+        a.step(2)
+        kept = {w: a.get(0, w) for w in what}
+        a.step(1)
+        b.build_H(0)
+        b.density(0)
+        b.kernel_update(0)
+        for w in what:
+            b.set(0, w, kept[w])
+        b.step(1)
+        for w in (X.R, X.NHIST):   # functions of what was set alone
+            assert np.array_equal(a.get(0, w), b.get(0, w))
+        assert np.max(np.abs(a.get(0, X.Q) - b.get(0, X.Q))) < tol
+        assert np.max(np.abs(a.get(0, X.F) - b.get(0, X.F))) < 10 * tol
+        assert np.max(np.abs(a.get(0, X.V) - b.get(0, X.V))) < 1e-3 * tol   # half a kick: 1e-4 A/fs per eV/A
+
+
+@pytest.mark.parametrize("prec,nsys,steps", [("fp64", 1, 1), ("fp16x3", 1, 3), ("fp16x3", 3, 2)])
+def test_calls_from_one_state_repeat(X, prec, nsys, steps):
+    # near the exact kernel K r = n - n*, so a step that takes the K r of the call before multiplies the deviation
+    # by -kappa; from a state set whole every call gives the same bits, however many there are
+    p = model_params(X, prec=prec, mu_tol=1e-9 if prec == "fp64" else 1e-3, rep_A=40.0)
+    systems = [sysdict(synth.make_system(24 - i, 1705 + i)) for i in range(nsys)]
+    what = (X.R, X.V, X.NHIST, X.F, X.KR, X.MU)
+    with X.Context(p, systems) as ctx:
+        state = []
+        for i in range(nsys):
+            ctx.set(i, X.N, random_n(systems[i]["natoms"], 6 + i, scale=0.01))
+            ctx.build_H(i)
+            ctx.density(i)
+            ctx.kernel_update(i)
+            state.append({w: ctx.get(i, w) for w in what})
+        first = None
+        for call in range(40):
+            for i in range(nsys):
+                for w in what:
+                    ctx.set(i, w, state[i][w])
+            ctx.step(steps)
+            got = [ctx.get(i, w) for i in range(nsys) for w in what + (X.Q,)]
+            first = first or got
+            assert all(np.array_equal(a, b) for a, b in zip(first, got)), call

@@ -568,3 +568,33 @@ def test_calls_from_one_state_repeat(X, prec, nsys, steps):
             got = [ctx.get(i, w) for i in range(nsys) for w in what + (X.Q,)]
             first = first or got
             assert all(np.array_equal(a, b) for a, b in zip(first, got)), call
+
+
+@pytest.mark.parametrize("prec,tol_f", [("fp64", 1e-8), ("fp16x3", 1e-4)])
+@pytest.mark.parametrize("nat", [24, 300])
+def test_forces_follow_moved_positions(X, prec, tol_f, nat):
+    # atoms moved by set(R) without a new Hamiltonian: D, q and n stay those of the old one, every force term is
+    # taken at the new R.  A uniform shift cannot tell (the Coulomb terms do not change under it); here the
+    # displacements differ, and Coulomb forces of the old R would miss by hundreds of tolerances
+    s = synth.make_system(nat, 29, **({"L": 7.0} if nat == 24 else {}))
+    p = model_params(X, prec=prec, rep_A=40.0, mu_tol=1e-9 if prec == "fp64" else 1e-3)
+    m = oracle_model(p)
+    n = random_n(nat, 30, scale=0.3)
+    ref = O.evaluate(s.R, s.L, s.Z, n, m, None, with_kernel=False, with_forces=False)
+    R2 = s.R + np.random.default_rng(31).normal(scale=0.05, size=(nat, 3))
+    want = O.forces(R2, s.L, m, ref.dens.D, ref.q, n)
+    bare = O.Model(Te=p.Te, n_sq=p.n_sq, rep_A=p.rep_A, rep_rho=p.rep_rho, coulomb_k=0.0)
+    coul = lambda R, F: F - O.forces(R, s.L, bare, ref.dens.D, ref.q, n, np.zeros((nat, nat, 3)))
+    stale = want - coul(R2, want) + coul(s.R, O.forces(s.R, s.L, m, ref.dens.D, ref.q, n))
+    assert np.max(np.abs(stale - want)) > 100 * tol_f
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, n)
+        ctx.set(0, X.MU, [ref.dens.mu])
+        ctx.build_H(0)
+        ctx.set(0, X.R, R2)
+        ctx.density(0)
+        F = ctx.get(0, X.F)
+        ctx.density(0)   # and again, from what the first call left
+        F2 = ctx.get(0, X.F)
+    assert np.max(np.abs(F - want)) < tol_f
+    assert np.max(np.abs(F2 - want)) < tol_f

@@ -808,7 +808,7 @@ __global__ void gj_eliminate_kernel(int n, int k, double* __restrict__ A, double
 
 cudaError_t launch_gauss_jordan(cudaStream_t s, int n, double* A, double* B, double* f, double* flag) {
   if (n < 1 || n > 65535) return cudaErrorInvalidValue;
-  if (gj_smem(n) <= kGjMaxSmem) {   // n <= 456
+  if (gj_smem(n) <= kGjMaxSmem) {   // n <= 463
     RET(cudaFuncSetAttribute(gj_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGjMaxSmem));
     gj_cluster_kernel<<<kGjCtas, kGjThreads, gj_smem(n), s>>>(n, A, B, flag);
     note_launch();

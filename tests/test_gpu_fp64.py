@@ -598,3 +598,26 @@ def test_forces_follow_moved_positions(X, prec, tol_f, nat):
         F2 = ctx.get(0, X.F)
     assert np.max(np.abs(F - want)) < tol_f
     assert np.max(np.abs(F2 - want)) < tol_f
+
+
+def test_exact_kernel_beyond_the_cluster(X):
+    # 470 atoms: the inverse by launches (up to 463 fit the shared memory of a cluster).  K (w - v) = v as above
+    import torch
+    nat = 470
+    s = synth.make_system(nat, 13)
+    p = model_params(X, kernel_mode=1, prec="fp16x3", kernel_prec=1)
+    v = random_n(nat, 17)
+    with X.Context(p, [sysdict(s)]) as ctx:
+        ctx.set(0, X.N, random_n(nat, 18))
+        ctx.build_H(0)
+        ctx.density(0)
+        before = X.binding.launch_count()
+        ctx.kernel_exact(0)
+        assert X.binding.launch_count() - before > 2 * nat   # a search and an elimination per step
+        K = ctx.get(0, X.KMAT)
+        vd = torch.tensor(v, dtype=torch.float64, device="cuda")
+        wd = torch.zeros_like(vd)
+        ctx.response(0, vd.data_ptr(), wd.data_ptr())
+        torch.cuda.synchronize()
+    # single products: the responses, and so J and w, are good to a few 2^-11
+    assert np.linalg.norm(K @ (wd.cpu().numpy() - v) - v) < 1e-1 * np.linalg.norm(v)

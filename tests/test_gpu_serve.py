@@ -69,3 +69,35 @@ def test_lockstep_batch_equals_solo_runs():
                 got = [ctx.get(i, w) for w in (X.Q, X.R, X.NHIST, X.KR, X.F, X.MU)]
                 for a, b in zip(solo[i], got):
                     assert np.array_equal(a, b), (prec, i, float(np.max(np.abs(a - b))))
+
+
+@pytest.mark.parametrize("prec", ["fp16x3", "fp64"])
+def test_lockstep_of_18_with_energies_equals_solo_runs(prec):
+    # more systems than side streams (8) and than the jobs of one list (16), one padded size, with the energy
+    # monitor inside the group: every trajectory and its energies are those of its own run, to the bit
+    import paper_1705_10845_gb300 as X
+    import synth
+    X.build.build()
+    X.load()
+    systems = []
+    for i in range(18):
+        s = synth.make_system(15 + (7 * i) % 18, 100 + i)
+        systems.append(dict(natoms=s.natoms, L=s.L, R=s.R, V=s.V, Z=s.Z, mass=s.mass))
+    fp64 = prec == "fp64"
+    p = X.default_params(rank_m=2, mix_alpha=0.06, kernel_c=1 - 1 / 0.06, prec=prec, scf_mode=1, kernel_auto=1,
+                         scf_tol=1e-9 if fp64 else 1e-5, mu_tol=1e-9 if fp64 else 1e-3, rep_A=40.0, rep_rho=0.3,
+                         kernel_prec=1, mu_prec=1, scf_max_iter=300, energy_every=1)
+    what = (X.Q, X.R, X.NHIST, X.KR, X.F, X.MU, X.ENERGY)
+    solo = []
+    for sd in systems:
+        with X.Context(p, [sd]) as ctx:
+            ctx.scf(0)
+            ctx.step(3)
+            solo.append([ctx.get(0, w) for w in what])
+    with X.Context(p, systems) as ctx:
+        ctx.scf(-1)
+        ctx.step(3)
+        for i in range(len(systems)):
+            for a, w in zip(solo[i], what):
+                b = ctx.get(i, w)
+                assert np.array_equal(a, b), (i, w, float(np.max(np.abs(a - b))))

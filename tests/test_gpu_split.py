@@ -583,3 +583,13 @@ int main(int argc, char** argv) {   // t0, n, then eigenvalues of T_0: sum_k 2^(
     print("entropy off by", off, "corrections of the spectrum", own, "of the padding", pad)
     assert abs(pad) > 1e-4
     assert abs(off - own) < 0.5 * abs(pad)
+
+
+@pytest.mark.parametrize("n,nprob", [(128, 64), (256, 24), (256, 64), (640, 16), (1024, 3)])
+@pytest.mark.parametrize("sym", [0, 1, 2])
+@pytest.mark.parametrize("prec,single", [("fp16x3", False), ("fp16x3", True), ("bf16x3", False), ("tf32x3", False)])
+def test_group_with_other_tiles_than_one_product(X, n, nprob, sym, prec, single):
+    # one product of these sizes takes 32-wide tiles (dense 1024 64-wide), a group 64- or 128-wide ones,
+    # by their waves over the SMs: a lockstep group gives the bits of its systems' own runs only if the width does not matter
+    err, flag = X.binding.selftest_gemm_group(n, prec, sym, single, nprob)
+    assert flag == 0 and err == 0.0

@@ -25,7 +25,9 @@
 // smaller) therefore never share an accumulator.  A pair product (pairs = 2) adds
 // the swapped operands as a second K range, C = A B^T + B A^T.  Every mbarrier
 // wait is bounded: on timeout the kernel records an error code and leaves its
-// loops, and TMEM is always released.
+// loops, waits (again bounded) for the copies and MMAs it has in flight, so that
+// none of them lands in the shared memory or TMEM of the CTA that comes next, and
+// releases TMEM.
 //
 // TF32 operands (fmt = 2, persistent kernel only) are FP32 words whose low 13
 // mantissa bits are zero.  A 128-byte swizzle row then holds 32 elements, and
@@ -45,6 +47,7 @@
 
 #include "operand.cuh"
 #include "precision.h"
+#include "ring.h"
 #include "tc.h"
 
 namespace xl {
@@ -111,6 +114,15 @@ __device__ __forceinline__ bool mbar_wait_fast(uint64_t* bar, uint32_t parity) {
     if (done) return true;
   }
   return false;
+}
+
+// After a wait that gave up: the copies that the ring's producer has in flight (each wait bounded; the first
+// that gives up ends it).
+__device__ __forceinline__ void drain_ring(uint64_t* full, int stages, uint32_t slot, uint32_t ph, bool first) {
+  for (int s = 0; s < stages; ++s) {
+    const int u = ring_last_use(slot, ph, first, s);
+    if (u >= 0 && !mbar_wait(&full[s], (uint32_t)u)) return;
+  }
 }
 
 __device__ __forceinline__ void prefetch_l2(const void* p) {
@@ -652,7 +664,8 @@ __global__ void __launch_bounds__(192, 1)
     if (lane == 0) {
       KSeg q;
       kseg_begin(a, nk, q);
-      for (int kb = 0; kb < total; ++kb, kseg_next(a, nk, q)) {
+      int kb = 0;
+      for (; kb < total; ++kb, kseg_next(a, nk, q)) {
         const int s = kb % STAGES;
         const uint32_t ph = (kb / STAGES) & 1;
         if (kb >= STAGES && !mbar_wait_fast(&empty[s], ph ^ 1)) {
@@ -666,7 +679,10 @@ __global__ void __launch_bounds__(192, 1)
         tma_load_2d(sA + s * A_BYTES, ma, kk, tm * BM, &full[s]);
         tma_load_2d(sB + s * B_BYTES, mb, kk, tn * BN, &full[s]);
       }
-      if (!ok) atomicExch(a.err, 1);
+      if (!ok) {
+        atomicExch(a.err, 1);
+        drain_ring(full, STAGES, kb % STAGES, (kb / STAGES) & 1, kb < STAGES);
+      }
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -827,7 +843,7 @@ struct PCfg {
   static constexpr uint32_t TMEM_COLS = (ONCE ? 4 : 2) * BN;   // ONCE: two accumulators for corrections
   static constexpr int B_BYTES = BN * BK * 2;
   static constexpr int STAGE_TILE = 32 * 33 * 4;
-  static constexpr int SMEM = STG * (A_BYTES + B_BYTES) + NEPI * STAGE_TILE + (2 * STG + 4) * 8 + 16 + 1024;
+  static constexpr int SMEM = STG * (A_BYTES + B_BYTES) + NEPI * STAGE_TILE + (2 * STG + 5) * 8 + 16 + 1024;
 };
 
 // ---- the two single-thread loops of the persistent kernel: 32-bit shared addresses throughout ----
@@ -909,7 +925,8 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
   uint64_t* empty = full + STG;
   uint64_t* acc_full = empty + STG;        // [2]
   uint64_t* acc_free = acc_full + 2;       // [2]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 4);
+  uint64_t* drain = acc_full + 4;          // completion of the last MMAs after a wait that gave up
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -922,6 +939,7 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
     mbar_init(&acc_full[1], 1);
     mbar_init(&acc_free[0], Cfg::NEPI);
     mbar_init(&acc_free[1], Cfg::NEPI);
+    mbar_init(drain, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1004,6 +1022,7 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
           }
         }
       }
+      if (*abort_flag) drain_ring(full, STG, slot, ph, first);
     } else if (warp == 1 && lane == 0) {
       constexpr uint32_t idesc_f16 = instr_desc(BN, 0);
       constexpr uint32_t idesc_bf16 = instr_desc(BN, 1);
@@ -1076,6 +1095,10 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
           atomicExch(a.err, 2);
           *abort_flag = 1;
         }
+      }
+      if (*abort_flag) {
+        bar_commit(smem_u32(drain));
+        mbar_wait(drain, 0);
       }
     }
   } else {
@@ -1351,6 +1374,8 @@ __global__ void __launch_bounds__(192, 1)
           tma_load_2d_pair(sB + s * PB_BYTES, mb, kk, brow, bar);
         }
       }
+      // both CTAs' copies signal the leader's barriers
+      if (leader && *abort_flag) drain_ring(full, PSTAGES, g % PSTAGES, (g / PSTAGES) & 1, g < PSTAGES);
     }
   } else if (warp == 1) {
     if (lane == 0 && leader) {

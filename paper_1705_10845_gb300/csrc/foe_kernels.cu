@@ -230,14 +230,19 @@ __global__ void __launch_bounds__(kVecThreads) probe_expand_kernel(double scale,
   __syncthreads();
   m = __reduce_max_sync(0xffffffffu, top[threadIdx.x & (kVecThreads / 32 - 1)]);
   const int ex = m >> 20;   // biased exponent; 0 and 2047: nothing to scale
-  const int e = (ex == 0 || ex == 2047) ? 0 : min(ex - 1022, 1022);
-  const double down = ldexp(1.0, -e);
-  if (threadIdx.x == 0) J.scal[3] = ldexp(1.0, e);
-  for (int a = threadIdx.x; a < J.np; a += kVecThreads) J.dvec[a] = (a < 4 * J.nat) ? scale * (pot[a >> 2] - pbar) * down : 0.0;
+  const int e = (ex == 0 || ex == 2047) ? 0 : max(-900, min(ex - 1022, 900));
+  const double f = scale * __hiloint2double((1023 - e) << 20, 0);   // scale 2^-e
+  if (threadIdx.x == 0) J.scal[3] = __hiloint2double((1023 + e) << 20, 0);
+  for (int I = threadIdx.x; I < J.nat; I += kVecThreads) {
+    const double x = f * (pot[I] - pbar);
+    for (int a = 4 * I; a < 4 * I + 4; ++a) J.dvec[a] = x;
+  }
+  for (int a = 4 * J.nat + threadIdx.x; a < J.np; a += kVecThreads) J.dvec[a] = 0.0;
 }
 
-// With d1 taken back by 2^e: mu1 = -sum d1 / sum dmu;  w_I = sum_{a in I} (d1_a + mu1 dmu_a)  (one block per job).
-// A unit probe's w - e_u is column u of J - I (row-major nat x nat at Jm), next to a column of the identity at B.
+// mu1 = -sum d1 / sum dmu;  w_I = sum_{a in I} (d1_a + mu1 dmu_a)  (one block per job), for the d1 of the
+// scaled probe; the results are taken back by 2^e (up).  A unit probe's w - e_u is column u of J - I
+// (row-major nat x nat at Jm), next to a column of the identity at B.
 template <int NJ>
 __global__ void __launch_bounds__(kVecThreads) probe_finish_kernel(const __grid_constant__ JobList<ProbeJob, NJ> L) {
   grid_wait();
@@ -247,19 +252,20 @@ __global__ void __launch_bounds__(kVecThreads) probe_finish_kernel(const __grid_
   const double up = J.scal[3];
   double s1 = 0.0, s2 = 0.0;
   for (int a = threadIdx.x; a < J.N; a += kVecThreads) {
-    s1 += d1[a] * up;
+    s1 += d1[a];
     s2 += dmu[a];
   }
   block_sum2(s1, s2, sh);
   const double mu1 = (s2 != 0.0) ? -s1 / s2 : 0.0;
   if (threadIdx.x == 0) {
-    J.scal[0] = s1;
+    J.scal[0] = s1 * up;
     J.scal[1] = s2;
-    J.scal[2] = mu1;
+    J.scal[2] = mu1 * up;
   }
   for (int I = threadIdx.x; I < J.nat; I += kVecThreads) {
     double t = 0.0;
-    for (int a = 4 * I; a < 4 * I + 4; ++a) t += fma(mu1, dmu[a], d1[a] * up);   // d1 up is exact
+    for (int a = 4 * I; a < 4 * I + 4; ++a) t += d1[a] + mu1 * dmu[a];
+    t *= up;
     if (J.w) J.w[I] = t;
     if (J.unit >= 0) {
       const size_t o = (size_t)I * J.nat + J.unit;

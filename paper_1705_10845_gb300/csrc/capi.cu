@@ -475,7 +475,6 @@ xlbomd_status forces(xlbomd_ctx* ctx, Sys& S) {
 // density matrix, charges (and forces) from the final mu pass
 xlbomd_status density_finish(xlbomd_ctx* ctx, Sys& S, const MuSearch& ms, bool with_forces) {
   cudaStream_t st = ctx->stream;
-  const xlbomd_params& p = ctx->p;
   ms.finish(S);
   CK(ctx->eng->density_out(st, S.mats, S.N, ms.dmu, S.dmu_diag, S.ddiag, S.Dm));
   CK(launch_charges(st, S.nat, S.ddiag, S.Z, S.nh, S.q, S.r));

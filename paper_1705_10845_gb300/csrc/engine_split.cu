@@ -1407,8 +1407,8 @@ done:
 }
 
 // Grouped products against single products: nprob seeded operand pairs, each product computed
-// alone and then all of them in one grouped launch (with 128- and 256-wide tiles where n allows
-// both); result = [max |C_group - C_single| over the problems and widths, error flag].
+// alone and then all of them in one grouped launch, twice (each at the tile width that its number of
+// tiles picks); result = [max |C_group - C_single| over the problems, error flag].
 int selftest_gemm_group(int n, int prec, int mode, int nprob, double* result) {
   if (n % 128 || n <= 0 || nprob < 2 || nprob > kMaxGroup || !is_split_prec(prec)) return -1;
   const int esz = operand_bytes(prec);

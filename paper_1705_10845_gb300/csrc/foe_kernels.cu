@@ -597,9 +597,10 @@ namespace {
 // cluster: column j lives in CTA j mod 8, one warp per column.  Per step the warp that holds the pivot
 // column searches it and sends the row exchange, 1/pivot and the factors to all CTAs; every warp then
 // updates its own columns, and the next pivot column goes first, so that its search and the cluster
-// barrier run beside the rest of the update (a CTA has 2 FP64 FMAs a clock: 0.3 us a step at n = 96).  The
-// factors are held three deep: a CTA arrives for step k + 1 when it enters step k, done with k - 1.
-// n = 96 takes 237 us; as a search and an elimination launch per step it took 1340.
+// barrier run beside the rest of the update.  The factors are held three deep: a CTA arrives for step k + 1
+// when it enters step k, done with k - 1.  At n = 96 the update's FP64 work is 0.3 us a step (a CTA has 2
+// FMAs a clock); the 2.5 us a step that were measured (237 us in all; as a search and an elimination
+// launch per step 1340) are the chain of search, division, remote stores and cluster barrier.
 constexpr int kGjCtas = 8, kGjThreads = 512, kGjMaxSmem = 227 * 1024;
 
 __host__ __device__ inline size_t gj_smem(int n) {

@@ -175,16 +175,6 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_
       : "memory");
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
@@ -1191,9 +1181,11 @@ __global__ void __launch_bounds__(PCfg<BN>::THREADS, 1)
 // of the B tile in its own shared memory and rows 128 r .. of the accumulator in its own TMEM.
 // The tensor cores of both SMs read both CTAs' operands, so each SM stages half as many B bytes
 // per flop as the one-SM product: 32 KB per 64-wide K block instead of 48 KB, six ring stages
-// instead of four, a third less shared-memory traffic per flop.  The accumulator modes (single
-// products alternating accumulators, split products with chunked FP32 folds) are those of the
-// one-SM persistent kernel, run by both CTAs' epilogue warps on their own TMEM lanes.
+// instead of four, a third less shared-memory traffic per flop.  Single products alternate
+// accumulators from tile to tile.  Split products start from the corrections and fold 1024-long
+// chunks of hi*hi into them through TMEM, by both CTAs' epilogue warps on their own TMEM lanes: another
+// order of sums than the one-SM kernel's (512-long chunks in registers), so the two agree to the error
+// bound of a product and not to the bit.
 //
 // Roles.  Both CTAs: warp 0 lane 0 loads the CTA's A and B halves of each K block by TMA,
 // signalling the leader CTA's (rank 0) full barrier; warps 2-5 run the epilogue.  Leader only:
@@ -1719,6 +1711,9 @@ int tiles_of(int n, int width, bool sym, const TcTiles& t) {
 // their corrections apart from the rest, so their results differ from the others' in rounding; a size
 // always takes one kind, whatever the number of problems.)  The times of a 128 x w tile relative to
 // w = 128 hardly depend on n: a CTA's K loop is bound by the ring's turn-around, about 2 us at any width.
+// Above 3072 every second padded size (no multiple of 256) takes 128-wide tiles.  That costs little: dense
+// split products in TFLOP/s of 16-bit work, 128-wide n = 3200, 4992, 6272, 8064: 1078, 1297, 1394, 1410;
+// 256-wide 3328, 5120, 6400, 8192: 1014, 1289, 1350, 1461 (fewer and larger tiles, an emptier last wave).
 int pick_width(int n, int nprob, const TcArgs& a, const TcTiles& t) {
   static const int cost[kTcWidths] = {68, 75, 100, 150};
   if (n > kOnceMaxN && n % 256 == 0) return 3;

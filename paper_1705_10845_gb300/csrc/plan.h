@@ -12,8 +12,9 @@
 // steps to 1e-8; with S_k and S_{k-1}, which cost one pass over memory, |R| <= 0.017 and one correction of
 // order 5 (four products) gives 1.4e-9.  Every factor is a function of one matrix, so all products run in
 // symmetric-output mode (half the tiles); the residual Q used to be a dense product.  An expansion of
-// 10 levels takes 25-30 dense-equivalent products instead of 59-64: charges and forces of 4096 atoms in
-// FP16x3 1349 -> 732 ms, of 100 atoms in FP64 254.8 -> 198.1 ms, their errors against 64 bits no larger.
+// 10 levels takes 25-30 dense-equivalent products instead of 59-64 (corrected to 1e-8; 34-40 to the FP64
+// path's 1e-16): charges and forces of 4096 atoms in FP16x3 1349 -> 732 ms, of 100 atoms in FP64 254.8 ->
+// 198.1 ms, their errors against 64 bits no larger.
 #pragma once
 #include <algorithm>
 #include <cmath>

@@ -223,8 +223,8 @@ cudaError_t launch_absmax(cudaStream_t s, int n, const double* x, double* out);
 cudaError_t launch_fill_history(cudaStream_t s, int nat, int kmax, double* nh);
 cudaError_t launch_axpy(cudaStream_t s, int n, double a, const double* x, double* y);
 cudaError_t launch_diag_sum(cudaStream_t s, int n, int np, const double* X, double* out);
-// exact kernel (foe_kernels.cu): B <- (A)^-1 B by Gauss-Jordan with partial pivoting (A row-major n x n, destroyed;
-// f: n doubles of work; *flag set to 1 on a zero or non-finite pivot)
+// exact kernel (foe_kernels.cu): B <- A^-1 by Gauss-Jordan with partial pivoting; B holds the identity on entry (both
+// row-major n x n, A is used up; f: n doubles of work; *flag set to 1 on a zero or non-finite pivot)
 cudaError_t launch_gauss_jordan(cudaStream_t s, int n, double* A, double* B, double* f, double* flag);
 // accumulated rank-1 kernel (foe_kernels.cu), row-major n x n FP64 matrices:
 // M = a I; y = M^T x; v <- v/|v| (flag 1 if |v| > 0); u = w - t; out = 1 + a.b;
